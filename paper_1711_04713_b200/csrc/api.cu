@@ -127,16 +127,21 @@ static int dispatch(const GemmProblem& g, int32_t algo) {
     if (!aligned16(g.workspace)) return ADAPTION_ERR_ALIGNMENT;
     return launch_pack_taps(g);
   }
+  // (an inner product is asked for its split-K workspace by the persistent kernel's rule, whichever
+  // kernel runs it)
+  const bool cluster = algo != ADAPTION_ALGO_DIRECT && cluster_path_preferred(g);
+  if (cluster && g.is_conv) return launch_cluster(g);
   const bool tensor_ok = tensor_path_supported(g);
-  if (algo == ADAPTION_ALGO_TENSOR && !tensor_ok) return ADAPTION_ERR_UNSUPPORTED;
+  if (algo == ADAPTION_ALGO_TENSOR && !tensor_ok && !cluster) return ADAPTION_ERR_UNSUPPORTED;
   if (algo != ADAPTION_ALGO_DIRECT && tensor_ok) {
     const size_t need = tensor_path_workspace(g);
     if (need > 0) {
       if (g.workspace == nullptr || g.workspace_bytes < need) return ADAPTION_ERR_WORKSPACE;
       if (!aligned16(g.workspace)) return ADAPTION_ERR_ALIGNMENT;
     }
-    return launch_tensor(g);
+    return cluster ? launch_cluster(g) : launch_tensor(g);
   }
+  if (cluster) return launch_cluster(g);
   return launch_direct(g);
 }
 
@@ -145,6 +150,7 @@ static int dispatch(const GemmProblem& g, int32_t algo) {
 // convolution itself needs there): only its horizontal pair maxima when the tensor-core path can
 // store those (half the bytes), else all of it; a pooling pass then writes y.
 struct ConvPoolPlan {
+  bool cluster = false;      // the cluster kernel pools in its epilogue: no temporary planes
   bool fused = false;        // the layer kernel stores horizontal maxima
   size_t conv_ws = 0;        // bytes the convolution needs at the start of the workspace
   size_t plane = 0;          // bytes of one temporary plane
@@ -159,6 +165,13 @@ static ConvPoolPlan plan_conv_pool(GemmProblem g, int32_t algo) {
   g.y.hi = planes == 2 ? reinterpret_cast<void*>(uintptr_t(256)) : nullptr;
   g.y.q16 = nullptr;
   const bool packs = algo != ADAPTION_ALGO_DIRECT && pack_taps_applicable(g);
+  g.pool2x2 = true;
+  if (algo != ADAPTION_ALGO_DIRECT && !packs && cluster_path_preferred(g)) {
+    pl.cluster = true;
+    pl.total = 256;          // never touched; the call always takes a workspace
+    return pl;
+  }
+  g.pool2x2 = false;
   if (algo != ADAPTION_ALGO_DIRECT) {
     if (packs) {
       pl.conv_ws = pack_taps_workspace(g);
@@ -263,6 +276,7 @@ size_t adaption_lp_conv_workspace_bytes(const adaption_conv_shape* h_shape, adap
                          nullptr, g) != ADAPTION_OK)
     return 0;
   if (pack_taps_applicable(g)) return pack_taps_workspace(g);
+  if (cluster_path_preferred(g)) return 0;
   return tensor_path_supported(g) ? tensor_path_workspace(g) : 0;
 }
 
@@ -322,6 +336,10 @@ int adaption_lp_conv_pool_fwd(const adaption_conv_shape* h_shape, adaption_qtens
   const ConvPoolPlan pl = plan_conv_pool(g, algo);
   if (d_workspace == nullptr || workspace_bytes < pl.total) return ADAPTION_ERR_WORKSPACE;
   if (!aligned16(d_workspace)) return ADAPTION_ERR_ALIGNMENT;
+  if (pl.cluster) {          // one kernel does both phases
+    g.pool2x2 = true;
+    return (phases & ADAPTION_PHASE_CONV) ? launch_cluster(g) : ADAPTION_OK;
+  }
   // temporary planes for the convolution's own (or half-pooled) output
   uint8_t* ws = static_cast<uint8_t*>(d_workspace);
   adaption_qtensor t = y;
