@@ -57,7 +57,7 @@ EXPORTS = [
     "adaption_quantize_stochastic", "adaption_bit_histogram", "adaption_width_histogram",
     "adaption_choose_frac_bits_from_hist", "adaption_choose_frac_bits_from_widths",
     "adaption_lp_act_stochastic", "adaption_lp_conv_pool_workspace_bytes", "adaption_lp_conv_pool_fwd",
-    "adaption_quantize_batch", "adaption_debug_set", "adaption_lp_conv_fwd_stochastic",
+    "adaption_quantize_batch", "adaption_quantize_batch_stochastic", "adaption_debug_set", "adaption_lp_conv_fwd_stochastic",
     "adaption_lp_ip_fwd_stochastic",
 ]
 HIST_BINS = 17
@@ -91,6 +91,7 @@ def load(path: str | None = None):
     lib.adaption_lp_conv_fwd.argtypes = [C.POINTER(adaption_conv_shape), adaption_qtensor, adaption_qtensor,
                                          P, I32, I32, I32, I32, adaption_qtensor, P, P, SZ, P]
     lib.adaption_quantize_batch.argtypes = [C.POINTER(adaption_quantize_item), I32, P]
+    lib.adaption_quantize_batch_stochastic.argtypes = [C.POINTER(adaption_quantize_item), C.POINTER(C.c_uint64), I32, P]
     lib.adaption_lp_conv_fwd_stochastic.argtypes = [C.POINTER(adaption_conv_shape), adaption_qtensor,
                                                     adaption_qtensor, P, I32, I32, I32, adaption_qtensor,
                                                     C.c_uint64, P, P, SZ, P]
@@ -245,6 +246,13 @@ def adaption_quantize_batch(items, n_items: int | None = None):
     """``items``: a ctypes array from quantize_items() (the tensors it names must stay alive)."""
     n = len(items) if n_items is None else n_items
     _check(load().adaption_quantize_batch(items, n, _stream()), "adaption_quantize_batch")
+
+
+def adaption_quantize_batch_stochastic(items, seeds):
+    """``items`` as for adaption_quantize_batch, one seed per item."""
+    arr = (C.c_uint64 * len(items))(*[int(v) & 0xFFFFFFFFFFFFFFFF for v in seeds])
+    _check(load().adaption_quantize_batch_stochastic(items, arr, len(items), _stream()),
+           "adaption_quantize_batch_stochastic")
 
 
 def adaption_quantize_stochastic(x: torch.Tensor, outer: int, inner: int, out: QTensor, seed: int,

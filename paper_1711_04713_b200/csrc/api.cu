@@ -22,6 +22,7 @@ int maxpool_impl(const adaption_qtensor&, int32_t, int32_t, int32_t, int32_t, co
 
 int quantize_stochastic_impl(const float*, size_t, size_t, const adaption_qtensor&, const adaption_qfmt*, int32_t,
                              uint64_t, adaption_stats*, cudaStream_t);
+int quantize_batch_stochastic_impl(const adaption_quantize_item*, const uint64_t*, int32_t, cudaStream_t);
 int requant_stochastic_impl(const adaption_qtensor&, size_t, size_t, int32_t, const adaption_qtensor&,
                             const adaption_qfmt*, uint64_t, adaption_stats*, cudaStream_t);
 int bit_histogram_impl(const float*, size_t, uint64_t*, cudaStream_t);
@@ -208,6 +209,11 @@ int adaption_quantize(const float* d_x, size_t outer, size_t inner, adaption_qte
 
 int adaption_quantize_batch(const adaption_quantize_item* h_items, int32_t n_items, void* stream) {
   return quantize_batch_impl(h_items, n_items, reinterpret_cast<cudaStream_t>(stream));
+}
+
+int adaption_quantize_batch_stochastic(const adaption_quantize_item* h_items, const uint64_t* h_seeds, int32_t n_items,
+                                       void* stream) {
+  return quantize_batch_stochastic_impl(h_items, h_seeds, n_items, reinterpret_cast<cudaStream_t>(stream));
 }
 
 int adaption_quantize_stochastic(const float* d_x, size_t outer, size_t inner, adaption_qtensor out,

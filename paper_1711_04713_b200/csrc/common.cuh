@@ -45,8 +45,8 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
       k0 += 0x9E3779B9u;
       k1 += 0xBB67AE85u;
     }
-    const uint32_t hi0 = __umulhi(0xD2511F53u, c0), lo0 = 0xD2511F53u * c0;
-    const uint32_t hi1 = __umulhi(0xCD9E8D57u, c2), lo1 = 0xCD9E8D57u * c2;
+    const uint64_t p0 = (uint64_t)0xD2511F53u * c0, p1 = (uint64_t)0xCD9E8D57u * c2;
+    const uint32_t hi0 = (uint32_t)(p0 >> 32), lo0 = (uint32_t)p0, hi1 = (uint32_t)(p1 >> 32), lo1 = (uint32_t)p1;
     const uint32_t n0 = hi1 ^ c1 ^ k0, n2 = hi0 ^ c3 ^ k1;
     c0 = n0; c1 = lo1; c2 = n2; c3 = lo0;
   }
@@ -136,6 +136,25 @@ __device__ __forceinline__ void flush_counts_warp(const Counts& c, adaption_stat
     if (z) atomicAdd((unsigned long long*)&stats->zeros, (unsigned long long)z);
     if (p) atomicAdd((unsigned long long*)&stats->sat_pos, (unsigned long long)p);
     if (n) atomicAdd((unsigned long long*)&stats->sat_neg, (unsigned long long)n);
+  }
+}
+
+// One atomic per block and counter; every thread of the block must call, once.
+__device__ __forceinline__ void flush_counts_block(const Counts& c, adaption_stats* stats) {
+  __shared__ uint32_t sums[3];
+  if (threadIdx.x < 3) sums[threadIdx.x] = 0u;
+  __syncthreads();
+  const uint32_t z = warp_sum(c.zeros), p = warp_sum(c.sat_pos), n = warp_sum(c.sat_neg);
+  if ((threadIdx.x & 31) == 0) {
+    if (z) atomicAdd(&sums[0], z);
+    if (p) atomicAdd(&sums[1], p);
+    if (n) atomicAdd(&sums[2], n);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (sums[0]) atomicAdd((unsigned long long*)&stats->zeros, (unsigned long long)sums[0]);
+    if (sums[1]) atomicAdd((unsigned long long*)&stats->sat_pos, (unsigned long long)sums[1]);
+    if (sums[2]) atomicAdd((unsigned long long*)&stats->sat_neg, (unsigned long long)sums[2]);
   }
 }
 

@@ -1,5 +1,4 @@
-// HBM-bound kernels: dynamic-range measurement, the fp32 -> fixed-point quantizer (LPAct with an
-// fp32 input is the same kernel with the ReLU flag), fixed-point format conversion, 2x2 max-pool.
+// HBM-bound kernels: dynamic-range measurement, fixed-point format conversion, 2x2 max-pool.
 // All of them are coalesced streaming kernels sized to a multiple of the SM count.
 #include <atomic>
 
@@ -85,62 +84,7 @@ __global__ void choose_fmt_kernel(const float* __restrict__ d_max_abs, int32_t n
   d_fmt->frac_bits = n_bits - 1 - m;
 }
 
-// ------------------------------------------------------------------------------------------
-// Quantizer (paper Sec. 2): q = saturate(round_half_away(x * 2^f)).  x * 2^f is exact in fp32;
-// the tie rule is applied on the exact fractional part (trunc + exact remainder), never on a
-// rounded sum.
-// ------------------------------------------------------------------------------------------
-// `scale2` is 2^(f+1): z = trunc(2 * x * 2^f) is taken with the saturating float->int conversion
-// (NaN -> 0, +-Inf and anything beyond int32 -> INT_MAX / INT_MIN), and the nearest integer with
-// ties away from zero is sign(z) * ((|z| + 1) >> 1): for 2y = n + e, 0 <= e < 1,
-// floor(y + 1/2) = floor((n + 1) / 2 + e / 2) = (n + 1) >> 1 because (n + 1) / 2 is an integer or a
-// half-integer and e / 2 < 1/2.  Only integer work follows the one conversion.
-__device__ __forceinline__ int32_t quantize_f32(float x, float scale2, int relu, int32_t qmin,
-                                                int32_t qmax, bool counted, Counts& c) {
-  int32_t z = __float2int_rz(x * scale2);
-  if (relu) z = max(z, 0);
-  const uint32_t a = (uint32_t)(z < 0 ? -(long long)z : (long long)z);   // |z| up to 2^31
-  const int32_t mag = (int32_t)((a + 1u) >> 1);                          // <= 2^30
-  const int32_t r = z < 0 ? -mag : mag;
-  const int32_t q = min(max(r, qmin), qmax);
-  c.sat_pos += (counted && r > qmax);
-  c.sat_neg += (counted && r < qmin);
-  c.zeros += (counted && q == 0);
-  return q;
-}
-
-// Four elements at once for the dense kernel; the counters are derived per group (clipping is
-// detected by OR-ing r ^ q and only then counted exactly).
-__device__ __forceinline__ void quantize_f32x4(const float4 v, float scale2, int relu, int32_t qmin,
-                                               int32_t qmax, Counts& c, int32_t (&q)[4]) {
-  const float x[4] = {v.x, v.y, v.z, v.w};
-  int32_t r[4], clipped = 0, nonzero = 0;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    int32_t z = __float2int_rz(x[k] * scale2);
-    if (relu) z = max(z, 0);
-    const uint32_t a = (uint32_t)(z < 0 ? -(long long)z : (long long)z);
-    const int32_t mag = (int32_t)((a + 1u) >> 1);
-    r[k] = z < 0 ? -mag : mag;
-    q[k] = min(max(r[k], qmin), qmax);
-    clipped |= r[k] ^ q[k];
-    nonzero += min(abs(q[k]), 1);
-  }
-  c.zeros += 4 - nonzero;
-  if (clipped != 0) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      c.sat_pos += (r[k] > qmax);
-      c.sat_neg += (r[k] < qmin);
-    }
-  }
-}
-
-// 2^(frac_bits + 1), the scale quantize_f32 expects
-__device__ __forceinline__ float scale_of(int32_t frac_bits) {
-  return __int_as_float((128 + frac_bits) << 23);
-}
-
+// Stored planes as words of four elements.
 struct QuantOut {
   uint32_t* hi;   // words of 4 bytes
   uint32_t* lo;
@@ -164,92 +108,6 @@ __device__ __forceinline__ void store4(const QuantOut& o, size_t word, int32_t q
     v.y = (uint32_t)(q2 & 0xffff) | ((uint32_t)(q3 & 0xffff) << 16);
     o.q16[word] = v;
   }
-}
-
-// Dense rows (inner == c_stride): the tensor is one flat array; one float4 in, one 4-byte word
-// per plane out, four independent groups in flight per thread.
-__global__ void __launch_bounds__(256) quantize_flat_kernel(const float4* __restrict__ x, size_t n4,
-                                                            QuantOut out, int32_t frac_bits,
-                                                            const adaption_qfmt* __restrict__ d_fmt,
-                                                            int relu, int32_t qmin, int32_t qmax,
-                                                            adaption_stats* __restrict__ stats) {
-  pdl_prologue();
-  if (d_fmt != nullptr) frac_bits = d_fmt->frac_bits;
-  const float scale = scale_of(frac_bits);
-  Counts c;
-  const size_t nthreads = (size_t)gridDim.x * blockDim.x;
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (; i + 3 * nthreads < n4; i += 4 * nthreads) {
-    float4 v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = __ldcs(x + i + u * nthreads);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      int32_t q[4];
-      quantize_f32x4(v[u], scale, relu, qmin, qmax, c, q);
-      store4(out, i + u * nthreads, q[0], q[1], q[2], q[3]);
-    }
-  }
-  for (; i < n4; i += nthreads) {
-    int32_t q[4];
-    quantize_f32x4(__ldcs(x + i), scale, relu, qmin, qmax, c, q);
-    store4(out, i, q[0], q[1], q[2], q[3]);
-  }
-  if (stats != nullptr) flush_counts_warp(c, stats);
-}
-
-// Rows with channel padding (inner < c_stride) or unaligned input: one thread per group of sixteen
-// stored channels (one 16-byte vector per plane); padding channels receive zeros and are not
-// counted.
-__global__ void __launch_bounds__(256) quantize_rows_kernel(const float* __restrict__ x, size_t outer,
-                                                            int64_t inner, int64_t c_stride,
-                                                            QuantOut out, int32_t frac_bits,
-                                                            const adaption_qfmt* __restrict__ d_fmt,
-                                                            int relu, int32_t qmin, int32_t qmax,
-                                                            adaption_stats* __restrict__ stats) {
-  pdl_prologue();
-  if (d_fmt != nullptr) frac_bits = d_fmt->frac_bits;
-  const float scale = scale_of(frac_bits);
-  Counts c;
-  const int64_t groups_per_row = c_stride / 16;
-  const size_t total = outer * (size_t)groups_per_row;
-  const size_t nthreads = (size_t)gridDim.x * blockDim.x;
-  const bool small = total <= 0xffffffffull;      // 32-bit division whenever the group index fits
-  for (size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += nthreads) {
-    const size_t row = small ? (size_t)((uint32_t)g / (uint32_t)groups_per_row) : g / groups_per_row;
-    const int64_t c0 = (int64_t)(g - row * groups_per_row) * 16;
-    const float* __restrict__ src = x + row * (size_t)inner + c0;
-    const int nreal = (int)min((int64_t)16, max((int64_t)0, inner - c0));
-    uint32_t lo[4], hi[4], h16[8];
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      if (4 * w >= nreal) {               // only padding from here on: zeros, nothing to compute
-        lo[w] = hi[w] = h16[2 * w] = h16[2 * w + 1] = 0u;
-        continue;
-      }
-      int32_t q[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const bool real = 4 * w + u < nreal;
-        const float v = real ? __ldg(src + 4 * w + u) : 0.0f;
-        q[u] = quantize_f32(v, scale, relu, qmin, qmax, real, c);
-      }
-      lo[w] = (uint32_t)(q[0] & 255) | ((uint32_t)(q[1] & 255) << 8) | ((uint32_t)(q[2] & 255) << 16) |
-              ((uint32_t)(q[3] & 255) << 24);
-      hi[w] = (uint32_t)((q[0] >> 8) & 255) | ((uint32_t)((q[1] >> 8) & 255) << 8) |
-              ((uint32_t)((q[2] >> 8) & 255) << 16) | ((uint32_t)((q[3] >> 8) & 255) << 24);
-      h16[2 * w] = (uint32_t)(q[0] & 0xffff) | ((uint32_t)(q[1] & 0xffff) << 16);
-      h16[2 * w + 1] = (uint32_t)(q[2] & 0xffff) | ((uint32_t)(q[3] & 0xffff) << 16);
-    }
-    reinterpret_cast<uint4*>(out.lo)[g] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-    if (out.planes == 2) reinterpret_cast<uint4*>(out.hi)[g] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-    if (out.q16 != nullptr) {
-      uint4* d = reinterpret_cast<uint4*>(out.q16) + 2 * g;
-      d[0] = make_uint4(h16[0], h16[1], h16[2], h16[3]);
-      d[1] = make_uint4(h16[4], h16[5], h16[6], h16[7]);
-    }
-  }
-  if (stats != nullptr) flush_counts_warp(c, stats);
 }
 
 // Requantization of a stored value (|v| <= 2^15, |shift| <= 15): everything fits in 32 bits.
@@ -510,155 +368,6 @@ static QuantOut quant_out_of(const adaption_qtensor& t) {
   o.lo = reinterpret_cast<uint32_t*>(t.lo);
   o.q16 = reinterpret_cast<uint2*>(t.q16);
   return o;
-}
-
-int quantize_impl(const float* d_x, size_t outer, size_t inner, const adaption_qtensor& out,
-                  const adaption_qfmt* d_fmt, int32_t relu, int32_t rounding, adaption_stats* d_stats,
-                  cudaStream_t stream) {
-  if (rounding == ADAPTION_ROUND_STOCHASTIC) return ADAPTION_ERR_UNSUPPORTED;
-  if (rounding != ADAPTION_ROUND_DETERMINISTIC) return ADAPTION_ERR_INVALID_ARG;
-  int rc = check_qtensor_out(out, (int64_t)inner);
-  if (rc != ADAPTION_OK) return rc;
-  if (outer == 0 || inner == 0) return ADAPTION_OK;
-  if (d_x == nullptr) return ADAPTION_ERR_INVALID_ARG;
-  if ((reinterpret_cast<uintptr_t>(d_x) & 3u) != 0) return ADAPTION_ERR_ALIGNMENT;
-  const int32_t qmin = -(1 << (out.fmt.n_bits - 1)), qmax = (1 << (out.fmt.n_bits - 1)) - 1;
-  const QuantOut qo = quant_out_of(out);
-  if ((int64_t)inner == out.c_stride && aligned16(d_x)) {
-    const size_t n4 = outer * inner / 4;
-    const int grid = stream_grid((n4 + 3) / 4, 256, 8);
-    launch_after_predecessor(quantize_flat_kernel, dim3(grid), dim3(256), stream, reinterpret_cast<const float4*>(d_x), n4, qo,
-                                                   out.fmt.frac_bits, d_fmt, relu, qmin, qmax, d_stats);
-  } else {
-    const size_t groups = outer * (size_t)(out.c_stride / 16);
-    const int grid = stream_grid(groups, 256, 8);
-    launch_after_predecessor(quantize_rows_kernel, dim3(grid), dim3(256), stream, d_x, outer, (int64_t)inner, out.c_stride, qo,
-                                                   out.fmt.frac_bits, d_fmt, relu, qmin, qmax, d_stats);
-  }
-  return cuda_status(cudaGetLastError());
-}
-
-// ------------------------------------------------------------------------------------------
-// Several dense tensors in one launch (the weights and biases of a whole network, quantized anew
-// in every forward pass): the tensors are cut into chunks of 1024 float4, numbered across the
-// batch; a block walks the chunks with the grid's stride and looks up the tensor a chunk belongs
-// to in the launch parameters (first_chunk is the running sum).  Per element the work is that of
-// quantize_flat_kernel.
-constexpr int kBatchItems = 40;
-constexpr int kBatchChunk4 = 1024;      // float4 per chunk: four per thread of a 256-thread block
-
-struct BatchItem {
-  const float4* x;
-  uint32_t* hi;
-  uint32_t* lo;
-  uint2* q16;
-  const adaption_qfmt* d_fmt;
-  unsigned long long n4;            // float4 in this tensor
-  unsigned long long first_chunk;   // chunks of the tensors before it
-  int32_t frac_bits, qmin, qmax, planes;
-};
-
-struct BatchArgs {
-  BatchItem item[kBatchItems];
-  unsigned long long total_chunks;
-  int32_t n;
-};
-
-__global__ void __launch_bounds__(256) quantize_batch_kernel(const __grid_constant__ BatchArgs a) {
-  pdl_prologue();
-  Counts unused;
-  // Chunks come in increasing order, so the search for a chunk's tensor only moves forward; the
-  // tensor's fields are copied to registers when it changes, not once per chunk (they sit in an
-  // array of the kernel's parameters, which a varying index can only reach through loads).
-  int t = -1;
-  const float4* x = nullptr;
-  QuantOut o{};
-  unsigned long long n4 = 0, first = 0;
-  float scale = 1.0f;
-  int32_t qmin = 0, qmax = 0;
-  for (unsigned long long chunk = blockIdx.x; chunk < a.total_chunks; chunk += gridDim.x) {
-    int nt = t < 0 ? 0 : t;
-    while (nt + 1 < a.n && a.item[nt + 1].first_chunk <= chunk) ++nt;
-    if (nt != t) {
-      t = nt;
-      const BatchItem& it = a.item[t];
-      x = it.x;
-      o.hi = it.hi; o.lo = it.lo; o.q16 = it.q16; o.planes = it.planes;
-      n4 = it.n4;
-      first = it.first_chunk;
-      scale = scale_of(it.d_fmt != nullptr ? it.d_fmt->frac_bits : it.frac_bits);
-      qmin = it.qmin;
-      qmax = it.qmax;
-    }
-    const unsigned long long base = (chunk - first) * kBatchChunk4 + threadIdx.x;
-    float4 v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const unsigned long long i = base + u * 256;
-      v[u] = i < n4 ? __ldcs(x + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const unsigned long long i = base + u * 256;
-      if (i < n4) {
-        int32_t q[4];
-        quantize_f32x4(v[u], scale, 0, qmin, qmax, unused, q);
-        store4(o, (size_t)i, q[0], q[1], q[2], q[3]);
-      }
-    }
-  }
-}
-
-int quantize_batch_impl(const adaption_quantize_item* h_items, int32_t n_items, cudaStream_t stream) {
-  if (n_items < 0 || (n_items > 0 && h_items == nullptr)) return ADAPTION_ERR_INVALID_ARG;
-  // validate everything before the first launch
-  for (int32_t k = 0; k < n_items; ++k) {
-    const adaption_quantize_item& h = h_items[k];
-    if (h.outer < 0 || h.inner < 0) return ADAPTION_ERR_INVALID_ARG;
-    int rc = check_qtensor_out(h.q, h.inner);
-    if (rc != ADAPTION_OK) return rc;
-    if (h.outer == 0 || h.inner == 0) continue;
-    if (h.d_x == nullptr) return ADAPTION_ERR_INVALID_ARG;
-    if ((reinterpret_cast<uintptr_t>(h.d_x) & 3u) != 0) return ADAPTION_ERR_ALIGNMENT;
-  }
-  BatchArgs args;
-  args.n = 0;
-  args.total_chunks = 0;
-  auto flush = [&]() -> int {
-    if (args.n == 0) return ADAPTION_OK;
-    const int grid = stream_grid((size_t)args.total_chunks, 1, 8);
-    launch_after_predecessor(quantize_batch_kernel, dim3(grid), dim3(256), stream, args);
-    args.n = 0;
-    args.total_chunks = 0;
-    return cuda_status(cudaGetLastError());
-  };
-  for (int32_t k = 0; k < n_items; ++k) {
-    const adaption_quantize_item& h = h_items[k];
-    if (h.outer == 0 || h.inner == 0) continue;
-    const bool dense = h.inner == h.q.c_stride && aligned16(h.d_x);
-    if (!dense) {               // padded rows: the row kernel, on its own
-      int rc = quantize_impl(h.d_x, (size_t)h.outer, (size_t)h.inner, h.q, h.d_fmt, 0,
-                             ADAPTION_ROUND_DETERMINISTIC, nullptr, stream);
-      if (rc != ADAPTION_OK) return rc;
-      continue;
-    }
-    BatchItem& it = args.item[args.n];
-    const QuantOut qo = quant_out_of(h.q);
-    it.x = reinterpret_cast<const float4*>(h.d_x);
-    it.hi = qo.hi; it.lo = qo.lo; it.q16 = qo.q16; it.planes = qo.planes;
-    it.d_fmt = h.d_fmt;
-    it.n4 = (unsigned long long)h.outer * (unsigned long long)h.inner / 4;   // c_stride is a multiple of 16
-    it.first_chunk = args.total_chunks;
-    it.frac_bits = h.q.fmt.frac_bits;
-    it.qmin = -(1 << (h.q.fmt.n_bits - 1));
-    it.qmax = (1 << (h.q.fmt.n_bits - 1)) - 1;
-    args.total_chunks += (it.n4 + kBatchChunk4 - 1) / kBatchChunk4;
-    if (++args.n == kBatchItems) {
-      int rc = flush();
-      if (rc != ADAPTION_OK) return rc;
-    }
-  }
-  return flush();
 }
 
 int requant_impl(const adaption_qtensor& in, size_t outer, size_t inner, int32_t relu,

@@ -230,7 +230,7 @@ class LPNetwork:
     def _quantize_params_stochastic(self, measure: bool, threshold: float):
         """Weights and biases with rounding_scheme STOCHASTIC: formats as in the deterministic case
         (from max|w| or the thresholded allocation), values by the stochastic quantizer."""
-        li = 0
+        entries, seeds = [], []
         for L in self.layers:
             if L.type not in ("conv", "ip"):
                 continue
@@ -240,11 +240,11 @@ class LPNetwork:
                 L.w_max_dev.zero_()
                 B.adaption_measure_range(L.w_f32, self.n_bits, L.w_max_dev, L.w_fmt_dev)
                 L.w.frac_bits = L.b.frac_bits = int(L.w_fmt_dev.cpu()[1])
-            sw, sb, _ = rounding_seeds(self.rounding_seed, li)
-            B.adaption_quantize_stochastic(L.w_f32, L.w.outer, L.w.inner, L.w, sw)
-            B.adaption_quantize_stochastic(L.b_f32, 1, L.K, L.b, sb)
-            L.extra["li"] = li
-            li += 1
+            L.extra["li"] = len(seeds) // 2
+            seeds += rounding_seeds(self.rounding_seed, L.extra["li"])[:2]
+            entries.append((L.w_f32, L.w.outer, L.w.inner, L.w, None))
+            entries.append((L.b_f32, 1, L.K, L.b, None))
+        B.adaption_quantize_batch_stochastic(B.quantize_items(entries), seeds)
 
     @staticmethod
     def helper_launches(L: _Layer) -> int:
@@ -255,8 +255,8 @@ class LPNetwork:
         return 2 if L.type == "conv" and L.C <= 4 else 1
 
     def param_quantize_launches(self) -> int:
-        """Kernel launches of one quantize_params(measure=False): dense tensors share one launch per
-        40, a tensor with padded rows takes one of its own."""
+        """Kernel launches of one quantize_params(measure=False): 40 dense tensors share a launch, and so do
+        40 with padded rows."""
         dense = padded = 0
         for L in self.layers:
             if L.type in ("conv", "ip"):
@@ -265,7 +265,7 @@ class LPNetwork:
                         dense += 1
                     else:
                         padded += 1
-        return (dense + 39) // 40 + padded
+        return (dense + 39) // 40 + (padded + 39) // 40
 
     # ------------------------------------------------------------------ one layer
     def _workspace(self, L: _Layer, x: B.QTensor) -> torch.Tensor | None:

@@ -1,0 +1,84 @@
+"""GPU parity of the quantizer where a tensor is cut into chunks of padded rows or shares a launch with
+others: chunk edges inside a block of four elements, rows longer than a chunk, unaligned inputs, special
+values at the edges of the range; deterministic and stochastic rounding."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import reference as orc
+from oracle import stochastic as orc_st
+from paper_1711_04713_b200 import binding as B
+from tests.util import Guards, dev, from_qtensor, q16_of, stats_tuple
+
+pytestmark = pytest.mark.gpu
+
+# outer, inner, pitch: one element per row; odd rows whose chunks start anywhere in a block of four;
+# exactly one chunk, one row more; a pitch of a whole chunk; rows of several segments
+SHAPES = [(700, 1, 16), (513, 3, 16), (1025, 7, 32), (64, 50, 64), (65, 50, 64), (3, 4081, 4096), (2, 4097, 4112),
+          (3, 9001, 9008), (5, 17, 12304), (300, 16, 16)]
+
+
+def _values(rng, shape, n_bits, f):
+    x = (rng.standard_normal(shape) * 2.0 ** (n_bits - 1 - f) * 0.6).astype(np.float32)
+    grid = (rng.integers(-(1 << n_bits), 1 << n_bits, shape) / 2).astype(np.float32) * np.float32(2.0 ** -f)
+    x = np.where(rng.random(shape) < 0.2, grid, x).astype(np.float32)         # grid values and ties
+    special = np.array([np.nan, np.inf, -np.inf, -0.0, 1e-45, -1e-45, 3e38, -2.0 ** -60], np.float32)
+    k = min(x.size, special.size)
+    x.ravel()[rng.choice(x.size, k, replace=False)] = special[:k]
+    return x
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("n_bits,f", [(16, 12), (8, 5)])
+@pytest.mark.parametrize("offset", [0, 3])
+@pytest.mark.parametrize("relu", [False, True])
+def test_rows(shape, n_bits, f, offset, relu):
+    outer, inner, pitch = shape
+    rng = np.random.default_rng(outer + inner + offset)
+    x = _values(rng, (outer, inner), n_bits, f)
+    src = torch.zeros(outer * inner + offset, device="cuda")
+    src[offset:] = dev(x.ravel())
+    xr = np.where(x > 0, x, 0).astype(np.float32) if relu else x
+    for seed in (None, 0x1234567890 + outer):
+        guards = Guards()
+        y = guards.qtensor(outer, inner, n_bits, f, pitch, with_q16=True)
+        st = B.new_stats()
+        if seed is None:
+            B.adaption_lp_act(src[offset:], None, outer, inner, relu, y, None, B.ROUND_DETERMINISTIC, st)
+            want, cnt = orc.quantize(xr, n_bits, f)
+            cnt = (cnt.zeros, cnt.sat_pos, cnt.sat_neg)
+        else:
+            B.adaption_quantize_stochastic(src[offset:], outer, inner, y, seed, relu, None, st)
+            want, cnt = orc_st.quantize_stochastic(x, n_bits, f, seed, relu)
+        assert np.array_equal(from_qtensor(y), want)
+        assert np.array_equal(q16_of(y), want)
+        assert y.padding_is_zero()
+        assert stats_tuple(st) == tuple(cnt)
+        guards.check()
+
+
+@pytest.mark.parametrize("stochastic", [False, True])
+def test_many_tensors_in_one_launch(stochastic):
+    """More tensors than one launch takes, dense and padded in turn, small and large, formats on host and device."""
+    rng = np.random.default_rng(3)
+    shapes = [(1 + (7 * k) % 90, [16, 50, 3, 128, 1][k % 5]) for k in range(45)] + [(3000, 64), (9, 5000)]
+    guards, entries, host, seeds = Guards(), [], [], []
+    for k, (outer, inner) in enumerate(shapes):
+        n = 16 if k % 3 else 8
+        f = n - 3
+        x = _values(rng, (outer, inner), n, f)
+        y = guards.qtensor(outer, inner, n, f if k % 4 else 0, None, with_q16=k % 2 == 0)
+        fmt = None if k % 4 else torch.tensor([n, f], dtype=torch.int32, device="cuda")
+        entries.append((dev(x), outer, inner, y, fmt))
+        host.append((x, n, f))
+        seeds.append(0xFFFFFFFF00000000 + 1000 * k)
+    items = B.quantize_items(entries)
+    if stochastic:
+        B.adaption_quantize_batch_stochastic(items, seeds)
+    else:
+        B.adaption_quantize_batch(items)
+    for (x, n, f), (_, _, _, y, _), seed in zip(host, entries, seeds):
+        want = orc_st.quantize_stochastic(x, n, f, seed, False)[0] if stochastic else orc.quantize(x, n, f)[0]
+        assert np.array_equal(from_qtensor(y), want)
+        assert y.padding_is_zero()
+    guards.check()
