@@ -1,13 +1,15 @@
-"""Thin ctypes binding of the C ABI in include/adaption.h (argument marshalling only).
+"""Thin binding of the C ABI in include/adaption.h (argument marshalling only).
 
 Every function here has the name of the C entry point it calls.  Device memory comes from
 torch tensors (``QTensor`` wraps the byte planes of one fixed-point tensor); all arithmetic runs
-in the CUDA library.  Importing this module never builds or falls back to anything: if the
-shared library is missing, ``load()`` raises.
+in the CUDA library.  The structures and the calls off the hot path go through ctypes, the marshalling of
+the others is native code (csrc/host_binding.cpp).  Importing this module never builds or falls back to
+anything: if a shared library is missing, ``load()`` raises.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -63,6 +65,7 @@ EXPORTS = [
 HIST_BINS = 17
 
 _lib = None
+_native = None          # csrc/host_binding.cpp, bound to the library by load()
 
 
 class AdaptionError(RuntimeError):
@@ -72,8 +75,9 @@ class AdaptionError(RuntimeError):
 
 
 def load(path: str | None = None):
-    """Load lib/libadaption.so (built in-tree by build.build_library).  Raises if it is absent."""
-    global _lib
+    """Load lib/libadaption.so (built in-tree by build.build_library) and the marshalling module beside it.
+    Raises if one is absent."""
+    global _lib, _native
     if _lib is not None:
         return _lib
     path = path or _build.LIB_PATH
@@ -127,8 +131,32 @@ def load(path: str | None = None):
         if name not in ("adaption_lp_conv_workspace_bytes", "adaption_lp_ip_workspace_bytes",
                         "adaption_lp_conv_pool_workspace_bytes", "adaption_status_string"):
             getattr(lib, name).restype = C.c_int
+    if not os.path.exists(_build.NATIVE_PATH):
+        raise RuntimeError(f"native half of the binding not built: {_build.NATIVE_PATH} is missing "
+                           "(run `python -m paper_1711_04713_b200.build`)")
+    spec = importlib.util.spec_from_file_location("_adaption_native", _build.NATIVE_PATH)
+    native = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(native)
+    native.bind(os.path.abspath(path), AdaptionError, *_stream_getters())
+    _native = native
     _lib = lib
     return lib
+
+
+def _stream_getters():
+    """(current device, raw handle of the current stream of a device)."""
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if device is None or stream is None:
+        return torch.cuda.current_device, lambda d: torch.cuda.current_stream(d).cuda_stream
+    return device, stream
+
+
+def _calls():
+    """The marshalling module, bound to the library."""
+    if _native is None:
+        load()
+    return _native
 
 
 def adaption_debug_set(name: str, value: int = 0):
@@ -223,53 +251,43 @@ def read_stats(stats: torch.Tensor) -> adaption_stats:
 def adaption_measure_range(x: torch.Tensor, n_bits: int, d_max_abs: torch.Tensor,
                            d_fmt_out: torch.Tensor | None):
     """x: fp32 CUDA tensor (contiguous); d_max_abs: 1 fp32; d_fmt_out: 2 int32 (n_bits, frac_bits)."""
-    _check(load().adaption_measure_range(_ptr(x), x.numel(), n_bits, _ptr(d_max_abs), _ptr(d_fmt_out),
-                                         _stream()), "adaption_measure_range")
+    _calls().measure_range(x, n_bits, d_max_abs, d_fmt_out)
 
 
 def adaption_quantize(x: torch.Tensor, outer: int, inner: int, out: QTensor,
                       d_fmt: torch.Tensor | None = None, rounding: int = ROUND_DETERMINISTIC,
                       d_stats: torch.Tensor | None = None):
-    _check(load().adaption_quantize(_ptr(x), outer, inner, out.c_struct(), _ptr(d_fmt), rounding,
-                                    _ptr(d_stats), _stream()), "adaption_quantize")
+    _calls().quantize(x, outer, inner, out, d_fmt, rounding, d_stats)
 
 
 def quantize_items(entries) -> "C.Array":
     """Host array of adaption_quantize_item from (x, outer, inner, out, d_fmt or None) tuples."""
     arr = (adaption_quantize_item * len(entries))()
-    for it, (x, outer, inner, out, d_fmt) in zip(arr, entries):
-        it.d_x, it.outer, it.inner, it.q, it.d_fmt = _ptr(x), outer, inner, out.c_struct(), _ptr(d_fmt)
+    _calls().fill_items(arr, entries)
     return arr
 
 
 def adaption_quantize_batch(items, n_items: int | None = None):
     """``items``: a ctypes array from quantize_items() (the tensors it names must stay alive)."""
-    n = len(items) if n_items is None else n_items
-    _check(load().adaption_quantize_batch(items, n, _stream()), "adaption_quantize_batch")
+    _calls().quantize_batch(items, len(items) if n_items is None else n_items)
 
 
 def adaption_quantize_batch_stochastic(items, seeds):
     """``items`` as for adaption_quantize_batch, one seed per item."""
     arr = (C.c_uint64 * len(items))(*[int(v) & 0xFFFFFFFFFFFFFFFF for v in seeds])
-    _check(load().adaption_quantize_batch_stochastic(items, arr, len(items), _stream()),
-           "adaption_quantize_batch_stochastic")
+    _calls().quantize_batch_stochastic(items, arr, len(items))
 
 
 def adaption_quantize_stochastic(x: torch.Tensor, outer: int, inner: int, out: QTensor, seed: int,
                                  relu: bool = False, d_fmt: torch.Tensor | None = None,
                                  d_stats: torch.Tensor | None = None):
-    _check(load().adaption_quantize_stochastic(_ptr(x), outer, inner, out.c_struct(), _ptr(d_fmt), int(relu),
-                                               seed & 0xFFFFFFFFFFFFFFFF, _ptr(d_stats), _stream()),
-           "adaption_quantize_stochastic")
+    _calls().quantize_stochastic(x, outer, inner, out, seed, relu, d_fmt, d_stats)
 
 
 def adaption_lp_act_stochastic(x_f32: torch.Tensor | None, x_q: QTensor | None, outer: int, inner: int, relu: bool,
                                out: QTensor, seed: int, d_fmt: torch.Tensor | None = None,
                                d_stats: torch.Tensor | None = None):
-    xq = None if x_q is None else C.byref(x_q.c_struct())
-    _check(load().adaption_lp_act_stochastic(_ptr(x_f32), xq, outer, inner, int(relu), out.c_struct(), _ptr(d_fmt),
-                                             seed & 0xFFFFFFFFFFFFFFFF, _ptr(d_stats), _stream()),
-           "adaption_lp_act_stochastic")
+    _calls().lp_act_stochastic(x_f32, x_q, outer, inner, relu, out, seed, d_fmt, d_stats)
 
 
 def new_hist(device="cuda") -> torch.Tensor:
@@ -278,12 +296,11 @@ def new_hist(device="cuda") -> torch.Tensor:
 
 
 def adaption_bit_histogram(x: torch.Tensor, d_hist: torch.Tensor):
-    _check(load().adaption_bit_histogram(_ptr(x), x.numel(), _ptr(d_hist), _stream()), "adaption_bit_histogram")
+    _calls().bit_histogram(x, d_hist)
 
 
 def adaption_width_histogram(x: QTensor, d_hist: torch.Tensor):
-    _check(load().adaption_width_histogram(x.c_struct(), x.outer, x.inner, _ptr(d_hist), _stream()),
-           "adaption_width_histogram")
+    _calls().width_histogram(x, d_hist)
 
 
 def adaption_choose_frac_bits_from_hist(hist, n_bits: int, threshold: float) -> int:
@@ -307,9 +324,7 @@ def adaption_choose_frac_bits_from_widths(hist, frac_bits: int, n_bits: int, thr
 def adaption_lp_act(x_f32: torch.Tensor | None, x_q: QTensor | None, outer: int, inner: int, relu: bool,
                     out: QTensor, d_fmt: torch.Tensor | None = None, rounding: int = ROUND_DETERMINISTIC,
                     d_stats: torch.Tensor | None = None):
-    xq = None if x_q is None else C.byref(x_q.c_struct())
-    _check(load().adaption_lp_act(_ptr(x_f32), xq, outer, inner, int(relu), out.c_struct(), _ptr(d_fmt),
-                                  rounding, _ptr(d_stats), _stream()), "adaption_lp_act")
+    _calls().lp_act(x_f32, x_q, outer, inner, relu, out, d_fmt, rounding, d_stats)
 
 
 def conv_shape(N, H, W, Cin, K, R, S, pad, stride) -> adaption_conv_shape:
@@ -324,31 +339,35 @@ def adaption_lp_conv_workspace_bytes(shape: adaption_conv_shape, fx: adaption_qf
 def adaption_lp_conv_fwd(shape: adaption_conv_shape, x: QTensor, w: QTensor, bias_q: torch.Tensor | None,
                          bias_frac_bits: int, relu: bool, mode: int, algo: int, y: QTensor | None,
                          d_stats: torch.Tensor, workspace: torch.Tensor | None = None):
-    ys = y.c_struct() if y is not None else adaption_qtensor()
-    wsb = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load().adaption_lp_conv_fwd(C.byref(shape), x.c_struct(), w.c_struct(), _ptr(bias_q),
-                                       bias_frac_bits, int(relu), mode, algo, ys, _ptr(d_stats),
-                                       _ptr(workspace), wsb, _stream()), "adaption_lp_conv_fwd")
+    _calls().conv_fwd(shape, x, w, bias_q, bias_frac_bits, relu, mode, algo, y, d_stats, workspace)
 
 
 def adaption_lp_conv_fwd_stochastic(shape: adaption_conv_shape, x: QTensor, w: QTensor, bias_q: torch.Tensor | None,
                                     bias_frac_bits: int, relu: bool, algo: int, y: QTensor, seed: int,
                                     d_stats: torch.Tensor, workspace: torch.Tensor | None = None):
-    wsb = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load().adaption_lp_conv_fwd_stochastic(C.byref(shape), x.c_struct(), w.c_struct(), _ptr(bias_q),
-                                                  bias_frac_bits, int(relu), algo, y.c_struct(),
-                                                  seed & 0xFFFFFFFFFFFFFFFF, _ptr(d_stats), _ptr(workspace), wsb,
-                                                  _stream()), "adaption_lp_conv_fwd_stochastic")
+    _calls().conv_fwd_stochastic(shape, x, w, bias_q, bias_frac_bits, relu, algo, y, seed, d_stats, workspace)
 
 
 def adaption_lp_ip_fwd_stochastic(B: int, K: int, O: int, x: QTensor, w: QTensor, bias_q: torch.Tensor | None,
                                   bias_frac_bits: int, relu: bool, algo: int, y: QTensor, seed: int,
                                   d_stats: torch.Tensor, workspace: torch.Tensor | None = None):
-    wsb = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load().adaption_lp_ip_fwd_stochastic(B, K, O, x.c_struct(), w.c_struct(), _ptr(bias_q), bias_frac_bits,
-                                                int(relu), algo, y.c_struct(), seed & 0xFFFFFFFFFFFFFFFF,
-                                                _ptr(d_stats), _ptr(workspace), wsb, _stream()),
-           "adaption_lp_ip_fwd_stochastic")
+    _calls().ip_fwd_stochastic(B, K, O, x, w, bias_q, bias_frac_bits, relu, algo, y, seed, d_stats, workspace)
+
+
+def conv_workspace_bytes(shape: adaption_conv_shape, x: QTensor, w: QTensor, algo: int = ALGO_AUTO) -> int:
+    """adaption_lp_conv_workspace_bytes for operands at hand."""
+    return _calls().conv_workspace(shape, x, w, algo)
+
+
+def conv_pool_workspace_bytes(shape: adaption_conv_shape, x: QTensor, w: QTensor, y: QTensor,
+                              algo: int = ALGO_AUTO) -> int:
+    """adaption_lp_conv_pool_workspace_bytes for operands at hand."""
+    return _calls().conv_pool_workspace(shape, x, w, y, algo)
+
+
+def ip_workspace_bytes(B: int, K: int, O: int, x: QTensor, w: QTensor, algo: int = ALGO_AUTO) -> int:
+    """adaption_lp_ip_workspace_bytes for operands at hand."""
+    return _calls().ip_workspace(B, K, O, x, w, algo)
 
 
 def adaption_lp_conv_pool_workspace_bytes(shape: adaption_conv_shape, fx: adaption_qfmt, fw: adaption_qfmt,
@@ -360,10 +379,7 @@ def adaption_lp_conv_pool_workspace_bytes(shape: adaption_conv_shape, fx: adapti
 def adaption_lp_conv_pool_fwd(shape: adaption_conv_shape, x: QTensor, w: QTensor, bias_q: torch.Tensor | None,
                               bias_frac_bits: int, relu: bool, algo: int, y: QTensor, d_stats: torch.Tensor,
                               workspace: torch.Tensor | None, phases: int = 3):
-    wsb = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load().adaption_lp_conv_pool_fwd(C.byref(shape), x.c_struct(), w.c_struct(), _ptr(bias_q), bias_frac_bits,
-                                            int(relu), algo, phases, y.c_struct(), _ptr(d_stats), _ptr(workspace),
-                                            wsb, _stream()), "adaption_lp_conv_pool_fwd")
+    _calls().conv_pool_fwd(shape, x, w, bias_q, bias_frac_bits, relu, algo, y, d_stats, workspace, phases)
 
 
 def adaption_lp_ip_workspace_bytes(B: int, K: int, O: int, fx: adaption_qfmt, fw: adaption_qfmt,
@@ -374,11 +390,7 @@ def adaption_lp_ip_workspace_bytes(B: int, K: int, O: int, fx: adaption_qfmt, fw
 def adaption_lp_ip_fwd(B: int, K: int, O: int, x: QTensor, w: QTensor, bias_q: torch.Tensor | None,
                        bias_frac_bits: int, relu: bool, mode: int, algo: int, y: QTensor | None,
                        d_stats: torch.Tensor, workspace: torch.Tensor | None = None):
-    ys = y.c_struct() if y is not None else adaption_qtensor()
-    wsb = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load().adaption_lp_ip_fwd(B, K, O, x.c_struct(), w.c_struct(), _ptr(bias_q), bias_frac_bits,
-                                     int(relu), mode, algo, ys, _ptr(d_stats), _ptr(workspace), wsb,
-                                     _stream()), "adaption_lp_ip_fwd")
+    _calls().ip_fwd(B, K, O, x, w, bias_q, bias_frac_bits, relu, mode, algo, y, d_stats, workspace)
 
 
 STATIC_WORKSPACE_BYTES = 4 << 20
@@ -390,15 +402,11 @@ def adaption_lp_ip_fwd_static_ws(B: int, K: int, O: int, x: QTensor, w: QTensor,
     """adaption_lp_ip_fwd without a workspace argument: the library's built-in scratch array is used.
     For callers that must not allocate; shapes whose workspace exceeds STATIC_WORKSPACE_BYTES raise
     AdaptionError(ERR_WORKSPACE).  Calls that may overlap on the GPU must be ordered by the caller."""
-    ys = y.c_struct() if y is not None else adaption_qtensor()
-    _check(load().adaption_lp_ip_fwd_static_ws(B, K, O, x.c_struct(), w.c_struct(), _ptr(bias_q),
-                                               bias_frac_bits, int(relu), mode, algo, ys, _ptr(d_stats),
-                                               _stream()), "adaption_lp_ip_fwd_static_ws")
+    _calls().ip_fwd_static_ws(B, K, O, x, w, bias_q, bias_frac_bits, relu, mode, algo, y, d_stats)
 
 
 def adaption_maxpool2x2(x: QTensor, N: int, H: int, W: int, Cc: int, y: QTensor):
-    _check(load().adaption_maxpool2x2(x.c_struct(), N, H, W, Cc, y.c_struct(), _stream()),
-           "adaption_maxpool2x2")
+    _calls().maxpool(x, N, H, W, Cc, y)
 
 
 def adaption_probe_i8_peak(bn: int, pair: bool, iters: int, d_cycles: torch.Tensor, d_status: torch.Tensor,

@@ -5,12 +5,14 @@ import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
 CSRC = os.path.join(_PKG, "csrc")
 LIB_DIR = os.path.join(_PKG, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "libadaption.so")
+NATIVE_PATH = os.path.join(LIB_DIR, "_adaption_native.so")      # native half of binding.py
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
@@ -31,18 +33,32 @@ def sources() -> list[str]:
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not os.path.exists(LIB_PATH) or not os.path.exists(NATIVE_PATH):
         return True
-    t = os.path.getmtime(LIB_PATH)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(_ROOT, "include", "*.h"))
+    t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(NATIVE_PATH))
+    deps = sources() + glob.glob(os.path.join(CSRC, "*.c*")) + glob.glob(os.path.join(_ROOT, "include", "*.h"))
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_native() -> str:
+    """Compile the argument marshalling (a CPython extension module) into lib/_adaption_native.so."""
+    tmp = NATIVE_PATH + f".{os.getpid()}.tmp"
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        raise RuntimeError("g++ not found: the native half of the binding cannot be built")
+    subprocess.check_call([cxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I",
+                           sysconfig.get_paths()["include"], "-I", os.path.join(_ROOT, "include"), "-o", tmp,
+                           os.path.join(CSRC, "host_binding.cpp"), "-ldl"])
+    os.replace(tmp, NATIVE_PATH)
+    return NATIVE_PATH
+
+
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into lib/libadaption.so."""
+    """Compile every .cu under csrc/ into lib/libadaption.so, and the native half of the binding beside it."""
     if not force and not is_stale():
         return LIB_PATH
     os.makedirs(LIB_DIR, exist_ok=True)
+    build_native()
     tmp = LIB_PATH + f".{os.getpid()}.tmp"
     cmd = [_nvcc()] + NVCC_FLAGS + ["-I", os.path.join(_ROOT, "include"), "-I", CSRC]
     if verbose:
@@ -50,6 +66,7 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     cmd += ["-o", tmp] + sources()
     subprocess.check_call(cmd)
     os.replace(tmp, LIB_PATH)
+    os.utime(NATIVE_PATH)
     return LIB_PATH
 
 

@@ -270,9 +270,9 @@ class LPNetwork:
     # ------------------------------------------------------------------ one layer
     def _workspace(self, L: _Layer, x: B.QTensor) -> torch.Tensor | None:
         if L.type == "conv":
-            need = B.adaption_lp_conv_workspace_bytes(L.shape, x.fmt(), L.w.fmt(), x.c_stride, self.algo)
+            need = B.conv_workspace_bytes(L.shape, x, L.w, self.algo)
         else:
-            need = B.adaption_lp_ip_workspace_bytes(L.N, L.ip_k, L.K, x.fmt(), L.w.fmt(), self.algo)
+            need = B.ip_workspace_bytes(L.N, L.ip_k, L.K, x, L.w, self.algo)
         if need == 0:
             return None
         if L.workspace is None or L.workspace.numel() < need:
@@ -290,8 +290,7 @@ class LPNetwork:
 
     def _run_conv_pool(self, L: _Layer, P: _Layer, x: B.QTensor, phases: int = 3) -> B.QTensor:
         P.y.frac_bits = L.y.frac_bits
-        need = B.adaption_lp_conv_pool_workspace_bytes(L.shape, x.fmt(), L.w.fmt(), P.y.fmt(), x.c_stride,
-                                                       P.y.c_stride, self.algo)
+        need = B.conv_pool_workspace_bytes(L.shape, x, L.w, P.y, self.algo)
         if P.workspace is None or P.workspace.numel() < need:
             P.workspace = torch.empty(need, dtype=torch.uint8, device=self.device)
         B.adaption_lp_conv_pool_fwd(L.shape, x, L.w, L.b.q16, L.b.frac_bits, L.relu, self.algo, P.y, L.stats,
