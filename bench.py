@@ -409,9 +409,9 @@ def run_gpu(args):
             i += 1
         return a
 
-    # kernels of ours per step: range (2) + input LPAct (1) + weight/bias quantization (dense tensors
+    # kernels of ours per step: range (1) + input LPAct (1) + weight/bias quantization (dense tensors
     # batched into one launch) + one per layer (+1 finalize where K is split, +2 first-layer tap packing)
-    launches_step = (3 + net.param_quantize_launches() + len(net.layers) +
+    launches_step = (2 + net.param_quantize_launches() + len(net.layers) +
                      sum(net.helper_launches(L) for L in gemm_layers))
 
     sampler = ClockSampler(local_rank)

@@ -23,12 +23,10 @@ namespace {
 constexpr int kBins = ADAPTION_HIST_BINS;
 constexpr int kWarps = 8;
 
-__device__ __forceinline__ int bits_of_f32(float x, bool& valid) {
-  const uint32_t u = __float_as_uint(x) & 0x7fffffffu;
-  valid = u <= 0x7f800000u;                    // not NaN
-  const int e = (int)(u >> 23) - 127;          // |x| in [2^e, 2^(e+1)); Inf: e = 128
-  const int b = e >= 0 ? e + 1 : 0;
-  return b < kBins - 1 ? b : kBins - 1;
+// bits needed by |x| without the upper bound; 129 for +-Inf and NaN
+__device__ __forceinline__ int open_bits_of_f32(float x) {
+  const uint32_t u = __float_as_uint(x);
+  return max((int)((u << 1) >> 24) - 126, 0);   // |x| in [2^e, 2^(e+1)) has the biased exponent e + 127
 }
 
 __device__ __forceinline__ int width_of_q(int32_t q) {
@@ -60,10 +58,37 @@ __device__ __forceinline__ void block_flush(PrivateHist& h, unsigned long long* 
   }
 }
 
-__device__ __forceinline__ void count_f32(PrivateHist& h, float x) {
-  bool valid;
-  const int b = bits_of_f32(x, valid);
-  if (valid) h.c[b][threadIdx.x] += 1u;
+__device__ __forceinline__ void count_bin(PrivateHist& h, float x, int b) {
+  if ((__float_as_uint(x) & 0x7fffffffu) <= 0x7f800000u) h.c[min(b, kBins - 1)][threadIdx.x] += 1u;     // not NaN
+}
+
+// The four lowest bins (|x| < 8: nearly all weights and activations) are counted in the bytes of one register:
+// a shift by 8 * bin adds nothing for the higher bins, which take the shared-memory counters.  (All elements through
+// shared memory: 166 us for 268 M elements against 151, 7.3 us for 7 M against 5.5; five blocks per SM beat eight,
+// 160 and 6.2 us.)
+__device__ __forceinline__ uint32_t shl1(int n) {
+  uint32_t r;
+  asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(n));          // 0 for n > 31
+  return r;
+}
+struct LowBins {
+  uint32_t bytes = 0;
+  int left = 255;                               // elements until a byte could overflow
+};
+__device__ __forceinline__ void spill(PrivateHist& h, LowBins& l) {
+#pragma unroll
+  for (int b = 0; b < 4; ++b) h.c[b][threadIdx.x] += (l.bytes >> (8 * b)) & 255u;
+  l = LowBins();
+}
+__device__ __forceinline__ void count4(PrivateHist& h, LowBins& l, const float4 v) {
+  const int b0 = open_bits_of_f32(v.x), b1 = open_bits_of_f32(v.y), b2 = open_bits_of_f32(v.z), b3 = open_bits_of_f32(v.w);
+  l.bytes += shl1(8 * b0) + shl1(8 * b1) + shl1(8 * b2) + shl1(8 * b3);
+  if (max(max(b0, b1), max(b2, b3)) >= 4) {
+    if (b0 >= 4) count_bin(h, v.x, b0);
+    if (b1 >= 4) count_bin(h, v.y, b1);
+    if (b2 >= 4) count_bin(h, v.z, b2);
+    if (b3 >= 4) count_bin(h, v.w, b3);
+  }
 }
 
 // head: elements before the first 16-byte boundary, then n4 float4, then the tail
@@ -72,22 +97,30 @@ __global__ void __launch_bounds__(kThreadsHist) bit_histogram_kernel(const float
                                                                      unsigned long long* __restrict__ d_hist) {
   __shared__ PrivateHist h;
   hist_clear(h);
+  pdl_prologue();
   const size_t nthreads = (size_t)gridDim.x * blockDim.x;
   const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const float4* __restrict__ x4 = reinterpret_cast<const float4*>(x + head);
-  size_t i = tid;
-  for (; i + nthreads < n4; i += 2 * nthreads) {
-    const float4 a = __ldcs(x4 + i), b = __ldcs(x4 + i + nthreads);
-    count_f32(h, a.x); count_f32(h, a.y); count_f32(h, a.z); count_f32(h, a.w);
-    count_f32(h, b.x); count_f32(h, b.y); count_f32(h, b.z); count_f32(h, b.w);
+  LowBins low;
+  constexpr int kVecs = 4;                     // float4 in flight per thread
+  constexpr size_t kChunk = (size_t)kThreadsHist * kVecs;
+  for (size_t base = blockIdx.x * kChunk + threadIdx.x; base < n4; base += gridDim.x * kChunk) {
+    float4 v[kVecs];
+#pragma unroll
+    for (int u = 0; u < kVecs; ++u)
+      if (base + u * kThreadsHist < n4) v[u] = __ldcs(x4 + base + u * kThreadsHist);
+#pragma unroll
+    for (int u = 0; u < kVecs; ++u)
+      if (base + u * kThreadsHist < n4) count4(h, low, v[u]);
+    low.left -= 4 * kVecs;
+    if (low.left < 4 * kVecs) spill(h, low);
   }
-  for (; i < n4; i += nthreads) {
-    const float4 a = __ldcs(x4 + i);
-    count_f32(h, a.x); count_f32(h, a.y); count_f32(h, a.z); count_f32(h, a.w);
-  }
+  spill(h, low);
   const size_t tail0 = head + 4 * n4;
-  for (size_t j = tid; j < head + (numel - tail0); j += nthreads)
-    count_f32(h, x[j < head ? j : tail0 + (j - head)]);
+  for (size_t j = tid; j < head + (numel - tail0); j += nthreads) {
+    const float e = x[j < head ? j : tail0 + (j - head)];
+    count_bin(h, e, open_bits_of_f32(e));
+  }
   block_flush(h, d_hist);
 }
 
@@ -98,6 +131,7 @@ __global__ void __launch_bounds__(kThreadsHist) width_histogram_kernel(const uin
                                                                        unsigned long long* __restrict__ d_hist) {
   __shared__ PrivateHist h;
   hist_clear(h);
+  pdl_prologue();
   const int64_t groups_per_row = c_stride / 16;
   const size_t total = outer * (size_t)groups_per_row;
   const size_t nthreads = (size_t)gridDim.x * blockDim.x;
@@ -118,9 +152,9 @@ __global__ void __launch_bounds__(kThreadsHist) width_histogram_kernel(const uin
   block_flush(h, d_hist);
 }
 
-int grid_for(size_t items) {
+int grid_for(size_t items, int blocks_per_sm) {
   size_t want = (items + 32 * kWarps - 1) / (32 * kWarps);
-  const size_t cap = (size_t)num_sms() * 8;
+  const size_t cap = (size_t)num_sms() * blocks_per_sm;
   if (want < 1) want = 1;
   return (int)(want < cap ? want : cap);
 }
@@ -135,8 +169,8 @@ int bit_histogram_impl(const float* d_x, size_t numel, uint64_t* d_hist, cudaStr
   size_t head = ((16 - (reinterpret_cast<uintptr_t>(d_x) & 15u)) & 15u) / 4;
   if (head > numel) head = numel;
   const size_t n4 = (numel - head) / 4;
-  bit_histogram_kernel<<<grid_for(n4 / 2 + 64), 32 * kWarps, 0, stream>>>(
-      d_x, numel, head, n4, reinterpret_cast<unsigned long long*>(d_hist));
+  launch_after_predecessor(bit_histogram_kernel, dim3(grid_for(n4 / 4 + 64, 5)), dim3(32 * kWarps), stream, d_x, numel, head,
+                           n4, reinterpret_cast<unsigned long long*>(d_hist));
   return cuda_status(cudaGetLastError(), "bit_histogram_kernel launch");
 }
 
@@ -147,8 +181,8 @@ int width_histogram_impl(const adaption_qtensor& x, size_t outer, size_t inner, 
   if (rc != ADAPTION_OK) return rc;
   if ((reinterpret_cast<uintptr_t>(d_hist) & 7u) != 0) return ADAPTION_ERR_ALIGNMENT;
   if (outer == 0 || inner == 0) return ADAPTION_OK;
-  width_histogram_kernel<<<grid_for(outer * (size_t)(x.c_stride / 16)), 32 * kWarps, 0, stream>>>(
-      x.fmt.n_bits > 8 ? static_cast<const uint4*>(x.hi) : nullptr, static_cast<const uint4*>(x.lo), outer,
+  launch_after_predecessor(
+      width_histogram_kernel, dim3(grid_for(outer * (size_t)(x.c_stride / 16), 8)), dim3(32 * kWarps), stream, x.fmt.n_bits > 8 ? static_cast<const uint4*>(x.hi) : nullptr, static_cast<const uint4*>(x.lo), outer,
       (int64_t)inner, x.c_stride, reinterpret_cast<unsigned long long*>(d_hist));
   return cuda_status(cudaGetLastError(), "width_histogram_kernel launch");
 }

@@ -33,30 +33,42 @@ static inline int stream_grid(size_t work_items, int threads, int blocks_per_sm)
 // Dynamic range (paper Sec. 2.1, Sec. 2.3): max |x|, NaN ignored.  Non-negative floats order
 // like their bit patterns, so the cross-block reduction is an integer atomicMax.
 // ------------------------------------------------------------------------------------------
+// Decimal point from the maximum (Sec. 2.3): smallest m in [0, n-1] with max < 2^m.  For
+// max >= 1 with binary exponent e (max in [2^e, 2^(e+1))) that is e+1; Inf has e = 128.
+__device__ __forceinline__ int32_t frac_bits_of_max(int max_bits, int32_t n_bits) {
+  const int e = ((max_bits & 0x7fffffff) >> 23) - 127;
+  int m = e >= 0 ? e + 1 : 0;
+  if (m > n_bits - 1) m = n_bits - 1;
+  return n_bits - 1 - m;
+}
+
+constexpr int kRangeVecs = 4;       // float4 per thread and step, all in flight at once
+
+// One kernel measures and chooses: a block that raised the maximum writes the format that belongs to it and
+// looks again, until the maximum it reads back is the one it wrote for.  (Whoever writes last has read the maximum
+// after its write, so the format that stays is that of the final maximum; block 0 writes in any case, for the
+// calls whose tensor raises nothing.)  The format took a launch of its own before.
 __global__ void __launch_bounds__(256) range_max_abs_kernel(const float* __restrict__ x, size_t numel,
-                                                            size_t head, size_t n4,
-                                                            float* __restrict__ d_max_abs) {
+                                                            size_t head, size_t n4, float* d_max_abs, int32_t n_bits,
+                                                            adaption_qfmt* d_fmt) {
   pdl_prologue();
   float m = 0.0f;
-  const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t nthreads = (size_t)gridDim.x * blockDim.x;
   // unaligned head and tail as scalars
-  if (tid < head) m = fmaxf(m, fabsf(x[tid]));
   const size_t tail_begin = head + n4 * 4;
-  if (tail_begin + tid < numel) m = fmaxf(m, fabsf(x[tail_begin + tid]));
-  const float4* __restrict__ x4 = reinterpret_cast<const float4*>(x + head);
-  size_t i = tid;
-  for (; i + 3 * nthreads < n4; i += 4 * nthreads) {
-    float4 a = __ldg(x4 + i), b = __ldg(x4 + i + nthreads), c = __ldg(x4 + i + 2 * nthreads),
-           d = __ldg(x4 + i + 3 * nthreads);
-    m = fmaxf(m, fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w))));
-    m = fmaxf(m, fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fmaxf(fabsf(b.z), fabsf(b.w))));
-    m = fmaxf(m, fmaxf(fmaxf(fabsf(c.x), fabsf(c.y)), fmaxf(fabsf(c.z), fabsf(c.w))));
-    m = fmaxf(m, fmaxf(fmaxf(fabsf(d.x), fabsf(d.y)), fmaxf(fabsf(d.z), fabsf(d.w))));
+  if (blockIdx.x == 0) {
+    if (threadIdx.x < head) m = fmaxf(m, fabsf(x[threadIdx.x]));
+    if (tail_begin + threadIdx.x < numel) m = fmaxf(m, fabsf(x[tail_begin + threadIdx.x]));
   }
-  for (; i < n4; i += nthreads) {
-    float4 a = __ldg(x4 + i);
-    m = fmaxf(m, fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w))));
+  const float4* __restrict__ x4 = reinterpret_cast<const float4*>(x + head);
+  constexpr size_t kChunk = 256 * kRangeVecs;
+  for (size_t base = blockIdx.x * kChunk + threadIdx.x; base < n4; base += gridDim.x * kChunk) {
+    float4 v[kRangeVecs];
+#pragma unroll
+    for (int u = 0; u < kRangeVecs; ++u)
+      v[u] = base + u * 256 < n4 ? __ldg(x4 + base + u * 256) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < kRangeVecs; ++u)
+      m = fmaxf(m, fmaxf(fmaxf(fabsf(v[u].x), fabsf(v[u].y)), fmaxf(fabsf(v[u].z), fabsf(v[u].w))));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -67,21 +79,29 @@ __global__ void __launch_bounds__(256) range_max_abs_kernel(const float* __restr
     float b = wmax[0];
 #pragma unroll
     for (int w = 1; w < 8; ++w) b = fmaxf(b, wmax[w]);
-    if (b > 0.0f) atomicMax(reinterpret_cast<int*>(d_max_abs), __float_as_int(b));
+    int* const bits = reinterpret_cast<int*>(d_max_abs);
+    const int mine = __float_as_int(b);
+    const int before = b > 0.0f ? atomicMax(bits, mine) : mine;
+    if (d_fmt != nullptr && (mine > before || blockIdx.x == 0)) {
+      int seen = *reinterpret_cast<volatile int*>(bits);
+      while (true) {
+        *reinterpret_cast<volatile int32_t*>(&d_fmt->n_bits) = n_bits;
+        *reinterpret_cast<volatile int32_t*>(&d_fmt->frac_bits) = frac_bits_of_max(seen, n_bits);
+        __threadfence();
+        const int now = *reinterpret_cast<volatile int*>(bits);
+        if (now == seen) break;           // (the maximum only grows, so this ends)
+        seen = now;
+      }
+    }
   }
 }
 
-// Decimal point from the maximum (Sec. 2.3): smallest m in [0, n-1] with max < 2^m.  For
-// max >= 1 with binary exponent e (max in [2^e, 2^(e+1))) that is e+1; Inf has e = 128.
+// The format alone, for a tensor without elements.
 __global__ void choose_fmt_kernel(const float* __restrict__ d_max_abs, int32_t n_bits,
                                   adaption_qfmt* __restrict__ d_fmt) {
   pdl_prologue();
-  const int bits = __float_as_int(*d_max_abs) & 0x7fffffff;
-  const int e = (bits >> 23) - 127;
-  int m = e >= 0 ? e + 1 : 0;
-  if (m > n_bits - 1) m = n_bits - 1;
   d_fmt->n_bits = n_bits;
-  d_fmt->frac_bits = n_bits - 1 - m;
+  d_fmt->frac_bits = frac_bits_of_max(__float_as_int(*d_max_abs), n_bits);
 }
 
 // Stored planes as words of four elements.
@@ -137,6 +157,7 @@ __global__ void __launch_bounds__(256) requant_rows_kernel(const uint32_t* __res
                                                            const adaption_qfmt* __restrict__ d_fmt,
                                                            RequantParams rq,
                                                            adaption_stats* __restrict__ stats) {
+  pdl_prologue();
   if (d_fmt != nullptr) out_frac_bits = d_fmt->frac_bits;
   rq.shift = in_frac_bits - out_frac_bits;
   Counts c;
@@ -231,6 +252,7 @@ __global__ void __launch_bounds__(256) requant_flat_kernel(const uint4* __restri
                                                            int32_t in_frac_bits, int32_t out_frac_bits,
                                                            const adaption_qfmt* __restrict__ d_fmt,
                                                            RequantParams rq, adaption_stats* __restrict__ stats) {
+  pdl_prologue();
   if (d_fmt != nullptr) out_frac_bits = d_fmt->frac_bits;
   rq.shift = in_frac_bits - out_frac_bits;
   const int32_t half = rq.shift > 0 ? 1 << (rq.shift - 1) : 0;
@@ -384,23 +406,19 @@ int requant_impl(const adaption_qtensor& in, size_t outer, size_t inner, int32_t
   if ((int64_t)inner == in.c_stride && in.c_stride == out.c_stride && out.q16 == nullptr) {
     const size_t n16 = outer * inner / 16;
     const int grid = stream_grid((n16 + 1) / 2, 256, 8);
-    if (in.fmt.n_bits > 8)
-      requant_flat_kernel<true><<<grid, 256, 0, stream>>>(
-          reinterpret_cast<const uint4*>(in.hi), reinterpret_cast<const uint4*>(in.lo), n16,
-          reinterpret_cast<uint4*>(out.hi), reinterpret_cast<uint4*>(out.lo), in.fmt.frac_bits,
-          out.fmt.frac_bits, d_fmt, rq, d_stats);
-    else
-      requant_flat_kernel<false><<<grid, 256, 0, stream>>>(
-          nullptr, reinterpret_cast<const uint4*>(in.lo), n16, reinterpret_cast<uint4*>(out.hi),
-          reinterpret_cast<uint4*>(out.lo), in.fmt.frac_bits, out.fmt.frac_bits, d_fmt, rq, d_stats);
+    const bool two = in.fmt.n_bits > 8;
+    launch_after_predecessor(two ? requant_flat_kernel<true> : requant_flat_kernel<false>, dim3(grid), dim3(256), stream,
+                             two ? reinterpret_cast<const uint4*>(in.hi) : nullptr, reinterpret_cast<const uint4*>(in.lo),
+                             n16, reinterpret_cast<uint4*>(out.hi), reinterpret_cast<uint4*>(out.lo), in.fmt.frac_bits,
+                             out.fmt.frac_bits, d_fmt, rq, d_stats);
     return cuda_status(cudaGetLastError());
   }
   const size_t groups = outer * (size_t)(out.c_stride / 4);
   const int grid = stream_grid(groups, 256, 8);
-  requant_rows_kernel<<<grid, 256, 0, stream>>>(
-      in.fmt.n_bits > 8 ? reinterpret_cast<const uint32_t*>(in.hi) : nullptr,
-      reinterpret_cast<const uint32_t*>(in.lo), in.c_stride, outer, (int64_t)inner, out.c_stride,
-      quant_out_of(out), in.fmt.frac_bits, out.fmt.frac_bits, d_fmt, rq, d_stats);
+  launch_after_predecessor(requant_rows_kernel, dim3(grid), dim3(256), stream,
+                           in.fmt.n_bits > 8 ? reinterpret_cast<const uint32_t*>(in.hi) : nullptr,
+                           reinterpret_cast<const uint32_t*>(in.lo), in.c_stride, outer, (int64_t)inner, out.c_stride,
+                           quant_out_of(out), in.fmt.frac_bits, out.fmt.frac_bits, d_fmt, rq, d_stats);
   return cuda_status(cudaGetLastError());
 }
 
@@ -414,13 +432,12 @@ int measure_range_impl(const float* d_x, size_t numel, int32_t n_bits, float* d_
     size_t head = ((16 - (reinterpret_cast<uintptr_t>(d_x) & 15u)) & 15u) / 4;
     if (head > numel) head = numel;
     const size_t n4 = (numel - head) / 4;
-    int grid = stream_grid((n4 + 3) / 4 + 4, 256, 8);
-    launch_after_predecessor(range_max_abs_kernel, dim3(grid), dim3(256), stream, d_x, numel, head, n4, d_max_abs);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return ADAPTION_ERR_CUDA;
-  }
-  if (d_fmt_out != nullptr)
+    const int grid = stream_grid((n4 + kRangeVecs - 1) / kRangeVecs, 256, 16);
+    launch_after_predecessor(range_max_abs_kernel, dim3(grid), dim3(256), stream, d_x, numel, head, n4, d_max_abs, n_bits,
+                             d_fmt_out);
+  } else if (d_fmt_out != nullptr) {
     launch_after_predecessor(choose_fmt_kernel, dim3(1), dim3(1), stream, (const float*)d_max_abs, n_bits, d_fmt_out);
+  }
   return cuda_status(cudaGetLastError());
 }
 

@@ -30,6 +30,7 @@ __global__ void __launch_bounds__(256) requant_stochastic_kernel(const uint4* __
                                                                  const adaption_qfmt* __restrict__ d_fmt, int relu,
                                                                  int32_t qmin, int32_t qmax, uint32_t key0,
                                                                  uint32_t key1, adaption_stats* __restrict__ stats) {
+  pdl_prologue();
   if (d_fmt != nullptr) out_frac_bits = d_fmt->frac_bits;
   const int shift = in_frac_bits - out_frac_bits;
   Counts c;
@@ -123,7 +124,8 @@ int requant_stochastic_impl(const adaption_qtensor& in, size_t outer, size_t inn
   size_t want = (groups + 255) / 256;
   const size_t cap = (size_t)num_sms() * 8;
   const int grid = (int)(want < cap ? (want < 1 ? 1 : want) : cap);
-  requant_stochastic_kernel<<<grid, 256, 0, stream>>>(
+  launch_after_predecessor(
+      requant_stochastic_kernel, dim3(grid), dim3(256), stream,
       in.fmt.n_bits > 8 ? static_cast<const uint4*>(in.hi) : nullptr, static_cast<const uint4*>(in.lo), in.c_stride,
       outer, (int64_t)inner, out.c_stride, o, in.fmt.frac_bits, out.fmt.frac_bits, d_fmt, relu ? 1 : 0, qmin, qmax,
       (uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32), d_stats);

@@ -445,7 +445,7 @@ class LPNetwork:
         if measure_input:
             # range of the incoming batch (monitoring; the calibrated input format stays in force)
             B.adaption_measure_range(x_f32, self.n_bits, self.x_max_dev, self.x_fmt_dev)
-            launches += 2
+            launches += 1
         self._quantize_input(x_f32)
         launches += 1
         if requantize_params:
