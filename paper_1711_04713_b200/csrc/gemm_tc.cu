@@ -52,13 +52,19 @@ constexpr int64_t kMaxKPerAccumulation = 32768;
 // epilogue variants (a template parameter of the kernel): generic 64-bit, the 32-bit fast path of
 // ReLU layers, generic with stochastic rounding
 constexpr int kEpiGeneric = 0, kEpiFast = 1, kEpiStochastic = 2;
+// main-loop variants: one full k-block per stage; several k-blocks per stage and / or resident weights; one
+// k-block per stage of which the last one of a tap has fewer steps (channel pitch no multiple of 128).  (Variants,
+// because the issuing warp's code decides the main loop's speed: with the bookkeeping of the third in the second
+// 64 x 224 x 224 x 64 -> 64 took 595 us against 515.)
+constexpr int kLoopPlain = 0, kLoopGrouped = 1, kLoopPartial = 2;
 
 struct TcParams {
   int M, N;
   int tile_m;                 // rows per tile: 128, or 256 for a CTA pair
   int tiles_m, tiles_n, splits, total_tiles;
   int num_kb, kb_per_split;
-  int BN, BK, ksteps;
+  int BN, BK;
+  int ksteps, ksteps_last;    // 32-byte steps of a k-block, of the last channel block of a tap
   uint32_t sbo, layout_type;
   int stages;
   uint32_t a_bytes, b_bytes, stage_bytes;
@@ -486,19 +492,21 @@ __device__ __forceinline__ void release_accumulators(unsigned long long* bar_ptr
 }
 
 // ---------------------------------------------------------------------------------- kernel
+// LOOP: the form of the main loop, see kLoopPlain.
 // GROUPED: stages hold several k-blocks and / or the weights are resident in shared memory (short
 // reductions); the plain variant keeps the issue loops free of that bookkeeping.
 // FAST: ReLU layer in requantizing mode whose shift lies in [9, 31] ([0, 31] with 8-bit operands
 // on both sides), N a multiple of 8, no split-K,
 // magnitudes within the 32-bit bounds of the fast epilogue: it then contains only that path.
 // 20 warps: one block per SM, 96 registers per thread.
-template <int NAX, int NBW, bool PAIR, bool GROUPED, int EPI>
+template <int NAX, int NBW, bool PAIR, int LOOP, int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
 lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
                const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
                const __grid_constant__ CUtensorMap map_y_hi, const __grid_constant__ CUtensorMap map_y_lo,
                const TcParams p) {
   constexpr int NACC = NAX + NBW - 1;
+  constexpr bool GROUPED = LOOP == kLoopGrouped, PARTIAL = LOOP == kLoopPartial;
   constexpr bool FAST = EPI == kEpiFast;
   constexpr bool STOCH = EPI == kEpiStochastic;
   extern __shared__ uint8_t smem_raw[];
@@ -702,7 +710,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       const uint32_t stage_u = p.stage_bytes >> 4, a_u = p.a_bytes >> 4, b_u = p.b_bytes >> 4;
       const uint32_t kb_u = p.kb_bytes >> 4;
       const uint32_t off_a1 = a_u, off_b0 = NAX * a_u;
-      const int ksteps = p.ksteps;
+      const int ksteps_full = p.ksteps;
       const uint32_t full_bar0 = smem_u32(&ctrl.full[0]), empty_bar0 = smem_u32(&ctrl.empty[0]);
       uint32_t tile_iter = 0, ph = 0;
       uint32_t a0 = ring_lo, full_bar = full_bar0, empty_bar = empty_bar0;
@@ -738,8 +746,14 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         uint32_t bres = bres_lo + (uint32_t)tc.kb_begin * bres_u;   // resident weights of this k-block
         const bool stagger = !GROUPED && NAX == 2 && NBW == 2 && p.tail_stagger != 0;
         const int kb_main_end = stagger ? tc.kb_end - 2 : tc.kb_end;
+        int cb = PARTIAL ? tc.kb_begin % p.cblks : 0;               // channel block of its tap
         for (int kb = tc.kb_begin; kb < kb_main_end; kb += kps) {
           const int nkb = GROUPED ? min(kps, tc.kb_end - kb) : 1;
+          int ksteps = ksteps_full;                                 // (fixed unless PARTIAL)
+          if (PARTIAL) {
+            if (cb == p.cblks - 1) ksteps = p.ksteps_last;
+            if (++cb == p.cblks) cb = 0;
+          }
           {
 #ifdef ADAPTION_TIMELINE
           const long long tw0 = clock64();
@@ -766,8 +780,9 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
               if (ksteps > 2) {
                 mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0 + 4u, a0 + off_a1 + 4u, b0 + 4u, b0 + b_u + 4u, dhi,
                                           id_ss, id_su, id_us, id_uu, 1u);
-                mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0 + 6u, a0 + off_a1 + 6u, b0 + 6u, b0 + b_u + 6u, dhi,
-                                          id_ss, id_su, id_us, id_uu, 1u);
+                if (!PARTIAL || ksteps > 3)
+                  mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0 + 6u, a0 + off_a1 + 6u, b0 + 6u, b0 + b_u + 6u, dhi,
+                                            id_ss, id_su, id_us, id_uu, 1u);
               }
             }
             if (GROUPED && nkb > 1) {
@@ -806,8 +821,14 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           // The two last k-blocks together, product by product.  (Integer accumulation: the order of
           // the MMAs does not matter.)  Both stages are handed back at the end.
           uint32_t st_a[2], st_full[2], st_empty[2], st_ph[2];
+          int st_ks[2];
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
+            st_ks[j] = ksteps_full;
+            if (PARTIAL) {
+              if (cb == p.cblks - 1) st_ks[j] = p.ksteps_last;
+              if (++cb == p.cblks) cb = 0;
+            }
             st_a[j] = a0; st_full[j] = full_bar; st_empty[j] = empty_bar; st_ph[j] = ph;
             a0 += stage_u;
             full_bar += 8u;
@@ -828,19 +849,19 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             const uint32_t off_b1 = off_b0 + b_u;
 #pragma unroll
             for (int j = 0; j < 2; ++j)
-              for (int ks = 0; ks < ksteps; ++ks)                     // lo * lo
+              for (int ks = 0; ks < st_ks[j]; ++ks)                     // lo * lo
                 mma_i8<PAIR>(d2, st_a[j] + off_a1 + 2u * ks, st_a[j] + off_b1 + 2u * ks, dhi, id_uu, 1u);
             tc_commit<PAIR>(smem_u32(&ctrl.part_full[0]));
 #pragma unroll
             for (int j = 0; j < 2; ++j)
-              for (int ks = 0; ks < ksteps; ++ks) {                   // hi * lo and lo * hi
+              for (int ks = 0; ks < st_ks[j]; ++ks) {                   // hi * lo and lo * hi
                 mma_i8<PAIR>(d1, st_a[j] + 2u * ks, st_a[j] + off_b1 + 2u * ks, dhi, id_su, 1u);
                 mma_i8<PAIR>(d1, st_a[j] + off_a1 + 2u * ks, st_a[j] + off_b0 + 2u * ks, dhi, id_us, 1u);
               }
             tc_commit<PAIR>(smem_u32(&ctrl.part_full[1]));
 #pragma unroll
             for (int j = 0; j < 2; ++j)
-              for (int ks = 0; ks < ksteps; ++ks)                     // hi * hi
+              for (int ks = 0; ks < st_ks[j]; ++ks)                     // hi * hi
                 mma_i8<PAIR>(d0, st_a[j] + 2u * ks, st_a[j] + off_b0 + 2u * ks, dhi, id_ss, 1u);
             tc_commit<PAIR>(st_empty[0]);
             tc_commit<PAIR>(st_empty[1]);
@@ -1166,7 +1187,7 @@ struct TcConfig {
   uint32_t tmem_cols = 32;
   int num_kb = 0, splits = 1, kb_per_split = 0;
   int tiles_m = 0, tiles_n = 0;
-  int cblks = 1;
+  int cblks = 1, ksteps_last = 0;
   bool b_resident = false;
   uint32_t b_res_bytes = 0;
   int kps = 1;
@@ -1201,8 +1222,15 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   if (g.is_conv) {
     const int64_t cs = g.x.c_stride;
     if (cs != g.w.c_stride || cs % 32 != 0 || cs > 65536) return c;
-    c.BK = cs % 128 == 0 ? 128 : (cs % 64 == 0 ? 64 : 32);
-    c.cblks = (int)(cs / c.BK);
+    // k-blocks of 128 bytes as soon as there are more than 64: bulk copies deliver one row per two cycles
+    // whatever its length, so narrow blocks cost as many rows each.  Where the pitch is no multiple of 128 the
+    // last block of a tap reaches past the pitch (the copy fills zeros without reading) and the MMAs skip
+    // the steps that are not there (in a grouped main loop they multiply the zeros: those loops wait for copies).
+    // 3x3 layers before -> now: 12 x 45 x 37 x 96 -> 168 at 12 bits 29.6 -> 25.0 us, 16 x 56 x 56 x 160 -> 128 at 16
+    // bits 44.8 -> 34.0, 16 x 56 x 56 x 96 -> 256 at 8 bits 34.8 -> 20.3.
+    c.BK = cs > 64 ? 128 : (int)cs;
+    c.cblks = (int)((cs + c.BK - 1) / c.BK);
+    c.ksteps_last = (int)(cs - (int64_t)(c.cblks - 1) * c.BK) / 32;
     c.num_kb = g.cs.R * g.cs.S * c.cblks;
     k_padded = (int64_t)g.cs.R * g.cs.S * cs;
     // im2col traversal limits of the tensor map (two spatial dimensions: 8-bit signed corners)
@@ -1368,7 +1396,7 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   return c;
 }
 
-template <int NAX, int NBW, bool PAIR, bool GROUPED, int EPI>
+template <int NAX, int NBW, bool PAIR, int LOOP, int EPI>
 int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
   // The dynamic shared-memory limit is a per-device attribute of the kernel: remember, per device
   // ordinal, the largest size it has been raised to (a racing thread at worst sets it once more).
@@ -1378,7 +1406,7 @@ int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t s
   if (cudaGetDevice(&dev) != cudaSuccess) return ADAPTION_ERR_CUDA;
   const bool cached = dev >= 0 && dev < kMaxDevices;
   if (!cached || smem > attr_size[dev].load(std::memory_order_acquire)) {
-    const cudaError_t ae = cudaFuncSetAttribute(lp_gemm_kernel<NAX, NBW, PAIR, GROUPED, EPI>,
+    const cudaError_t ae = cudaFuncSetAttribute(lp_gemm_kernel<NAX, NBW, PAIR, LOOP, EPI>,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (ae != cudaSuccess) return cuda_failure(ae, "lp_gemm_kernel shared-memory attribute");
     if (cached) {
@@ -1411,7 +1439,7 @@ int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t s
   cfg.attrs = n_attr ? attr : nullptr;
   cfg.numAttrs = n_attr;
   const cudaError_t le =
-      cudaLaunchKernelEx(&cfg, lp_gemm_kernel<NAX, NBW, PAIR, GROUPED, EPI>, maps[0], maps[1], maps[2], maps[3], maps[4],
+      cudaLaunchKernelEx(&cfg, lp_gemm_kernel<NAX, NBW, PAIR, LOOP, EPI>, maps[0], maps[1], maps[2], maps[3], maps[4],
                          maps[5], p);
   if (le != cudaSuccess) {
     (void)cudaGetLastError();
@@ -1420,22 +1448,25 @@ int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t s
   return cuda_status(cudaGetLastError(), "after lp_gemm_kernel launch");
 }
 
-template <int NAX, int NBW, bool PAIR, bool GROUPED>
+template <int NAX, int NBW, bool PAIR, int LOOP>
 int launch_epi(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
-  if (p.fast_relu != 0) return launch_kernel<NAX, NBW, PAIR, GROUPED, kEpiFast>(maps, p, grid, smem, stream);
-  if (p.st.enabled != 0) return launch_kernel<NAX, NBW, PAIR, GROUPED, kEpiStochastic>(maps, p, grid, smem, stream);
-  return launch_kernel<NAX, NBW, PAIR, GROUPED, kEpiGeneric>(maps, p, grid, smem, stream);
+  if (p.fast_relu != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiFast>(maps, p, grid, smem, stream);
+  if (p.st.enabled != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiStochastic>(maps, p, grid, smem, stream);
+  return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiGeneric>(maps, p, grid, smem, stream);
+}
+
+template <int NAX, int NBW, bool PAIR>
+int launch_loop(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
+  if (p.kps > 1 || p.b_resident != 0) return launch_epi<NAX, NBW, PAIR, kLoopGrouped>(maps, p, grid, smem, stream);
+  if (p.ksteps_last != p.ksteps) return launch_epi<NAX, NBW, PAIR, kLoopPartial>(maps, p, grid, smem, stream);
+  return launch_epi<NAX, NBW, PAIR, kLoopPlain>(maps, p, grid, smem, stream);
 }
 
 template <int NAX, int NBW>
 int launch_either(bool pair, const CUtensorMap* maps, const TcParams& p, int grid, size_t smem,
                   cudaStream_t stream) {
-  const bool grouped = p.kps > 1 || p.b_resident != 0;
-  if (pair)
-    return grouped ? launch_epi<NAX, NBW, true, true>(maps, p, grid, smem, stream)
-                   : launch_epi<NAX, NBW, true, false>(maps, p, grid, smem, stream);
-  return grouped ? launch_epi<NAX, NBW, false, true>(maps, p, grid, smem, stream)
-                 : launch_epi<NAX, NBW, false, false>(maps, p, grid, smem, stream);
+  return pair ? launch_loop<NAX, NBW, true>(maps, p, grid, smem, stream)
+              : launch_loop<NAX, NBW, false>(maps, p, grid, smem, stream);
 }
 
 
@@ -1611,6 +1642,7 @@ int launch_tensor(const GemmProblem& g) {
   p.total_tiles = c.tiles_m * c.tiles_n * c.splits;
   p.num_kb = c.num_kb; p.kb_per_split = c.kb_per_split;
   p.BN = c.BN; p.BK = c.BK; p.ksteps = c.BK / 32;
+  p.ksteps_last = g.is_conv ? c.ksteps_last : p.ksteps;
   p.sbo = (uint32_t)(8 * c.BK); p.layout_type = c.layout_type;
   p.stages = c.stages; p.a_bytes = c.a_bytes; p.b_bytes = c.b_bytes; p.stage_bytes = c.stage_bytes;
   p.kps = c.kps; p.kb_bytes = c.kb_bytes;
@@ -1620,8 +1652,9 @@ int launch_tensor(const GemmProblem& g) {
   p.split_hh = (c.nacc == 3 && c.acc_bufs == 1 && 4 * c.BN <= 512 && knob(kSplitHh) != 0) ? 1 : 0;
   if (p.split_hh) p.tmem_cols = 512;
   p.is_conv = g.is_conv ? 1 : 0;
+  p.cblks = c.cblks;
   if (g.is_conv) {
-    p.OH = g.OH; p.OW = g.OW; p.S = g.cs.S; p.cblks = c.cblks; p.w_pitch = (int)g.w.c_stride;
+    p.OH = g.OH; p.OW = g.OW; p.S = g.cs.S; p.w_pitch = (int)g.w.c_stride;
     p.stride_h = g.cs.stride_h; p.stride_w = g.cs.stride_w; p.pad_h = g.cs.pad_h; p.pad_w = g.cs.pad_w;
   }
   p.bias = g.bias; p.bias_shift = g.bias_shift;
@@ -1653,7 +1686,7 @@ int launch_tensor(const GemmProblem& g) {
       knob(kFast) != 0) {
     // 32-bit bounds of the fast epilogue (see fast_result): with a reduction of kred bytes per plane row
     // |hh| <= kred 2^14, |mid| <= kred 65280, |ll| <= kred 65025, and |C| < 2^(15 + bias_shift) + 2^(shift-1)
-    const long long kred = (long long)c.num_kb * c.BK;
+    const long long kred = g.is_conv ? (long long)g.cs.R * g.cs.S * g.x.c_stride : (long long)c.num_kb * c.BK;
     const long long cmax = (g.bias != nullptr ? (1ll << (15 + g.bias_shift)) : 0ll) +
                            (p.rq.shift > 0 ? 1ll << (p.rq.shift - 1) : 0ll);
     const long long hmax = kred * 16384 + (cmax >> 16) + 1;

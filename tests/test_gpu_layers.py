@@ -639,3 +639,20 @@ def test_layer_calls_from_two_host_threads():
     t2 = threading.Thread(target=work, args=(41, (5, 30, 30, 64, 64, 3, 1, 1, 16, 16, 16, True)))
     t1.start(); t2.start(); t1.join(); t2.join()
     assert not errors, errors
+
+
+PARTIAL_BLOCKS = [
+    # N, H, W, Cin, K, R, pad, stride, nx, nw, n_out, relu: channel pitches that are no multiple of 128 bytes
+    (6, 30, 30, 96, 168, 3, 1, 1, 12, 12, 12, True),      # one block of three steps per tap, two column tiles
+    (6, 30, 30, 160, 128, 3, 1, 1, 16, 16, 16, True),     # 128 + 32: every second block a single step
+    (4, 33, 31, 200, 72, 3, 1, 2, 16, 16, 16, False),     # pitch 224, stride 2, generic epilogue
+    (3, 28, 28, 192, 264, 3, 1, 1, 8, 8, 8, True),        # single pass, grouped stages, 256-column tiles
+    (8, 40, 40, 70, 64, 3, 1, 1, 8, 16, 16, True),        # pitch 96, 64-column tile, resident weights
+    (5, 26, 26, 288, 40, 1, 0, 1, 16, 8, 12, True),       # 1x1, three blocks
+]
+
+
+@pytest.mark.parametrize("case", PARTIAL_BLOCKS)
+@pytest.mark.parametrize("with_q16", [False, True])
+def test_conv_channel_pitch_not_a_multiple_of_128(case, with_q16, cta_mode):
+    run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_TENSOR, with_q16=with_q16)
