@@ -58,6 +58,26 @@ constexpr int kEpiGeneric = 0, kEpiFast = 1, kEpiStochastic = 2;
 // 64 x 224 x 224 x 64 -> 64 took 595 us against 515.)
 constexpr int kLoopPlain = 0, kLoopGrouped = 1, kLoopPartial = 2;
 
+// Division by a number fixed for the launch: q = (n * mul >> 32) >> shift for 0 <= n < 2^31 (mul =
+// ceil(2^(32 + shift) / d) with 2^(shift + 1) >= d > 2^shift; mul = 0 stands for d = 1).  An integer division costs a
+// warp twenty to thirty instructions, and the copying and issuing warps share their schedulers with the epilogue's.
+struct FastDiv {
+  uint32_t mul, shift;
+  int d;
+  __device__ __forceinline__ int quot(int n) const { return mul == 0u ? n : (int)(__umulhi((uint32_t)n, mul) >> shift); }
+};
+FastDiv fast_div(int d) {
+  FastDiv f;
+  f.d = d;
+  f.mul = 0;
+  f.shift = 0;
+  if (d > 1) {
+    while ((2ll << f.shift) < d) ++f.shift;
+    f.mul = (uint32_t)(((1ull << (32 + f.shift)) + (unsigned)d - 1) / (unsigned)d);
+  }
+  return f;
+}
+
 struct TcParams {
   int M, N;
   int tile_m;                 // rows per tile: 128, or 256 for a CTA pair
@@ -76,7 +96,8 @@ struct TcParams {
   // only activation planes and all weight k-blocks are loaded once per CTA at this offset
   int b_resident;
   uint32_t b_res_off;
-  int acc_bufs;
+  int acc_bufs, acc_shift;    // 1, 2 or 4 accumulator sets, and the power of two
+  FastDiv div_tiles_n, div_splits, div_ow, div_oh, div_s, div_cblks;
   // Three accumulators of 128 columns leave one quarter of TMEM free: the high accumulator then
   // alternates between the first and the last quarter from tile to tile (the other two stay put),
   // and the epilogue hands the low and middle accumulators back before it reads the high one, so
@@ -109,7 +130,7 @@ struct TcParams {
   // epilogue variants chosen on the host
   int fast_relu;              // launch the FAST kernel variant (paired 16-bit epilogue)
   int pool_w;                 // store max(row 2j, row 2j+1) of the tile: half of a 2x2 max-pool (staged only)
-  int epi_groups;             // 1, or 2: the epilogue warps form two groups that take alternate tiles
+  int epi_groups;             // 1, 2 or 4 groups of epilogue warps that take turns tile by tile
   int staged;                 // outputs leave through shared memory and bulk-tensor stores
   int stage_bufs;             // staging buffers per epilogue group: 1, or 2 used in turn (narrow tiles)
   uint32_t stage_off;         // offset of the staging planes from the ring base
@@ -187,10 +208,10 @@ struct TileCoord {
 };
 __device__ __forceinline__ TileCoord decode_tile(int t, const TcParams& p) {
   TileCoord tc;
-  const int tn = t % p.tiles_n;
-  const int rest = t / p.tiles_n;
-  const int split = rest % p.splits;
-  const int tm = rest / p.splits;
+  const int rest = p.div_tiles_n.quot(t);
+  const int tn = t - rest * p.tiles_n;
+  const int tm = p.div_splits.quot(rest);
+  const int split = rest - tm * p.splits;
   tc.m0 = tm * p.tile_m;
   tc.n0 = tn * p.BN;
   tc.kb_begin = split * p.kb_per_split;
@@ -579,7 +600,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       const CUtensorMap* my_map2 = &map_b1;
       const uint32_t my_off2 = NAX * p.a_bytes + (uint32_t)(NBW - 1) * p.b_bytes;
       uint32_t it = 0, ph = 0;
-      int s = 0;
+      int s = 0, turn = 0;                     // turn: s modulo nsub
       bool ok = true;
       if (b_res && warp == kProducerWarps - 1) {
         // the whole weight matrix of this (single) column tile, one copy per k-block and plane,
@@ -611,21 +632,32 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         int tap = 0, cb = 0, r = 0, sx = 0;       // position of kb in the (tap, channel block) order
         if (lane == 0 && warp == 0) TL_STAMP(0, (uint32_t)((t - worker) / workers), 0);
         if (p.is_conv) {
-          const int ow = m_begin % p.OW;
-          const int rest = m_begin / p.OW;
-          const int oh = rest % p.OH;
-          img = rest / p.OH;
+          const int rest = p.div_ow.quot(m_begin);
+          const int ow = m_begin - rest * p.OW;
+          img = p.div_oh.quot(rest);
+          const int oh = rest - img * p.OH;
           base_w = ow * p.stride_w - p.pad_w;
           base_h = oh * p.stride_h - p.pad_h;
-          tap = tc.kb_begin / p.cblks;
+          tap = p.div_cblks.quot(tc.kb_begin);
           cb = tc.kb_begin - tap * p.cblks;
-          r = tap / p.S;
+          r = p.div_s.quot(tap);
           sx = tap - r * p.S;
         }
         for (int kb = tc.kb_begin; kb < tc.kb_end; kb += kps, ++it) {
           if (it == (uint32_t)p.stall_at) { stalled = true; break; }
           const int nkb = GROUPED ? min(kps, tc.kb_end - kb) : 1;      // k-blocks in this stage
-          const bool my_turn = (s % nsub) == sub;     // ring slots have fixed owners
+          const bool my_turn = turn == sub;           // ring slots have fixed owners
+          if (++turn == nsub) turn = 0;
+          if (GROUPED && !my_turn) {
+            if (++s == p.stages) { s = 0; ph ^= 1u; turn = 0; }
+            continue;
+          }
+          if (GROUPED && nsub > 1 && p.is_conv) {     // (the stages in between were another warp's)
+            tap = p.div_cblks.quot(kb);
+            cb = kb - tap * p.cblks;
+            r = p.div_s.quot(tap);
+            sx = tap - r * p.S;
+          }
           uint32_t full = 0, dst = 0;
           if (my_turn) {                                  // this warp's turn for its plane
             ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&ctrl.empty[s]), ph ^ 1u, &ctrl, p));
@@ -661,7 +693,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
               }
             }
           }
-          if (++s == p.stages) { s = 0; ph ^= 1u; }
+          if (++s == p.stages) { s = 0; ph ^= 1u; turn = 0; }
         }
       }
       const bool is_b_loader = b_res && warp == kProducerWarps - 1;
@@ -725,8 +757,8 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       }
       for (int t = worker; t < p.total_tiles && ok; t += workers, ++tile_iter) {
         const TileCoord tc = decode_tile(t, p);
-        const uint32_t buf = tile_iter % (uint32_t)p.acc_bufs;
-        const uint32_t bph = (tile_iter / (uint32_t)p.acc_bufs) & 1u;
+        const uint32_t buf = tile_iter & (uint32_t)(p.acc_bufs - 1);
+        const uint32_t bph = (tile_iter >> p.acc_shift) & 1u;
         if (lane == 0) TL_STAMP(1, tile_iter, 0);
         ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&ctrl.tmem_empty[buf]), bph ^ 1u, &ctrl, p, false));
         // split release: barrier 0 above covers the middle and low accumulators, barriers 1 and 2
@@ -770,37 +802,17 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             // a0 / ak: low descriptor word of the first A plane of a k-block; the other planes and
             // the k-steps are fixed offsets (16-byte units) from it (weights: in the stage or
             // resident).  The first k-block is straight-line code; grouped stages loop over the rest.
-            {
-              const uint32_t b0 = b_res ? bres : a0 + off_b0;
-              mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0, a0 + off_a1, b0, b0 + b_u, dhi, id_ss, id_su, id_us,
-                                        id_uu, acc);
-              if (ksteps > 1)
-                mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0 + 2u, a0 + off_a1 + 2u, b0 + 2u, b0 + b_u + 2u, dhi,
-                                          id_ss, id_su, id_us, id_uu, 1u);
-              if (ksteps > 2) {
-                mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0 + 4u, a0 + off_a1 + 4u, b0 + 4u, b0 + b_u + 4u, dhi,
-                                          id_ss, id_su, id_us, id_uu, 1u);
-                if (!PARTIAL || ksteps > 3)
-                  mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0 + 6u, a0 + off_a1 + 6u, b0 + 6u, b0 + b_u + 6u, dhi,
-                                            id_ss, id_su, id_us, id_uu, 1u);
-              }
-            }
-            if (GROUPED && nkb > 1) {
-              uint32_t ak = a0 + kb_u, bk = bres + bres_u;
-              for (int j = 1; j < nkb; ++j, ak += kb_u, bk += bres_u) {
-                const uint32_t b0 = b_res ? bk : ak + off_b0;
-                mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, ak, ak + off_a1, b0, b0 + b_u, dhi, id_ss, id_su, id_us,
-                                          id_uu, 1u);
-                if (ksteps > 1)
-                  mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, ak + 2u, ak + off_a1 + 2u, b0 + 2u, b0 + b_u + 2u, dhi,
-                                            id_ss, id_su, id_us, id_uu, 1u);
-                if (ksteps > 2) {
-                  mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, ak + 4u, ak + off_a1 + 4u, b0 + 4u, b0 + b_u + 4u, dhi,
-                                            id_ss, id_su, id_us, id_uu, 1u);
-                  mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, ak + 6u, ak + off_a1 + 6u, b0 + 6u, b0 + b_u + 6u, dhi,
-                                            id_ss, id_su, id_us, id_uu, 1u);
+            mma_kblock<NAX, NBW, PAIR, PARTIAL>(d0, d1, d2, a0, off_a1, b_res ? bres : a0 + off_b0, b_u, dhi, id_ss, id_su,
+                                                id_us, id_uu, ksteps, acc);
+            if (GROUPED) {
+              // (unrolled: a loop here costs the issuing thread more than the narrow MMAs take)
+#pragma unroll
+              for (int j = 1; j < 4; ++j)
+                if (j < nkb) {
+                  const uint32_t ak = a0 + (uint32_t)j * kb_u;
+                  mma_kblock<NAX, NBW, PAIR, false>(d0, d1, d2, ak, off_a1, b_res ? bres + (uint32_t)j * bres_u : ak + off_b0,
+                                                    b_u, dhi, id_ss, id_su, id_us, id_uu, ksteps, 1u);
                 }
-              }
             }
             tc_commit<PAIR>(empty_bar);                        // stage reusable once these MMAs retire
           }
@@ -883,9 +895,9 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
   } else {
     // ------------------------------------------------------------------ epilogue warps
     const int quarter = warp & 3;          // TMEM lanes 32*quarter .. 32*quarter+31
-    // With two accumulator sets and narrow tiles the warps form two groups that take alternate
-    // tiles (and accumulator sets), so that one group's TMEM loads overlap the other's arithmetic;
-    // each group has its own barriers, constants and staging planes.
+    // With several accumulator sets the warps form groups that take turns tile by tile (each with an
+    // accumulator set, barriers, constants and staging planes of its own), so that one group's waits and
+    // TMEM loads overlap the others' arithmetic.
     const int groups = p.epi_groups;
     const int gwarps = kEpiWarps / groups, gthreads = 32 * gwarps;
     const int group = (warp - kFirstEpiWarp) / gwarps;
@@ -911,8 +923,8 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     int const_n0 = -1;          // first column of the tile whose constants are staged
     for (int t = worker + group * workers; t < p.total_tiles; t += groups * workers, tile_iter += (uint32_t)groups) {
       const TileCoord tc = decode_tile(t, p);
-      const uint32_t buf = tile_iter % (uint32_t)p.acc_bufs;
-      const uint32_t bph = (tile_iter / (uint32_t)p.acc_bufs) & 1u;
+      const uint32_t buf = tile_iter & (uint32_t)(p.acc_bufs - 1);
+      const uint32_t bph = (tile_iter >> p.acc_shift) & 1u;
       // per-column constants of this tile (the last barrier of the previous tile separates these
       // writes from its readers): bias aligned to the accumulator, plus the rounding half on the
       // fast path.  Kept when the tile covers the same columns as the previous one.
@@ -1267,6 +1279,7 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   c.tiles_n = (int)((g.N + c.BN - 1) / c.BN);
   c.acc_bufs = 512 / (c.nacc * c.BN);
   if (c.acc_bufs > kMaxAccBufs) c.acc_bufs = kMaxAccBufs;
+  if (c.acc_bufs == 3) c.acc_bufs = 2;
   if (c.acc_bufs < 1) return c;
   uint32_t cols = (uint32_t)(c.acc_bufs * c.nacc * c.BN);
   c.tmem_cols = 32;
@@ -1327,25 +1340,34 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   const int out_planes = g.y.fmt.n_bits > 8 ? 2 : 1;
   c.staged = g.mode == ADAPTION_MODE_REQUANT && c.splits == 1 && g.y.q16 == nullptr && g.y.lo != nullptr &&
              g.y.c_stride >= c.BN && g.y.c_stride % 16 == 0 && knob(kStaged) != 0;
-  // two epilogue groups when two tiles can be in flight in TMEM and their constants fit the halves
-  // of the per-column array
-  c.epi_groups = (c.acc_bufs >= 2 && c.acc_bufs % 2 == 0 && c.BN <= 64 &&
-                  knob(kEpiGroups) == 2) ? 2 : 1;
+  // As many epilogue groups as tiles can be in flight in TMEM, two for wide tiles: a group's chain per tile (wait,
+  // TMEM loads, arithmetic, staging, barrier, store) is mostly latency.  8 bits, batch 128: 3 -> 64 channels at 224 x 224
+  // 387 us with two groups, 349 with four; 64 -> 128 at 112 x 112 163 with one, 128 with two, 126 with four;
+  // 128 -> 256 at 56 x 56 106 with one, 90 with two; 3 -> 16 at 16 bits, batch 16 91 with two, 62 with four.
+  c.epi_groups = c.acc_bufs;
+  const int most_groups = c.BN <= 64 ? 4 : 2;
+  while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
   c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) : 0u;
   // dynamic shared memory: everything up to the per-block limit except the control block
   c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
   const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
-  // group short k-blocks so that a stage carries roughly 768 tensor-pipe cycles of work or more
+  // group short k-blocks so that a stage carries roughly 768 tensor-pipe cycles of work or more (512 with one
+  // product per step: 128 -> 128 channels at 112 x 112, 8 bits, batch 128 231 us with two k-blocks, 264 with three)
   {
     const int products = c.nax * c.nbw;
     const int cyc_per_kb = (c.BK / 32) * products * (c.BN >= 128 ? c.BN / 2 : 48);
-    int kps = (768 + cyc_per_kb - 1) / cyc_per_kb;
+    const int want = c.nacc == 1 ? 512 : 768;
+    int kps = (want + cyc_per_kb - 1) / cyc_per_kb;
     if (kps > 4) kps = 4;
     const int kps_env = knob(kKps);
     if (narrow_pair && c.pair) kps = 3;
     if (kps_env >= 1 && kps_env <= 4) kps = kps_env;
     if (kps > c.kb_per_split) kps = c.kb_per_split;
     if (kps < 1) kps = 1;
+    if (kps_env == 0) {                     // as few stages per tile, but even ones
+      const int per_tile = (c.kb_per_split + kps - 1) / kps;
+      kps = (c.kb_per_split + per_tile - 1) / per_tile;
+    }
     c.kps = kps;
   }
   c.kb_bytes = c.nax * c.a_bytes + c.nbw * c.b_bytes;
@@ -1369,7 +1391,7 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
     c.stage_bufs = 1;
   }
   if (c.stages > kMaxStages) c.stages = kMaxStages;
-  // Narrow tiles with two epilogue groups: a second staging buffer per group, so that a group does
+  // Narrow tiles with two epilogue groups (with four the other groups cover the wait): a second staging buffer per group, so that a group does
   // not wait for its previous tile's bulk store to have read shared memory - where the ring keeps at
   // least four stages beside it (short reductions with small stages, e.g. a packed first layer).
   if (c.staged && c.epi_groups == 2 && c.BN <= 64 && knob(kStageBufs) != 1) {
@@ -1648,7 +1670,15 @@ int launch_tensor(const GemmProblem& g) {
   p.kps = c.kps; p.kb_bytes = c.kb_bytes;
   p.b_resident = c.b_resident ? 1 : 0;
   p.b_res_off = (uint32_t)c.stages * c.stage_bytes;
-  p.acc_bufs = c.acc_bufs; p.tmem_cols = c.tmem_cols;
+  p.acc_bufs = c.acc_bufs;
+  p.acc_shift = c.acc_bufs == 4 ? 2 : (c.acc_bufs == 2 ? 1 : 0);
+  p.div_tiles_n = fast_div(c.tiles_n);
+  p.div_splits = fast_div(c.splits);
+  p.div_ow = fast_div(g.is_conv ? g.OW : 1);
+  p.div_oh = fast_div(g.is_conv ? g.OH : 1);
+  p.div_s = fast_div(g.is_conv ? g.cs.S : 1);
+  p.div_cblks = fast_div(c.cblks);
+  p.tmem_cols = c.tmem_cols;
   p.split_hh = (c.nacc == 3 && c.acc_bufs == 1 && 4 * c.BN <= 512 && knob(kSplitHh) != 0) ? 1 : 0;
   if (p.split_hh) p.tmem_cols = 512;
   p.is_conv = g.is_conv ? 1 : 0;

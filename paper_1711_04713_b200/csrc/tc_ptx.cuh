@@ -320,6 +320,72 @@ __device__ __forceinline__ void mma_kstep(uint32_t d0, uint32_t d1, uint32_t d2,
   }
 }
 
+// `STEPS` consecutive k-steps of one product, as one instruction sequence.
+#define ADAPTION_MMA_STEPS(CG, MORE)                                       \
+  asm volatile(                                                             \
+      "{\n"                                                                 \
+      ".reg .pred p, q;\n"                                                  \
+      ".reg .b32 x, y;\n"                                                   \
+      ".reg .b64 da, db;\n"                                                 \
+      "setp.ne.b32 p, %5, 0;\n"                                             \
+      "setp.eq.b32 q, %3, %3;\n"                                            \
+      "mov.b64 da, {%1, %3};\n"                                             \
+      "mov.b64 db, {%2, %3};\n"                                             \
+      "tcgen05.mma.cta_group::" CG ".kind::i8 [%0], da, db, %4, p;\n" MORE "}\n" ::"r"(d), \
+      "r"(a), "r"(b), "r"(dhi), "r"(id), "r"(acc)                            \
+      : "memory")
+#define ADAPTION_MMA_NEXT(CG, OFF)                                          \
+  "add.u32 x, %1, " OFF ";\n"                                               \
+  "add.u32 y, %2, " OFF ";\n"                                               \
+  "mov.b64 da, {x, %3};\n"                                                  \
+  "mov.b64 db, {y, %3};\n"                                                  \
+  "tcgen05.mma.cta_group::" CG ".kind::i8 [%0], da, db, %4, q;\n"
+template <bool PAIR>
+__device__ __forceinline__ void mma_single_kblock(uint32_t d, uint32_t a, uint32_t b, uint32_t dhi, uint32_t id,
+                                                  int ksteps, uint32_t acc) {
+  if (PAIR) {
+    if (ksteps == 4)
+      ADAPTION_MMA_STEPS("2", ADAPTION_MMA_NEXT("2", "2") ADAPTION_MMA_NEXT("2", "4") ADAPTION_MMA_NEXT("2", "6"));
+    else if (ksteps == 3)
+      ADAPTION_MMA_STEPS("2", ADAPTION_MMA_NEXT("2", "2") ADAPTION_MMA_NEXT("2", "4"));
+    else if (ksteps == 2)
+      ADAPTION_MMA_STEPS("2", ADAPTION_MMA_NEXT("2", "2"));
+    else
+      ADAPTION_MMA_STEPS("2", "");
+  } else {
+    if (ksteps == 4)
+      ADAPTION_MMA_STEPS("1", ADAPTION_MMA_NEXT("1", "2") ADAPTION_MMA_NEXT("1", "4") ADAPTION_MMA_NEXT("1", "6"));
+    else if (ksteps == 3)
+      ADAPTION_MMA_STEPS("1", ADAPTION_MMA_NEXT("1", "2") ADAPTION_MMA_NEXT("1", "4"));
+    else if (ksteps == 2)
+      ADAPTION_MMA_STEPS("1", ADAPTION_MMA_NEXT("1", "2"));
+    else
+      ADAPTION_MMA_STEPS("1", "");
+  }
+}
+#undef ADAPTION_MMA_STEPS
+#undef ADAPTION_MMA_NEXT
+
+// All k-steps of one k-block (1, 2 or 4 of them; with PARTIAL also 3).  a0: low descriptor word of the first
+// plane of A, b0 of B; the other planes and the k-steps are fixed offsets in 16-byte units.
+template <int NAX, int NBW, bool PAIR, bool PARTIAL>
+__device__ __forceinline__ void mma_kblock(uint32_t d0, uint32_t d1, uint32_t d2, uint32_t a0, uint32_t off_a1, uint32_t b0,
+                                           uint32_t b_u, uint32_t dhi, uint32_t id_ss, uint32_t id_su, uint32_t id_us,
+                                           uint32_t id_uu, int ksteps, uint32_t acc) {
+  if (NAX == 1 && NBW == 1) {
+    mma_single_kblock<PAIR>(d0, a0, b0, dhi, id_ss, ksteps, acc);
+    return;
+  }
+  const uint32_t a1 = a0 + off_a1, b1 = b0 + b_u;
+  mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0, a1, b0, b1, dhi, id_ss, id_su, id_us, id_uu, acc);
+  if (ksteps > 1) mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0 + 2u, a1 + 2u, b0 + 2u, b1 + 2u, dhi, id_ss, id_su, id_us, id_uu, 1u);
+  if (ksteps > 2) {
+    mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0 + 4u, a1 + 4u, b0 + 4u, b1 + 4u, dhi, id_ss, id_su, id_us, id_uu, 1u);
+    if (!PARTIAL || ksteps > 3)
+      mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0 + 6u, a1 + 6u, b0 + 6u, b1 + 6u, dhi, id_ss, id_su, id_us, id_uu, 1u);
+  }
+}
+
 // Instruction descriptor: int32 accumulate, 8-bit operands with independent signedness,
 // both K-major, M = 128, N = bn.
 __device__ __forceinline__ uint32_t make_idesc(bool a_signed, bool b_signed, int bn, int m) {

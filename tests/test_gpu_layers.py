@@ -656,3 +656,16 @@ PARTIAL_BLOCKS = [
 @pytest.mark.parametrize("with_q16", [False, True])
 def test_conv_channel_pitch_not_a_multiple_of_128(case, with_q16, cta_mode):
     run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_TENSOR, with_q16=with_q16)
+
+
+@pytest.mark.parametrize("case", [
+    (37, 64, 64, 32, 16, 3, 1, 1, 16, 16, 16, True),      # four groups, three accumulators of 32 columns
+    (37, 64, 64, 3, 64, 3, 1, 1, 8, 8, 8, True),          # four groups, packed taps, more tiles than CTAs
+    (9, 100, 101, 64, 64, 3, 1, 1, 8, 8, 8, False),       # four groups, signed outputs, ragged M
+    (20, 56, 56, 64, 128, 3, 1, 1, 8, 8, 8, True),        # two groups of wide tiles, resident weights
+    (20, 56, 56, 128, 136, 3, 1, 1, 8, 8, 8, True),       # two groups, CTA pairs, a second ragged column tile
+    (12, 56, 56, 128, 256, 3, 1, 1, 8, 8, 16, True),      # two groups of 256-column pair tiles
+    (6, 56, 56, 128, 128, 3, 1, 1, 16, 8, 16, True),      # two accumulators of 128 columns
+])
+def test_epilogue_groups_by_default(case):
+    run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_TENSOR if case[3] != 3 else B.ALGO_AUTO, with_q16=False)
