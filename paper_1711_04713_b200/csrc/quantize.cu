@@ -10,13 +10,14 @@
 //     instructions per element, so the rounding itself is single-precision arithmetic with one conversion.
 // Dense tensors (pitch == row length) are flat arrays: eight consecutive elements per thread and step.  With
 // channel padding a thread makes one 16-byte vector per plane; with a generator it quantizes the aligned blocks
-// of four that cover its up to sixteen elements and shifts the bytes into place.
+// of four that cover its up to sixteen elements and shifts the bytes into place, or, in large tensors, the lanes of
+// a warp share the blocks of several rows and assemble the vectors from shared memory.
 //
 // Measured (16 bits; before: integer arithmetic on unpacked values, as many blocks as fit walking the tensor
 // together): 268 M dense elements 275 -> 239 us (6.74 TB/s), 51 M with ReLU 55.6 -> 48.5; stochastic 558 -> 389 us
 // (4.1 TB/s, bound by the integer pipes); the parameters of VGG16 157 -> 132 us, stochastic 359 -> 249; 3.2 M pixels
-// of 3 channels 27.5 -> 28.4, stochastic 89.5 -> 34; 150001 rows of 50 in a pitch of 64 12.8 -> 12.5, stochastic
-// 40 -> 25 (chunks of rows assembled in shared memory took 18.5 and 27).
+// of 3 channels 27.5 -> 28.4, stochastic 89.5 -> 38; 150001 rows of 50 in a pitch of 64 12.8 -> 12.5, stochastic
+// 40 -> 19.4 (rows assembled in shared memory by a whole block took 18.5 and 27).
 #include "common.cuh"
 
 namespace adaption {
@@ -27,6 +28,7 @@ namespace {
 
 constexpr int kQThreads = 256;
 constexpr int kBatchItems = 40;
+constexpr int kFlatBytes = 1024;            // one plane of the rows a warp assembles at a time
 // Blocks per SM.  More than fit at a time: blocks then start in address order as others end, which the memory
 // system rewards (268 M dense elements, 16 bits: 236 us with 32 blocks of three chunks' worth per SM, 299 us with
 // the 6 that fit walking the tensor together).
@@ -42,7 +44,8 @@ struct QuantItem {
   unsigned long long count;                 // dense: groups of eight elements; padded: 16-byte vectors
   unsigned long long numel;
   long long inner;
-  uint32_t row_vecs;                        // padded: vectors per row
+  uint32_t row_vecs, inv_vecs;              // padded: vectors per row, ceil(2^32 / row_vecs)
+  int32_t warp_rows;                        // rows a warp assembles at a time; 0: one vector per thread
   int32_t aligned;                          // x on a boundary of 16 (1) or 32 bytes (2)
   int32_t frac_bits, qmin, qmax, planes;
   uint32_t key0, key1;
@@ -316,10 +319,82 @@ __device__ __forceinline__ void quantize_narrow_rows(const QuantItem& it, const 
   }
 }
 
+// sixteen bytes from byte `at` on, the first `real` of them, zeros behind
+__device__ __forceinline__ uint4 unaligned16(const uint32_t* words, int at, int real) {
+  const uint32_t* w = words + (at >> 2);
+  const uint32_t sh = 8u * (uint32_t)(at & 3);
+  uint32_t in[5], o[4];
+#pragma unroll
+  for (int j = 0; j < 5; ++j) in[j] = w[j];               // (the buffer has room for a word behind its end)
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int k = min(max(real - 4 * j, 0), 4);
+    o[j] = __funnelshift_r(in[j], in[j + 1], sh);
+    if (k < 4) o[j] &= (1u << (8 * k)) - 1u;
+  }
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// `warp_rows` rows (a multiple of four, so they start on a block boundary) per warp: the lanes quantize the rows'
+// blocks of four in input order, no element twice, and leave the bytes densely in shared memory; then each
+// lane picks up whole vectors of the padded rows from there.
+template <bool STOCH>
+__device__ __forceinline__ void quantize_rows_by_warp(const QuantItem& it, const QuantRule& rule, unsigned long long group,
+                                                      uint8_t* flat, Counts& c) {
+  const int lane = threadIdx.x & 31;
+  const unsigned long long row0 = group * (unsigned)it.warp_rows, outer = it.count;
+  if (row0 >= outer) return;
+  const int rows = (int)min((unsigned long long)it.warp_rows, outer - row0);
+  const int inner = (int)it.inner, n = rows * inner;                    // at most kFlatBytes
+  const unsigned long long f0 = row0 * (unsigned)inner;                 // a multiple of four
+  uint32_t* const flat_lo = reinterpret_cast<uint32_t*>(flat);
+  uint32_t* const flat_hi = reinterpret_cast<uint32_t*>(flat + kFlatBytes + 16);
+  __syncwarp();                                                         // (the previous rows have been picked up)
+  const int blocks = (n + 3) / 4;
+  constexpr int kAhead = 2;                                             // loads in flight per lane
+  for (int first = lane; first < blocks; first += 32 * kAhead) {
+    float4 v[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (first + 32 * u < blocks) load_block(it, f0 + 4u * (unsigned)(first + 32 * u), v[u]);
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int b = first + 32 * u;
+      if (b < blocks) {
+        uint32_t w0, w1;
+        quantize4<STOCH>(v[u], rule, (f0 >> 2) + (unsigned)b, min(4, n - 4 * b), c, w0, w1);
+        flat_lo[b] = low_bytes(w0, w1);
+        if (it.planes == 2) flat_hi[b] = high_bytes(w0, w1);
+      }
+    }
+  }
+  __syncwarp();
+  const int vecs = rows * (int)it.row_vecs;
+  uint4* const out_lo = reinterpret_cast<uint4*>(it.lo) + row0 * it.row_vecs;
+  uint4* const out_hi = reinterpret_cast<uint4*>(it.hi) + row0 * it.row_vecs;
+  for (int i = lane; i < vecs; i += 32) {
+    const int row = it.row_vecs == 1 ? i : (int)__umulhi((uint32_t)i, it.inv_vecs);
+    const int c0 = 16 * (i - row * (int)it.row_vecs), real = min(16, max(0, inner - c0));
+    uint4 l = make_uint4(0u, 0u, 0u, 0u), h = l;
+    if (real > 0) {
+      const int at = row * inner + c0;
+      l = unaligned16(flat_lo, at, real);
+      if (it.planes == 2) h = unaligned16(flat_hi, at, real);
+    }
+    __stcs(out_lo + i, l);
+    if (it.planes == 2) __stcs(out_hi + i, h);
+  }
+}
+
 // One 16-byte vector of a padded row per thread.
 template <bool STOCH>
 __device__ __forceinline__ void quantize_padded_chunk(const QuantItem& it, const QuantRule& rule, unsigned long long base,
-                                                      unsigned chunk, Counts& c) {
+                                                      unsigned chunk, uint8_t* flat, Counts& c) {
+  if (STOCH && it.warp_rows > 0) {
+    // (a chunk stands for one run of rows per warp)
+    quantize_rows_by_warp<STOCH>(it, rule, base / chunk * (kQThreads / 32) + (threadIdx.x >> 5), flat, c);
+    return;
+  }
   const unsigned long long g = base + threadIdx.x;
   if (it.row_vecs == 1 && it.inner <= 4) {
     quantize_narrow_rows<STOCH>(it, rule, g, g < it.count, c);
@@ -414,6 +489,10 @@ __device__ __forceinline__ void quantize_padded_chunk(const QuantItem& it, const
 
 template <bool STOCH, bool PADDED, int CAP>
 __global__ void __launch_bounds__(kQThreads, STOCH ? 4 : (PADDED ? 6 : 5)) quantize_kernel(const __grid_constant__ QuantArgs<CAP> a) {
+  constexpr int kFlat = 2 * (kFlatBytes + 16);
+  constexpr bool kByWarp = PADDED && STOCH;
+  __shared__ __align__(16) uint8_t flat[kByWarp ? kQThreads / 32 * kFlat : 16];
+  uint8_t* const my_flat = kByWarp ? flat + (threadIdx.x >> 5) * kFlat : flat;
   pdl_prologue();
   Counts c;
   // Chunks come in increasing order, so the search for a chunk's tensor only moves forward.
@@ -428,7 +507,7 @@ __global__ void __launch_bounds__(kQThreads, STOCH ? 4 : (PADDED ? 6 : 5)) quant
     const QuantItem& it = a.item[t];
     const unsigned long long base = (chunk - it.first_chunk) * (unsigned)a.chunk;
     if (PADDED)
-      quantize_padded_chunk<STOCH>(it, rule, base, (unsigned)a.chunk, c);
+      quantize_padded_chunk<STOCH>(it, rule, base, (unsigned)a.chunk, my_flat, c);
     else
       quantize_dense_chunk<STOCH>(it, rule, base, (unsigned)a.chunk, c);
   }
@@ -457,7 +536,17 @@ void make_item(QuantItem& it, const float* x, size_t outer, size_t inner, const 
   it.qmax = (1 << (q.fmt.n_bits - 1)) - 1;
   it.key0 = (uint32_t)seed;
   it.key1 = (uint32_t)(seed >> 32);
+  it.inv_vecs = it.row_vecs > 1 ? (uint32_t)(((1ull << 32) + it.row_vecs - 1) / it.row_vecs) : 0u;
+  it.warp_rows = 0;
   it.count = is_dense(x, inner, q) ? it.numel / 8 : (unsigned long long)outer * it.row_vecs;   // (pitches are multiples of 16)
+}
+
+// Padded tensors that a warp assembles several rows of at a time: with a generator (150001 rows of 50: 25.2 us with
+// one vector per thread, 19.4 this way; without one 13.6 and 14.1), where four rows fit, rows do not share
+// lanes (quantize_narrow_rows) and the tensor fills the chip with such runs of rows.
+bool by_warp(const QuantItem& it, bool stochastic) {
+  return stochastic && it.q16 == nullptr && it.inner * 4 <= kFlatBytes && (it.row_vecs > 1 || it.inner > 4) &&
+         it.count >= (unsigned long long)num_sms() * 1024;
 }
 
 template <bool STOCH, bool PADDED, int CAP>
@@ -472,8 +561,16 @@ int launch_quantize(QuantArgs<CAP>& a, cudaStream_t stream) {
   }
   a.total_chunks = 0;
   for (int k = 0; k < a.n; ++k) {
-    a.item[k].first_chunk = a.total_chunks;
-    a.total_chunks += (a.item[k].count + (unsigned)a.chunk - 1) / (unsigned)a.chunk;
+    QuantItem& it = a.item[k];
+    it.first_chunk = a.total_chunks;
+    if (PADDED && by_warp(it, STOCH)) {
+      it.warp_rows = (int32_t)(kFlatBytes / it.inner) & ~3;
+      it.count /= it.row_vecs;
+      const unsigned long long per_chunk = (unsigned long long)it.warp_rows * (kQThreads / 32);
+      a.total_chunks += (it.count + per_chunk - 1) / per_chunk;
+    } else {
+      a.total_chunks += (it.count + (unsigned)a.chunk - 1) / (unsigned)a.chunk;
+    }
   }
   const unsigned long long cap = (unsigned long long)num_sms() * kBlocksPerSm;
   const unsigned grid = (unsigned)(a.total_chunks < cap ? a.total_chunks : cap);

@@ -57,6 +57,27 @@ def test_rows(shape, n_bits, f, offset, relu):
         guards.check()
 
 
+@pytest.mark.parametrize("shape", [(76001, 17, 32), (40003, 50, 64), (20001, 256, 272), (160001, 5, 16)])
+def test_rows_of_a_large_tensor_stochastic(shape):
+    """Tensors large enough for a warp to assemble several rows at a time: odd row lengths, the longest rows,
+    a last run of rows that is not full."""
+    outer, inner, pitch = shape
+    rng = np.random.default_rng(outer)
+    x = _values(rng, (outer, inner), 16, 12)
+    want, cnt = orc_st.quantize_stochastic(x, 16, 12, 99 + inner, False)
+    for offset in (0, 1):
+        src = torch.zeros(outer * inner + offset, device="cuda")
+        src[offset:] = dev(x.ravel())
+        guards = Guards()
+        y = guards.qtensor(outer, inner, 16, 12, pitch)
+        st = B.new_stats()
+        B.adaption_quantize_stochastic(src[offset:], outer, inner, y, 99 + inner, False, None, st)
+        assert np.array_equal(from_qtensor(y), want)
+        assert y.padding_is_zero()
+        assert stats_tuple(st) == tuple(cnt)
+        guards.check()
+
+
 @pytest.mark.parametrize("stochastic", [False, True])
 def test_many_tensors_in_one_launch(stochastic):
     """More tensors than one launch takes, dense and padded in turn, small and large, formats on host and device."""
