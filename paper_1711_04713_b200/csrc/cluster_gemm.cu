@@ -216,6 +216,16 @@ __device__ __forceinline__ void finish_group(const long long (&v)[G], int nreal,
 #pragma unroll
     for (int j = 0; j < G; ++j) keep_range(v[j], p, vmax);
   } else if constexpr (KIND == kFinishStochastic) {
+    if (G == 8 && step == 1 && nreal == G && (index & 3) == 0) {     // two whole generator blocks
+#pragma unroll
+      for (int b = 0; b < G / 4; ++b) {
+        const uint64_t blk = (index >> 2) + (uint64_t)b;
+        const Philox4 r = philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), 0u, 0u, p.st.key0, p.st.key1);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) q[4 * b + j] = requant_value_stochastic(v[4 * b + j], p.rq, r.w[j], true, cnt);
+      }
+      return;
+    }
 #pragma unroll
     for (int j = 0; j < G; ++j) {
       q[j] = 0;
@@ -330,7 +340,7 @@ template <int KIND>
 __device__ __forceinline__ void finish_tile(const CgParams& p, const Slots& slots, const CgCtrl& ctrl, int cpo, int r0,
                                             int col_first) {
   // (eight at a time where the owned columns divide: 310 cycles per value and thread against 780)
-  const bool wide = KIND == kFinishRound && (cpo & 7) == 0;
+  const bool wide = (cpo & 7) == 0 && (KIND == kFinishRound || (KIND == kFinishStochastic && p.is_conv && p.N % 8 == 0));
   if (!p.is_conv) {
     if (wide)
       finish_inner_product<8, KIND>(p, slots, ctrl, cpo, r0, col_first);

@@ -50,8 +50,9 @@ constexpr int kThreads = 32 * (kFirstEpiWarp + kEpiWarps);
 // <= 128*255 per k, so a reduction of up to 32768 stays below 2^31.
 constexpr int64_t kMaxKPerAccumulation = 32768;
 // epilogue variants (a template parameter of the kernel): generic 64-bit, the 32-bit fast path of
-// ReLU layers, generic with stochastic rounding
-constexpr int kEpiGeneric = 0, kEpiFast = 1, kEpiStochastic = 2;
+// ReLU layers, generic with stochastic rounding, 32-bit with stochastic rounding (16 images, us: 3 -> 64 channels at
+// 224 x 224 243 -> 166, 128 -> 128 at 112 x 112 158 -> 103, the same at 8 bits 167 -> 51)
+constexpr int kEpiGeneric = 0, kEpiFast = 1, kEpiStochastic = 2, kEpiFastStochastic = 3;
 // main-loop variants: one full k-block per stage; several k-blocks per stage and / or resident weights; one
 // k-block per stage of which the last one of a tap has fewer steps (channel pitch no multiple of 128).  (Variants,
 // because the issuing warp's code decides the main loop's speed: with the bookkeeping of the third in the second
@@ -129,6 +130,7 @@ struct TcParams {
   int stall_at;
   // epilogue variants chosen on the host
   int fast_relu;              // launch the FAST kernel variant (paired 16-bit epilogue)
+  int fast_stochastic;        // ... the 32-bit one with stochastic rounding
   int pool_w;                 // store max(row 2j, row 2j+1) of the tile: half of a 2x2 max-pool (staged only)
   int epi_groups;             // 1, 2 or 4 groups of epilogue warps that take turns tile by tile
   int staged;                 // outputs leave through shared memory and bulk-tensor stores
@@ -371,6 +373,65 @@ __device__ __forceinline__ void philox_draws8(uint64_t i0, uint32_t k0, uint32_t
   for (int j = 0; j < 8; ++j) R[j] = off == 1 ? w[j + 1] : (off == 2 ? w[j + 2] : w[j + 3]);
 }
 
+// Eight consecutive outputs with stochastic rounding in 32-bit arithmetic (ReLU layers, 9 <= shift <= 31, with one
+// accumulator 1 <= shift <= 31, N a multiple of 8): with C = bias * 2^bias_shift and T, H as in fast_result
+// (without the rounding half) q = floor(v / 2^shift) is what fast_result returns, and the threshold
+// (v mod 2^shift) 2^(32 - shift) is the low 32 bits of v, v = 2^16 H + 2^8 T + (low byte of ll + Cl), shifted left.
+// Negative v give q <= -1, at most 0 after the draw: the packed maximum with zero is the ReLU.  N is a multiple
+// of 8, so the eight elements are two whole generator blocks.
+template <int NACC>
+__device__ __forceinline__ void stochastic8(const Acc8<NACC>& x, const int* cl, const int* ch, const TcParams& p,
+                                            bool row_ok, int m, int col, Counts& cnt, uint32_t* w) {
+  const bool counted = row_ok && col < p.N;
+  const int shift = p.rq.shift;
+  uint32_t R[8];
+  if (counted) {
+    const uint64_t b = ((uint64_t)m * (uint64_t)p.N + (uint64_t)col) >> 2;
+    const Philox4 r0 = philox4x32_10((uint32_t)b, (uint32_t)(b >> 32), 0u, 0u, p.st.key0, p.st.key1);
+    const Philox4 r1 = philox4x32_10((uint32_t)(b + 1), (uint32_t)((b + 1) >> 32), 0u, 0u, p.st.key0, p.st.key1);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { R[j] = r0.w[j]; R[4 + j] = r1.w[j]; }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) R[j] = 0xffffffffu;
+  }
+  int32_t q[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    int32_t f;
+    uint32_t v_lo;
+    if (NACC == 1) {
+      const int32_t v = x.a[0][j] + cl[j];
+      f = v >> shift;
+      v_lo = (uint32_t)v;
+    } else {
+      const int32_t l = x.a[NACC - 1][j] + cl[j];
+      const int32_t T = x.a[NACC - 2][j] + (l >> 8), H = (NACC == 3 ? x.a[0][j] : 0) + ch[j];
+      f = shift >= 16 ? (H + (T >> 8)) >> (shift - 16) : mad_lo(H, 1 << (16 - shift), T >> (shift - 8));
+      v_lo = ((uint32_t)H << 16) + ((uint32_t)T << 8) + ((uint32_t)l & 255u);
+    }
+    q[j] = f + (R[j] < (v_lo << (32 - shift)) ? 1 : 0);
+  }
+  const uint32_t qmax2 = (uint32_t)p.rq.qmax * 0x00010001u;
+  uint32_t nonzero = 0;
+  bool clipped = false;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t v = max_s16x2(pack_sat_s16x2(q[2 * j + 1], q[2 * j]), 0u);
+    const uint32_t c = min_s16x2(v, qmax2);
+    clipped |= (c & 0xffffu) == (uint32_t)p.rq.qmax || (c >> 16) == (uint32_t)p.rq.qmax;      // (maybe)
+    nonzero += min_s16x2(c, 0x00010001u);
+    w[j] = counted ? c : 0u;
+  }
+  if (counted) {
+    cnt.zeros += 8u - (nonzero & 0xffffu) - (nonzero >> 16);
+    if (clipped) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) cnt.sat_pos += q[j] > p.rq.qmax;
+    }
+  }
+}
+
 template <int NACC, bool RELU, bool STOCH>
 __device__ __forceinline__ void requant8(const Acc8<NACC>& x, const long long* c64, const TcParams& p, bool row_ok,
                                          int m, int col, Counts& cnt, uint32_t* w) {
@@ -529,7 +590,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
   constexpr int NACC = NAX + NBW - 1;
   constexpr bool GROUPED = LOOP == kLoopGrouped, PARTIAL = LOOP == kLoopPartial;
   constexpr bool FAST = EPI == kEpiFast;
-  constexpr bool STOCH = EPI == kEpiStochastic;
+  constexpr bool STOCH = EPI == kEpiStochastic, FASTST = EPI == kEpiFastStochastic;
   extern __shared__ uint8_t smem_raw[];
   __shared__ Ctrl ctrl;
 
@@ -933,10 +994,10 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           const int n = tc.n0 + c;
           long long b = 0;
           if (p.bias != nullptr && n < p.N && p.splits == 1) b = (long long)p.bias[n] * (1ll << p.bias_shift);
-          if (FAST) {
+          if (FAST || FASTST) {
             // two arrays of BN 32-bit words: C mod 2^16 and C div 2^16 (a single accumulator takes all
             // of C from the first), read four columns per load
-            const long long C = b + (p.rq.shift > 0 ? 1ll << (p.rq.shift - 1) : 0ll);
+            const long long C = b + (FAST && p.rq.shift > 0 ? 1ll << (p.rq.shift - 1) : 0ll);
             int* cw = reinterpret_cast<int*>(colconst);
             cw[c] = NACC == 1 ? (int)C : (int)(C & 0xffff);
             cw[p.BN + c] = (int)(C >> 16);
@@ -977,7 +1038,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       unsigned long long* const bar_hh = split ? &ctrl.tmem_empty[1u + hh_sel] : bar_rest;
       // Sixteen columns per step.  The accumulators are handed back to the issuing warp as soon as
       // the last step's values are in registers, before the arithmetic on them.
-      const bool storing = FAST || (p.splits == 1 && p.mode == ADAPTION_MODE_REQUANT);
+      const bool storing = FAST || FASTST || (p.splits == 1 && p.mode == ADAPTION_MODE_REQUANT);
       bool released = false;
       bool tile_ok = true;        // a later wait of this tile gave up: finish the tile, then leave together
       // Fast path with thirty-two columns per warp step: one TMEM load per accumulator, the low and
@@ -1117,7 +1178,11 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           partial_or_range8<NACC>(xb, bcol + 8, p, row_ok, m, col + 8, vmax);
         } else {
           uint32_t wq[8];
-          if (p.rq.relu) {
+          if (FASTST) {
+            const int* cl = reinterpret_cast<const int*>(colconst) + c0;
+            stochastic8<NACC>(xa, cl, cl + p.BN, p, row_ok, m, col, cnt, wq);
+            stochastic8<NACC>(xb, cl + 8, cl + p.BN + 8, p, row_ok, m, col + 8, cnt, wq + 4);
+          } else if (p.rq.relu) {
             requant8<NACC, true, STOCH>(xa, bcol, p, row_ok, m, col, cnt, wq);
             requant8<NACC, true, STOCH>(xb, bcol + 8, p, row_ok, m, col + 8, cnt, wq + 4);
           } else {
@@ -1473,6 +1538,7 @@ int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t s
 template <int NAX, int NBW, bool PAIR, int LOOP>
 int launch_epi(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
   if (p.fast_relu != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiFast>(maps, p, grid, smem, stream);
+  if (p.fast_stochastic != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiFastStochastic>(maps, p, grid, smem, stream);
   if (p.st.enabled != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiStochastic>(maps, p, grid, smem, stream);
   return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiGeneric>(maps, p, grid, smem, stream);
 }
@@ -1710,10 +1776,12 @@ int launch_tensor(const GemmProblem& g) {
   // finalize kernel when the reduction is split
   p.st = g.stochastic;
   if (g.mode != ADAPTION_MODE_REQUANT || c.splits > 1) p.st.enabled = 0;
-  if (g.mode == ADAPTION_MODE_REQUANT && c.splits == 1 && g.relu && !g.stochastic.enabled &&
-      p.rq.shift >= (single ? 0 : 9) &&
-      p.rq.shift <= 31 && g.N % 8 == 0 && cols_per_epi_warp >= 32 && cols_per_epi_warp % 32 == 0 &&
-      knob(kFast) != 0) {
+  // (its steps of 32 columns need that many per warp; the stochastic form takes 16, and with a shift of zero, where
+  // nothing is drawn, both do the same)
+  const bool draws = g.stochastic.enabled && p.rq.shift > 0;
+  if (g.mode == ADAPTION_MODE_REQUANT && c.splits == 1 && g.relu && p.rq.shift >= (single ? 0 : 9) &&
+      p.rq.shift <= 31 && g.N % 8 == 0 &&
+      (draws ? cols_per_epi_warp % 16 == 0 : cols_per_epi_warp >= 32 && cols_per_epi_warp % 32 == 0) && knob(kFast) != 0) {
     // 32-bit bounds of the fast epilogue (see fast_result): with a reduction of kred bytes per plane row
     // |hh| <= kred 2^14, |mid| <= kred 65280, |ll| <= kred 65025, and |C| < 2^(15 + bias_shift) + 2^(shift-1)
     const long long kred = g.is_conv ? (long long)g.cs.R * g.cs.S * g.x.c_stride : (long long)c.num_kb * c.BK;
@@ -1727,7 +1795,8 @@ int launch_tensor(const GemmProblem& g) {
       ok32 = ok32 && (hmax << (16 - p.rq.shift)) + (tmax >> (p.rq.shift - 8)) + 1 < lim;
     // single accumulator: s8 x s8 products only, the constant added in full
     if (single) ok32 = kred * 16384 + cmax < lim;
-    p.fast_relu = ok32 ? 1 : 0;
+    p.fast_relu = ok32 && !draws ? 1 : 0;
+    p.fast_stochastic = ok32 && draws ? 1 : 0;
   }
   const bool grouped_kernel = c.kps > 1 || c.b_resident;
   p.tail_stagger = (p.split_hh && p.fast_relu && !grouped_kernel && c.kb_per_split >= 3 && c.stages >= 3 &&

@@ -669,3 +669,19 @@ def test_conv_channel_pitch_not_a_multiple_of_128(case, with_q16, cta_mode):
 ])
 def test_epilogue_groups_by_default(case):
     run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_TENSOR if case[3] != 3 else B.ALGO_AUTO, with_q16=False)
+
+
+@pytest.mark.parametrize("case,fmts,f_out,mag", [
+    # shifts on both sides of 16, at the lowest of the 32-bit epilogue and below it, outputs that saturate
+    ((9, 40, 40, 16, 32, 7, 1, 1, 16, 16, 16, True), (13, 15), 10, None),     # BN = 32, four groups, shift 18
+    ((2, 24, 24, 128, 128, 3, 1, 1, 16, 16, 16, True), (4, 8), 3, (8, 8)),    # CTA pairs, shift 9
+    ((2, 24, 24, 128, 128, 3, 1, 1, 16, 16, 16, True), (4, 8), 4, (8, 8)),    # shift 8: the 64-bit epilogue
+    ((2, 24, 24, 128, 136, 3, 1, 1, 16, 16, 8, True), (8, 8), 1, (11, 11)),   # shift 15, 8-bit outputs that clip
+    ((5, 40, 40, 64, 64, 3, 1, 1, 8, 8, 8, True), (4, 7), 3, None),           # one accumulator, shift 8
+    ((5, 40, 40, 64, 64, 3, 1, 1, 8, 8, 8, True), (2, 2), 4, (4, 4)),         # one accumulator, shift 0: exact
+    ((3, 40, 40, 64, 72, 3, 1, 1, 16, 8, 16, True), (9, 7), 4, None),         # two accumulators, ragged column tile
+])
+def test_stochastic_rounding_in_32_bits(case, fmts, f_out, mag, cta_mode):
+    cnt = run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_TENSOR, f_out=f_out, fmts=fmts, mag_bits=mag,
+                        with_q16=False, stochastic_seed=0x123456789ABC + sum(case))
+    assert cnt.zeros > 0
