@@ -26,10 +26,15 @@ def calibration_loop(be, kinds: list[str], threshold: float = 0.0, group=None, d
     range, a REQUANT pass (and, with `threshold` > 0, the width histogram of that output and a second
     REQUANT pass if integer bits can go).  With a process group every range, histogram and counter
     is reduced over the replicas, so that all of them fix the same decimal points (each replica holds
-    its own shard of the batch, the weights are replicated).  Returns the per-layer records."""
+    its own shard of the batch, the weights are replicated).  Returns the per-layer records.
+
+    Only the ranges (and histograms) decide anything on the way.  A backend whose counters live on a device
+    may return None from quantize_input and requant_pass and hand all of them over afterwards through
+    ``counters(i)`` (None for the input), so that the host does not wait for every layer twice."""
     rec = []
     fx = be.input_frac_bits(threshold, group)
     rec.append({"type": "input", "frac_bits": fx, "stats": be.quantize_input(fx)})
+    layers = []
     for i, kind in enumerate(kinds):
         if kind == "pool":
             rec.append({"type": "pool", "frac_bits": be.pool(i)})
@@ -45,10 +50,16 @@ def calibration_loop(be, kinds: list[str], threshold: float = 0.0, group=None, d
             if f2 != f:
                 f = f2
                 st = be.requant_pass(i, f)
-        totals = replicas.sum_counters(int(st.zeros), int(st.sat_pos), int(st.sat_neg), device, group)
         rec.append({"type": kind, "name": be.layer_name(i), "frac_bits": f, "w_frac_bits": be.w_frac_bits(i),
-                    "max_abs_acc": A, "local_max_abs_acc": local, "acc_frac_bits": F, "stats": st,
-                    "counters_all_replicas": totals})
+                    "max_abs_acc": A, "local_max_abs_acc": local, "acc_frac_bits": F, "stats": st})
+        layers.append((i, rec[-1]))
+    if rec[0]["stats"] is None:
+        rec[0]["stats"] = be.counters(None)
+    for i, r in layers:
+        if r["stats"] is None:
+            r["stats"] = be.counters(i)
+        st = r["stats"]
+        r["counters_all_replicas"] = replicas.sum_counters(int(st.zeros), int(st.sat_pos), int(st.sat_neg), device, group)
     return rec
 
 
@@ -94,6 +105,7 @@ class _Layer:
     w_max_dev: torch.Tensor | None = None
     y: B.QTensor | None = None
     stats: torch.Tensor | None = None
+    row: int = 0             # of the network's ranges and counters
     workspace: torch.Tensor | None = None
     shape: object = None
     macs: int = 0
@@ -120,9 +132,16 @@ class LPNetwork:
         self.calibrated = False
         self.launches_per_forward = 0
 
-        self.x_fmt_dev = torch.zeros(2, dtype=torch.int32, device=device)
-        self.x_max_dev = torch.zeros(1, dtype=torch.float32, device=device)
-        self.x_stats = B.new_stats(device)
+        # What calibration clears and reads as one: (maximum, format) of the input and of every layer's weights as
+        # rows of four 32-bit words, and the counters of the input and of every layer.
+        n_layers = sum(p["type"] in ("conv", "ip") for p in params)
+        self._ranges = torch.zeros((n_layers + 1, 4), dtype=torch.int32, device=device)
+        self._all_stats = torch.zeros((n_layers + 1, B.STATS_BYTES), dtype=torch.uint8, device=device)
+        self._host_stats = torch.empty((n_layers + 1, B.STATS_BYTES), dtype=torch.uint8, pin_memory=True)
+        self._host_ranges = torch.empty((n_layers + 1, 4), dtype=torch.int32, pin_memory=True)
+        rows = iter(range(1, n_layers + 1))
+        self.x_max_dev, self.x_fmt_dev = self._range_views(0)
+        self.x_stats = self._all_stats[0]
         # A first convolution with few input channels gathers its taps into packed rows inside the
         # library (it needs no 32-byte pitch), so the network input keeps the smallest pitch.
         first = params[0] if params else None
@@ -180,11 +199,21 @@ class LPNetwork:
             if L.type in ("conv", "ip"):
                 L.b_f32 = torch.from_numpy(np.ascontiguousarray(p["b"])).to(device)
                 L.b = B.QTensor.empty(1, L.K, n_bits, 0, None, True, device)
-                L.w_fmt_dev = torch.zeros(2, dtype=torch.int32, device=device)
-                L.w_max_dev = torch.zeros(1, dtype=torch.float32, device=device)
-                L.stats = B.new_stats(device)
+                L.row = next(rows)
+                L.w_max_dev, L.w_fmt_dev = self._range_views(L.row)
+                L.stats = self._all_stats[L.row]
             self.layers.append(L)
         self.total_macs = sum(L.macs for L in self.layers)
+
+    def _range_views(self, row: int):
+        """(maximum, format) of one row of the ranges."""
+        return self._ranges[row, :1].view(torch.float32), self._ranges[row, 1:3]
+
+    def _to_host(self, src: torch.Tensor, dst: torch.Tensor) -> torch.Tensor:
+        """Copy to pinned memory and wait for it."""
+        dst.copy_(src, non_blocking=True)
+        torch.cuda.current_stream().synchronize()
+        return dst
 
     # ------------------------------------------------------------------ parameters
     def _fp32_fmt_by_threshold(self, t: torch.Tensor, threshold: float) -> int:
@@ -201,50 +230,49 @@ class LPNetwork:
             return self._quantize_params_stochastic(measure, threshold)
         if not measure:
             # fixed formats: every weight and bias tensor of the network in one library call
-            entries = []
-            for L in self.layers:
-                if L.type in ("conv", "ip"):
-                    entries.append((L.w_f32, L.w.outer, L.w.inner, L.w, None))
-                    entries.append((L.b_f32, 1, L.K, L.b, None))
-            B.adaption_quantize_batch(B.quantize_items(entries))
+            layers = [L for L in self.layers if L.type in ("conv", "ip")]
+            B.adaption_quantize_batch(B.quantize_items(self._parameter_entries(layers)))
             return
-        for L in self.layers:
-            if L.type not in ("conv", "ip"):
-                continue
-            if measure and threshold > 0:
+        layers = [L for L in self.layers if L.type in ("conv", "ip")]
+        self._weight_formats(layers, threshold)
+        B.adaption_quantize_batch(B.quantize_items(self._parameter_entries(layers)))
+
+    @staticmethod
+    def _parameter_entries(layers):
+        entries = []
+        for L in layers:
+            entries.append((L.w_f32, L.w.outer, L.w.inner, L.w, None))
+            entries.append((L.b_f32, 1, L.K, L.b, None))
+        return entries
+
+    def _weight_formats(self, layers, threshold: float):
+        """Decimal points of the weights, and of the biases with them: from max|w|, or from the thresholded
+        allocation."""
+        if threshold > 0:
+            for L in layers:
                 L.w.frac_bits = L.b.frac_bits = self._fp32_fmt_by_threshold(L.w_f32, threshold)
                 L.w_fmt_dev.copy_(torch.tensor([self.n_bits, L.w.frac_bits], dtype=torch.int32))
-                B.adaption_quantize(L.w_f32, L.w.outer, L.w.inner, L.w)
-                B.adaption_quantize(L.b_f32, 1, L.K, L.b)
-            elif measure:
-                L.w_max_dev.zero_()
-                B.adaption_measure_range(L.w_f32, self.n_bits, L.w_max_dev, L.w_fmt_dev)
-                B.adaption_quantize(L.w_f32, L.w.outer, L.w.inner, L.w, L.w_fmt_dev)
-                B.adaption_quantize(L.b_f32, 1, L.K, L.b, L.w_fmt_dev)
-        for L in self.layers:
-            if L.type in ("conv", "ip"):
-                f = int(L.w_fmt_dev.cpu()[1])
-                L.w.frac_bits = f
-                L.b.frac_bits = f
+            return
+        if not layers:
+            return
+        self._ranges[1:].zero_()
+        for L in layers:
+            B.adaption_measure_range(L.w_f32, self.n_bits, L.w_max_dev, L.w_fmt_dev)
+        host = self._to_host(self._ranges, self._host_ranges)
+        for L in layers:
+            L.w.frac_bits = L.b.frac_bits = int(host[L.row, 2])
 
     def _quantize_params_stochastic(self, measure: bool, threshold: float):
         """Weights and biases with rounding_scheme STOCHASTIC: formats as in the deterministic case
         (from max|w| or the thresholded allocation), values by the stochastic quantizer."""
-        entries, seeds = [], []
-        for L in self.layers:
-            if L.type not in ("conv", "ip"):
-                continue
-            if measure and threshold > 0:
-                L.w.frac_bits = L.b.frac_bits = self._fp32_fmt_by_threshold(L.w_f32, threshold)
-            elif measure:
-                L.w_max_dev.zero_()
-                B.adaption_measure_range(L.w_f32, self.n_bits, L.w_max_dev, L.w_fmt_dev)
-                L.w.frac_bits = L.b.frac_bits = int(L.w_fmt_dev.cpu()[1])
-            L.extra["li"] = len(seeds) // 2
-            seeds += rounding_seeds(self.rounding_seed, L.extra["li"])[:2]
-            entries.append((L.w_f32, L.w.outer, L.w.inner, L.w, None))
-            entries.append((L.b_f32, 1, L.K, L.b, None))
-        B.adaption_quantize_batch_stochastic(B.quantize_items(entries), seeds)
+        layers = [L for L in self.layers if L.type in ("conv", "ip")]
+        if measure:
+            self._weight_formats(layers, threshold)
+        seeds = []
+        for li, L in enumerate(layers):
+            L.extra["li"] = li
+            seeds += rounding_seeds(self.rounding_seed, li)[:2]
+        B.adaption_quantize_batch_stochastic(B.quantize_items(self._parameter_entries(layers)), seeds)
 
     @staticmethod
     def helper_launches(L: _Layer) -> int:
@@ -336,6 +364,9 @@ class LPNetwork:
         ``group`` (or an initialised default process group): data-parallel replicas, each calibrating
         on its own shard of the batch, agree on every decimal point (see ``calibration_loop``)."""
         self.quantize_params(measure=True, threshold=threshold)
+        # One clearing serves both passes of a layer: the range pass writes the range word, the storing pass the counts.
+        self._all_stats.zero_()
+        self._host_counters = None
         self._cal_x, self._cal_x_fmt, self._cal_in = x_f32, x_fmt, {}
         try:
             rec = calibration_loop(self, [L.type for L in self.layers], threshold, group, self.device)
@@ -357,20 +388,31 @@ class LPNetwork:
             return B.adaption_choose_frac_bits_from_hist(total, self.n_bits, threshold)
         self.x_max_dev.zero_()
         B.adaption_measure_range(x, self.n_bits, self.x_max_dev, self.x_fmt_dev)
-        local = float(self.x_max_dev.cpu()[0])
+        row = self._to_host(self._ranges[0], self._host_ranges[0])
+        local, frac_bits = float(row[:1].view(torch.float32)[0]), int(row[2])
         agreed = replicas.largest_float(local, self.device, group)
         if agreed != local:
             # fold the replicas' maximum in and let the library derive the format from it
             self.x_max_dev.fill_(agreed)
             B.adaption_measure_range(x[:0], self.n_bits, self.x_max_dev, self.x_fmt_dev)
-        return int(self.x_fmt_dev.cpu()[1])
+            frac_bits = int(self._to_host(self._ranges[0], self._host_ranges[0])[2])
+        return frac_bits
 
     def quantize_input(self, frac_bits: int):
-        self.x_stats.zero_()
         self.xq.frac_bits = frac_bits
         self._quantize_input(self._cal_x)
         self._cal_act = self.xq
-        return B.read_stats(self.x_stats)
+
+    def counters(self, i: int | None):
+        """Counters of the input (None) or of layer i after the last storing pass, all read at once."""
+        if self._host_counters is None:
+            self._all_stats.view(torch.int64)[:, 3] = 0           # (the ranges have been read)
+            self._host_counters = self._to_host(self._all_stats, self._host_stats).numpy().copy()
+        L = None if i is None else self.layers[i]
+        st = B.adaption_stats.from_buffer_copy(self._host_counters[0 if L is None else L.row].tobytes())
+        if st.status != 0:
+            raise B.AdaptionError(st.status, "input" if L is None else f"layer {L.name}")
+        return st
 
     def pool(self, i: int) -> int:
         self._cal_act = self._run_layer(self.layers[i], self._cal_act, B.MODE_REQUANT)
@@ -378,10 +420,9 @@ class LPNetwork:
 
     def range_pass(self, i: int) -> int:
         L = self.layers[i]
-        L.stats.zero_()
         self._cal_in[i] = self._cal_act
         self._run_layer(L, self._cal_act, B.MODE_RANGE)
-        st = B.read_stats(L.stats)
+        st = B.adaption_stats.from_buffer_copy(self._to_host(L.stats, self._host_stats[L.row]).numpy().tobytes())
         if st.status != 0:
             raise B.AdaptionError(st.status, f"layer {L.name} (range)")
         return int(st.max_abs_acc)
@@ -394,13 +435,10 @@ class LPNetwork:
 
     def requant_pass(self, i: int, frac_bits: int):
         L = self.layers[i]
+        if L.y is self._cal_act:            # a second storing pass of the same layer (thresholded allocation)
+            L.stats.zero_()
         L.y.frac_bits = frac_bits
-        L.stats.zero_()
         self._cal_act = self._run_layer(L, self._cal_in[i], B.MODE_REQUANT)
-        st = B.read_stats(L.stats)
-        if st.status != 0:
-            raise B.AdaptionError(st.status, f"layer {L.name}")
-        return st
 
     def width_histogram(self, i: int) -> list[int]:
         hist = B.new_hist(self.device)
