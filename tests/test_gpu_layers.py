@@ -685,3 +685,13 @@ def test_stochastic_rounding_in_32_bits(case, fmts, f_out, mag, cta_mode):
     cnt = run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_TENSOR, f_out=f_out, fmts=fmts, mag_bits=mag,
                         with_q16=False, stochastic_seed=0x123456789ABC + sum(case))
     assert cnt.zeros > 0
+
+
+@pytest.mark.parametrize("ws_offset", [0, 16])                # packed rows stored in one piece, in two halves
+@pytest.mark.parametrize("case", [
+    (2, 24, 24, 3, 264, 3, 1, 1, 16, 16, 16, True),           # two blocks of weight rows, the second ragged
+    (4, 16, 16, 1, 4104, 5, 2, 1, 16, 8, 16, False),          # more weight rows than the weight blocks hold at once
+    (1, 33, 32, 4, 8, 2, 0, 1, 8, 16, 8, True),               # one ragged block of weights, the last pixel block ragged
+])
+def test_packed_taps_weights_in_the_same_launch(case, ws_offset):
+    run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_AUTO, with_q16=False, ws_offset=ws_offset)
