@@ -905,7 +905,7 @@ int launch_cluster(const GemmProblem& g) {
     } else {
       if (i == 0 || w2)
         ok = encode_tiled_2d(&maps[i], wp[i], (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.w.c_stride, (uint32_t)c.BK,
-                             (uint32_t)kRows, swz);
+                             (uint32_t)kRows, swz, true);
       if (ok && (i == 0 || x2))
         ok = encode_tiled_2d(&maps[2 + i], xp[i], (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.x.c_stride, (uint32_t)c.BK,
                              (uint32_t)c.BN, swz);

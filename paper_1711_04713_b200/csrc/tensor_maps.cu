@@ -39,7 +39,7 @@ bool load_tensor_map_encoders() {
 }
 
 bool encode_tiled(CUtensorMap* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
-                  const uint32_t* box, const uint32_t* estr, CUtensorMapSwizzle swz) {
+                  const uint32_t* box, const uint32_t* estr, CUtensorMapSwizzle swz, bool long_rows) {
   cuuint64_t d[5], s[4];
   cuuint32_t b[5], e[5];
   for (int i = 0; i < rank; ++i) {
@@ -49,7 +49,8 @@ bool encode_tiled(CUtensorMap* map, const void* base, int rank, const uint64_t* 
     if (i > 0) s[i - 1] = strides[i - 1];
   }
   return g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, (cuuint32_t)rank, const_cast<void*>(base), d, s, b, e,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
+                        long_rows ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
