@@ -318,12 +318,14 @@ ADAPTION_API int adaption_probe_i8_peak(int32_t bn, int32_t pair, int32_t iters,
  *   "fast" 0       generic 64-bit epilogue instead of the 32-bit one        (default 1)
  *   "staged" 0     direct stores instead of shared-memory staging           (default 1)
  *   "stages" n     cap the depth of the shared-memory ring                  (default 0: none)
- *   "bk" 32|64, "bn" 32|64, "kps" 1..4, "bres" 0, "wide" 0, "epigroups" 1|2   narrower tiles etc.
+ *   "bk" 32|64, "bn" 32|64, "kps" 1..4, "bres" 0, "wide" 0, "epigroups" 1|2|4 narrower tiles etc.
  *   "split_hh" 0   three 128-column accumulators are handed back together            (default 1)
  *   "stagger" 0    the last k-blocks of a tile are issued like the others                 (default 1)
  *   "stage_bufs" 1 one output staging buffer per epilogue group even where two would fit (default 2)
  *   "cluster" 0|2  never / always the one-cluster-per-tile kernel where it can run      (default 1: heuristic)
  *   "cluster_size" 1|2|4|8, "cluster_bn" n   its cluster size and column width          (default 0: heuristic)
+ *   "pixels" 0|2|4 convolutions over a pitch of 32 channels without grouped pixels / in groups of two / of at most
+ *                  four whatever the number of tiles                                 (default 1: heuristic)
  *   "pdl" 0        layer kernels are launched without programmatic stream serialization (default 1)
  *   "timeout_us" t limit of every device-side wait in microseconds (default 0: two seconds)
  *   "stall_at" i   the copy-issuing warps of every block stop before their i-th stage with nothing

@@ -57,7 +57,8 @@ constexpr int kEpiGeneric = 0, kEpiFast = 1, kEpiStochastic = 2, kEpiFastStochas
 // k-block per stage of which the last one of a tap has fewer steps (channel pitch no multiple of 128).  (Variants,
 // because the issuing warp's code decides the main loop's speed: with the bookkeeping of the third in the second
 // 64 x 224 x 224 x 64 -> 64 took 595 us against 515.)
-constexpr int kLoopPlain = 0, kLoopGrouped = 1, kLoopPartial = 2;
+// kLoopPixels: neighbouring output pixels share a row of the GEMM, see PixelPlan.
+constexpr int kLoopPlain = 0, kLoopGrouped = 1, kLoopPartial = 2, kLoopPixels = 3;
 
 // Division by a number fixed for the launch: q = (n * mul >> 32) >> shift for 0 <= n < 2^31 (mul =
 // ceil(2^(32 + shift) / d) with 2^(shift + 1) >= d > 2^shift; mul = 0 stands for d = 1).  An integer division costs a
@@ -78,6 +79,31 @@ FastDiv fast_div(int d) {
   }
   return f;
 }
+
+// Pixel grouping (kLoopPixels), for convolutions of stride 1 over a pitch of 32 channels.  With G neighbouring pixels
+// taken as one of 32 G channels (the tensor is the same bytes) a row of the GEMM covers G output pixels, its G * ys
+// columns are (pixel p, output channel), and one copy of 128 rows of 32 G bytes serves what took up to 2 G copies of
+// 32-byte rows: copies deliver one row per two cycles whatever its length, and an MMA reads its 128 rows of activations
+// from shared memory whatever its columns.  The step of input pixel u (from the first output pixel's position, before
+// padding) meets output pixel p under tap u + pad - p: it runs for the pixels p where that is a tap, a range, on the
+// accumulator columns of that range.  The weights stay in shared memory as rows of one 32-byte step, taps in
+// descending order, so the B operand of such a range is a contiguous run of rows.
+// 16 bits, us: 16 x 112 x 112 x 16 -> 16, 7x7 112 -> 55 (G = 2); 16 x 112 x 112 x 32 -> 64, 5x5 72 -> 42; 64 x 56 x 56 x 32
+// -> 32, 3x3 27.6 -> 19.4.  (With 64-byte pixels in pairs 64 x 224 x 224 x 64 -> 64 gained nothing, 457 -> 452 us: there
+// the operand bytes that the MMAs read bound both.)
+constexpr int kMaxPixelBlocks = 8;
+struct PixelPlan {
+  int G;                      // pixels per row (1: not grouped)
+  int ys, ys_shift;           // columns per pixel (pitch of the output), a power of two
+  int n_valid;                // of which real output channels
+  int S;                      // filter taps per row
+  int blocks, first;          // groups of input pixels that a row of taps reaches; the one to begin with
+  uint32_t b_plane;           // bytes of one resident weight plane
+  uint32_t row_u;             // one filter row of it, in 16-byte units
+  // per block and 32-byte step: bits 17-22 columns / 8 (0: the step meets no pixel), below them the first column
+  uint32_t step[kMaxPixelBlocks][4];
+  uint32_t b_row[kMaxPixelBlocks][4];   // where its weights start in a filter row, in 16-byte units
+};
 
 struct TcParams {
   int M, N;
@@ -137,6 +163,7 @@ struct TcParams {
   int stage_bufs;             // staging buffers per epilogue group: 1, or 2 used in turn (narrow tiles)
   uint32_t stage_off;         // offset of the staging planes from the ring base
   uint32_t const_off;         // offset of the per-column epilogue constants (8 bytes per column and group)
+  PixelPlan px;
 };
 
 // Optional per-role time stamps of CTA 0 (development builds only: -DADAPTION_TIMELINE).
@@ -301,18 +328,34 @@ __device__ __forceinline__ int32_t fast_result(int32_t t, int32_t h, int shift) 
   if (WIDE) return (h + (t >> 8)) >> (shift - 16);
   return mad_lo(h, 1 << (16 - shift), t >> (shift - 8));
 }
-// sixteen of the thirty-two columns (`half` = 0 or 1) -> eight packed words; `t` and `h` hold T and H
+// sixteen of the thirty-two columns (`half` = 0 or 1; they begin at column `col`) -> eight packed words; `t` and `h`
+// hold T and H
 // (or, with a single accumulator, t holds the sum plus its constant)
-template <int NACC, bool WIDE>
+// real columns of the eight that begin at column `col` (0, or all eight where N is a multiple of 8)
+template <bool PIX>
+__device__ __forceinline__ int real_columns8(int col, const TcParams& p) {
+  const int n = PIX ? p.px.n_valid - (col & (p.px.ys - 1)) : p.N - col;
+  return min(max(n, 0), 8);
+}
+// index of an output element among the real ones, row-major over pixels and channels
+template <bool PIX>
+__device__ __forceinline__ uint64_t element_index(int m, int col, const TcParams& p) {
+  if (PIX)
+    return ((uint64_t)m * (uint64_t)p.px.G + (uint64_t)(col >> p.px.ys_shift)) * (uint64_t)p.px.n_valid +
+           (uint64_t)(col & (p.px.ys - 1));
+  return (uint64_t)m * (uint64_t)p.N + (uint64_t)col;
+}
+
+template <int NACC, bool WIDE, bool PIX>
 __device__ __forceinline__ void fast_outputs16(const int32_t (&t)[32], const int32_t (&h)[32], int half, int shift,
-                                               int32_t qmax, bool row_ok, int col, int N, Counts& cnt,
-                                               uint32_t (&w)[8]) {
+                                               int32_t qmax, bool row_ok, int col, const TcParams& p,
+                                               Counts& cnt, uint32_t (&w)[8]) {
   const uint32_t qmax2 = (uint32_t)qmax * 0x00010001u;
   const int32_t bound = qmax == 32767 ? 32767 : qmax + 1;      // a lane that reached this may have been clipped
 #pragma unroll
   for (int g = 0; g < 2; ++g) {
     const int base = 16 * half + 8 * g;
-    const bool counted = row_ok && col + base < N;
+    const bool counted = row_ok && real_columns8<PIX>(col + 8 * g, p) > 0;
     uint32_t top = 0, nonzero = 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -379,14 +422,14 @@ __device__ __forceinline__ void philox_draws8(uint64_t i0, uint32_t k0, uint32_t
 // (v mod 2^shift) 2^(32 - shift) is the low 32 bits of v, v = 2^16 H + 2^8 T + (low byte of ll + Cl), shifted left.
 // Negative v give q <= -1, at most 0 after the draw: the packed maximum with zero is the ReLU.  N is a multiple
 // of 8, so the eight elements are two whole generator blocks.
-template <int NACC>
+template <int NACC, bool PIX>
 __device__ __forceinline__ void stochastic8(const Acc8<NACC>& x, const int* cl, const int* ch, const TcParams& p,
                                             bool row_ok, int m, int col, Counts& cnt, uint32_t* w) {
-  const bool counted = row_ok && col < p.N;
+  const bool counted = row_ok && real_columns8<PIX>(col, p) > 0;
   const int shift = p.rq.shift;
   uint32_t R[8];
   if (counted) {
-    const uint64_t b = ((uint64_t)m * (uint64_t)p.N + (uint64_t)col) >> 2;
+    const uint64_t b = element_index<PIX>(m, col, p) >> 2;
     const Philox4 r0 = philox4x32_10((uint32_t)b, (uint32_t)(b >> 32), 0u, 0u, p.st.key0, p.st.key1);
     const Philox4 r1 = philox4x32_10((uint32_t)(b + 1), (uint32_t)((b + 1) >> 32), 0u, 0u, p.st.key0, p.st.key1);
 #pragma unroll
@@ -432,15 +475,15 @@ __device__ __forceinline__ void stochastic8(const Acc8<NACC>& x, const int* cl, 
   }
 }
 
-template <int NACC, bool RELU, bool STOCH>
+template <int NACC, bool RELU, bool STOCH, bool PIX>
 __device__ __forceinline__ void requant8(const Acc8<NACC>& x, const long long* c64, const TcParams& p, bool row_ok,
                                          int m, int col, Counts& cnt, uint32_t* w) {
-  const int nvalid = row_ok ? min(max(p.N - col, 0), 8) : 0;
+  const int nvalid = row_ok ? real_columns8<PIX>(col, p) : 0;
   int32_t q[8];
   if (STOCH && p.rq.shift > 0) {
     // stochastic rounding: element index = row-major index over the real M x N outputs
     uint32_t R[8];
-    if (nvalid > 0) philox_draws8((uint64_t)m * (uint64_t)p.N + (uint64_t)col, p.st.key0, p.st.key1, R);
+    if (nvalid > 0) philox_draws8(element_index<PIX>(m, col, p), p.st.key0, p.st.key1, R);
 #pragma unroll
     for (int j = 0; j < 8; ++j)
       q[j] = j < nvalid ? requant_value_stochastic(acc_value<NACC>(x, j) + c64[j], p.rq, R[j], true, cnt)
@@ -461,10 +504,10 @@ __device__ __forceinline__ void requant8(const Acc8<NACC>& x, const long long* c
 
 // What the epilogue does with eight accumulator columns of one row in the modes that store nothing:
 // split-K partial sums go to the int64 workspace, the range mode keeps the largest magnitude.
-template <int NACC>
+template <int NACC, bool PIX>
 __device__ __forceinline__ void partial_or_range8(const Acc8<NACC>& x, const long long* c64, const TcParams& p,
                                                   bool row_ok, int m, int col, long long& vmax) {
-  if (p.splits > 1) {
+  if (!PIX && p.splits > 1) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const long long v = acc_value<NACC>(x, j);
@@ -472,12 +515,13 @@ __device__ __forceinline__ void partial_or_range8(const Acc8<NACC>& x, const lon
         atomicAdd((unsigned long long*)(p.ws + (long long)m * p.ws_ld + col + j), (unsigned long long)v);
     }
   } else {
+    const int nvalid = row_ok ? real_columns8<PIX>(col, p) : 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       long long v = acc_value<NACC>(x, j) + c64[j];
       if (p.rq.relu && v < 0) v = 0;
       v = v < 0 ? -v : v;
-      if (row_ok && col + j < p.N) vmax = v > vmax ? v : vmax;
+      if (j < nvalid) vmax = v > vmax ? v : vmax;
     }
   }
 }
@@ -586,9 +630,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
                const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
                const __grid_constant__ CUtensorMap map_y_hi, const __grid_constant__ CUtensorMap map_y_lo,
-               const TcParams p) {
+               const __grid_constant__ TcParams p) {
   constexpr int NACC = NAX + NBW - 1;
-  constexpr bool GROUPED = LOOP == kLoopGrouped, PARTIAL = LOOP == kLoopPartial;
+  constexpr bool GROUPED = LOOP == kLoopGrouped, PARTIAL = LOOP == kLoopPartial, PIX = LOOP == kLoopPixels;
   constexpr bool FAST = EPI == kEpiFast;
   constexpr bool STOCH = EPI == kEpiStochastic, FASTST = EPI == kEpiFastStochastic;
   extern __shared__ uint8_t smem_raw[];
@@ -645,7 +689,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     // Planes that are streamed through the ring: all of them, or only the activation planes when
     // the weights are resident.  With fewer streamed planes than producer warps, several warps
     // share a plane and take turns stage by stage.
-    const bool b_res = GROUPED && p.b_resident;
+    const bool b_res = PIX || (GROUPED && p.b_resident);
     const int nact = b_res ? NAX : NPLANES;
     const int kps = GROUPED ? p.kps : 1;
     const int nsub = nact >= kProducerWarps ? 1 : kProducerWarps / nact;   // warps per streamed plane
@@ -668,7 +712,20 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         // all reporting to one barrier
         // (in a pair each CTA fetches its own half of the weight rows; the bytes of both are counted
         // on the leader's barrier, which the leader arms for both)
-        if (elect_one()) {
+        if (PIX) {
+          if (elect_one()) {
+            const uint32_t bar = smem_u32(&ctrl.b_ready);
+            mbar_expect_tx(bar, NBW * p.px.b_plane);
+            uint32_t dst = ring + p.b_res_off;
+            for (int row = 0; row < p.num_kb; row += p.px.blocks, dst += p.px.row_u * 16u) {
+              const int r = p.div_s.quot(row);
+              for (int tap = 0; tap < p.px.S; ++tap)
+                for (int bplane = 0; bplane < NBW; ++bplane)
+                  tma_load_2d<false>(dst + (uint32_t)bplane * p.px.b_plane + (uint32_t)((p.px.S - 1 - tap) * p.px.ys) * 32u,
+                                     bplane == 0 ? &map_b0 : &map_b1, bar, (r * p.px.S + tap) * p.w_pitch, 0);
+            }
+          }
+        } else if (elect_one()) {
           uint32_t bar = smem_u32(&ctrl.b_ready);
           if (rank == 0) mbar_expect_tx(bar, (PAIR ? 2u : 1u) * (uint32_t)p.num_kb * NBW * p.b_bytes);
           if (PAIR) bar = mapa_rank(bar, 0);
@@ -709,11 +766,11 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           const int nkb = GROUPED ? min(kps, tc.kb_end - kb) : 1;      // k-blocks in this stage
           const bool my_turn = turn == sub;           // ring slots have fixed owners
           if (++turn == nsub) turn = 0;
-          if (GROUPED && !my_turn) {
+          if ((GROUPED || PIX) && !my_turn) {
             if (++s == p.stages) { s = 0; ph ^= 1u; turn = 0; }
             continue;
           }
-          if (GROUPED && nsub > 1 && p.is_conv) {     // (the stages in between were another warp's)
+          if ((GROUPED || PIX) && nsub > 1 && p.is_conv) {     // (the stages in between were another warp's)
             tap = p.div_cblks.quot(kb);
             cb = kb - tap * p.cblks;
             r = p.div_s.quot(tap);
@@ -733,7 +790,11 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           for (int j = 0; j < nkb; ++j) {
             if (my_turn && elect_one()) {
               if (p.is_conv) {
-                if (is_a)
+                if (PIX) {
+                  int d = sx + p.px.first;                     // (the block order begins with a full one)
+                  if (d >= p.px.blocks) d -= p.px.blocks;
+                  tma_load_im2col<false>(dst + my_off, my_map, full, 0, base_w, base_h, img, (uint16_t)d, (uint16_t)r);
+                } else if (is_a)
                   tma_load_im2col<PAIR>(dst + my_off, my_map, full, cb * p.BK, base_w, base_h, img, (uint16_t)sx,
                                         (uint16_t)r);
                 else
@@ -794,10 +855,12 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     // The warp walks the stages in uniform control flow; one elected lane issues.
     if (rank == 0) {
       const int tile_rows = PAIR ? 2 * kBM : kBM;
-      const uint32_t id_ss = make_idesc(true, true, p.BN, tile_rows);
-      const uint32_t id_su = make_idesc(true, false, p.BN, tile_rows);
-      const uint32_t id_us = make_idesc(false, true, p.BN, tile_rows);
-      const uint32_t id_uu = make_idesc(false, false, p.BN, tile_rows);
+      const int id_n = PIX ? 0 : p.BN;                              // (PIX: filled in step by step)
+      const uint32_t id_ss = make_idesc(true, true, id_n, tile_rows);
+      const uint32_t id_su = make_idesc(true, false, id_n, tile_rows);
+      const uint32_t id_us = make_idesc(false, true, id_n, tile_rows);
+      const uint32_t id_uu = make_idesc(false, false, id_n, tile_rows);
+      const uint32_t dhi_b = smem_desc_hi(256, 6);                  // PIX: weight rows of 32 bytes
       const uint32_t dhi = smem_desc_hi(p.sbo, p.layout_type);
       const uint32_t ring_lo = smem_desc_lo(ring);
       const uint32_t stage_u = p.stage_bytes >> 4, a_u = p.a_bytes >> 4, b_u = p.b_bytes >> 4;
@@ -809,7 +872,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       uint32_t a0 = ring_lo, full_bar = full_bar0, empty_bar = empty_bar0;
       int s = 0;
       bool ok = true;
-      const bool b_res = GROUPED && p.b_resident;
+      const bool b_res = PIX || (GROUPED && p.b_resident);
       const int kps = GROUPED ? p.kps : 1;
       const uint32_t bres_lo = smem_desc_lo(ring + p.b_res_off), bres_u = NBW * b_u;
       if (b_res) {
@@ -837,9 +900,11 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         const uint32_t d0 = dset + hh_sel * (uint32_t)(3 * p.BN);
         const uint32_t d1 = dset + (uint32_t)p.BN, d2 = dset + 2u * (uint32_t)p.BN;
         uint32_t bres = bres_lo + (uint32_t)tc.kb_begin * bres_u;   // resident weights of this k-block
-        const bool stagger = !GROUPED && NAX == 2 && NBW == 2 && p.tail_stagger != 0;
+        const bool stagger = !GROUPED && !PIX && NAX == 2 && NBW == 2 && p.tail_stagger != 0;
         const int kb_main_end = stagger ? tc.kb_end - 2 : tc.kb_end;
         int cb = PARTIAL ? tc.kb_begin % p.cblks : 0;               // channel block of its tap
+        int pb = 0;                                                 // block of input pixels
+        uint32_t pb_row = bres_lo;                                  // weights of the filter row
         for (int kb = tc.kb_begin; kb < kb_main_end; kb += kps) {
           const int nkb = GROUPED ? min(kps, tc.kb_end - kb) : 1;
           int ksteps = ksteps_full;                                 // (fixed unless PARTIAL)
@@ -863,8 +928,21 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             // a0 / ak: low descriptor word of the first A plane of a k-block; the other planes and
             // the k-steps are fixed offsets (16-byte units) from it (weights: in the stage or
             // resident).  The first k-block is straight-line code; grouped stages loop over the rest.
-            mma_kblock<NAX, NBW, PAIR, PARTIAL>(d0, d1, d2, a0, off_a1, b_res ? bres : a0 + off_b0, b_u, dhi, id_ss, id_su,
-                                                id_us, id_uu, ksteps, acc);
+            if (PIX) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const uint32_t e = p.px.step[pb][i];
+                if (e != 0u) {
+                  const uint32_t col = e & 0x1ffu, n = e & ~0x1ffu, a = a0 + 2u * (uint32_t)i;
+                  const uint32_t b = pb_row + p.px.b_row[pb][i];
+                  mma_kstep<NAX, NBW, false>(d0 + col, d1 + col, d2 + col, a, a + off_a1, b, b + (p.px.b_plane >> 4), dhi,
+                                             id_ss + n, id_su + n, id_us + n, id_uu + n, i == 0 ? acc : 1u, dhi_b);
+                }
+              }
+            } else {
+              mma_kblock<NAX, NBW, PAIR, PARTIAL>(d0, d1, d2, a0, off_a1, b_res ? bres : a0 + off_b0, b_u, dhi, id_ss, id_su,
+                                                  id_us, id_uu, ksteps, acc);
+            }
             if (GROUPED) {
               // (unrolled: a loop here costs the issuing thread more than the narrow MMAs take)
 #pragma unroll
@@ -879,6 +957,9 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           }
           }
           if (GROUPED) bres += (uint32_t)nkb * bres_u;
+          if (PIX) {
+            if (++pb == p.px.blocks) { pb = 0; pb_row += p.px.row_u; }
+          }
           a0 += stage_u;
           full_bar += 8u;
           empty_bar += 8u;
@@ -968,10 +1049,11 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     const int col_begin = min(p.BN, (ew >> 2) * cols_per_warp);
     const int col_end = min(p.BN, col_begin + cols_per_warp);
     const int row = quarter * 32 + lane;   // row of the tile (and of this CTA's staging planes)
-    const int planes_bytes = kBM * p.BN * p.rq.out_planes;
+    const int plane_bytes = kBM * (PIX && p.pool_w ? p.BN >> 1 : p.BN);
+    const int planes_bytes = plane_bytes * p.rq.out_planes;
     const uint32_t stage_group = ring + p.stage_off + (uint32_t)(group * planes_bytes * p.stage_bufs);
     uint32_t stage_lo = stage_group;
-    uint32_t stage_hi = stage_lo + (uint32_t)(kBM * p.BN);
+    uint32_t stage_hi = stage_lo + (uint32_t)plane_bytes;
     uint32_t stage_turn = 0;
     // per-column epilogue constants of the current tile, one array per group, behind the staging planes
     long long* colconst = reinterpret_cast<long long*>(smem_raw + (ring - smem_u32(smem_raw)) + p.const_off) +
@@ -993,7 +1075,9 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         for (int c = 32 * ew + lane; c < p.BN; c += gthreads) {
           const int n = tc.n0 + c;
           long long b = 0;
-          if (p.bias != nullptr && n < p.N && p.splits == 1) b = (long long)p.bias[n] * (1ll << p.bias_shift);
+          const int ch = PIX ? n & (p.px.ys - 1) : n;
+          if (p.bias != nullptr && ch < (PIX ? p.px.n_valid : p.N) && p.splits == 1)
+            b = (long long)p.bias[ch] * (1ll << p.bias_shift);
           if (FAST || FASTST) {
             // two arrays of BN 32-bit words: C mod 2^16 and C div 2^16 (a single accumulator takes all
             // of C from the first), read four columns per load
@@ -1011,7 +1095,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       // (with two buffers in turn: the store from two tiles ago)
       if (p.stage_bufs == 2) {
         stage_lo = stage_group + stage_turn * (uint32_t)planes_bytes;
-        stage_hi = stage_lo + (uint32_t)(kBM * p.BN);
+        stage_hi = stage_lo + (uint32_t)plane_bytes;
         stage_turn ^= 1u;
         if (p.staged && store_leader) bulk_wait_read_all_but_one();
       } else if (p.staged && store_leader) {
@@ -1051,18 +1135,33 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           if (split) release_accumulators<PAIR>(bar_hh, lane);
           released = true;
         }
-        for (int c0 = col_begin; c0 < col_end; c0 += 32) {
+        for (int cv = col_begin; cv < col_end; cv += 32) {
           int32_t t[32], h[32];
+          // two runs of sixteen columns, next to each other; grouped pixels that are pooled in pairs: the same
+          // channels of two neighbouring pixels
+          int c0 = cv, run = 16;
+          const bool pool_px = PIX && p.pool_w != 0;
+          if (pool_px) {
+            run = p.px.ys;
+            c0 = (cv & ~(2 * run - 1)) + ((cv & (2 * run - 1)) >> 1);
+          }
           const int4* cl4 = reinterpret_cast<const int4*>(reinterpret_cast<const int*>(colconst) + c0);
           const int4* ch4 = reinterpret_cast<const int4*>(reinterpret_cast<const int*>(colconst) + p.BN + c0);
+          const int run4 = (run >> 2) - 4;       // what the second run's constants are further on
+          const auto load32 = [&](uint32_t at, int32_t (&r)[32]) {
+            if (PIX)
+              tmem_ld16x2(at, (uint32_t)run, r);
+            else
+              tmem_ld32(at, r);
+          };
           if (NACC == 3) {
-            tmem_ld32(taddr + (uint32_t)(c0 + 2 * p.BN), t);       // ll
-            if (!stagger) tmem_ld32(taddr + (uint32_t)(c0 + p.BN), h);   // mid
+            load32(taddr + (uint32_t)(c0 + 2 * p.BN), t);       // ll
+            if (!stagger) load32(taddr + (uint32_t)(c0 + p.BN), h);   // mid
           } else if (NACC == 2) {
-            tmem_ld32(taddr + (uint32_t)(c0 + p.BN), t);           // weight 1
-            tmem_ld32(taddr + (uint32_t)c0, h);                    // weight 2^8
+            load32(taddr + (uint32_t)(c0 + p.BN), t);           // weight 1
+            load32(taddr + (uint32_t)c0, h);                    // weight 2^8
           } else {
-            tmem_ld32(taddr + (uint32_t)c0, t);
+            load32(taddr + (uint32_t)c0, t);
           }
           tmem_ld_wait();
           pin_after_wait32(t);
@@ -1071,7 +1170,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             // fold the constant into the low accumulator while the middle one completes, then fetch it
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-              const int4 c = cl4[j];
+              const int4 c = cl4[j + (PIX && j >= 4 ? run4 : 0)];
               t[4 * j + 0] = (t[4 * j + 0] + c.x) >> 8;
               t[4 * j + 1] = (t[4 * j + 1] + c.y) >> 8;
               t[4 * j + 2] = (t[4 * j + 2] + c.z) >> 8;
@@ -1079,21 +1178,21 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             }
             tile_ok = wait_bar_inline(smem_u32(&ctrl.part_full[1]), bph, &ctrl, p) && tile_ok;
             tc_fence_after();
-            tmem_ld32(taddr + (uint32_t)(c0 + p.BN), h);           // mid
+            load32(taddr + (uint32_t)(c0 + p.BN), h);           // mid
             tmem_ld_wait();
             pin_after_wait32(h);
 #pragma unroll
             for (int j = 0; j < 32; ++j) t[j] += h[j];             // T
           }
           // the low and middle accumulators are in registers: with the split release they go back now
-          if (split && c0 + 32 >= col_end) {
+          if (split && cv + 32 >= col_end) {
             release_accumulators<PAIR>(bar_rest, lane);
             if (lane == 0 && (ew & 3) == 0) TL_STAMP(2 + (ew >> 2), tile_iter, 3);
           }
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             if (NACC == 3 && stagger) break;
-            const int4 c = cl4[j];
+            const int4 c = cl4[j + (PIX && j >= 4 ? run4 : 0)];
             if (NACC >= 2) {                                       // T = mid + floor((ll + Cl) / 2^8)
               t[4 * j + 0] = h[4 * j + 0] + ((t[4 * j + 0] + c.x) >> 8);
               t[4 * j + 1] = h[4 * j + 1] + ((t[4 * j + 1] + c.y) >> 8);
@@ -1108,11 +1207,11 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
               tile_ok = wait_bar_inline(smem_u32(&ctrl.tmem_full[buf]), bph, &ctrl, p) && tile_ok;
               tc_fence_after();
             }
-            tmem_ld32(taddr + hh_off + (uint32_t)c0, h);           // hh
+            load32(taddr + hh_off + (uint32_t)c0, h);           // hh
             tmem_ld_wait();
             pin_after_wait32(h);
           }
-          if (c0 + 32 >= col_end) {
+          if (cv + 32 >= col_end) {
             release_accumulators<PAIR>(bar_hh, lane);
             if (lane == 0 && (ew & 3) == 0) TL_STAMP(2 + (ew >> 2), tile_iter, 4);
             released = true;
@@ -1120,7 +1219,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           if (NACC >= 2) {                                         // H = hh + Ch
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-              const int4 c = ch4[j];
+              const int4 c = ch4[j + (PIX && j >= 4 ? run4 : 0)];
               if (NACC == 3) {
                 h[4 * j + 0] += c.x; h[4 * j + 1] += c.y; h[4 * j + 2] += c.z; h[4 * j + 3] += c.w;
               } else {
@@ -1128,17 +1227,27 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
               }
             }
           }
-          const int col = tc.n0 + c0;
           const bool wide = NACC == 1 || p.rq.shift >= 16;
+          uint32_t left[8];
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
             uint32_t wq[8];
+            const int col = tc.n0 + c0 + half * run;
             if (wide)
-              fast_outputs16<NACC, true>(t, h, half, p.rq.shift, p.rq.qmax, row_ok, col, p.N, cnt, wq);
+              fast_outputs16<NACC, true, PIX>(t, h, half, p.rq.shift, p.rq.qmax, row_ok, col, p, cnt, wq);
             else
-              fast_outputs16<NACC, false>(t, h, half, p.rq.shift, p.rq.qmax, row_ok, col, p.N, cnt, wq);
+              fast_outputs16<NACC, false, PIX>(t, h, half, p.rq.shift, p.rq.qmax, row_ok, col, p, cnt, wq);
             const int chunk = (c0 >> 4) + half;
-            if (p.staged && p.pool_w) {
+            if (pool_px) {
+              // the right pixel of a pair: its maximum with the left one, one chunk of the pooled row
+#pragma unroll
+              for (int j = 0; j < 8; ++j) left[j] = half == 0 ? wq[j] : max_s16x2(left[j], wq[j]);
+              if (half == 1) {
+                const uint32_t off = staged_offset(row, cv >> 5, p.BN >> 1);
+                st_shared_v4(stage_lo + off, plane_lo(left));
+                if (p.rq.out_planes == 2) st_shared_v4(stage_hi + off, plane_hi(left));
+              }
+            } else if (p.staged && p.pool_w) {
 #pragma unroll
               for (int j = 0; j < 8; ++j) wq[j] = max_s16x2(wq[j], __shfl_xor_sync(0xffffffffu, wq[j], 1));
               if ((lane & 1) == 0) {
@@ -1151,7 +1260,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
               st_shared_v4(stage_lo + off, plane_lo(wq));
               if (p.rq.out_planes == 2) st_shared_v4(stage_hi + off, plane_hi(wq));
             } else {
-              store16_global(wq, p, row_ok, m, col + 16 * half);
+              store16_global(wq, p, row_ok, m, col);
             }
           }
         }
@@ -1174,20 +1283,20 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         const int col = tc.n0 + c0;
         const long long* bcol = colconst + c0;
         if (!storing) {
-          partial_or_range8<NACC>(xa, bcol, p, row_ok, m, col, vmax);
-          partial_or_range8<NACC>(xb, bcol + 8, p, row_ok, m, col + 8, vmax);
+          partial_or_range8<NACC, PIX>(xa, bcol, p, row_ok, m, col, vmax);
+          partial_or_range8<NACC, PIX>(xb, bcol + 8, p, row_ok, m, col + 8, vmax);
         } else {
           uint32_t wq[8];
           if (FASTST) {
             const int* cl = reinterpret_cast<const int*>(colconst) + c0;
-            stochastic8<NACC>(xa, cl, cl + p.BN, p, row_ok, m, col, cnt, wq);
-            stochastic8<NACC>(xb, cl + 8, cl + p.BN + 8, p, row_ok, m, col + 8, cnt, wq + 4);
+            stochastic8<NACC, PIX>(xa, cl, cl + p.BN, p, row_ok, m, col, cnt, wq);
+            stochastic8<NACC, PIX>(xb, cl + 8, cl + p.BN + 8, p, row_ok, m, col + 8, cnt, wq + 4);
           } else if (p.rq.relu) {
-            requant8<NACC, true, STOCH>(xa, bcol, p, row_ok, m, col, cnt, wq);
-            requant8<NACC, true, STOCH>(xb, bcol + 8, p, row_ok, m, col + 8, cnt, wq + 4);
+            requant8<NACC, true, STOCH, PIX>(xa, bcol, p, row_ok, m, col, cnt, wq);
+            requant8<NACC, true, STOCH, PIX>(xb, bcol + 8, p, row_ok, m, col + 8, cnt, wq + 4);
           } else {
-            requant8<NACC, false, STOCH>(xa, bcol, p, row_ok, m, col, cnt, wq);
-            requant8<NACC, false, STOCH>(xb, bcol + 8, p, row_ok, m, col + 8, cnt, wq + 4);
+            requant8<NACC, false, STOCH, PIX>(xa, bcol, p, row_ok, m, col, cnt, wq);
+            requant8<NACC, false, STOCH, PIX>(xb, bcol + 8, p, row_ok, m, col + 8, cnt, wq + 4);
           }
           if (p.staged && p.pool_w) {
             // Horizontal half of a 2x2 max-pool: rows 2j and 2j+1 of the tile are neighbouring
@@ -1221,8 +1330,9 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         epi_bar_sync(group, gthreads);
       }
       if (p.staged && store_leader) {
-        const int m_first = (tc.m0 + (int)rank * kBM) >> (p.pool_w ? 1 : 0);     // row of the stored tensor
-        for (int sub = 0; sub * 128 < p.BN; ++sub) {
+        const int m_first = (tc.m0 + (int)rank * kBM) >> (p.pool_w && !PIX ? 1 : 0);     // row of the stored tensor
+        const int y_cols = PIX && p.pool_w ? p.BN >> 1 : p.BN;
+        for (int sub = 0; sub * 128 < y_cols; ++sub) {
           const uint32_t so = (uint32_t)sub * (uint32_t)(kBM * 128);
           tma_store_2d(&map_y_lo, stage_lo + so, tc.n0 + sub * 128, m_first);
           if (p.rq.out_planes == 2) tma_store_2d(&map_y_hi, stage_hi + so, tc.n0 + sub * 128, m_first);
@@ -1277,6 +1387,7 @@ struct TcConfig {
   int stage_bufs = 1;
   size_t smem_bytes = 0;
   size_t workspace_bytes = 0;
+  PixelPlan px{};              // px.G > 1: pixels grouped (make_pixel_config)
 };
 
 TcConfig make_config_impl(const GemmProblem& g, bool allow_wide);
@@ -1483,6 +1594,104 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   return c;
 }
 
+// The tile configuration with groups of G pixels (see PixelPlan), or one that is not ok.
+TcConfig make_pixel_config(const GemmProblem& g, int G) {
+  TcConfig c;
+  const int S = g.cs.S, R = g.cs.R, pad = g.cs.pad_w;
+  const bool storing = g.mode == ADAPTION_MODE_REQUANT;
+  const int64_t ys = storing ? g.y.c_stride : (g.N + 31) / 32 * 32;
+  c.nax = g.x.fmt.n_bits > 8 ? 2 : 1;
+  c.nbw = g.w.fmt.n_bits > 8 ? 2 : 1;
+  c.nacc = c.nax + c.nbw - 1;
+  if ((ys != 32 && ys != 64 && ys != 128) || g.N > ys || g.cs.W % G != 0 || g.OW % G != 0 ||
+      G * ys > (c.nacc == 1 ? 256 : 128))
+    return c;
+  PixelPlan& px = c.px;
+  px.G = G;
+  px.ys = (int)ys;
+  px.ys_shift = ys == 32 ? 5 : (ys == 64 ? 6 : 7);
+  px.n_valid = (int)g.N;
+  px.S = S;
+  px.row_u = (uint32_t)(S * ys * 2);
+  px.b_plane = (uint32_t)(R * S * 32 * ys);
+  const int lead = (pad + G - 1) / G;                       // groups before the first output pixel's
+  px.blocks = lead + (S - 1 - pad + 2 * G - 1) / G;         // (pad < S)
+  if (px.blocks > kMaxPixelBlocks) return c;
+  px.first = -1;
+  uint32_t step[kMaxPixelBlocks][4] = {}, b_row[kMaxPixelBlocks][4] = {};
+  for (int d = 0; d < px.blocks; ++d)
+    for (int i = 0; i < G; ++i) {
+      const int u = (d - lead) * G + i;
+      int lo = u + pad - (S - 1), hi = u + pad;             // output pixels that see input pixel u under a tap
+      if (lo < 0) lo = 0;
+      if (hi > G - 1) hi = G - 1;
+      if (lo > hi) continue;
+      step[d][i] = (uint32_t)((hi - lo + 1) * ys / 8) << 17 | (uint32_t)(lo * ys);
+      b_row[d][i] = (uint32_t)((S - 1 - (u + pad - lo)) * ys * 2);
+      if (i == 0 && hi - lo + 1 == G && px.first < 0) px.first = d;
+    }
+  // the first MMA of a tile overwrites the accumulators: it has to cover all their columns
+  if (px.first < 0) return c;
+  for (int d = 0; d < px.blocks; ++d) {
+    const int from = (d + px.first) % px.blocks;
+    std::memcpy(px.step[d], step[from], sizeof(step[0]));
+    std::memcpy(px.b_row[d], b_row[from], sizeof(b_row[0]));
+  }
+  c.BK = G * 32;
+  c.ksteps_last = G;
+  c.swizzle = G == 4 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+  c.layout_type = G == 4 ? 2u : 4u;
+  c.BN = G * px.ys;
+  c.num_kb = c.kb_per_split = R * px.blocks;
+  // (same limits of the tensor map as in make_config_impl)
+  const int up_w = g.OW / G - g.cs.W / G - lead, up_h = g.cs.pad_h - (R - 1);
+  if (lead > 128 || g.cs.pad_h > 128 || up_w < -128 || up_h < -128 || up_w > 127 || up_h > 127) return c;
+  c.tiles_m = (int)((g.M / G + kBM - 1) / kBM);
+  c.tiles_n = 1;
+  // Too few tiles leave SMs without one: 112 x 112 x 16 -> 16, 7x7, 16 bits, ungrouped against grouped: one image (46 tiles)
+  // 14.7 us against 15.6, two 25.0 against 17.6, four 37 against 26; 112 x 112 x 32 -> 64, 5x5: one image (49) 10.5
+  // against 12.4, four (196) 22.6 against 18.8.
+  if (c.tiles_m < num_sms() / 2 && knob(kPixels) < 2) return c;
+  c.acc_bufs = 512 / (c.nacc * c.BN);
+  if (c.acc_bufs > kMaxAccBufs) c.acc_bufs = kMaxAccBufs;
+  if (c.acc_bufs == 3) c.acc_bufs = 2;
+  while (c.tmem_cols < (uint32_t)(c.acc_bufs * c.nacc * c.BN)) c.tmem_cols <<= 1;
+  c.a_bytes = (uint32_t)(kBM * c.BK);
+  c.kb_bytes = c.stage_bytes = c.nax * c.a_bytes;
+  const int out_planes = g.y.fmt.n_bits > 8 ? 2 : 1;
+  c.staged = storing && g.y.q16 == nullptr && g.y.lo != nullptr;
+  c.epi_groups = c.acc_bufs;
+  const int most_groups = c.BN <= 64 ? 4 : 2;
+  while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
+  c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) / (g.pool_w ? 2u : 1u) : 0u;
+  c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
+  const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
+  c.b_resident = true;
+  c.b_res_bytes = c.nbw * px.b_plane;
+  if (c.b_res_bytes + 3 * c.stage_bytes + 1024 > budget) return c;
+  c.stages = (int)((budget - 1024 - c.b_res_bytes) / c.stage_bytes);
+  if (c.stages > kMaxStages) c.stages = kMaxStages;
+  c.stage_off = (uint32_t)(((size_t)c.stages * c.stage_bytes + c.b_res_bytes + 1023) & ~(size_t)1023);
+  c.smem_bytes = (size_t)c.stage_off + 1024 + c.stage_out_bytes + c.const_bytes;
+  c.ok = true;
+  return c;
+}
+
+// Grouped pixels where they apply: the widest groups whose weights and stages fit.
+TcConfig make_pixel_config(const GemmProblem& g) {
+  if (knob(kPixels) == 0 || !g.is_conv || g.x.c_stride != 32 || g.w.c_stride != 32 || g.N > 128 || g.cs.stride_w != 1 ||
+      g.cs.stride_h > 8 || g.cs.R > 255 || g.cs.pad_w >= g.cs.S || g.M > (int64_t)1 << 30 ||
+      (int64_t)g.cs.R * g.cs.S * 32 > kMaxKPerAccumulation)
+    return TcConfig();
+  for (Knob k : {kSplits, kPair, kStaged, kStages, kBK, kBN, kKps, kBres, kWide, kSplitHh, kStageBufs})
+    if (knob(k) != kKnobDefaults[k]) return TcConfig();        // an override of the other tiles asks for them
+  for (int G = knob(kPixels) > 1 ? knob(kPixels) : 4; G > 1; G /= 2) {
+    const TcConfig c = make_pixel_config(g, G);
+    if (c.ok) return c;
+  }
+  return TcConfig();
+}
+
 template <int NAX, int NBW, bool PAIR, int LOOP, int EPI>
 int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
   // The dynamic shared-memory limit is a per-device attribute of the kernel: remember, per device
@@ -1553,6 +1762,7 @@ int launch_loop(const CUtensorMap* maps, const TcParams& p, int grid, size_t sme
 template <int NAX, int NBW>
 int launch_either(bool pair, const CUtensorMap* maps, const TcParams& p, int grid, size_t smem,
                   cudaStream_t stream) {
+  if (p.px.G > 1) return launch_epi<NAX, NBW, false, kLoopPixels>(maps, p, grid, smem, stream);
   return pair ? launch_loop<NAX, NBW, true>(maps, p, grid, smem, stream)
               : launch_loop<NAX, NBW, false>(maps, p, grid, smem, stream);
 }
@@ -1685,9 +1895,49 @@ int tensor_path_tiles(const GemmProblem& g, bool* split) {
 
 size_t tensor_path_workspace(const GemmProblem& g) { return make_config(g).workspace_bytes; }
 
+// The 32-bit epilogues: 1 = rounding to nearest (kEpiFast), 2 = stochastic (kEpiFastStochastic), 0 = neither applies.
+int fast_epilogue(const GemmProblem& g, const TcConfig& c, const RequantParams& rq) {
+  const bool single = c.nacc == 1;
+  // (its steps of 32 columns need that many per warp: tiles of 64 columns need the two warp groups, tiles of 32 take
+  // the generic epilogue; the stochastic form takes 16, and with a shift of zero, where nothing is drawn, both do the same)
+  const int cols_per_epi_warp = c.BN / (kEpiWarps / c.epi_groups / 4);
+  const bool draws = g.stochastic.enabled && rq.shift > 0;
+  if (!(g.mode == ADAPTION_MODE_REQUANT && c.splits == 1 && g.relu && rq.shift >= (single ? 0 : 9) && rq.shift <= 31 &&
+        g.N % 8 == 0 && (draws ? cols_per_epi_warp % 16 == 0 : cols_per_epi_warp >= 32 && cols_per_epi_warp % 32 == 0) &&
+        knob(kFast) != 0))
+    return 0;
+  // 32-bit bounds of the fast epilogue (see fast_result): with a reduction of kred bytes per plane row
+  // |hh| <= kred 2^14, |mid| <= kred 65280, |ll| <= kred 65025, and |C| < 2^(15 + bias_shift) + 2^(shift-1)
+  const long long kred = g.is_conv ? (long long)g.cs.R * g.cs.S * g.x.c_stride : (long long)c.num_kb * c.BK;
+  const long long cmax = (g.bias != nullptr ? (1ll << (15 + g.bias_shift)) : 0ll) +
+                         (rq.shift > 0 ? 1ll << (rq.shift - 1) : 0ll);
+  const long long hmax = kred * 16384 + (cmax >> 16) + 1;
+  const long long tmax = kred * 65280 + ((kred * 65025 + 65535) >> 8) + 1;
+  const long long lim = 1ll << 31;
+  bool ok32 = kred * 65025 + 65535 < lim && tmax < lim && hmax + (tmax >> 8) + 1 < lim;
+  if (rq.shift < 16 && !single) ok32 = ok32 && (hmax << (16 - rq.shift)) + (tmax >> (rq.shift - 8)) + 1 < lim;
+  // single accumulator: s8 x s8 products only, the constant added in full
+  if (single) ok32 = kred * 16384 + cmax < lim;
+  return ok32 ? (draws ? 2 : 1) : 0;
+}
+
 int launch_tensor(const GemmProblem& g) {
-  const TcConfig c = make_config(g);
+  const RequantParams rq = g.mode == ADAPTION_MODE_REQUANT ? make_requant(g.acc_frac_bits, g.y.fmt, g.relu)
+                                                           : RequantParams{0, g.relu ? 1 : 0, 0, 0, 1};
+  // (with grouped pixels only the rounding 32-bit epilogue pools)
+  TcConfig c = make_pixel_config(g);
+  if (!c.ok || (g.pool_w && !(c.staged && fast_epilogue(g, c, rq) == 1))) c = make_config(g);
   if (!c.ok) return ADAPTION_ERR_UNSUPPORTED;
+  const int G = c.px.G > 1 ? c.px.G : 1;       // output pixels per row
+  const int64_t M = g.M / G, N = G > 1 ? c.BN : g.N, y_stride = g.y.c_stride * G;
+  // the convolution that the copies of the activations see
+  adaption_conv_shape cs = g.cs;
+  const int OW = g.OW / G;
+  if (G > 1) {
+    cs.W /= G;
+    cs.pad_w = (g.cs.pad_w + G - 1) / G;
+    cs.S = cs.W - OW + 2 * cs.pad_w + 1;        // (the filter width that gives OW)
+  }
   if (!load_tensor_map_encoders()) return ADAPTION_ERR_CUDA;
 
   // plane 0 is the high byte plane when there are two, else the single plane
@@ -1698,38 +1948,45 @@ int launch_tensor(const GemmProblem& g) {
   for (int i = 0; i < 2; ++i) {
     bool ok;
     if (g.is_conv)
-      ok = encode_im2col_nhwc(&maps[i], xa[i], g.cs, g.x.c_stride, (uint32_t)c.BK, (uint32_t)kBM, c.swizzle);
+      ok = encode_im2col_nhwc(&maps[i], xa[i], cs, g.x.c_stride * G, (uint32_t)c.BK, (uint32_t)kBM, c.swizzle);
     else
       ok = encode_tiled_2d(&maps[i], xa[i], (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.x.c_stride,
                            (uint32_t)c.BK, (uint32_t)c.a_rows, c.swizzle);
     if (!ok) return ADAPTION_ERR_CUDA;
     const uint64_t wk = g.is_conv ? (uint64_t)g.cs.R * g.cs.S * g.w.c_stride : (uint64_t)g.K;
     const uint64_t wpitch = g.is_conv ? wk : (uint64_t)g.w.c_stride;
-    if (!encode_tiled_2d(&maps[2 + i], wb[i], wk, (uint64_t)g.N, wpitch, (uint32_t)c.BK,
-                         (uint32_t)(c.pair ? c.BN / 2 : c.BN), c.swizzle))
+    const bool rows32 = G > 1;                 // grouped pixels: weight rows of one 32-byte step
+    if (!encode_tiled_2d(&maps[2 + i], wb[i], wk, (uint64_t)g.N, wpitch, rows32 ? 32u : (uint32_t)c.BK,
+                         (uint32_t)(rows32 ? c.px.ys : (c.pair ? c.BN / 2 : c.BN)),
+                         rows32 ? CU_TENSOR_MAP_SWIZZLE_32B : c.swizzle))
       return ADAPTION_ERR_CUDA;
   }
 
   if (c.staged) {
-    const int ybox = c.BN < 128 ? c.BN : 128;       // wider tiles leave as several stores of 128 columns
+    // rows and columns of a stored tile: pooling halves the rows, or with grouped pixels the columns
+    const bool halve_rows = g.pool_w && G == 1, halve_cols = g.pool_w && G > 1;
+    const int ycols = halve_cols ? c.BN / 2 : c.BN;
+    const int ybox = ycols < 128 ? ycols : 128;     // wider tiles leave as several stores of 128 columns
+    const uint64_t ypitch = (uint64_t)(halve_cols ? y_stride / 2 : y_stride);
     const CUtensorMapSwizzle yswz = ybox == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
                                                 : (ybox == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
     const void* planes[2] = {g.y.hi, g.y.lo};
     for (int i = 0; i < 2; ++i) {
       if (planes[i] == nullptr) continue;      // single-plane outputs have no high plane
-      if (!encode_tiled_2d(&maps[4 + i], planes[i], (uint64_t)g.y.c_stride, (uint64_t)(g.pool_w ? g.M / 2 : g.M),
-                           (uint64_t)g.y.c_stride, (uint32_t)ybox, (uint32_t)(g.pool_w ? kBM / 2 : kBM), yswz))
+      if (!encode_tiled_2d(&maps[4 + i], planes[i], ypitch, (uint64_t)(halve_rows ? M / 2 : M), ypitch, (uint32_t)ybox,
+                           (uint32_t)(halve_rows ? kBM / 2 : kBM), yswz))
         return ADAPTION_ERR_CUDA;
     }
   }
 
   TcParams p;
   std::memset(&p, 0, sizeof(p));
-  p.M = (int)g.M; p.N = (int)g.N; p.tile_m = c.tile_m;
+  p.M = (int)M; p.N = (int)N; p.tile_m = c.tile_m;
   p.tiles_m = c.tiles_m; p.tiles_n = c.tiles_n; p.splits = c.splits;
   p.total_tiles = c.tiles_m * c.tiles_n * c.splits;
   p.num_kb = c.num_kb; p.kb_per_split = c.kb_per_split;
   p.BN = c.BN; p.BK = c.BK; p.ksteps = c.BK / 32;
+  p.px = c.px;
   p.ksteps_last = g.is_conv ? c.ksteps_last : p.ksteps;
   p.sbo = (uint32_t)(8 * c.BK); p.layout_type = c.layout_type;
   p.stages = c.stages; p.a_bytes = c.a_bytes; p.b_bytes = c.b_bytes; p.stage_bytes = c.stage_bytes;
@@ -1740,9 +1997,10 @@ int launch_tensor(const GemmProblem& g) {
   p.acc_shift = c.acc_bufs == 4 ? 2 : (c.acc_bufs == 2 ? 1 : 0);
   p.div_tiles_n = fast_div(c.tiles_n);
   p.div_splits = fast_div(c.splits);
-  p.div_ow = fast_div(g.is_conv ? g.OW : 1);
+  p.div_ow = fast_div(g.is_conv ? OW : 1);
   p.div_oh = fast_div(g.is_conv ? g.OH : 1);
-  p.div_s = fast_div(g.is_conv ? g.cs.S : 1);
+  const int taps_s = G > 1 ? c.px.blocks : g.cs.S;       // k-blocks per filter row and channel block
+  p.div_s = fast_div(g.is_conv ? taps_s : 1);
   p.div_cblks = fast_div(c.cblks);
   p.tmem_cols = c.tmem_cols;
   p.split_hh = (c.nacc == 3 && c.acc_bufs == 1 && 4 * c.BN <= 512 && knob(kSplitHh) != 0) ? 1 : 0;
@@ -1750,16 +2008,14 @@ int launch_tensor(const GemmProblem& g) {
   p.is_conv = g.is_conv ? 1 : 0;
   p.cblks = c.cblks;
   if (g.is_conv) {
-    p.OH = g.OH; p.OW = g.OW; p.S = g.cs.S; p.w_pitch = (int)g.w.c_stride;
-    p.stride_h = g.cs.stride_h; p.stride_w = g.cs.stride_w; p.pad_h = g.cs.pad_h; p.pad_w = g.cs.pad_w;
+    p.OH = g.OH; p.OW = OW; p.S = taps_s; p.w_pitch = (int)g.w.c_stride;
+    p.stride_h = g.cs.stride_h; p.stride_w = g.cs.stride_w; p.pad_h = g.cs.pad_h; p.pad_w = cs.pad_w;
   }
   p.bias = g.bias; p.bias_shift = g.bias_shift;
   p.mode = g.mode;
+  p.rq = rq;
   if (g.mode == ADAPTION_MODE_REQUANT) {
-    p.rq = make_requant(g.acc_frac_bits, g.y.fmt, g.relu);
-    p.y_hi = (int8_t*)g.y.hi; p.y_lo = (uint8_t*)g.y.lo; p.y_q16 = g.y.q16; p.y_stride = g.y.c_stride;
-  } else {
-    p.rq = RequantParams{0, g.relu ? 1 : 0, 0, 0, 1};
+    p.y_hi = (int8_t*)g.y.hi; p.y_lo = (uint8_t*)g.y.lo; p.y_q16 = g.y.q16; p.y_stride = y_stride;
   }
   if (g.pool_w && !(c.staged && g.M % 2 == 0)) return ADAPTION_ERR_UNSUPPORTED;
   p.pool_w = g.pool_w ? 1 : 0;
@@ -1768,36 +2024,13 @@ int launch_tensor(const GemmProblem& g) {
   p.stage_bufs = c.stage_bufs;
   p.stage_off = c.stage_off;
   p.const_off = c.stage_off + c.stage_out_bytes;
-  const bool single = c.nacc == 1;
-  // (its epilogue takes 32 columns per warp step: tiles of 64 columns need the two warp groups,
-  // tiles of 32 columns take the generic epilogue)
-  const int cols_per_epi_warp = c.BN / (kEpiWarps / c.epi_groups / 4);
   // stochastic rounding happens where the value is requantized: in this kernel's epilogue, or in the
   // finalize kernel when the reduction is split
   p.st = g.stochastic;
   if (g.mode != ADAPTION_MODE_REQUANT || c.splits > 1) p.st.enabled = 0;
-  // (its steps of 32 columns need that many per warp; the stochastic form takes 16, and with a shift of zero, where
-  // nothing is drawn, both do the same)
-  const bool draws = g.stochastic.enabled && p.rq.shift > 0;
-  if (g.mode == ADAPTION_MODE_REQUANT && c.splits == 1 && g.relu && p.rq.shift >= (single ? 0 : 9) &&
-      p.rq.shift <= 31 && g.N % 8 == 0 &&
-      (draws ? cols_per_epi_warp % 16 == 0 : cols_per_epi_warp >= 32 && cols_per_epi_warp % 32 == 0) && knob(kFast) != 0) {
-    // 32-bit bounds of the fast epilogue (see fast_result): with a reduction of kred bytes per plane row
-    // |hh| <= kred 2^14, |mid| <= kred 65280, |ll| <= kred 65025, and |C| < 2^(15 + bias_shift) + 2^(shift-1)
-    const long long kred = g.is_conv ? (long long)g.cs.R * g.cs.S * g.x.c_stride : (long long)c.num_kb * c.BK;
-    const long long cmax = (g.bias != nullptr ? (1ll << (15 + g.bias_shift)) : 0ll) +
-                           (p.rq.shift > 0 ? 1ll << (p.rq.shift - 1) : 0ll);
-    const long long hmax = kred * 16384 + (cmax >> 16) + 1;
-    const long long tmax = kred * 65280 + ((kred * 65025 + 65535) >> 8) + 1;
-    const long long lim = 1ll << 31;
-    bool ok32 = kred * 65025 + 65535 < lim && tmax < lim && hmax + (tmax >> 8) + 1 < lim;
-    if (p.rq.shift < 16 && !single)
-      ok32 = ok32 && (hmax << (16 - p.rq.shift)) + (tmax >> (p.rq.shift - 8)) + 1 < lim;
-    // single accumulator: s8 x s8 products only, the constant added in full
-    if (single) ok32 = kred * 16384 + cmax < lim;
-    p.fast_relu = ok32 && !draws ? 1 : 0;
-    p.fast_stochastic = ok32 && draws ? 1 : 0;
-  }
+  const int fast = fast_epilogue(g, c, rq);
+  p.fast_relu = fast == 1 ? 1 : 0;
+  p.fast_stochastic = fast == 2 ? 1 : 0;
   const bool grouped_kernel = c.kps > 1 || c.b_resident;
   p.tail_stagger = (p.split_hh && p.fast_relu && !grouped_kernel && c.kb_per_split >= 3 && c.stages >= 3 &&
                     c.nax == 2 && c.nbw == 2 && knob(kStagger) != 0) ? 1 : 0;

@@ -183,7 +183,7 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
 // its own 128 rows of A and half of the B rows, and receives its 128 rows of the result in its TMEM.
 template <bool PAIR>
 __device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
-                                       uint32_t idesc, uint32_t accumulate) {
+                                       uint32_t idesc, uint32_t accumulate, uint32_t b_desc_hi) {
   if (PAIR)
     asm volatile(
         "{\n"
@@ -191,10 +191,10 @@ __device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint32_t a_lo, uint32_t 
         ".reg .b64 da, db;\n"
         "setp.ne.b32 p, %5, 0;\n"
         "mov.b64 da, {%1, %3};\n"
-        "mov.b64 db, {%2, %3};\n"
+        "mov.b64 db, {%2, %6};\n"
         "tcgen05.mma.cta_group::2.kind::i8 [%0], da, db, %4, p;\n"
         "}\n" ::"r"(d_tmem),
-        "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
+        "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(b_desc_hi)
         : "memory");
   else
     asm volatile(
@@ -203,11 +203,16 @@ __device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint32_t a_lo, uint32_t 
         ".reg .b64 da, db;\n"
         "setp.ne.b32 p, %5, 0;\n"
         "mov.b64 da, {%1, %3};\n"
-        "mov.b64 db, {%2, %3};\n"
+        "mov.b64 db, {%2, %6};\n"
         "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %4, p;\n"
         "}\n" ::"r"(d_tmem),
-        "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
+        "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(b_desc_hi)
         : "memory");
+}
+template <bool PAIR>
+__device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
+                                       uint32_t accumulate) {
+  mma_i8<PAIR>(d_tmem, a_lo, b_lo, desc_hi, idesc, accumulate, desc_hi);
 }
 // sixteen consecutive columns: the first eight into `lo`, the next eight into `hi`
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, int32_t (&lo)[8], int32_t (&hi)[8]) {
@@ -232,6 +237,20 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, int32_t (&r)[32]) {
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr)
       : "memory");
+}
+// two runs of sixteen columns, `step` columns apart
+__device__ __forceinline__ void tmem_ld16x2(uint32_t taddr, uint32_t step, int32_t (&r)[32]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[16 * h + 0]), "=r"(r[16 * h + 1]), "=r"(r[16 * h + 2]), "=r"(r[16 * h + 3]), "=r"(r[16 * h + 4]),
+          "=r"(r[16 * h + 5]), "=r"(r[16 * h + 6]), "=r"(r[16 * h + 7]), "=r"(r[16 * h + 8]), "=r"(r[16 * h + 9]),
+          "=r"(r[16 * h + 10]), "=r"(r[16 * h + 11]), "=r"(r[16 * h + 12]), "=r"(r[16 * h + 13]),
+          "=r"(r[16 * h + 14]), "=r"(r[16 * h + 15])
+        : "r"(taddr + (h ? step : 0u))
+        : "memory");
 }
 __device__ __forceinline__ void pin_after_wait32(int32_t (&r)[32]) {
   asm volatile(""
@@ -269,8 +288,8 @@ __device__ __forceinline__ uint32_t smem_desc_lo(uint32_t saddr) {
 
 // One 32-byte k-step of a tile, issued as a single instruction sequence so that the issuing thread
 // spends as few instructions per MMA as possible (its instruction stream, not the tensor pipe, is
-// what limits the mainloop otherwise).  Operand descriptors: low words a0/a1/b0/b1, shared high
-// word dhi.  acc = 0 overwrites the accumulators (first k-step of a tile).
+// what limits the mainloop otherwise).  Operand descriptors: low words a0/a1/b0/b1, high word dhi
+// for A and dhb for B.  acc = 0 overwrites the accumulators (first k-step of a tile).
 #define ADAPTION_MMA_KSTEP_2X2(CG)                                                              \
   asm volatile(                                                                                 \
       "{\n"                                                                                     \
@@ -280,21 +299,22 @@ __device__ __forceinline__ uint32_t smem_desc_lo(uint32_t saddr) {
       "setp.eq.b32 q, %7, %7;\n"                                                                \
       "mov.b64 da0, {%3, %7};\n"                                                                \
       "mov.b64 da1, {%4, %7};\n"                                                                \
-      "mov.b64 db0, {%5, %7};\n"                                                                \
-      "mov.b64 db1, {%6, %7};\n"                                                                \
+      "mov.b64 db0, {%5, %13};\n"                                                               \
+      "mov.b64 db1, {%6, %13};\n"                                                               \
       "tcgen05.mma.cta_group::" CG ".kind::i8 [%0], da0, db0, %8, p;\n"                         \
       "tcgen05.mma.cta_group::" CG ".kind::i8 [%1], da0, db1, %9, p;\n"                         \
       "tcgen05.mma.cta_group::" CG ".kind::i8 [%1], da1, db0, %10, q;\n"                        \
       "tcgen05.mma.cta_group::" CG ".kind::i8 [%2], da1, db1, %11, p;\n"                        \
       "}\n" ::"r"(d0),                                                                          \
       "r"(d1), "r"(d2), "r"(a0), "r"(a1), "r"(b0), "r"(b1), "r"(dhi), "r"(id_ss), "r"(id_su),  \
-      "r"(id_us), "r"(id_uu), "r"(acc)                                                          \
+      "r"(id_us), "r"(id_uu), "r"(acc), "r"(dhb)                                                \
       : "memory")
 
 template <bool PAIR>
 __device__ __forceinline__ void mma_kstep_2x2(uint32_t d0, uint32_t d1, uint32_t d2, uint32_t a0, uint32_t a1,
                                               uint32_t b0, uint32_t b1, uint32_t dhi, uint32_t id_ss,
-                                              uint32_t id_su, uint32_t id_us, uint32_t id_uu, uint32_t acc) {
+                                              uint32_t id_su, uint32_t id_us, uint32_t id_uu, uint32_t acc,
+                                              uint32_t dhb) {
   // hi*hi -> d0 (weight 2^16); hi*lo and lo*hi -> d1 (weight 2^8); lo*lo -> d2 (weight 1)
   if (PAIR)
     ADAPTION_MMA_KSTEP_2X2("2");
@@ -306,18 +326,25 @@ __device__ __forceinline__ void mma_kstep_2x2(uint32_t d0, uint32_t d1, uint32_t
 template <int NAX, int NBW, bool PAIR>
 __device__ __forceinline__ void mma_kstep(uint32_t d0, uint32_t d1, uint32_t d2, uint32_t a0, uint32_t a1,
                                           uint32_t b0, uint32_t b1, uint32_t dhi, uint32_t id_ss, uint32_t id_su,
-                                          uint32_t id_us, uint32_t id_uu, uint32_t acc) {
+                                          uint32_t id_us, uint32_t id_uu, uint32_t acc, uint32_t dhb) {
   if (NAX == 2 && NBW == 2) {
-    mma_kstep_2x2<PAIR>(d0, d1, d2, a0, a1, b0, b1, dhi, id_ss, id_su, id_us, id_uu, acc);
+    mma_kstep_2x2<PAIR>(d0, d1, d2, a0, a1, b0, b1, dhi, id_ss, id_su, id_us, id_uu, acc, dhb);
   } else if (NAX == 2 && NBW == 1) {
-    mma_i8<PAIR>(d0, a0, b0, dhi, id_ss, acc);          // hi*w    weight 2^8
-    mma_i8<PAIR>(d1, a1, b0, dhi, id_us, acc);          // lo*w    weight 1
+    mma_i8<PAIR>(d0, a0, b0, dhi, id_ss, acc, dhb);          // hi*w    weight 2^8
+    mma_i8<PAIR>(d1, a1, b0, dhi, id_us, acc, dhb);          // lo*w    weight 1
   } else if (NAX == 1 && NBW == 2) {
-    mma_i8<PAIR>(d0, a0, b0, dhi, id_ss, acc);          // x*hi    weight 2^8
-    mma_i8<PAIR>(d1, a0, b1, dhi, id_su, acc);          // x*lo    weight 1
+    mma_i8<PAIR>(d0, a0, b0, dhi, id_ss, acc, dhb);          // x*hi    weight 2^8
+    mma_i8<PAIR>(d1, a0, b1, dhi, id_su, acc, dhb);          // x*lo    weight 1
   } else {
-    mma_i8<PAIR>(d0, a0, b0, dhi, id_ss, acc);
+    mma_i8<PAIR>(d0, a0, b0, dhi, id_ss, acc, dhb);
   }
+}
+
+template <int NAX, int NBW, bool PAIR>
+__device__ __forceinline__ void mma_kstep(uint32_t d0, uint32_t d1, uint32_t d2, uint32_t a0, uint32_t a1,
+                                          uint32_t b0, uint32_t b1, uint32_t dhi, uint32_t id_ss, uint32_t id_su,
+                                          uint32_t id_us, uint32_t id_uu, uint32_t acc) {
+  mma_kstep<NAX, NBW, PAIR>(d0, d1, d2, a0, a1, b0, b1, dhi, id_ss, id_su, id_us, id_uu, acc, dhi);
 }
 
 // `STEPS` consecutive k-steps of one product, as one instruction sequence.
