@@ -157,6 +157,7 @@ struct TcParams {
   // epilogue variants chosen on the host
   int fast_relu;              // launch the FAST kernel variant (paired 16-bit epilogue)
   int fast_stochastic;        // ... the 32-bit one with stochastic rounding
+  int fast_range;             // range mode: 32-bit keys decide what is worth the exact 64-bit value
   int pool_w;                 // store max(row 2j, row 2j+1) of the tile: half of a 2x2 max-pool (staged only)
   int epi_groups;             // 1, 2 or 4 groups of epilogue warps that take turns tile by tile
   int staged;                 // outputs leave through shared memory and bulk-tensor stores
@@ -523,6 +524,40 @@ __device__ __forceinline__ void partial_or_range8(const Acc8<NACC>& x, const lon
       v = v < 0 ? -v : v;
       if (j < nvalid) vmax = v > vmax ? v : vmax;
     }
+  }
+}
+
+// The range mode where 32 bits hold the parts (see fast_result; C without a rounding half): floor(v / 2^16) = H + floor(T / 2^8)
+// costs six operations a value, the exact 64-bit |v| about fifteen.  `key` is floor(max |v| / 2^16) over what the warp has
+// seen; only eight columns in which some lane reaches it are looked at exactly (for a negative v the complement of its
+// quotient is compared, at most |v| / 2^16 and never below floor((|v| - 1) / 2^16), so no larger magnitude is missed).
+// With a single accumulator v itself is compared.  Columns past N add up to zero; rows past M are left out.
+// 16 images, us: 3 -> 64 channels at 224 x 224 117 -> 83, 64 -> 64 149 -> 105; 64 -> 128 at 112 x 112 65 -> 57; 8 bits, 128 ->
+// 128 at 112 x 112 41 -> 28.
+template <int NACC>
+__device__ __forceinline__ void fast_range8(const Acc8<NACC>& x, const int* cl, const int* ch, const TcParams& p, bool row_ok,
+                                            long long& vmax, int32_t& key) {
+  const int32_t flip = p.rq.relu ? 0 : -1;
+  int32_t best = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    int32_t f;
+    if (NACC == 1) {
+      f = x.a[0][j] + cl[j];
+    } else {
+      const int32_t T = x.a[NACC - 2][j] + ((x.a[NACC - 1][j] + cl[j]) >> 8);
+      f = (NACC == 3 ? x.a[0][j] : 0) + ch[j] + (T >> 8);
+    }
+    best = max(best, f ^ ((f >> 31) & flip));
+  }
+  if (__any_sync(0xffffffffu, row_ok && best >= key)) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      long long v = acc_value<NACC>(x, j) + (NACC == 1 ? (long long)cl[j] : (long long)ch[j] * 65536ll + (long long)cl[j]);
+      if (v < 0) v = p.rq.relu ? 0 : -v;
+      if (row_ok && v > vmax) vmax = v;
+    }
+    key = __reduce_max_sync(0xffffffffu, (int32_t)min(NACC == 1 ? vmax + 1 + flip : vmax >> 16, 0x7fffffffll));
   }
 }
 
@@ -1062,6 +1097,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     uint32_t tile_iter = (uint32_t)group;
     Counts cnt;
     long long vmax = 0;
+    int32_t key = 0;
     bool ok = true;
     int const_n0 = -1;          // first column of the tile whose constants are staged
     for (int t = worker + group * workers; t < p.total_tiles; t += groups * workers, tile_iter += (uint32_t)groups) {
@@ -1078,7 +1114,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           const int ch = PIX ? n & (p.px.ys - 1) : n;
           if (p.bias != nullptr && ch < (PIX ? p.px.n_valid : p.N) && p.splits == 1)
             b = (long long)p.bias[ch] * (1ll << p.bias_shift);
-          if (FAST || FASTST) {
+          if (FAST || FASTST || (EPI == kEpiGeneric && p.fast_range)) {
             // two arrays of BN 32-bit words: C mod 2^16 and C div 2^16 (a single accumulator takes all
             // of C from the first), read four columns per load
             const long long C = b + (FAST && p.rq.shift > 0 ? 1ll << (p.rq.shift - 1) : 0ll);
@@ -1282,7 +1318,11 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         if (!have) break;
         const int col = tc.n0 + c0;
         const long long* bcol = colconst + c0;
-        if (!storing) {
+        if (EPI == kEpiGeneric && p.fast_range) {
+          const int* cl = reinterpret_cast<const int*>(colconst) + c0;
+          fast_range8<NACC>(xa, cl, cl + p.BN, p, row_ok, vmax, key);
+          fast_range8<NACC>(xb, cl + 8, cl + p.BN + 8, p, row_ok, vmax, key);
+        } else if (!storing) {
           partial_or_range8<NACC, PIX>(xa, bcol, p, row_ok, m, col, vmax);
           partial_or_range8<NACC, PIX>(xb, bcol + 8, p, row_ok, m, col + 8, vmax);
         } else {
@@ -1895,6 +1935,23 @@ int tensor_path_tiles(const GemmProblem& g, bool* split) {
 
 size_t tensor_path_workspace(const GemmProblem& g) { return make_config(g).workspace_bytes; }
 
+// 32-bit bounds of the fast epilogues (see fast_result): with a reduction of kred bytes per plane row
+// |hh| <= kred 2^14, |mid| <= kred 65280, |ll| <= kred 65025, and |C| < 2^(15 + bias_shift) + 2^(shift-1).
+// Shift 0: no rounding half is added, and the result is floor(v / 2^16) (range mode) or, with one accumulator, v.
+bool fits_32_bits(const GemmProblem& g, const TcConfig& c, int shift) {
+  const bool single = c.nacc == 1;
+  const long long kred = g.is_conv ? (long long)g.cs.R * g.cs.S * g.x.c_stride : (long long)c.num_kb * c.BK;
+  const long long cmax = (g.bias != nullptr ? (1ll << (15 + g.bias_shift)) : 0ll) + (shift > 0 ? 1ll << (shift - 1) : 0ll);
+  const long long hmax = kred * 16384 + (cmax >> 16) + 1;
+  const long long tmax = kred * 65280 + ((kred * 65025 + 65535) >> 8) + 1;
+  const long long lim = 1ll << 31;
+  // single accumulator: s8 x s8 products only, the constant added in full
+  if (single) return kred * 16384 + cmax < lim;
+  bool ok = kred * 65025 + 65535 < lim && tmax < lim && hmax + (tmax >> 8) + 1 < lim;
+  if (shift > 0 && shift < 16) ok = ok && (hmax << (16 - shift)) + (tmax >> (shift - 8)) + 1 < lim;
+  return ok;
+}
+
 // The 32-bit epilogues: 1 = rounding to nearest (kEpiFast), 2 = stochastic (kEpiFastStochastic), 0 = neither applies.
 int fast_epilogue(const GemmProblem& g, const TcConfig& c, const RequantParams& rq) {
   const bool single = c.nacc == 1;
@@ -1906,19 +1963,7 @@ int fast_epilogue(const GemmProblem& g, const TcConfig& c, const RequantParams& 
         g.N % 8 == 0 && (draws ? cols_per_epi_warp % 16 == 0 : cols_per_epi_warp >= 32 && cols_per_epi_warp % 32 == 0) &&
         knob(kFast) != 0))
     return 0;
-  // 32-bit bounds of the fast epilogue (see fast_result): with a reduction of kred bytes per plane row
-  // |hh| <= kred 2^14, |mid| <= kred 65280, |ll| <= kred 65025, and |C| < 2^(15 + bias_shift) + 2^(shift-1)
-  const long long kred = g.is_conv ? (long long)g.cs.R * g.cs.S * g.x.c_stride : (long long)c.num_kb * c.BK;
-  const long long cmax = (g.bias != nullptr ? (1ll << (15 + g.bias_shift)) : 0ll) +
-                         (rq.shift > 0 ? 1ll << (rq.shift - 1) : 0ll);
-  const long long hmax = kred * 16384 + (cmax >> 16) + 1;
-  const long long tmax = kred * 65280 + ((kred * 65025 + 65535) >> 8) + 1;
-  const long long lim = 1ll << 31;
-  bool ok32 = kred * 65025 + 65535 < lim && tmax < lim && hmax + (tmax >> 8) + 1 < lim;
-  if (rq.shift < 16 && !single) ok32 = ok32 && (hmax << (16 - rq.shift)) + (tmax >> (rq.shift - 8)) + 1 < lim;
-  // single accumulator: s8 x s8 products only, the constant added in full
-  if (single) ok32 = kred * 16384 + cmax < lim;
-  return ok32 ? (draws ? 2 : 1) : 0;
+  return fits_32_bits(g, c, rq.shift) ? (draws ? 2 : 1) : 0;
 }
 
 int launch_tensor(const GemmProblem& g) {
@@ -2031,6 +2076,7 @@ int launch_tensor(const GemmProblem& g) {
   const int fast = fast_epilogue(g, c, rq);
   p.fast_relu = fast == 1 ? 1 : 0;
   p.fast_stochastic = fast == 2 ? 1 : 0;
+  p.fast_range = g.mode == ADAPTION_MODE_RANGE && c.splits == 1 && knob(kFast) != 0 && fits_32_bits(g, c, 0) ? 1 : 0;
   const bool grouped_kernel = c.kps > 1 || c.b_resident;
   p.tail_stagger = (p.split_hh && p.fast_relu && !grouped_kernel && c.kb_per_split >= 3 && c.stages >= 3 &&
                     c.nax == 2 && c.nbw == 2 && knob(kStagger) != 0) ? 1 : 0;

@@ -695,3 +695,35 @@ def test_stochastic_rounding_in_32_bits(case, fmts, f_out, mag, cta_mode):
 ])
 def test_packed_taps_weights_in_the_same_launch(case, ws_offset):
     run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_AUTO, with_q16=False, ws_offset=ws_offset)
+
+
+@pytest.mark.parametrize("nx,nw", [(16, 16), (16, 8), (8, 8)])
+@pytest.mark.parametrize("relu", [True, False])
+@pytest.mark.parametrize("where", ["first", "last", "equal quotients", "one more", "minus one"])
+def test_range_keeps_the_largest_magnitude(nx, nw, relu, where):
+    """One 1x1 convolution whose accumulators are put in place one by one: the largest magnitude sits in the first or
+    the last output, differs from the second largest in its low 16 bits only, or by one, or is -1."""
+    N, H, W, Cin, K = 5, 40, 41, 64, 72
+    xq, wq = np.zeros((N, H, W, Cin), np.int64), np.zeros((K, 1, 1, Cin), np.int64)
+    top = (1 << (nx - 1)) - 1
+    wq[:, 0, 0, 0] = (1 << (nw - 1)) - 1
+    wq[:, 0, 0, 1] = 1
+    wq[1::2] *= -1
+    if where == "minus one":
+        xq[3, 7, 9, 1] = 1
+    else:
+        xq[0 if where == "first" else -1, 0 if where == "first" else -1, 0 if where == "first" else -1, 0] = top
+        xq[2, 3, 4, 0] = top - 1
+        if where in ("equal quotients", "one more"):
+            xq[1, 1, 1, :2] = top, (top if where == "equal quotients" else 1)
+    bq = np.zeros(K, np.int16)
+    bq[-1] = -3 if where == "minus one" else 0
+    acc = orc.conv_acc(xq, wq, (0, 0), (1, 1))
+    fx, fw = nx - 3, nw - 1
+    x, w = to_qtensor(xq.reshape(-1, Cin), nx, fx, 64), to_qtensor(wq.reshape(-1, Cin), nw, fw, 64)
+    for bias in (None, bq):
+        st = B.new_stats()
+        B.adaption_lp_conv_fwd(B.conv_shape(N, H, W, Cin, K, 1, 1, 0, 1), x, w, dev(bias) if bias is not None else None,
+                               fx + fw, relu, B.MODE_RANGE, B.ALGO_TENSOR, None, st, None)
+        assert B.read_stats(st).status == 0
+        assert int(B.read_stats(st).max_abs_acc) == orc.epilogue_range(acc, bias, fx + fw, fx + fw, relu)
