@@ -336,6 +336,9 @@ ADAPTION_API int adaption_probe_i8_peak(int32_t bn, int32_t pair, int32_t iters,
  * do not change overrides while another host thread is inside a layer call. */
 ADAPTION_API int adaption_debug_set(const char* h_name, int32_t value);
 
+/* Kernels that calls of the calling host thread have launched so far (memsets and copies are not counted). */
+ADAPTION_API uint64_t adaption_launches(void);
+
 ADAPTION_API const char* adaption_status_string(int status);
 
 #ifdef __cplusplus

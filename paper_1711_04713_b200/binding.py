@@ -60,7 +60,7 @@ EXPORTS = [
     "adaption_choose_frac_bits_from_hist", "adaption_choose_frac_bits_from_widths",
     "adaption_lp_act_stochastic", "adaption_lp_conv_pool_workspace_bytes", "adaption_lp_conv_pool_fwd",
     "adaption_quantize_batch", "adaption_quantize_batch_stochastic", "adaption_debug_set", "adaption_lp_conv_fwd_stochastic",
-    "adaption_lp_ip_fwd_stochastic",
+    "adaption_lp_ip_fwd_stochastic", "adaption_launches",
 ]
 HIST_BINS = 17
 
@@ -131,6 +131,8 @@ def load(path: str | None = None):
         if name not in ("adaption_lp_conv_workspace_bytes", "adaption_lp_ip_workspace_bytes",
                         "adaption_lp_conv_pool_workspace_bytes", "adaption_status_string"):
             getattr(lib, name).restype = C.c_int
+    lib.adaption_launches.argtypes = []
+    lib.adaption_launches.restype = C.c_uint64
     if not os.path.exists(_build.NATIVE_PATH):
         raise RuntimeError(f"native half of the binding not built: {_build.NATIVE_PATH} is missing "
                            "(run `python -m paper_1711_04713_b200.build`)")
@@ -162,6 +164,11 @@ def _calls():
 def adaption_debug_set(name: str, value: int = 0):
     """Test / experiment override of the tensor-core path's heuristics (see the header)."""
     _check(load().adaption_debug_set(name.encode(), int(value)), f"adaption_debug_set({name})")
+
+
+def adaption_launches() -> int:
+    """Kernels this host thread's calls have launched so far."""
+    return load().adaption_launches()
 
 
 def status_string(status: int) -> str:

@@ -35,6 +35,9 @@ int probe_i8_peak(int bn, int pair, int iters, int commit_every, unsigned long l
 int num_sms();
 int debug_set(const char* name, int value);
 
+static thread_local uint64_t t_launches = 0;
+void count_launch() { ++t_launches; }
+
 // Longest reduction the direct kernels and the int64 workspace can take without overflow:
 // |q_x * q_w| <= 2^30, so 2^31 terms still leave a sign bit and headroom for the bias.
 static const int64_t kMaxReduction = (int64_t)1 << 31;
@@ -431,6 +434,8 @@ int adaption_probe_i8_peak(int32_t bn, int32_t pair, int32_t iters, int32_t comm
   return probe_i8_peak(bn, pair ? 1 : 0, iters, commit_every, reinterpret_cast<unsigned long long*>(d_cycles), d_status,
                        reinterpret_cast<cudaStream_t>(stream));
 }
+
+uint64_t adaption_launches(void) { return t_launches; }
 
 int adaption_debug_set(const char* h_name, int32_t value) { return debug_set(h_name, value); }
 

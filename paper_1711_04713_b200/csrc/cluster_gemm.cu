@@ -839,6 +839,7 @@ int launch_cg(const CUtensorMap* maps, const CgParams& p, int grid, size_t smem,
   }
   cfg.attrs = n_attr ? attr : nullptr;
   cfg.numAttrs = n_attr;
+  count_launch();
   const cudaError_t le = cudaLaunchKernelEx(&cfg, lp_cluster_kernel<NAX, NBW>, maps[0], maps[1], maps[2], maps[3], p);
   if (le != cudaSuccess) {
     (void)cudaGetLastError();

@@ -227,6 +227,7 @@ __device__ __forceinline__ void pdl_prologue() {
   pdl_launch_dependents();
 }
 
+void count_launch();     // one more kernel launched by this host thread (adaption_launches)
 bool pdl_enabled();      // process-wide switch (adaption_debug_set "pdl")
 
 // Launch of a kernel whose first statement is pdl_prologue().
@@ -245,6 +246,7 @@ inline cudaError_t launch_after_predecessor(void (*kernel)(KArgs...), dim3 grid,
     cfg.attrs = attr;
     cfg.numAttrs = 1;
   }
+  count_launch();
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 

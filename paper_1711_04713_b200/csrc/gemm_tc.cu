@@ -1774,6 +1774,7 @@ int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t s
   }
   cfg.attrs = n_attr ? attr : nullptr;
   cfg.numAttrs = n_attr;
+  count_launch();
   const cudaError_t le =
       cudaLaunchKernelEx(&cfg, lp_gemm_kernel<NAX, NBW, PAIR, LOOP, EPI>, maps[0], maps[1], maps[2], maps[3], maps[4],
                          maps[5], p);

@@ -274,14 +274,6 @@ class LPNetwork:
             seeds += rounding_seeds(self.rounding_seed, li)[:2]
         B.adaption_quantize_batch_stochastic(B.quantize_items(self._parameter_entries(layers)), seeds)
 
-    @staticmethod
-    def helper_launches(L: _Layer) -> int:
-        """Launches beside the layer's own kernel when it runs with a workspace: the tap packing of a
-        first layer with at most 4 channels (activations, weights), else the split-K finalize."""
-        if L.workspace is None:
-            return 0
-        return 2 if L.type == "conv" and L.C <= 4 else 1
-
     def param_quantize_launches(self) -> int:
         """Kernel launches of one quantize_params(measure=False): 40 dense tensors share a launch, and so do
         40 with padded rows."""
@@ -479,32 +471,25 @@ class LPNetwork:
         """One forward pass with the calibrated formats; enqueues work only (no host sync).
         Returns the output QTensor and the number of kernel launches issued."""
         assert self.calibrated
-        launches = 0
+        before = B.adaption_launches()
         if measure_input:
             # range of the incoming batch (monitoring; the calibrated input format stays in force)
             B.adaption_measure_range(x_f32, self.n_bits, self.x_max_dev, self.x_fmt_dev)
-            launches += 1
         self._quantize_input(x_f32)
-        launches += 1
         if requantize_params:
             self.quantize_params(measure=False)
-            launches += self.param_quantize_launches()
         a = self.xq
         i = 0
         while i < len(self.layers):
             L = self.layers[i]
             if self.fused_pool_after(i):
                 a = self._run_conv_pool(L, self.layers[i + 1], a)
-                launches += 1
                 i += 1
             else:
                 a = self._run_layer(L, a, B.MODE_REQUANT)
-            launches += 1
-            if L.workspace is not None and L.type != "pool":
-                launches += self.helper_launches(L)
             i += 1
-        self.launches_per_forward = launches
-        return a, launches
+        self.launches_per_forward = B.adaption_launches() - before
+        return a, self.launches_per_forward
 
     def zero_stats(self):
         self.x_stats.zero_()
