@@ -727,3 +727,21 @@ def test_range_keeps_the_largest_magnitude(nx, nw, relu, where):
                                fx + fw, relu, B.MODE_RANGE, B.ALGO_TENSOR, None, st, None)
         assert B.read_stats(st).status == 0
         assert int(B.read_stats(st).max_abs_acc) == orc.epilogue_range(acc, bias, fx + fw, fx + fw, relu)
+
+
+@pytest.mark.parametrize("case,f_in,shift_outs", [
+    ((6, 40, 40, 64, 64, 3, 1, 1, 8, 8, 8, True), (4, 7), (0, 1, 2, 5)),     # clipping from none to nearly all
+    ((5, 31, 33, 128, 136, 3, 1, 1, 8, 8, 8, True), (4, 7), (1,)),           # ragged rows and column tile, pairs
+    ((9, 24, 24, 3, 40, 3, 1, 1, 8, 8, 8, True), (6, 7), (0, 2)),            # packed taps, columns past N in the tile
+    ((6, 40, 40, 64, 64, 3, 1, 1, 8, 8, 4, True), (4, 7), (1,)),             # bound 7: the 16-bit form
+])
+def test_8_bit_outputs_four_to_a_word(case, f_in, shift_outs, cta_mode):
+    rng = np.random.default_rng(sum(case))
+    algo = B.ALGO_TENSOR if case[3] != 3 else B.ALGO_AUTO
+    run_conv_case(rng, *case, algo, with_q16=False)
+    clipped = [run_conv_case(rng, *case, algo, f_out=f_in[0] - 3 + d, fmts=f_in, with_q16=False).sat_pos
+               for d in shift_outs]
+    assert max(clipped) > 0
+    # shift 1, the lowest of the form, and shift 0 below it, on small accumulators
+    for f_out in (3, 4) if case[10] == 8 else (3,):
+        run_conv_case(rng, *case, algo, f_out=f_out, fmts=(2, 2), mag_bits=(3, 2), with_q16=False)
