@@ -254,3 +254,17 @@ def test_quantize_batch_matches_oracle():
         B.adaption_quantize_batch(B.quantize_items(entries[:1] + [(keep[0][0], 4, 16, bad, None)]))
     torch.cuda.synchronize()
     assert int(checks[0][1].lo.min()) == 0x11 and int(checks[0][1].lo.max()) == 0x11
+
+
+@pytest.mark.parametrize("vectors", [-2, 0, 2])
+def test_format_change_around_the_size_from_which_more_blocks_run(vectors):
+    """Dense 8-bit rows of 16 around 16 blocks of 256 pairs of vectors per SM, against the oracle."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    outer = sms * 16 * 256 * 2 + vectors
+    q = np.random.default_rng(outer).integers(-128, 128, size=(outer, 16)).astype(np.int16)
+    xin, out = to_qtensor(q, 8, 5, 16), B.QTensor.empty(outer, 16, 8, 3, 16)
+    st = B.new_stats()
+    B.adaption_lp_act(None, xin, outer, 16, True, out, None, B.ROUND_DETERMINISTIC, st)
+    want, cnt = orc.requantize(q, 5, True, 8, 3)
+    assert np.array_equal(from_qtensor(out), want)
+    assert stats_tuple(st) == (cnt.zeros, cnt.sat_pos, cnt.sat_neg)
