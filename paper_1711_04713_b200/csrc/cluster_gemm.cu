@@ -12,8 +12,9 @@
 // Operands:
 //   convolution    rows = output pixels: a box of bn images x bh rows x bw columns with
 //                  bn * bh * bw <= 128, fetched per filter tap by one tiled copy (zero fill outside the image,
-//                  element strides for strided layers), so tensors of any size qualify and the tile's
-//                  shape can follow the 2x2 windows of a pool; columns = output channels
+//                  element strides for strided layers), so tensors of few bytes qualify and the tile's
+//                  shape can follow the 2x2 windows of a pool; columns = output channels.  A row of outputs is
+//                  at most 16 boxes: widths up to 2048, with a pool (boxes of at most 64 columns) up to 1024
 //   inner product  rows = 128 output channels, columns = the batch rows: the weights take the
 //                  128-row side of the MMA, so a batch of 1 to 16 costs 16 columns instead of 128 rows
 // K-blocks are 128 bytes of one tap's channels.  Where the channel pitch is no multiple of 128 the copy's
@@ -853,7 +854,8 @@ int launch_cg(const CUtensorMap* maps, const CgParams& p, int grid, size_t smem,
 // Whether this layer runs here rather than on the persistent kernel.
 bool cluster_path_preferred(const GemmProblem& g) {
   const int mode = knob(kCluster);
-  if (mode == 0) return false;
+  // (pair maxima are stored by the persistent kernel alone; a plan with planes of half the rows has chosen it)
+  if (mode == 0 || g.pool_w) return false;
   // an override of the persistent kernel's tiles asks for that kernel
   for (Knob k : {kSplits, kPair, kFast, kStaged, kStages, kBK, kBN, kKps, kBres, kWide, kEpiGroups, kSplitHh, kStagger,
                  kStageBufs})
@@ -874,6 +876,7 @@ bool cluster_path_preferred(const GemmProblem& g) {
 }
 
 int launch_cluster(const GemmProblem& g) {
+  if (g.pool_w) return ADAPTION_ERR_UNSUPPORTED;
   const CgPlan c = make_plan(g, g.pool2x2);
   if (!c.ok) return ADAPTION_ERR_UNSUPPORTED;
   if (!load_tensor_map_encoders()) return ADAPTION_ERR_CUDA;

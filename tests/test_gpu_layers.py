@@ -503,6 +503,17 @@ def test_conv_with_fused_pool(case, with_q16):
     guards.check()
 
 
+@pytest.mark.parametrize("case", [
+    # wider than the pooled boxes of the cluster kernel reach, so few tiles that it would take the layer unpooled
+    (1, 2, 1200, 64, 64, 3, 1, 1, 16, 16, 16, True), (1, 2, 1200, 64, 64, 3, 1, 1, 8, 8, 8, True),
+    (1, 4, 1054, 108, 20, 3, 1, 1, 16, 16, 16, True), (1, 6, 1348, 124, 110, 3, 1, 1, 12, 12, 12, True),
+    (1, 2, 1024, 64, 64, 3, 1, 1, 16, 16, 16, True),      # the widest that it pools itself
+    (1, 2, 2050, 64, 40, 3, 1, 1, 16, 16, 16, False),     # too wide for it in either form
+])
+def test_pool_of_wide_low_images(case):
+    test_conv_with_fused_pool(case, False)
+
+
 # ------------------------------------------------------------------ stochastic rounding in the layer epilogue
 STOCHASTIC_CONV = [
     # N, H, W, Cin, K, R, pad, stride, nx, nw, n_out, relu
