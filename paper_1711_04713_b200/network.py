@@ -428,7 +428,8 @@ class LPNetwork:
     def requant_pass(self, i: int, frac_bits: int):
         L = self.layers[i]
         if L.y is self._cal_act:            # a second storing pass of the same layer (thresholded allocation)
-            L.stats.zero_()
+            # its counts replace the first one's; the status stays, it is read once both have run
+            L.stats[:B.adaption_stats.status.offset].zero_()
         L.y.frac_bits = frac_bits
         self._cal_act = self._run_layer(L, self._cal_in[i], B.MODE_REQUANT)
 
