@@ -543,10 +543,16 @@ void make_item(QuantItem& it, const float* x, size_t outer, size_t inner, const 
 
 // Padded tensors that a warp assembles several rows of at a time: with a generator (150001 rows of 50: 25.2 us with
 // one vector per thread, 19.4 this way; without one 13.6 and 14.1), where four rows fit, rows do not share
-// lanes (quantize_narrow_rows) and the tensor fills the chip with such runs of rows.
-bool by_warp(const QuantItem& it, bool stochastic) {
-  return stochastic && it.q16 == nullptr && it.inner * 4 <= kFlatBytes && (it.row_vecs > 1 || it.inner > 4) &&
-         it.count >= (unsigned long long)num_sms() * 1024;
+// lanes (quantize_narrow_rows) and the tensor fills the chip with such runs of rows.  The vectors of a run are
+// divided by row_vecs through a reciprocal whose error is below row_vecs / 2^32: exact while vectors * row_vecs < 2^32
+// (one element per row: pitches up to 32 KB; 256 elements: up to 512 KB).
+int rows_by_warp(const QuantItem& it, bool stochastic) {
+  if (!stochastic || it.q16 != nullptr || it.inner * 4 > kFlatBytes || (it.row_vecs == 1 && it.inner <= 4) ||
+      it.count < (unsigned long long)num_sms() * 1024)
+    return 0;
+  const int rows = (int)(kFlatBytes / it.inner) & ~3;
+  const unsigned long long vecs = it.row_vecs < (1u << 16) ? (unsigned long long)rows * it.row_vecs : 1ull << 32;
+  return vecs * it.row_vecs < 1ull << 32 ? rows : 0;
 }
 
 template <bool STOCH, bool PADDED, int CAP>
@@ -563,8 +569,8 @@ int launch_quantize(QuantArgs<CAP>& a, cudaStream_t stream) {
   for (int k = 0; k < a.n; ++k) {
     QuantItem& it = a.item[k];
     it.first_chunk = a.total_chunks;
-    if (PADDED && by_warp(it, STOCH)) {
-      it.warp_rows = (int32_t)(kFlatBytes / it.inner) & ~3;
+    if (PADDED) it.warp_rows = rows_by_warp(it, STOCH);
+    if (it.warp_rows > 0) {
       it.count /= it.row_vecs;
       const unsigned long long per_chunk = (unsigned long long)it.warp_rows * (kQThreads / 32);
       a.total_chunks += (it.count + per_chunk - 1) / per_chunk;

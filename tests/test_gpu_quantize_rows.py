@@ -57,7 +57,10 @@ def test_rows(shape, n_bits, f, offset, relu):
         guards.check()
 
 
-@pytest.mark.parametrize("shape", [(76001, 17, 32), (40003, 50, 64), (20001, 256, 272), (160001, 5, 16)])
+# (the last four: the widest pitch at which the rows of a run are told apart by a multiplication, and the pitches
+# from which a run of as many rows has too many vectors for it)
+@pytest.mark.parametrize("shape", [(76001, 17, 32), (40003, 50, 64), (20001, 256, 272), (160001, 5, 16),
+                                   (1030, 1, 32752), (1030, 1, 33024), (1030, 1, 65520), (230, 5, 74144)])
 def test_rows_of_a_large_tensor_stochastic(shape):
     """Tensors large enough for a warp to assemble several rows at a time: odd row lengths, the longest rows,
     a last run of rows that is not full."""
