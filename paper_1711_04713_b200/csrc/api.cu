@@ -121,6 +121,13 @@ static int build_ip_problem(int64_t B, int64_t K, int64_t O, const adaption_qten
   return ADAPTION_OK;
 }
 
+// Whether the layer runs on the cluster kernel.  ADAPTION_ALGO_TENSOR asks for shapes that the persistent kernel
+// takes and is refused for all others: the few outputs of a tensor below its limits may run here, but only by AUTO.
+static bool runs_on_clusters(const GemmProblem& g, int32_t algo) {
+  return algo != ADAPTION_ALGO_DIRECT && cluster_path_preferred(g) &&
+         (algo != ADAPTION_ALGO_TENSOR || tensor_path_supported(g));
+}
+
 static int dispatch(const GemmProblem& g, int32_t algo) {
   if (algo != ADAPTION_ALGO_AUTO && algo != ADAPTION_ALGO_TENSOR && algo != ADAPTION_ALGO_DIRECT)
     return ADAPTION_ERR_INVALID_ARG;
@@ -133,10 +140,10 @@ static int dispatch(const GemmProblem& g, int32_t algo) {
   }
   // (an inner product is asked for its split-K workspace by the persistent kernel's rule, whichever
   // kernel runs it)
-  const bool cluster = algo != ADAPTION_ALGO_DIRECT && cluster_path_preferred(g);
+  const bool cluster = runs_on_clusters(g, algo);
   if (cluster && g.is_conv) return launch_cluster(g);
   const bool tensor_ok = tensor_path_supported(g);
-  if (algo == ADAPTION_ALGO_TENSOR && !tensor_ok && !cluster) return ADAPTION_ERR_UNSUPPORTED;
+  if (algo == ADAPTION_ALGO_TENSOR && !tensor_ok) return ADAPTION_ERR_UNSUPPORTED;
   if (algo != ADAPTION_ALGO_DIRECT && tensor_ok) {
     const size_t need = tensor_path_workspace(g);
     if (need > 0) {
@@ -170,7 +177,7 @@ static ConvPoolPlan plan_conv_pool(GemmProblem g, int32_t algo) {
   g.y.q16 = nullptr;
   const bool packs = algo != ADAPTION_ALGO_DIRECT && pack_taps_applicable(g);
   g.pool2x2 = true;
-  if (algo != ADAPTION_ALGO_DIRECT && !packs && cluster_path_preferred(g)) {
+  if (!packs && runs_on_clusters(g, algo)) {
     pl.cluster = true;
     pl.total = 256;          // never touched; the call always takes a workspace
     return pl;

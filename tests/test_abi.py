@@ -122,3 +122,23 @@ def test_threshold_allocation_host_helper_matches_oracle(lib):
             B.adaption_choose_frac_bits_from_hist([0] * ba.HIST_BINS, 16, bad)
     with pytest.raises(B.AdaptionError):
         B.adaption_choose_frac_bits_from_hist([0] * ba.HIST_BINS, 17, 0.0)
+
+
+@pytest.mark.parametrize("shape", [(1, 8, 8, 64, 32, 3, 1, 1), (1, 163, 1, 3, 2, 3, 3, 3), (4, 14, 14, 128, 128, 3, 1, 1)])
+@pytest.mark.parametrize("n_bits", [8, 16])
+def test_tensor_only_calls_below_the_tensor_path_are_refused(lib, shape, n_bits):
+    """Convolutions over less than 128 KiB: ALGO_TENSOR is refused on the host, whatever kernel AUTO has for them."""
+    N, H, W, C, K, R, pad, stride = shape
+    fake, pitch = 4096, B.pad_to(C, 32)
+    x = B.adaption_qtensor(fake, fake, None, B.adaption_qfmt(n_bits, 3), pitch)
+    y = B.adaption_qtensor(fake, fake, None, B.adaption_qfmt(n_bits, 3), B.pad_to(K, 32))
+    shp = ctypes.byref(B.conv_shape(N, H, W, C, K, R, R, pad, stride))
+    for mode in (B.MODE_REQUANT, B.MODE_RANGE):
+        assert lib.adaption_lp_conv_fwd(shp, x, x, None, 0, 1, mode, B.ALGO_TENSOR, y, fake, None, 0,
+                                        None) == B.ERR_UNSUPPORTED
+    assert lib.adaption_lp_conv_fwd_stochastic(shp, x, x, None, 0, 1, B.ALGO_TENSOR, y, 1, fake, None, 0,
+                                               None) == B.ERR_UNSUPPORTED
+    if ((H + 2 * pad - R) // stride + 1) % 2 == 0 and ((W + 2 * pad - R) // stride + 1) % 2 == 0:
+        need = lib.adaption_lp_conv_pool_workspace_bytes(shp, x.fmt, x.fmt, y.fmt, pitch, y.c_stride, B.ALGO_TENSOR)
+        assert lib.adaption_lp_conv_pool_fwd(shp, x, x, None, 0, 1, B.ALGO_TENSOR, B.PHASE_CONV, y, fake, fake, need,
+                                             None) == B.ERR_UNSUPPORTED
