@@ -220,15 +220,17 @@ PyObject* fill_items(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   Py_RETURN_NONE;
 }
 
-// items, n
+// items (None: a null pointer, which the library takes with n = 0 and refuses otherwise), n
 PyObject* quantize_batch(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   ARGS(2)
   int32_t n;
   void* st;
   Buffer b;
-  if (!i32(a[1], &n) || !b.get(a[0], n > 0 ? (size_t)n * sizeof(adaption_quantize_item) : 0, "items") || !current_stream(&st))
+  if (!i32(a[1], &n) ||
+      (a[0] != Py_None && !b.get(a[0], n > 0 ? (size_t)n * sizeof(adaption_quantize_item) : 0, "items")) ||
+      !current_stream(&st))
     return nullptr;
-  CALL(p_adaption_quantize_batch((const adaption_quantize_item*)b.b.buf, n, st))
+  CALL(p_adaption_quantize_batch(b.held ? (const adaption_quantize_item*)b.b.buf : nullptr, n, st))
   return answer(rc, "adaption_quantize_batch");
 }
 

@@ -106,3 +106,11 @@ def test_many_tensors_in_one_launch(stochastic):
         assert np.array_equal(from_qtensor(y), want)
         assert y.padding_is_zero()
     guards.check()
+
+
+def test_a_batch_without_tensors():
+    """No array at all is fine for no tensors, and an invalid argument of the library for any."""
+    B.adaption_quantize_batch(None, 0)
+    with pytest.raises(B.AdaptionError) as e:
+        B.adaption_quantize_batch(None, 1)
+    assert e.value.status == B.ERR_INVALID_ARG
