@@ -194,6 +194,18 @@ def cta_mode(request, _default_overrides):
     return request.param
 
 
+@pytest.fixture(params=["chosen", "persistent"])
+def kernel(request, _default_overrides):
+    """Run a case on the kernel that the heuristics choose (layers with few output tiles: one cluster per tile), and
+    on the persistent kernel with one output pixel per row, whose tiles the case is about."""
+    if request.param == "persistent":
+        B.adaption_debug_set("cluster", 0)
+        B.adaption_debug_set("pixels", 0)
+
+
+on_both_kernels = pytest.mark.usefixtures("kernel")
+
+
 @pytest.mark.parametrize("case", TC_CONV)
 def test_conv_tensor(case, cta_mode):
     N, H, W, Cin, K, R, pad, stride, nx, nw, n_out, relu = case
@@ -246,6 +258,7 @@ def test_single_pass_fast_epilogue_every_shift(shift, n_out, K, Cin, cta_mode):
         assert cnt.sat_pos > 0   # the case does exercise saturation
 
 
+@on_both_kernels
 def test_epilogue_variants_agree():
     """Cross-path identity: the generic 64-bit epilogue with direct stores, the staged stores and the
     fast paired path all give the oracle's bits on the same case."""
@@ -333,6 +346,7 @@ WIDE_CONV = [
 ]
 
 
+@on_both_kernels
 @pytest.mark.parametrize("case", WIDE_CONV)
 @pytest.mark.parametrize("with_q16", [False, True])
 @pytest.mark.parametrize("wide", [1, 0])
@@ -341,11 +355,13 @@ def test_conv_single_pass_wide_tiles(case, with_q16, wide):
     run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_TENSOR, with_q16=with_q16)
 
 
+@on_both_kernels
 def test_ip_single_pass_wide_tiles():
     run_ip_case(np.random.default_rng(77), 1100, 1152, 384, 8, 8, 8, True, B.ALGO_TENSOR, with_q16=False)
     run_ip_case(np.random.default_rng(78), 2048, 2304, 256, 8, 8, 8, False, B.ALGO_TENSOR, with_q16=True)
 
 
+@on_both_kernels
 @pytest.mark.parametrize("groups", [1, 2])
 @pytest.mark.parametrize("with_q16", [False, True])
 def test_epilogue_groups_agree(groups, with_q16):
@@ -365,8 +381,10 @@ def test_ip_tensor_staged_stores(case, cta_mode):
     run_ip_case(np.random.default_rng(sum(case) + 1), Bsz, K, O, nx, nw, n_out, relu, B.ALGO_TENSOR, with_q16=False)
 
 
+@on_both_kernels
 def test_ip_tensor_split_k_paths():
-    # long reduction with few output tiles: the library splits K and needs its workspace
+    # long reduction with few output tiles: asked for the workspace of a split reduction, which the persistent
+    # kernel uses (the cluster kernel takes the shape by default, and leaves the workspace alone)
     need = run_ip_case(np.random.default_rng(11), 64, 25088, 256, 16, 16, 16, True, B.ALGO_TENSOR)
     assert need == 64 * 256 * 8
     # forcing other split factors gives the same bits
@@ -451,9 +469,15 @@ POOL_CONV = [
     (5, 16, 16, 128, 128, 1, 0, 1, 16, 16, 16, True),     # 1x1 filter
     (4, 32, 32, 64, 64, 3, 1, 1, 16, 16, 16, True),       # 64 -> 64 channels: CTA pair, 64-column tiles, two epilogue groups
     (3, 26, 30, 64, 40, 3, 1, 1, 16, 16, 16, True),       # same with a ragged M tail and 40 channels
+    (3, 22, 26, 128, 136, 3, 1, 1, 16, 16, 16, True),     # pair tiles, a ragged last one in both directions
+    (3, 26, 30, 64, 40, 3, 1, 1, 8, 8, 8, True),          # 8 bits: outputs four to a word, one column tile
+    (3, 22, 26, 128, 136, 3, 1, 1, 8, 8, 8, True),        # same, a second ragged column tile
+    (3, 22, 26, 128, 264, 3, 1, 1, 8, 8, 8, True),        # same, 256-column pair tiles
+    (3, 22, 26, 128, 264, 3, 1, 1, 8, 8, 16, True),       # 256-column pair tiles, 16-bit outputs
 ]
 
 
+@on_both_kernels
 @pytest.mark.parametrize("case", POOL_CONV)
 @pytest.mark.parametrize("with_q16", [False, True])
 def test_conv_with_fused_pool(case, with_q16):
@@ -540,6 +564,7 @@ def test_conv_stochastic_rounding(case, with_q16, cta_mode):
     assert cnt.zeros > 0
 
 
+@on_both_kernels
 @pytest.mark.parametrize("shift_case", [(13, 15, 12), (4, 8, 12), (2, 3, 9), (0, 0, 0)])
 def test_conv_stochastic_rounding_across_shifts(shift_case):
     """Long and short right shifts, an exact left shift (more fractional bits out than in) and shift 0."""
@@ -548,11 +573,13 @@ def test_conv_stochastic_rounding_across_shifts(shift_case):
                   B.ALGO_TENSOR, f_out=f_out, with_q16=False, mag_bits=(6, 6), fmts=(fx, fw), stochastic_seed=99)
 
 
+@on_both_kernels
 @pytest.mark.parametrize("case", [(70, 1000, 260, 16, 16, 16, False), (64, 25088, 250, 16, 16, 16, True),
                                   (130, 256, 128, 8, 8, 8, True), (5, 64, 33, 16, 8, 16, False)])
 @pytest.mark.parametrize("algo", [B.ALGO_AUTO, B.ALGO_DIRECT])
 def test_ip_stochastic_rounding(case, algo):
-    """Inner products, including a split reduction (the finalize kernel rounds) and the plain kernel."""
+    """Inner products, including a reduction that the persistent kernel splits (the finalize kernel rounds) and the
+    plain kernel."""
     if algo == B.ALGO_DIRECT and case[1] > 2000:
         pytest.skip("the plain kernel takes too long on the long reduction")
     run_ip_case(np.random.default_rng(sum(case) + 9), *case, algo, stochastic_seed=0xFEEDFACE + case[0])
@@ -608,6 +635,7 @@ def test_device_side_wait_runs_out_and_the_next_call_is_exact(mode, stall_at):
     run_conv_case(np.random.default_rng(22), *case, B.ALGO_TENSOR, with_q16=False)
 
 
+@on_both_kernels
 def test_left_shift_of_accumulators_beyond_2_to_the_48():
     """An inner product long enough for |acc| = 2^48 (262144 products of -32768 * -32768) requantized
     to MORE fractional bits than the accumulator has: the exact product acc * 2^15 does not fit 64 bits
@@ -669,6 +697,7 @@ def test_conv_channel_pitch_not_a_multiple_of_128(case, with_q16, cta_mode):
     run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_TENSOR, with_q16=with_q16)
 
 
+@on_both_kernels
 @pytest.mark.parametrize("case", [
     (37, 64, 64, 32, 16, 3, 1, 1, 16, 16, 16, True),      # four groups, three accumulators of 32 columns
     (37, 64, 64, 3, 64, 3, 1, 1, 8, 8, 8, True),          # four groups, packed taps, more tiles than CTAs

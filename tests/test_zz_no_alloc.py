@@ -22,6 +22,17 @@ from tests.util import dev, from_qtensor, stats_tuple, to_qtensor
 pytestmark = pytest.mark.gpu
 
 
+@pytest.fixture(autouse=True, params=["persistent", "chosen"])
+def _kernel(request):
+    """The persistent kernel, which splits the long reductions and uses the scratch, and the one that the heuristics
+    choose (one cluster per tile, which is asked for the same bytes and leaves them alone)."""
+    B.adaption_debug_set("reset")
+    if request.param == "persistent":
+        B.adaption_debug_set("cluster", 0)
+    yield
+    B.adaption_debug_set("reset")
+
+
 def _case(seed, Bsz, K, O, relu):
     rng = np.random.default_rng(seed)
     xq = rng.integers(-32768, 32768, (Bsz, K)).astype(np.int16)
@@ -35,7 +46,7 @@ def _run_both(seed, Bsz, K, O, relu, f_out, uses_scratch=True):
     x, w, bias, host = _case(seed, Bsz, K, O, relu)
     need = B.adaption_lp_ip_workspace_bytes(Bsz, K, O, x.fmt(), w.fmt(), B.ALGO_TENSOR)
     if uses_scratch:
-        assert 0 < need <= B.STATIC_WORKSPACE_BYTES      # the split-K (scratch-using) path is exercised
+        assert 0 < need <= B.STATIC_WORKSPACE_BYTES      # a reduction that the persistent kernel splits
     else:
         assert need == 0                                 # an unsplit reduction: the array is not touched
     ws_bytes = max(need, 16)
