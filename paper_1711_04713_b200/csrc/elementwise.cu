@@ -31,8 +31,10 @@ static inline int stream_grid(size_t work_items, int threads, int blocks_per_sm)
 
 // Format changes of stored tensors: sixteen blocks per SM where there is work for them.  Twice as many as fit at a time,
 // so that they start in address order (512 x 2^19 elements, 16 bits 202 us with eight, 180 with sixteen; with 32 175,
-// but 3 M x 16 elements 37, 35 and 42: every block also ends with its counters); with less work a part
-// of a second wave costs more than the order gives (12.8 M elements, 8 bits 10.7 us against 11.4).
+// but 3 M x 16 elements 37, 35 and 42: every block also ends with its counters, added up over the block first, because
+// one atomic per warp took longer than the tensor: 200000 rows of 17 at 8 bits 16.1 us, 12.7 this way, 30000 of 40 8.4 and
+// 4.8); with less work a part of a second wave costs more than the order gives (12.8 M elements, 8 bits 10.7 us against
+// 11.4).
 static inline int requant_grid(size_t work_items) {
   const int many = stream_grid(work_items, 256, 16);
   return many == num_sms() * 16 ? many : stream_grid(work_items, 256, 8);
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(256) requant_rows_kernel(const uint32_t* __res
     }
     store4(out, g, q[0], q[1], q[2], q[3]);
   }
-  if (stats != nullptr) flush_counts_warp(c, stats);
+  if (stats != nullptr) flush_counts_block(c, stats);
 }
 
 // Dense rows on both sides (pitch == inner extent, no int16 copy): the tensor is one flat array,
@@ -288,7 +290,7 @@ __global__ void __launch_bounds__(256) requant_flat_kernel(const uint4* __restri
   }
   for (; i < n16; i += nthreads)
     one(i, __ldcs(in_lo + i), TWO_PLANES_IN ? __ldcs(in_hi + i) : make_uint4(0, 0, 0, 0));
-  if (stats != nullptr) flush_counts_warp(c, stats);
+  if (stats != nullptr) flush_counts_block(c, stats);
 }
 
 // ------------------------------------------------------------------------------------------
