@@ -578,7 +578,12 @@ int launch_quantize(QuantArgs<CAP>& a, cudaStream_t stream) {
       a.total_chunks += (it.count + (unsigned)a.chunk - 1) / (unsigned)a.chunk;
     }
   }
-  const unsigned long long cap = (unsigned long long)num_sms() * kBlocksPerSm;
+  // Padded rows without a generator: with few chunks per SM a block of one or two chunks costs more in its start and its
+  // counters than the order gives (1 M rows, us, 32 blocks per SM and 12: of 1 element 10.0, 8.5, of 5 13.8, 12.6, of 13
+  // 19.2, 18.0; 3 M rows of 13 50.9, 51.4).  Rows that share lanes gain at any size (3 M rows of 3 27.5, 27.0).
+  const bool narrow = PADDED && a.n == 1 && a.item[0].row_vecs == 1 && a.item[0].inner <= 4;
+  const bool few = PADDED && !STOCH && (narrow || a.total_chunks < (unsigned long long)num_sms() * 64);
+  const unsigned long long cap = (unsigned long long)num_sms() * (few ? 12 : kBlocksPerSm);
   const unsigned grid = (unsigned)(a.total_chunks < cap ? a.total_chunks : cap);
   const cudaError_t e = launch_after_predecessor(quantize_kernel<STOCH, PADDED, CAP>, dim3(grid), dim3(kQThreads), stream, a);
   if (e != cudaSuccess) (void)cudaGetLastError();

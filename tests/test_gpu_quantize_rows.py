@@ -81,6 +81,23 @@ def test_rows_of_a_large_tensor_stochastic(shape):
         guards.check()
 
 
+@pytest.mark.parametrize("shape", [(460001, 3, 16), (460001, 9, 16), (230001, 17, 32)])
+@pytest.mark.parametrize("relu", [False, True])
+def test_blocks_of_several_chunks(shape, relu):
+    """Tensors of more chunks than there are blocks, without a generator; the last chunk is not full."""
+    outer, inner, pitch = shape
+    x = _values(np.random.default_rng(outer), (outer, inner), 16, 12)
+    want, cnt = orc.quantize(np.where(x > 0, x, 0).astype(np.float32) if relu else x, 16, 12)
+    guards = Guards()
+    y = guards.qtensor(outer, inner, 16, 12, pitch)
+    st = B.new_stats()
+    B.adaption_lp_act(dev(x), None, outer, inner, relu, y, None, B.ROUND_DETERMINISTIC, st)
+    assert np.array_equal(from_qtensor(y), want)
+    assert y.padding_is_zero()
+    assert stats_tuple(st) == (cnt.zeros, cnt.sat_pos, cnt.sat_neg)
+    guards.check()
+
+
 @pytest.mark.parametrize("stochastic", [False, True])
 def test_many_tensors_in_one_launch(stochastic):
     """More tensors than one launch takes, dense and padded in turn, small and large, formats on host and device."""
