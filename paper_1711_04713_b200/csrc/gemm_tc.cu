@@ -1553,9 +1553,12 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   // Single-pass (8-bit) layers with many output channels take 256-column pair tiles: one int32
   // accumulator per tile leaves room for two sets of 256 columns, and a 256 x 256 tile halves the
   // operand bytes per MMA cycle, which is what limits the int8 rate (see make_config's pair notes).
+  // (not for short reductions over partial blocks where the channel count is no multiple of 8: the 64-bit epilogue
+  // bounds those and pays for every column of the last tile; 45 x 16 x 14 pixels, 3x3, 69 -> 294 24.7 us against 18.7)
+  const bool partial = g.is_conv && c.ksteps_last != c.BK / 32;
   const bool wide = allow_wide && c.nacc == 1 && c.BK == 128 && g.N >= 256 && c.num_kb >= 9 && g.M >= 1024 &&
                     (num_sms() % 2) == 0 && forced_bn == 0 && knob(kPair) != 0 &&
-                    knob(kWide) != 0;
+                    knob(kWide) != 0 && !(partial && g.N % 8 != 0 && c.num_kb < 16);
   if (wide) c.BN = 256;
   c.tiles_m = (int)((g.M + kBM - 1) / kBM);
   c.tiles_n = (int)((g.N + c.BN - 1) / c.BN);
@@ -1634,7 +1637,7 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
   const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
   // group short k-blocks so that a stage carries roughly 768 tensor-pipe cycles of work or more (512 with one
-  // product per step: 128 -> 128 channels at 112 x 112, 8 bits, batch 128 231 us with two k-blocks, 264 with three)
+  // product per step: 128 -> 128 channels at 112 x 112, 8 bits, batch 128 231 us with two k-blocks, 264 with three).
   {
     const int products = c.nax * c.nbw;
     const int cyc_per_kb = (c.BK / 32) * products * (c.BN >= 128 ? c.BN / 2 : 48);

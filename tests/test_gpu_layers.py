@@ -483,6 +483,10 @@ POOL_CONV = [
 def test_conv_with_fused_pool(case, with_q16):
     """adaption_lp_conv_pool_fwd equals convolution, epilogue and 2x2 max-pool of the oracle; its
     counters are those of the convolution's own output."""
+    run_pool_case(case, with_q16)
+
+
+def run_pool_case(case, with_q16):
     N, H, W, Cin, K, R, pad, stride, nx, nw, n_out, relu = case
     rng = np.random.default_rng(sum(case))
     cs = B.pad_to(Cin, 32) if Cin != 20 else 48
@@ -535,7 +539,7 @@ def test_conv_with_fused_pool(case, with_q16):
     (1, 2, 2050, 64, 40, 3, 1, 1, 16, 16, 16, False),     # too wide for it in either form
 ])
 def test_pool_of_wide_low_images(case):
-    test_conv_with_fused_pool(case, False)
+    run_pool_case(case, False)
 
 
 # ------------------------------------------------------------------ stochastic rounding in the layer epilogue
@@ -709,6 +713,18 @@ def test_conv_channel_pitch_not_a_multiple_of_128(case, with_q16, cta_mode):
 ])
 def test_epilogue_groups_by_default(case):
     run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_TENSOR if case[3] != 3 else B.ALGO_AUTO, with_q16=False)
+
+
+@on_both_kernels
+@pytest.mark.parametrize("case", [
+    # tiles whose stages, columns or epilogue groups depend on the pitch, the widths and the channel count at once
+    (6, 30, 30, 96, 294, 3, 1, 1, 8, 8, 8, True),         # partial blocks, 294 channels: columns by 128
+    (6, 30, 30, 96, 296, 3, 1, 1, 8, 8, 8, True),         # same, a multiple of 8: by 256
+])
+def test_tiles_chosen_by_pitch_widths_and_channels(case):
+    run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_AUTO, with_q16=False)
+    if case[1] == case[2]:
+        run_pool_case(case, False)
 
 
 @pytest.mark.parametrize("case,fmts,f_out,mag", [
