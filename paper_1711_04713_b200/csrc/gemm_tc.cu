@@ -1636,15 +1636,18 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   // dynamic shared memory: everything up to the per-block limit except the control block
   c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
   const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
-  // group short k-blocks so that a stage carries roughly 768 tensor-pipe cycles of work or more (512 with one
-  // product per step: 128 -> 128 channels at 112 x 112, 8 bits, batch 128 231 us with two k-blocks, 264 with three).
+  // group short k-blocks so that a stage carries roughly 768 tensor-pipe cycles of work or more.  512 with one product
+  // per step (128 -> 128 channels at 112 x 112, 8 bits, batch 128 231 us with two k-blocks, 264 with three), but not for
+  // convolutions of more than twelve k-blocks on 128 columns, whose weights cannot stay resident beside either ring (18 to
+  // 48 blocks 10 % faster with three; 8 x 74 x 194 pixels, 5x5, 112 -> 103 63 us against 56; an inner product of 512 rows,
+  // 4096 -> 4096, has 12.1 with two, 13.4 with three).
   // Two accumulators over partial blocks (a pitch that is no multiple of 128): one block per stage, because the grouped
   // loop multiplies the zeros behind the pitch (128 columns 10 to 15 % faster, 64 columns 6 to 9; 19 x 35 x 12 pixels, 5x5,
   // 302 -> 259 70 us against 58; tiles of 32 columns wait for copies either way).
   {
     const int products = c.nax * c.nbw;
     const int cyc_per_kb = (c.BK / 32) * products * (c.BN >= 128 ? c.BN / 2 : 48);
-    const int want = c.nacc == 1 ? 512 : 768;
+    const int want = c.nacc == 1 && !(g.is_conv && c.BN == 128 && c.num_kb > 12) ? 512 : 768;
     int kps = (want + cyc_per_kb - 1) / cyc_per_kb;
     if (kps > 4) kps = 4;
     if (c.nacc == 2 && partial && c.BN >= 64) kps = 1;

@@ -721,6 +721,8 @@ def test_epilogue_groups_by_default(case):
     (7, 30, 30, 96, 136, 3, 1, 1, 16, 8, 16, True),       # two accumulators, partial blocks: one block per stage, pairs
     (7, 30, 30, 160, 72, 1, 0, 1, 8, 16, 8, False),       # same without pairs, two blocks
     (7, 30, 30, 70, 60, 3, 1, 1, 16, 8, 16, True),        # same, 64 columns
+    (7, 30, 30, 160, 120, 3, 1, 1, 8, 8, 8, True),        # one accumulator, 18 blocks: three per stage
+    (6, 30, 31, 128, 100, 5, 2, 1, 8, 8, 8, True),        # 25 blocks, the last stage a single one
     (6, 30, 30, 96, 294, 3, 1, 1, 8, 8, 8, True),         # partial blocks, 294 channels: columns by 128
     (6, 30, 30, 96, 296, 3, 1, 1, 8, 8, 8, True),         # same, a multiple of 8: by 256
 ])
