@@ -1629,8 +1629,15 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   // TMEM loads, arithmetic, staging, barrier, store) is mostly latency.  8 bits, batch 128: 3 -> 64 channels at 224 x 224
   // 387 us with two groups, 349 with four; 64 -> 128 at 112 x 112 163 with one, 128 with two, 126 with four;
   // 128 -> 256 at 56 x 56 106 with one, 90 with two; 3 -> 16 at 16 bits, batch 16 91 with two, 62 with four.
+  // Stored outputs of a channel count that is no multiple of 8 take the 64-bit epilogue, whose steps of 16 columns four
+  // groups do not share: two for those where a tile has the k-blocks to cover a longer chain (60 layers of up to 31
+  // channels and at least nine blocks 5 % faster on average, at best 40; 16 bits, 36 x 97 x 139 pixels, 3x3, 23 -> 11 82 us
+  // against 67; 8 bits, 14 x 71 x 165, 3x3, 166 -> 9 47 against 34.  One block, 58 x 60 x 176, 3 -> 31 53 with four, 58
+  // with two; 64 columns gain 2 to 4 % beyond nine blocks).
   c.epi_groups = c.acc_bufs;
-  const int most_groups = c.BN <= 64 ? 4 : 2;
+  const bool two_groups = g.is_conv && g.mode == ADAPTION_MODE_REQUANT && g.N % 8 != 0 &&
+                          c.num_kb >= (c.BN == 32 ? 9 : 10);
+  const int most_groups = c.BN <= 64 && !two_groups ? 4 : 2;
   while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
   c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) : 0u;
   // dynamic shared memory: everything up to the per-block limit except the control block

@@ -725,6 +725,9 @@ def test_epilogue_groups_by_default(case):
     (6, 30, 31, 128, 100, 5, 2, 1, 8, 8, 8, True),        # 25 blocks, the last stage a single one
     (6, 30, 30, 96, 294, 3, 1, 1, 8, 8, 8, True),         # partial blocks, 294 channels: columns by 128
     (6, 30, 30, 96, 296, 3, 1, 1, 8, 8, 8, True),         # same, a multiple of 8: by 256
+    (23, 40, 40, 32, 11, 3, 1, 1, 16, 16, 16, True),      # 11 channels: two epilogue groups, more tiles than CTAs
+    (9, 40, 41, 166, 9, 3, 1, 1, 8, 8, 8, True),          # same, one accumulator
+    (9, 40, 41, 130, 43, 3, 1, 1, 8, 16, 8, True),        # same, 64 columns
 ])
 def test_tiles_chosen_by_pitch_widths_and_channels(case):
     run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_AUTO, with_q16=False)
