@@ -940,7 +940,8 @@ int launch_cluster(const GemmProblem& g) {
   if (g.mode == ADAPTION_MODE_REQUANT) {
     p.rq = make_requant(g.acc_frac_bits, g.y.fmt, g.relu);
     p.y_hi = (int8_t*)g.y.hi; p.y_lo = (uint8_t*)g.y.lo; p.y_q16 = g.y.q16; p.y_stride = g.y.c_stride;
-    p.y_cols = (int)g.y.c_stride;
+    // (columns are counted in 32 bits, and at most 2^20 are outputs: padding further out than 2^30 is not zeroed)
+    p.y_cols = (int)(g.y.c_stride < (1 << 30) ? g.y.c_stride : 1 << 30);
   } else {
     p.rq = RequantParams{0, g.relu ? 1 : 0, 0, 0, 1};
     p.st.enabled = 0;

@@ -106,6 +106,19 @@ def test_pitch_beyond_the_last_tile_is_zeroed():
     guards.check()
 
 
+def test_output_pitch_beyond_32_bits():
+    """Rows 2^31 + 16 elements apart: the outputs are stored where they belong (outputs of 8 bits, two rows)."""
+    rng = np.random.default_rng(12)
+    xq, wq = _rand_q(rng, (2, 64), 8, 0.4), _rand_q(rng, (8, 64), 8)
+    want, _ = orc.epilogue(orc.ip_acc(xq, wq), None, 0, 13, True, 8, 2)
+    pitch = (1 << 31) + 16
+    y = B.QTensor(2, 8, pitch, 8, 2, torch.full((2 * pitch,), 0x3C, dtype=torch.uint8, device="cuda"))
+    B.adaption_lp_ip_fwd(2, 64, 8, to_qtensor(xq, 8, 6), to_qtensor(wq, 8, 7), None, 0, True, B.MODE_REQUANT, B.ALGO_AUTO,
+                         y, B.new_stats(), None)
+    got = torch.stack([y.lo[:8], y.lo[pitch:pitch + 8]]).cpu().numpy()
+    assert np.array_equal(got.view(np.int8), want)
+
+
 def test_device_side_wait_runs_out():
     """The copying warps stop before their second stage with nothing in flight; the waits of the others
     run out, the kernel says so in the stats word and returns, and the next call is exact."""
