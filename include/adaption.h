@@ -68,7 +68,8 @@ enum { ADAPTION_MODE_REQUANT = 0, ADAPTION_MODE_RANGE = 1 };
 
 /* Kernel choice for the layer calls.  AUTO takes the tensor-core path whenever the shape
  * allows it; DIRECT forces the plain integer kernel, TENSOR fails with
- * ADAPTION_ERR_UNSUPPORTED where the tensor-core path cannot run. */
+ * ADAPTION_ERR_UNSUPPORTED where the tensor-core path cannot run (convolutions over less than 128 KiB
+ * among them, some of which AUTO runs as thread-block clusters). */
 enum { ADAPTION_ALGO_AUTO = 0, ADAPTION_ALGO_TENSOR = 1, ADAPTION_ALGO_DIRECT = 2 };
 
 typedef struct adaption_qfmt {
@@ -233,7 +234,8 @@ ADAPTION_API int adaption_lp_ip_fwd_stochastic(int64_t B, int64_t K, int64_t O, 
  * (the quantizer is monotone, so pooling the stored integers is exact); d_stats counts the
  * convolution's own outputs, before pooling.  Requantizing mode only.  The convolution's output
  * lives in the workspace: where the tensor-core path can, only the maxima of horizontal pixel
- * pairs are stored there (half the bytes written and read back), otherwise all of it.
+ * pairs are stored there (half the bytes written and read back), otherwise all of it.  (Layers with
+ * few output tiles pool inside their kernel: y is then written in the convolution's phase.)
  * phases: ADAPTION_PHASE_CONV | ADAPTION_PHASE_POOL runs the whole layer pair; the two phases may
  * also be issued by two calls with otherwise identical arguments (convolution first, same stream
  * order, workspace untouched in between), e.g. to time them apart.

@@ -140,7 +140,7 @@ struct TcParams {
   const int16_t* bias;
   int bias_shift;
   RequantParams rq;
-  StochasticParams st;         // stochastic rounding in the requantization (generic epilogue only)
+  StochasticParams st;         // stochastic rounding in the requantization
   int mode;
   int8_t* y_hi;
   uint8_t* y_lo;
@@ -261,7 +261,7 @@ __device__ __forceinline__ long long combine(int32_t a0, int32_t a1, int32_t a2)
 // (shift >= 1): v / 2^shift rounded half away from zero, saturated to [qmin, qmax].  The shifted
 // value is narrowed to 32 bits with saturation first, so clamping and counting are 32-bit work.
 // With ReLU the value is non-negative and the lower bound cannot be crossed.
-template <bool RELU, bool COUNT_ALL>
+template <bool RELU>
 __device__ __forceinline__ int32_t requant_shift_right(long long v, long long half, int shift, int32_t qmin,
                                                        int32_t qmax, bool counted, Counts& c) {
   if (RELU) v = v < 0 ? 0ll : v;
@@ -272,15 +272,9 @@ __device__ __forceinline__ int32_t requant_shift_right(long long v, long long ha
   const int32_t rh = (int32_t)(r >> 32);
   const int32_t rs = (rh == (r32 >> 31)) ? r32 : (rh < 0 ? (int32_t)0x80000000 : 0x7fffffff);
   const int32_t q = min(max(rs, qmin), qmax);
-  if (COUNT_ALL) {
-    c.sat_pos += (rs > qmax);
-    if (!RELU) c.sat_neg += (rs < qmin);
-    c.zeros += (q == 0);
-  } else {
-    c.sat_pos += (counted && rs > qmax);
-    if (!RELU) c.sat_neg += (counted && rs < qmin);
-    c.zeros += (counted && q == 0);
-  }
+  c.sat_pos += (counted && rs > qmax);
+  if (!RELU) c.sat_neg += (counted && rs < qmin);
+  c.zeros += (counted && q == 0);
   return q;
 }
 
@@ -330,9 +324,6 @@ __device__ __forceinline__ int32_t fast_result(int32_t t, int32_t h, int shift) 
   if (WIDE) return (h + (t >> 8)) >> (shift - 16);
   return mad_lo(h, 1 << (16 - shift), t >> (shift - 8));
 }
-// sixteen of the thirty-two columns (`half` = 0 or 1; they begin at column `col`) -> eight packed words; `t` and `h`
-// hold T and H
-// (or, with a single accumulator, t holds the sum plus its constant)
 // real columns of the eight that begin at column `col` (0, or all eight where N is a multiple of 8)
 template <bool PIX>
 __device__ __forceinline__ int real_columns8(int col, const TcParams& p) {
@@ -348,6 +339,8 @@ __device__ __forceinline__ uint64_t element_index(int m, int col, const TcParams
   return (uint64_t)m * (uint64_t)p.N + (uint64_t)col;
 }
 
+// sixteen of the thirty-two columns (`half` = 0 or 1; they begin at column `col`) -> eight packed words; `t` and `h`
+// hold T and H (or, with a single accumulator, t holds the sum plus its constant)
 template <int NACC, bool WIDE, bool PIX>
 __device__ __forceinline__ void fast_outputs16(const int32_t (&t)[32], const int32_t (&h)[32], int half, int shift,
                                                int32_t qmax, bool row_ok, int col, const TcParams& p,
@@ -540,8 +533,8 @@ __device__ __forceinline__ void requant8(const Acc8<NACC>& x, const long long* c
     const long long half = 1ll << (p.rq.shift - 1);
 #pragma unroll
     for (int j = 0; j < 8; ++j)
-      q[j] = requant_shift_right<RELU, false>(acc_value<NACC>(x, j) + c64[j], half, p.rq.shift, p.rq.qmin, p.rq.qmax,
-                                              j < nvalid, cnt);
+      q[j] = requant_shift_right<RELU>(acc_value<NACC>(x, j) + c64[j], half, p.rq.shift, p.rq.qmin, p.rq.qmax, j < nvalid,
+                                       cnt);
   } else {
 #pragma unroll
     for (int j = 0; j < 8; ++j) q[j] = requant_value(acc_value<NACC>(x, j) + c64[j], p.rq, j < nvalid, cnt);
@@ -655,12 +648,12 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t sr
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // the bulk stores committed so far have read their shared-memory source
+__device__ __forceinline__ void bulk_wait_read_all() {
+  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
 // ... all but the most recent group have (two staging buffers in turn)
 __device__ __forceinline__ void bulk_wait_read_all_but_one() {
   asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-}
-__device__ __forceinline__ void bulk_wait_read_all() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 // ... and have completed
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
@@ -700,12 +693,10 @@ __device__ __forceinline__ void release_accumulators(unsigned long long* bar_ptr
 }
 
 // ---------------------------------------------------------------------------------- kernel
-// LOOP: the form of the main loop, see kLoopPlain.
-// GROUPED: stages hold several k-blocks and / or the weights are resident in shared memory (short
-// reductions); the plain variant keeps the issue loops free of that bookkeeping.
-// FAST: ReLU layer in requantizing mode whose shift lies in [9, 31] ([0, 31] with 8-bit operands
-// on both sides), N a multiple of 8, no split-K,
-// magnitudes within the 32-bit bounds of the fast epilogue: it then contains only that path.
+// LOOP: the form of the main loop, see kLoopPlain (GROUPED, PARTIAL and PIX below).
+// EPI: the epilogue, see kEpiGeneric.  The 32-bit ones (FAST, FASTST) are launched for ReLU layers in requantizing mode whose
+// shift lies in [9, 31] ([0, 31] with 8-bit operands on both sides), N a multiple of 8, no split-K, magnitudes within
+// their bounds (fast_epilogue), and contain only that path.
 // 20 warps: one block per SM, 96 registers per thread.
 template <int NAX, int NBW, bool PAIR, int LOOP, int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
