@@ -14,10 +14,10 @@
 // a warp share the blocks of several rows and assemble the vectors from shared memory.
 //
 // Measured (16 bits; before: integer arithmetic on unpacked values, as many blocks as fit walking the tensor
-// together): 268 M dense elements 275 -> 239 us (6.74 TB/s), 51 M with ReLU 55.6 -> 48.5; stochastic 558 -> 389 us
-// (4.1 TB/s, bound by the integer pipes); the parameters of VGG16 157 -> 132 us, stochastic 359 -> 249; 3.2 M pixels
+// together): 268 M dense elements 275 -> 239 us (6.74 TB/s), 51 M with ReLU 55.6 -> 48.5; stochastic 558 -> 332 us
+// (4.9 TB/s; 385 before the rounding below took five instructions); the parameters of VGG16 157 -> 132 us, stochastic 359 -> 249 (56 M of 2-D weights 97 -> 84 since); 3.2 M pixels
 // of 3 channels 27.5 -> 28.4, stochastic 89.5 -> 38; 150001 rows of 50 in a pitch of 64 12.8 -> 12.5, stochastic
-// 40 -> 19.4 (rows assembled in shared memory by a whole block took 18.5 and 27).
+// 40 -> 19.2 (rows assembled in shared memory by a whole block took 18.5 and 27).
 #include "common.cuh"
 
 namespace adaption {
@@ -61,7 +61,7 @@ struct QuantArgs {
 
 struct QuantRule {
   float scale, y_max;                       // y_max: qmax
-  int32_t qmin, qmax, relu, wide;           // wide: more than 8 bits
+  int32_t qmin, qmax, relu, counted;
   uint32_t qmin2, qmax2;                    // both lanes
   uint32_t key0, key1;
 };
@@ -89,86 +89,64 @@ __device__ __forceinline__ int32_t round_away(float y) {
   return __float2int_rz(__fadd_rz(y, h));
 }
 
-// Stochastic rounding of y, |y| <= 2^15 + 2: floor(y) + 1 iff draw < T, T = floor(frac(y) 2^32).
-// An integer u converted with rounding down compares with a float like u itself: f > u iff f > RD(u).
-//
-// In general, with a = |y| and t = frac(a) 2^32 (exact steps):
-//   y >= 0: up iff floor(t) > draw;  y < 0: frac(y) = 1 - frac(a), so the magnitude grows iff t > ~draw
-//   (T = 2^32 - ceil(t); draw < T iff ceil(t) <= ~draw; never for t = 0).
-__device__ __forceinline__ int32_t round_stochastic(float y, uint32_t draw) {
-  const float a = fabsf(y);
-  const float m = __fadd_rd(a, 8388608.0f);               // 2^23 + floor(a)
-  const float t = (a - (m - 8388608.0f)) * 4294967296.0f;
-  const int32_t s = __float_as_int(y) >> 31;
-  const float tf = (s == 0 && t < 8388608.0f) ? __fadd_rd(t, 8388608.0f) - 8388608.0f : t;
-  const bool up = tf > __uint2float_rd(draw ^ (uint32_t)s);
-  const int32_t mag = __float_as_int(m) - 0x4B000000 + (up ? 1 : 0);
-  return (mag ^ s) - s;
+// Stochastic rounding of y, |y| <= 2^15 + 2: floor(y) + 1 iff draw < T, T = floor(frac(y) 2^32), without a branch.
+// With d = (draw + 1) 2^-32 the value goes up iff frac(y) >= d, so the result is floor(y - d) + 1, or, the same number,
+// floor(y + (1 - d)).  ~draw as a signed integer is -(draw + 1) where d <= 1/2 and 2^32 - (draw + 1) above, one of the
+// two summands in units of 2^-32, at most 1/2 in magnitude; it is converted with rounding down, and so is the sum (a
+// rounded-down sum has the floor of the exact one).  Rounding the summand changes no decision:
+//   d <= 1/2: frac(y) >= d is asked with d rounded up.  frac(y) is a float wherever that can matter (y > 0 or y <= -1/2:
+//     a multiple of the last place of y, below 1; for -1/2 < y < 0 it is above 1/2, and rounded d is not).
+//   d > 1/2: 1 - frac(y) <= 1 - d is asked with 1 - d rounded down.  1 - frac(y) is a float (y < 0 or y >= 1/2), or above
+//     1/2 and so above 1 - d.
+// Five instructions a value; bringing frac(y) and the draw to one scale and comparing them took eight where a test of
+// all four values allowed it and fourteen elsewhere.  The result is the low half of the returned word (the sum carries
+// 1.5 * 2^23).
+__device__ __forceinline__ uint32_t round_stochastic(float y, uint32_t draw) {
+  const int32_t k = (int32_t)~draw;
+  const float m = __fadd_rd(__fmaf_rd(__int2float_rd(k), 2.3283064365386963e-10f, y), 12582912.0f);
+  return __float_as_uint(m) + ((uint32_t)k >> 31);
 }
-// Where y = 0 or 1 <= |y| <= 2^15, frac(y) is a multiple of 2^-23 and so exact in single precision for
-// either sign, and t = frac(y) 2^32 is an integer: up iff t > draw.  The result is the low half of the returned word.
-__device__ __forceinline__ uint32_t round_stochastic_common(float y, uint32_t draw) {
-  float m = __fadd_rd(y, 12582912.0f);                    // 1.5 * 2^23 + floor(y): its low bits are floor(y)
-  const float t = (y - (m - 12582912.0f)) * 4294967296.0f;
-  if (t > __uint2float_rd(draw)) m += 1.0f;
-  return __float_as_uint(m);
-}
-// largest magnitude; NaN if one of them is
-__device__ __forceinline__ float max_abs_nan(float a, float b) {
+// largest of three magnitudes; NaN if one of them is
+__device__ __forceinline__ float max_abs_nan(float a, float b, float c) {
   float d;
-  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(fabsf(a)), "f"(fabsf(b)));
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
 
 // Four consecutive elements -> two words of two 16-bit lanes.  Elements that are not there are passed as 0
 // and left out by the caller's count of real ones.
 template <bool STOCH>
-__device__ __forceinline__ void quantize4(const float4 v, const QuantRule& r, unsigned long long block, int real,
+__device__ __forceinline__ void quantize4(const float4 v, const QuantRule& r, uint32_t block, uint32_t block_hi, int real,
                                           Counts& c, uint32_t& w0, uint32_t& w1) {
   const float x[4] = {v.x, v.y, v.z, v.w};
-  int32_t q[4];
   if constexpr (STOCH) {
-    const Philox4 rnd = philox4x32_10((uint32_t)block, (uint32_t)(block >> 32), 0u, 0u, r.key0, r.key1);
+    const Philox4 rnd = philox4x32_10(block, block_hi, 0u, 0u, r.key0, r.key1);
     float y[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       y[k] = x[k] * r.scale;
       if (r.relu) y[k] = fmaxf(y[k], 0.0f);                // (NaN -> 0)
     }
-    // largest magnitude; NaN if one of them is
-    const float top = max_abs_nan(max_abs_nan(y[0], y[1]), max_abs_nan(y[2], y[3]));
-    bool common = false;
-    if (r.wide) {         // (narrow formats have many values between 0 and 1: the general form throughout)
-      uint32_t least = 0xffffffffu;
+    const float top = max_abs_nan(max_abs_nan(y[0], y[1], y[2]), y[3], 0.0f);
+    uint32_t m[4];
+    if (top <= r.y_max) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) least = min(least, 2u * __float_as_uint(y[k]) - 1u);     // (0 becomes the largest)
-      common = top <= r.y_max && least >= 2u * 0x3f800000u - 1u;
-    }
-    if (common) {
-      uint32_t m[4];
+      for (int k = 0; k < 4; ++k) m[k] = round_stochastic(y[k], rnd.w[k]);
+    } else {                                               // something may saturate, or is no number
+      const float y_lo = (float)r.qmin - 2.0f, y_hi = r.y_max + 2.0f;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) m[k] = round_stochastic_common(y[k], rnd.w[k]);
-      w0 = __byte_perm(m[0], m[1], 0x5410);
-      w1 = __byte_perm(m[2], m[3], 0x5410);
-    } else {
-      if (!(top <= r.y_max)) {                             // something may saturate, or is no number
-        const float y_lo = (float)r.qmin - 2.0f, y_hi = r.y_max + 2.0f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float yk = y[k] != y[k] ? 0.0f : fminf(fmaxf(y[k], y_lo), y_hi);
-          const int32_t e = round_stochastic(yk, rnd.w[k]);
-          q[k] = min(max(e, r.qmin), r.qmax);
-          c.sat_pos += e > r.qmax;
-          c.sat_neg += e < r.qmin;
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) q[k] = round_stochastic(y[k], rnd.w[k]);
+      for (int k = 0; k < 4; ++k) {
+        const float yk = y[k] != y[k] ? 0.0f : fminf(fmaxf(y[k], y_lo), y_hi);
+        const int32_t e = (int32_t)round_stochastic(yk, rnd.w[k]) - 0x4B400000;
+        m[k] = (uint32_t)min(max(e, r.qmin), r.qmax);
+        c.sat_pos += e > r.qmax;
+        c.sat_neg += e < r.qmin;
       }
-      w0 = __byte_perm((uint32_t)q[0], (uint32_t)q[1], 0x5410);
-      w1 = __byte_perm((uint32_t)q[2], (uint32_t)q[3], 0x5410);
     }
+    w0 = __byte_perm(m[0], m[1], 0x5410);
+    w1 = __byte_perm(m[2], m[3], 0x5410);
   } else {
+    int32_t q[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) q[k] = round_away(x[k] * r.scale);
     w0 = pack_sat2(q[0], q[1]);
@@ -198,9 +176,11 @@ __device__ __forceinline__ void quantize4(const float4 v, const QuantRule& r, un
       }
     }
   }
-  // zero lanes: min(|w|, 1) per lane, counted as bits
-  const uint32_t nz = __vcmpne2(w0, 0u), nz1 = __vcmpne2(w1, 0u);
-  c.zeros += (uint32_t)(real - __popc((nz & 0x00010001u) | (nz1 & 0x00020002u)));
+  // zero lanes, counted as bits (parameters are quantized without counters)
+  if (!STOCH || r.counted) {
+    const uint32_t nz = __vcmpne2(w0, 0u), nz1 = __vcmpne2(w1, 0u);
+    c.zeros += (uint32_t)(real - __popc((nz & 0x00010001u) | (nz1 & 0x00020002u)));
+  }
 }
 
 __device__ __forceinline__ uint32_t low_bytes(uint32_t w0, uint32_t w1) { return __byte_perm(w0, w1, 0x6420); }
@@ -219,7 +199,7 @@ __device__ __forceinline__ void load8(const float* p, bool aligned32, float4 (&v
   }
 }
 
-__device__ __forceinline__ QuantRule rule_of(const QuantItem& it, int relu) {
+__device__ __forceinline__ QuantRule rule_of(const QuantItem& it, int relu, bool counted) {
   QuantRule r;
   const int32_t f = it.d_fmt != nullptr ? it.d_fmt->frac_bits : it.frac_bits;
   r.scale = __int_as_float((127 + f) << 23);
@@ -227,7 +207,7 @@ __device__ __forceinline__ QuantRule rule_of(const QuantItem& it, int relu) {
   r.qmin = it.qmin;
   r.qmax = it.qmax;
   r.relu = relu;
-  r.wide = it.planes == 2;
+  r.counted = counted;
   r.qmin2 = (uint32_t)(it.qmin & 0xffff) * 0x00010001u;
   r.qmax2 = (uint32_t)it.qmax * 0x00010001u;
   r.key0 = it.key0;
@@ -240,6 +220,8 @@ template <bool STOCH>
 __device__ __forceinline__ void quantize_dense_chunk(const QuantItem& it, const QuantRule& rule, unsigned long long base,
                                                      unsigned chunk, Counts& c) {
   const unsigned long long end = min(it.count, base + chunk);
+  // (chunks are powers of two: a chunk's generator blocks share the high word, and the first two rounds' work on it)
+  const uint32_t block_hi = (uint32_t)(base >> 31);
   float4 v[2][2];
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
@@ -251,8 +233,8 @@ __device__ __forceinline__ void quantize_dense_chunk(const QuantItem& it, const 
     const unsigned long long i = base + u * kQThreads + threadIdx.x;
     if (i < end) {
       uint32_t w[4];
-      quantize4<STOCH>(v[u][0], rule, 2 * i, 4, c, w[0], w[1]);
-      quantize4<STOCH>(v[u][1], rule, 2 * i + 1, 4, c, w[2], w[3]);
+      quantize4<STOCH>(v[u][0], rule, (uint32_t)(2 * i), block_hi, 4, c, w[0], w[1]);
+      quantize4<STOCH>(v[u][1], rule, (uint32_t)(2 * i) + 1u, block_hi, 4, c, w[2], w[3]);
       // (streaming stores: the planes are read much later)
       __stcs(reinterpret_cast<uint2*>(it.lo) + i, make_uint2(low_bytes(w[0], w[1]), low_bytes(w[2], w[3])));
       if (it.planes == 2)
@@ -286,7 +268,7 @@ __device__ __forceinline__ void quantize_narrow_rows(const QuantItem& it, const 
   if (sub < inner && i < it.numel) {
     float4 v;
     load_block(it, i, v);
-    quantize4<STOCH>(v, rule, block, (int)min(4ull, it.numel - i), c, w0, w1);
+    quantize4<STOCH>(v, rule, (uint32_t)block, (uint32_t)(block >> 32), (int)min(4ull, it.numel - i), c, w0, w1);
   }
   const uint32_t l = low_bytes(w0, w1), h = high_bytes(w0, w1);
   const int at = inner * sub;                         // place of this row's first byte among the 4 * inner
@@ -362,7 +344,8 @@ __device__ __forceinline__ void quantize_rows_by_warp(const QuantItem& it, const
       const int b = first + 32 * u;
       if (b < blocks) {
         uint32_t w0, w1;
-        quantize4<STOCH>(v[u], rule, (f0 >> 2) + (unsigned)b, min(4, n - 4 * b), c, w0, w1);
+        const unsigned long long blk = (f0 >> 2) + (unsigned)b;
+        quantize4<STOCH>(v[u], rule, (uint32_t)blk, (uint32_t)(blk >> 32), min(4, n - 4 * b), c, w0, w1);
         flat_lo[b] = low_bytes(w0, w1);
         if (it.planes == 2) flat_hi[b] = high_bytes(w0, w1);
       }
@@ -420,7 +403,7 @@ __device__ __forceinline__ void quantize_padded_chunk(const QuantItem& it, const
         if (4 * t + 1 < real) v.y = __ldg(src + 1);
         if (4 * t + 2 < real) v.z = __ldg(src + 2);
         if (4 * t + 3 < real) v.w = __ldg(src + 3);
-        quantize4<false>(v, rule, 0, min(4, real - 4 * t), c, wq[2 * t], wq[2 * t + 1]);
+        quantize4<false>(v, rule, 0u, 0u, min(4, real - 4 * t), c, wq[2 * t], wq[2 * t + 1]);
         wl[t] = low_bytes(wq[2 * t], wq[2 * t + 1]);
         wh[t] = high_bytes(wq[2 * t], wq[2 * t + 1]);
       }
@@ -456,7 +439,7 @@ __device__ __forceinline__ void quantize_padded_chunk(const QuantItem& it, const
       if (lo > 2 || hi < 3) v[t].z = 0.f;
       if (hi < 4) v[t].w = 0.f;
       uint32_t w0, w1;
-      quantize4<STOCH>(v[t], rule, b0 + (unsigned)t, hi - lo, c, w0, w1);
+      quantize4<STOCH>(v[t], rule, (uint32_t)(b0 + (unsigned)t), (uint32_t)((b0 + (unsigned)t) >> 32), hi - lo, c, w0, w1);
       wl[t] = low_bytes(w0, w1);
       wh[t] = high_bytes(w0, w1);
       if (it.q16 != nullptr) {
@@ -487,8 +470,10 @@ __device__ __forceinline__ void quantize_padded_chunk(const QuantItem& it, const
   }
 }
 
+// With a generator three blocks per SM for a single tensor, registers for more independent chains: 268 M elements 345 us with
+// four, 331 with three; a batch 83.6 and 91.
 template <bool STOCH, bool PADDED, int CAP>
-__global__ void __launch_bounds__(kQThreads, STOCH ? 4 : (PADDED ? 6 : 5)) quantize_kernel(const __grid_constant__ QuantArgs<CAP> a) {
+__global__ void __launch_bounds__(kQThreads, STOCH ? (CAP == 1 ? 3 : 4) : (PADDED ? 6 : 5)) quantize_kernel(const __grid_constant__ QuantArgs<CAP> a) {
   constexpr int kFlat = 2 * (kFlatBytes + 16);
   constexpr bool kByWarp = PADDED && STOCH;
   __shared__ __align__(16) uint8_t flat[kByWarp ? kQThreads / 32 * kFlat : 16];
@@ -497,12 +482,12 @@ __global__ void __launch_bounds__(kQThreads, STOCH ? 4 : (PADDED ? 6 : 5)) quant
   Counts c;
   // Chunks come in increasing order, so the search for a chunk's tensor only moves forward.
   int t = 0;
-  QuantRule rule = rule_of(a.item[0], a.relu);
+  QuantRule rule = rule_of(a.item[0], a.relu, a.stats != nullptr);
   for (unsigned long long chunk = blockIdx.x; chunk < a.total_chunks; chunk += gridDim.x) {
     if (CAP > 1) {
       const int was = t;
       while (t + 1 < a.n && a.item[t + 1].first_chunk <= chunk) ++t;
-      if (t != was) rule = rule_of(a.item[t], a.relu);
+      if (t != was) rule = rule_of(a.item[t], a.relu, a.stats != nullptr);
     }
     const QuantItem& it = a.item[t];
     const unsigned long long base = (chunk - it.first_chunk) * (unsigned)a.chunk;

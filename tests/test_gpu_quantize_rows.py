@@ -131,3 +131,25 @@ def test_a_batch_without_tensors():
     with pytest.raises(B.AdaptionError) as e:
         B.adaption_quantize_batch(None, 1)
     assert e.value.status == B.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("n_bits,f", [(16, 14), (8, 7), (4, 3)])
+def test_stochastic_decisions_next_to_the_draw(n_bits, f):
+    """Values whose fraction lies on, next to, or a last place of single precision away from the draw that decides them,
+    of both signs and all magnitudes down to 2^-40: the rounding in single precision takes no other side than exact arithmetic."""
+    n, seed = 1 << 16, 0xABCDEF0123456789
+    rng = np.random.default_rng(n_bits)
+    r = orc_st.draws(n, seed).astype(np.float64)
+    whole = rng.integers(-3, 4, n).astype(np.float64)
+    y = (whole + (r + rng.integers(-1, 3, n)) * 2.0 ** -32).astype(np.float32)
+    tiny = (rng.choice([-1.0, 1.0], n) * rng.uniform(1, 2, n) * 2.0 ** rng.integers(-40, 0, n)).astype(np.float32)
+    y = np.where(rng.random(n) < 0.25, tiny, y).astype(np.float32)
+    y = np.nextafter(y, y + rng.integers(-1, 2, n).astype(np.float32)).astype(np.float32)
+    x = (y * np.float32(2.0 ** -f)).reshape(-1, 64)                       # (exact: a power of two)
+    guards = Guards()
+    q, st = guards.qtensor(x.shape[0], 64, n_bits, f, 64), B.new_stats()
+    B.adaption_quantize_stochastic(dev(x), x.shape[0], 64, q, seed, False, None, st)
+    want, cnt = orc_st.quantize_stochastic(x, n_bits, f, seed, False)
+    assert np.array_equal(from_qtensor(q), want)
+    assert stats_tuple(st) == tuple(cnt)
+    guards.check()
