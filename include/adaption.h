@@ -235,7 +235,8 @@ ADAPTION_API int adaption_lp_ip_fwd_stochastic(int64_t B, int64_t K, int64_t O, 
  * convolution's own outputs, before pooling.  Requantizing mode only.  The convolution's output
  * lives in the workspace: where the tensor-core path can, only the maxima of horizontal pixel
  * pairs are stored there (half the bytes written and read back), otherwise all of it.  (Layers with
- * few output tiles pool inside their kernel: y is then written in the convolution's phase.)
+ * few output tiles, and those whose image sizes are covered by 128-pixel boxes, pool inside their kernel: y is
+ * then written in the convolution's phase.)
  * phases: ADAPTION_PHASE_CONV | ADAPTION_PHASE_POOL runs the whole layer pair; the two phases may
  * also be issued by two calls with otherwise identical arguments (convolution first, same stream
  * order, workspace untouched in between), e.g. to time them apart.

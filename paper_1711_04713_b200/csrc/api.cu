@@ -163,6 +163,7 @@ static int dispatch(const GemmProblem& g, int32_t algo) {
 struct ConvPoolPlan {
   bool cluster = false;      // the cluster kernel pools in its epilogue: no temporary planes
   bool fused = false;        // the layer kernel stores horizontal maxima
+  bool boxes = false;        // it pools whole windows (where y has no int16 copy): the temporary planes stay untouched
   size_t conv_ws = 0;        // bytes the convolution needs at the start of the workspace
   size_t plane = 0;          // bytes of one temporary plane
   size_t total = 0;
@@ -191,6 +192,11 @@ static ConvPoolPlan plan_conv_pool(GemmProblem g, int32_t algo) {
       pl.conv_ws = tensor_path_workspace(g);
       pl.fused = tensor_path_can_pool(g);
     }
+  }
+  if (algo != ADAPTION_ALGO_DIRECT && !packs && tensor_path_supported(g)) {
+    g.box_pool = true;
+    pl.boxes = tensor_path_can_pool_boxes(g);
+    g.box_pool = false;
   }
   pl.conv_ws = (pl.conv_ws + 255) & ~(size_t)255;
   const size_t rows = pl.fused ? (size_t)g.M / 2 : (size_t)g.M;
@@ -355,6 +361,10 @@ int adaption_lp_conv_pool_fwd(const adaption_conv_shape* h_shape, adaption_qtens
   if (pl.cluster) {          // one kernel does both phases
     g.pool2x2 = true;
     return (phases & ADAPTION_PHASE_CONV) ? launch_cluster(g) : ADAPTION_OK;
+  }
+  if (pl.boxes && y.q16 == nullptr) {
+    g.box_pool = true;
+    return (phases & ADAPTION_PHASE_CONV) ? launch_tensor(g) : ADAPTION_OK;
   }
   // temporary planes for the convolution's own (or half-pooled) output
   uint8_t* ws = static_cast<uint8_t*>(d_workspace);

@@ -114,21 +114,6 @@ __device__ __forceinline__ bool cg_wait(uint32_t bar, uint32_t parity, CgCtrl* c
   return cg_wait_slow(bar, parity, ctrl, p);
 }
 
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
-      "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z)
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z,
-                                            int w) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
-      "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w)
-      : "memory");
-}
 __device__ __forceinline__ void st_shared_pair(uint32_t addr, long long a, long long b) {
   asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(addr), "l"(a), "l"(b) : "memory");
 }
@@ -445,11 +430,11 @@ lp_cluster_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_const
           if (planes == 2) tma_load_2d<false>(dst + pb, m1, full, kb * p.BK, is_a ? r0 : c0);
         } else if (is_a) {
           const int x = ow0 * p.stride_w - p.pad_w + sx, y = oh0 * p.stride_h - p.pad_h + r;
-          tma_load_4d(dst, m0, full, cb * p.BK, x, y, img0);
-          if (planes == 2) tma_load_4d(dst + pb, m1, full, cb * p.BK, x, y, img0);
+          tma_load_4d<false>(dst, m0, full, cb * p.BK, x, y, img0);
+          if (planes == 2) tma_load_4d<false>(dst + pb, m1, full, cb * p.BK, x, y, img0);
         } else {
-          tma_load_3d(dst, m0, full, cb * p.BK, tap, c0);
-          if (planes == 2) tma_load_3d(dst + pb, m1, full, cb * p.BK, tap, c0);
+          tma_load_3d<false>(dst, m0, full, cb * p.BK, tap, c0);
+          if (planes == 2) tma_load_3d<false>(dst + pb, m1, full, cb * p.BK, tap, c0);
         }
       }
       __syncwarp();
@@ -855,7 +840,7 @@ int launch_cg(const CUtensorMap* maps, const CgParams& p, int grid, size_t smem,
 bool cluster_path_preferred(const GemmProblem& g) {
   const int mode = knob(kCluster);
   // (pair maxima are stored by the persistent kernel alone; a plan with planes of half the rows has chosen it)
-  if (mode == 0 || g.pool_w) return false;
+  if (mode == 0 || g.pool_w || g.box_pool) return false;
   // an override of the persistent kernel's tiles asks for that kernel
   for (Knob k : {kSplits, kPair, kFast, kStaged, kStages, kBK, kBN, kKps, kBres, kWide, kEpiGroups, kSplitHh, kStagger,
                  kStageBufs})

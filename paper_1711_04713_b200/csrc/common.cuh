@@ -271,6 +271,8 @@ struct GemmProblem {
   // Tensor-core path only: y receives max(row 2j, row 2j+1) of the layer's output as its row j (the
   // horizontal half of a 2x2 max-pool; y then has M / 2 rows).  Counters still refer to all M rows.
   bool pool_w = false;
+  // Tensor-core path only: y receives the 2x2 / stride-2 max-pool of the layer's output, from tiles that are boxes of pixels.
+  bool box_pool = false;
   // Cluster path only: y receives the 2x2 / stride-2 max-pool of the layer's output.
   bool pool2x2 = false;
   // rounding_scheme STOCHASTIC for the requantization of this layer (REQUANT mode only)
@@ -281,6 +283,7 @@ int launch_direct(const GemmProblem& p);
 bool tensor_path_supported(const GemmProblem& p);
 size_t tensor_path_workspace(const GemmProblem& p);
 int launch_tensor(const GemmProblem& p);
+bool tensor_path_can_pool_boxes(const GemmProblem& p);   // whether launch_tensor takes `p`, which has box_pool set
 bool tensor_path_can_pool(const GemmProblem& p);   // whether launch_tensor takes `p` with pool_w set
 int tensor_path_tiles(const GemmProblem& p, bool* split);   // its output tiles (0: cannot run), and whether it splits K
 // Layers with few output tiles: one cluster of CTAs per tile (no workspace).  The decision depends on

@@ -105,6 +105,19 @@ struct PixelPlan {
   uint32_t b_row[kMaxPixelBlocks][4];   // where its weights start in a filter row, in 16-byte units
 };
 
+// Tiles whose 128 rows are a box of 2^w x 2^h x 2^n pixels (columns fastest, then rows, then images) instead of
+// consecutive pixels: whole 2x2 windows of a max-pool lie in one tile, even in one warp, so the epilogue stores their
+// maxima, a quarter of the bytes, and no pooling pass reads the layer back.
+// Against storing pair maxima and pooling them vertically, us: 16 bits, 64 x 224 x 224 x 64 -> 64 531 -> 439, 64 x 112 x 112 x
+// 128 -> 128 345 -> 312, 64 x 56 x 56 x 256 -> 256 287 -> 270, 64 x 28 x 28 x 512 -> 512 263 -> 251; 8 bits, 128 images 448 ->
+// 435, 221 -> 174, 160 -> 131, 145 -> 129; one image 18 -> 15, 15 -> 13.
+struct BoxPlan {
+  int on, pool;
+  int w, h, n;                // powers of two, as exponents
+  int tiles_w, tiles_h, images;
+  FastDiv div_w, div_h;
+};
+
 struct TcParams {
   int M, N;
   int tile_m;                 // rows per tile: 128, or 256 for a CTA pair
@@ -166,6 +179,7 @@ struct TcParams {
   uint32_t stage_off;         // offset of the staging planes from the ring base
   uint32_t const_off;         // offset of the per-column epilogue constants (8 bytes per column and group)
   PixelPlan px;
+  BoxPlan box;
 };
 
 // Optional per-role time stamps of CTA 0 (development builds only: -DADAPTION_TIMELINE).
@@ -248,6 +262,20 @@ __device__ __forceinline__ TileCoord decode_tile(int t, const TcParams& p) {
   tc.kb_begin = split * p.kb_per_split;
   tc.kb_end = min(p.num_kb, tc.kb_begin + p.kb_per_split);
   return tc;
+}
+
+// First pixel of box `b`.
+struct BoxCoord {
+  int ow, oh, img;
+};
+__device__ __forceinline__ BoxCoord decode_box(int b, const BoxPlan& x) {
+  BoxCoord c;
+  const int rest = x.div_w.quot(b);
+  const int ib = x.div_h.quot(rest);
+  c.ow = (b - rest * x.tiles_w) << x.w;
+  c.oh = (rest - ib * x.tiles_h) << x.h;
+  c.img = ib << x.n;
+  return c;
 }
 
 template <int NACC>
@@ -630,15 +658,52 @@ __device__ __forceinline__ void store16_global(const uint32_t* w, const TcParams
 // chunks swizzled the way the bulk-tensor store expects for that row length, which also keeps the
 // 16-byte writes of a quarter warp on distinct banks) and leave as one bulk-tensor store per plane.
 // (Rows longer than the 128-byte swizzle span are kept as sub-planes of 128 columns, one store each.)
-__device__ __forceinline__ uint32_t staged_offset(int row, int chunk, int bn) {
+__device__ __forceinline__ uint32_t staged_offset(int row, int chunk, int bn, int rows = kBM) {
   const int sub = chunk >> 3;
   const int w = bn < 128 ? bn : 128;                       // row length of a (sub-)plane
   uint32_t off = (uint32_t)row * (uint32_t)w + (uint32_t)(chunk & 7) * 16u;
   off ^= ((off >> 7) & (uint32_t)((w >> 4) - 1) & 7u) << 4;
-  return off + (uint32_t)sub * (uint32_t)(kBM * 128);
+  return off + (uint32_t)sub * (uint32_t)(rows * 128);
 }
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint4 v) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void st_shared_b32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// 2x2 windows of a box tile: the four lanes of a window (they differ in lane bits 1 and `down`) hold sixteen channels of a
+// pixel each.  Every exchange hands over the half that the partner keeps, so each lane ends with the maxima of four
+// channels, `first` being the first of them.  16-bit values in pairs (eight words in, two out) or bytes 0 .. 127 (four in,
+// one out).
+template <bool BYTES, int WORDS>
+__device__ __forceinline__ void window_max(uint32_t (&w)[WORDS], int lane, int down, int& first) {
+  const bool right = (lane & 1) != 0, lower = (lane & down) != 0;
+#pragma unroll
+  for (int j = 0; j < WORDS / 2; ++j) {
+    const uint32_t other = __shfl_xor_sync(0xffffffffu, right ? w[j] : w[j + WORDS / 2], 1);
+    const uint32_t mine = right ? w[j + WORDS / 2] : w[j];
+    w[j] = BYTES ? max_bytes7(mine, other) : max_s16x2(mine, other);
+  }
+#pragma unroll
+  for (int j = 0; j < WORDS / 4; ++j) {
+    const uint32_t other = __shfl_xor_sync(0xffffffffu, lower ? w[j] : w[j + WORDS / 4], down);
+    const uint32_t mine = lower ? w[j + WORDS / 4] : w[j];
+    w[j] = BYTES ? max_bytes7(mine, other) : max_s16x2(mine, other);
+  }
+  first = (right ? 8 : 0) + (lower ? 4 : 0);
+}
+__device__ __forceinline__ void store_window_max(uint32_t (&wq)[8], int lane, int down, int window, int chunk, const TcParams& p,
+                                                 uint32_t stage_lo, uint32_t stage_hi) {
+  int first;
+  window_max<false>(wq, lane, down, first);
+  const uint32_t off = staged_offset(window, chunk, p.BN, kBM / 4) + (uint32_t)first;
+  st_shared_b32(stage_lo + off, __byte_perm(wq[0], wq[1], 0x6420));
+  if (p.rq.out_planes == 2) st_shared_b32(stage_hi + off, __byte_perm(wq[0], wq[1], 0x7531));
+}
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t src, int x, int y, int z, int w) {
+  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(map),
+               "r"(src), "r"(x), "r"(y), "r"(z), "r"(w)
                : "memory");
 }
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int x, int y) {
@@ -822,13 +887,20 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         int img = 0, base_h = 0, base_w = 0;
         int tap = 0, cb = 0, r = 0, sx = 0;       // position of kb in the (tap, channel block) order
         if (lane == 0 && warp == 0) TL_STAMP(0, (uint32_t)((t - worker) / workers), 0);
-        if (p.is_conv) {
+        if (p.box.on) {
+          const BoxCoord bc = decode_box(m_begin >> 7, p.box);
+          img = bc.img;
+          base_w = bc.ow - p.pad_w;
+          base_h = bc.oh - p.pad_h;
+        } else if (p.is_conv) {
           const int rest = p.div_ow.quot(m_begin);
           const int ow = m_begin - rest * p.OW;
           img = p.div_oh.quot(rest);
           const int oh = rest - img * p.OH;
           base_w = ow * p.stride_w - p.pad_w;
           base_h = oh * p.stride_h - p.pad_h;
+        }
+        if (p.is_conv) {
           tap = p.div_cblks.quot(tc.kb_begin);
           cb = tc.kb_begin - tap * p.cblks;
           r = p.div_s.quot(tap);
@@ -867,7 +939,9 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                   int d = sx + p.px.first;                     // (the block order begins with a full one)
                   if (d >= p.px.blocks) d -= p.px.blocks;
                   tma_load_im2col<false>(dst + my_off, my_map, full, 0, base_w, base_h, img, (uint16_t)d, (uint16_t)r);
-                } else if (is_a)
+                } else if (is_a && p.box.on)
+                  tma_load_4d<PAIR>(dst + my_off, my_map, full, cb * p.BK, base_w + sx, base_h + r, img);
+                else if (is_a)
                   tma_load_im2col<PAIR>(dst + my_off, my_map, full, cb * p.BK, base_w, base_h, img, (uint16_t)sx,
                                         (uint16_t)r);
                 else
@@ -1122,8 +1196,12 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     const int col_begin = min(p.BN, (ew >> 2) * cols_per_warp);
     const int col_end = min(p.BN, col_begin + cols_per_warp);
     const int row = quarter * 32 + lane;   // row of the tile (and of this CTA's staging planes)
-    const int plane_bytes = kBM * (PIX && p.pool_w ? p.BN >> 1 : p.BN);
+    const int plane_rows = p.box.pool ? kBM / 4 : kBM;
+    const int plane_bytes = plane_rows * (PIX && p.pool_w ? p.BN >> 1 : p.BN);
     const int planes_bytes = plane_bytes * p.rq.out_planes;
+    // box tiles: the lane of the pixel below, and the row of the stored tile that a 2x2 window becomes
+    const int down = 1 << p.box.w;
+    const int window = ((row >> (p.box.w + 1)) << (p.box.w - p.box.pool)) | ((row & (down - 1)) >> 1);
     const uint32_t stage_group = ring + p.stage_off + (uint32_t)(group * planes_bytes * p.stage_bufs);
     uint32_t stage_lo = stage_group;
     uint32_t stage_hi = stage_lo + (uint32_t)plane_bytes;
@@ -1185,8 +1263,16 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       if (lane == 0 && (ew & 3) == 0) TL_STAMP(2 + (ew >> 2), tile_iter, 1);
       if (!w) { ok = false; break; }
       tc_fence_after();
-      const int m = tc.m0 + (int)rank * kBM + row;
-      const bool row_ok = m < p.M;
+      int m = tc.m0 + (int)rank * kBM + row;
+      bool row_ok = m < p.M;
+      BoxCoord bc{0, 0, 0};
+      if (!PIX && p.box.on) {
+        bc = decode_box(m >> 7, p.box);
+        const int ow = bc.ow + (row & (down - 1)), oh = bc.oh + ((row >> p.box.w) & ((1 << p.box.h) - 1));
+        const int img = bc.img + (row >> (p.box.w + p.box.h));
+        row_ok = ow < p.OW && oh < p.OH && img < p.box.images;
+        m = (img * p.OH + oh) * p.OW + ow;
+      }
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * (uint32_t)(NACC * p.BN);
       // where this tile's high accumulator lives, and the barrier that hands it back
       const bool split = NACC == 3 && p.split_hh != 0;
@@ -1310,6 +1396,12 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             if (NACC == 1 && p.byte_out) {
               uint32_t b[4];
               fast_bytes16<PIX>(t, half, p.rq.shift, row_ok, col, p, cnt, b);
+              if (!PIX && p.box.pool) {
+                int first;
+                window_max<true>(b, lane, down, first);
+                st_shared_b32(stage_lo + staged_offset(window, (c0 >> 4) + half, p.BN, kBM / 4) + (uint32_t)first, b[0]);
+                continue;
+              }
               uint32_t at = staged_offset(row, (c0 >> 4) + half, p.BN);
               bool mine = true;
               if (pool_px) {
@@ -1331,7 +1423,9 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             else
               fast_outputs16<NACC, false, PIX>(t, h, half, p.rq.shift, p.rq.qmax, row_ok, col, p, cnt, wq);
             const int chunk = (c0 >> 4) + half;
-            if (pool_px) {
+            if (!PIX && p.box.pool) {
+              store_window_max(wq, lane, down, window, chunk, p, stage_lo, stage_hi);
+            } else if (pool_px) {
               // the right pixel of a pair: its maximum with the left one, one chunk of the pooled row
 #pragma unroll
               for (int j = 0; j < 8; ++j) left[j] = half == 0 ? wq[j] : max_s16x2(left[j], wq[j]);
@@ -1395,7 +1489,9 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             requant8<NACC, false, STOCH, PIX>(xa, bcol, p, row_ok, m, col, cnt, wq);
             requant8<NACC, false, STOCH, PIX>(xb, bcol + 8, p, row_ok, m, col + 8, cnt, wq + 4);
           }
-          if (p.staged && p.pool_w) {
+          if (!PIX && p.box.pool) {
+            store_window_max(wq, lane, down, window, c0 >> 4, p, stage_lo, stage_hi);
+          } else if (p.staged && p.pool_w) {
             // Horizontal half of a 2x2 max-pool: rows 2j and 2j+1 of the tile are neighbouring
             // pixels of one image row (even width, tiles start at even rows) and sit in neighbouring
             // lanes; the maximum of the packed 16-bit values is stored once, as row j.
@@ -1426,7 +1522,15 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       } else {
         epi_bar_sync(group, gthreads);
       }
-      if (p.staged && store_leader) {
+      if (!PIX && p.box.on && p.staged && store_leader) {
+        const int ow = bc.ow >> p.box.pool, oh = bc.oh >> p.box.pool;
+        for (int sub = 0; sub * 128 < p.BN; ++sub) {
+          const uint32_t so = (uint32_t)sub * (uint32_t)(plane_rows * 128);
+          tma_store_4d(&map_y_lo, stage_lo + so, tc.n0 + sub * 128, ow, oh, bc.img);
+          if (p.rq.out_planes == 2) tma_store_4d(&map_y_hi, stage_hi + so, tc.n0 + sub * 128, ow, oh, bc.img);
+        }
+        bulk_commit();
+      } else if (p.staged && store_leader) {
         const int m_first = (tc.m0 + (int)rank * kBM) >> (p.pool_w && !PIX ? 1 : 0);     // row of the stored tensor
         const int y_cols = PIX && p.pool_w ? p.BN >> 1 : p.BN;
         for (int sub = 0; sub * 128 < y_cols; ++sub) {
@@ -1485,7 +1589,43 @@ struct TcConfig {
   size_t smem_bytes = 0;
   size_t workspace_bytes = 0;
   PixelPlan px{};              // px.G > 1: pixels grouped (make_pixel_config)
+  BoxPlan box{};               // box.on: tiles are boxes of pixels
 };
+
+// Boxes of 2^w x 2^h x 2^n pixels over OW x OH pixels of `images` images.
+BoxPlan box_plan(int w, int h, int n, int OW, int OH, int images, bool pool) {
+  BoxPlan b{};
+  b.on = 1;
+  b.pool = pool ? 1 : 0;
+  b.w = w; b.h = h; b.n = n;
+  b.images = images;
+  b.tiles_w = (OW + (1 << w) - 1) >> w;
+  b.tiles_h = (OH + (1 << h) - 1) >> h;
+  b.div_w = fast_div(b.tiles_w);
+  b.div_h = fast_div(b.tiles_h);
+  return b;
+}
+int64_t box_count(const BoxPlan& b) {
+  return (int64_t)b.tiles_w * b.tiles_h * ((b.images + (1 << b.n) - 1) >> b.n);
+}
+// The boxes of 128 pixels with whole 2x2 windows that cover a layer with the fewest tiles, wide ones before narrow ones.
+// A window's rows have to lie in one warp of 32: at most 16 columns.  (box.on = 0: more than one tile in sixteen would be
+// margin; the pooling pass that boxes save takes 7 to 20 % of the layer.)
+BoxPlan pool_boxes(const GemmProblem& g) {
+  BoxPlan best{};
+  int64_t fewest = 0;
+  for (int w = 4; w >= 1; --w)
+    for (int h = 7 - w; h >= 1; --h) {
+      const BoxPlan b = box_plan(w, h, 7 - w - h, g.OW, g.OH, g.cs.N, true);
+      const int64_t n = box_count(b);
+      if (!best.on || n < fewest) {
+        best = b;
+        fewest = n;
+      }
+    }
+  if (fewest * kBM * 16 > g.M * 17 || fewest > (1 << 23)) best.on = 0;
+  return best;
+}
 
 TcConfig make_config_impl(const GemmProblem& g, bool allow_wide);
 
@@ -1552,6 +1692,12 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
                     knob(kWide) != 0 && !(partial && g.N % 8 != 0 && c.num_kb < 16);
   if (wide) c.BN = 256;
   c.tiles_m = (int)((g.M + kBM - 1) / kBM);
+  if (g.box_pool) {
+    if (!g.is_conv || g.cs.stride_h != 1 || g.cs.stride_w != 1) return c;
+    c.box = pool_boxes(g);
+    if (!c.box.on) return c;
+    c.tiles_m = (int)box_count(c.box);
+  }
   c.tiles_n = (int)((g.N + c.BN - 1) / c.BN);
   c.acc_bufs = 512 / (c.nacc * c.BN);
   if (c.acc_bufs > kMaxAccBufs) c.acc_bufs = kMaxAccBufs;
@@ -1602,7 +1748,7 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   if (pair_env == 1 && c.splits == 1 && (sms % 2) == 0) c.pair = true;
   if (c.pair) {
     c.tile_m = 2 * kBM;
-    c.tiles_m = (int)((g.M + c.tile_m - 1) / c.tile_m);
+    c.tiles_m = g.box_pool ? (c.tiles_m + 1) / 2 : (int)((g.M + c.tile_m - 1) / c.tile_m);
   }
   // Inner products on a small batch: only the rows that exist are staged (the MMA still covers 128
   // rows; the rest reads whatever follows in the stage and lands in accumulator rows nobody stores).
@@ -1630,7 +1776,7 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
                           c.num_kb >= (c.BN == 32 ? 9 : 10);
   const int most_groups = c.BN <= 64 && !two_groups ? 4 : 2;
   while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
-  c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) : 0u;
+  c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) / (c.box.pool ? 4u : 1u) : 0u;
   // dynamic shared memory: everything up to the per-block limit except the control block
   c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
   const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
@@ -1996,6 +2142,17 @@ extern "C" __attribute__((visibility("default"))) int adaption_debug_timeline(lo
 
 bool tensor_path_supported(const GemmProblem& g) { return make_config(g).ok; }
 
+// The whole 2x2 max-pool in the layer's epilogue (`g.box_pool`): box tiles.  (The columns of a pitch behind the last tile's
+// would stay unwritten.  Layers over 32 channels are grouped by pixels, which gains more than the pooling pass costs.)
+bool tensor_path_can_pool_boxes(const GemmProblem& g) {
+  if (knob(kBox) == 0) return false;
+  GemmProblem half = g;
+  half.box_pool = false;
+  if (make_pixel_config(half).ok) return false;
+  const TcConfig c = make_config(g);
+  return c.ok && c.box.on && c.staged && c.splits == 1 && g.y.c_stride <= (int64_t)c.tiles_n * c.BN;
+}
+
 // The horizontal half of a 2x2 max-pool can ride on the staged stores of a requantizing layer.
 bool tensor_path_can_pool(const GemmProblem& g) {
   const TcConfig c = make_config(g);
@@ -2045,7 +2202,8 @@ int launch_tensor(const GemmProblem& g) {
   const RequantParams rq = g.mode == ADAPTION_MODE_REQUANT ? make_requant(g.acc_frac_bits, g.y.fmt, g.relu)
                                                            : RequantParams{0, g.relu ? 1 : 0, 0, 0, 1};
   // (with grouped pixels only the rounding 32-bit epilogue pools)
-  TcConfig c = make_pixel_config(g);
+  TcConfig c;
+  if (!g.box_pool) c = make_pixel_config(g);
   if (!c.ok || (g.pool_w && !(c.staged && fast_epilogue(g, c, rq) == 1))) c = make_config(g);
   if (!c.ok) return ADAPTION_ERR_UNSUPPORTED;
   const int G = c.px.G > 1 ? c.px.G : 1;       // output pixels per row
@@ -2067,7 +2225,12 @@ int launch_tensor(const GemmProblem& g) {
   std::memset(maps, 0, sizeof(maps));
   for (int i = 0; i < 2; ++i) {
     bool ok;
-    if (g.is_conv)
+    if (c.box.on) {
+      const uint64_t px = (uint64_t)g.x.c_stride, W = (uint64_t)g.cs.W, H = (uint64_t)g.cs.H;
+      const uint64_t dims[4] = {px, W, H, (uint64_t)g.cs.N}, strides[3] = {px, px * W, px * W * H};
+      const uint32_t box[4] = {(uint32_t)c.BK, 1u << c.box.w, 1u << c.box.h, 1u << c.box.n};
+      ok = encode_tiled(&maps[i], xa[i], 4, dims, strides, box, nullptr, c.swizzle);
+    } else if (g.is_conv)
       ok = encode_im2col_nhwc(&maps[i], xa[i], cs, g.x.c_stride * G, (uint32_t)c.BK, (uint32_t)kBM, c.swizzle);
     else
       ok = encode_tiled_2d(&maps[i], xa[i], (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.x.c_stride,
@@ -2093,6 +2256,14 @@ int launch_tensor(const GemmProblem& g) {
     const void* planes[2] = {g.y.hi, g.y.lo};
     for (int i = 0; i < 2; ++i) {
       if (planes[i] == nullptr) continue;      // single-plane outputs have no high plane
+      if (c.box.on) {
+        const int half = c.box.pool;
+        const uint64_t W = (uint64_t)(g.OW >> half), H = (uint64_t)(g.OH >> half);
+        const uint64_t dims[4] = {ypitch, W, H, (uint64_t)g.cs.N}, strides[3] = {ypitch, ypitch * W, ypitch * W * H};
+        const uint32_t box[4] = {(uint32_t)ybox, 1u << (c.box.w - half), 1u << (c.box.h - half), 1u << c.box.n};
+        if (!encode_tiled(&maps[4 + i], planes[i], 4, dims, strides, box, nullptr, yswz)) return ADAPTION_ERR_CUDA;
+        continue;
+      }
       if (!encode_tiled_2d(&maps[4 + i], planes[i], ypitch, (uint64_t)(halve_rows ? M / 2 : M), ypitch, (uint32_t)ybox,
                            (uint32_t)(halve_rows ? kBM / 2 : kBM), yswz))
         return ADAPTION_ERR_CUDA;
@@ -2107,6 +2278,7 @@ int launch_tensor(const GemmProblem& g) {
   p.num_kb = c.num_kb; p.kb_per_split = c.kb_per_split;
   p.BN = c.BN; p.BK = c.BK; p.ksteps = c.BK / 32;
   p.px = c.px;
+  p.box = c.box;
   p.ksteps_last = g.is_conv ? c.ksteps_last : p.ksteps;
   p.sbo = (uint32_t)(8 * c.BK); p.layout_type = c.layout_type;
   p.stages = c.stages; p.a_bytes = c.a_bytes; p.b_bytes = c.b_bytes; p.stage_bytes = c.stage_bytes;
@@ -2138,6 +2310,7 @@ int launch_tensor(const GemmProblem& g) {
     p.y_hi = (int8_t*)g.y.hi; p.y_lo = (uint8_t*)g.y.lo; p.y_q16 = g.y.q16; p.y_stride = y_stride;
   }
   if (g.pool_w && !(c.staged && g.M % 2 == 0)) return ADAPTION_ERR_UNSUPPORTED;
+  if (g.box_pool && !(c.staged && c.box.pool)) return ADAPTION_ERR_UNSUPPORTED;
   p.pool_w = g.pool_w ? 1 : 0;
   p.epi_groups = c.epi_groups;
   p.staged = c.staged ? 1 : 0;

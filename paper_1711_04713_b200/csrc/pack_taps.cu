@@ -163,6 +163,7 @@ GemmProblem packed_problem(const GemmProblem& g, uint8_t* ws) {
   const PackLayout l = layout_of(g);
   GemmProblem q = g;
   q.is_conv = false;
+  q.box_pool = false;
   q.K = kPackK;
   const bool x2 = g.x.fmt.n_bits > 8, w2 = g.w.fmt.n_bits > 8;
   q.x.lo = ws;
