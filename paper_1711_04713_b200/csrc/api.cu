@@ -163,7 +163,8 @@ static int dispatch(const GemmProblem& g, int32_t algo) {
 struct ConvPoolPlan {
   bool cluster = false;      // the cluster kernel pools in its epilogue: no temporary planes
   bool fused = false;        // the layer kernel stores horizontal maxima
-  bool boxes = false;        // it pools whole windows (where y has no int16 copy): the temporary planes stay untouched
+  // it pools whole windows (where y has no int16 copy): the temporary planes stay untouched; taps: without packing them
+  bool boxes = false, taps = false;
   size_t conv_ws = 0;        // bytes the convolution needs at the start of the workspace
   size_t plane = 0;          // bytes of one temporary plane
   size_t total = 0;
@@ -193,10 +194,12 @@ static ConvPoolPlan plan_conv_pool(GemmProblem g, int32_t algo) {
       pl.fused = tensor_path_can_pool(g);
     }
   }
-  if (algo != ADAPTION_ALGO_DIRECT && !packs && tensor_path_supported(g)) {
+  if (algo != ADAPTION_ALGO_DIRECT && (packs || tensor_path_supported(g))) {
     g.box_pool = true;
+    g.taps = packs;
     pl.boxes = tensor_path_can_pool_boxes(g);
-    g.box_pool = false;
+    pl.taps = packs;
+    g.box_pool = g.taps = false;
   }
   pl.conv_ws = (pl.conv_ws + 255) & ~(size_t)255;
   const size_t rows = pl.fused ? (size_t)g.M / 2 : (size_t)g.M;
@@ -364,6 +367,7 @@ int adaption_lp_conv_pool_fwd(const adaption_conv_shape* h_shape, adaption_qtens
   }
   if (pl.boxes && y.q16 == nullptr) {
     g.box_pool = true;
+    g.taps = pl.taps;
     return (phases & ADAPTION_PHASE_CONV) ? launch_tensor(g) : ADAPTION_OK;
   }
   // temporary planes for the convolution's own (or half-pooled) output

@@ -273,6 +273,8 @@ struct GemmProblem {
   bool pool_w = false;
   // Tensor-core path only: y receives the 2x2 / stride-2 max-pool of the layer's output, from tiles that are boxes of pixels.
   bool box_pool = false;
+  // Tensor-core path only: a first layer over pixels of 16 bytes, read without packing.
+  bool taps = false;
   // Cluster path only: y receives the 2x2 / stride-2 max-pool of the layer's output.
   bool pool2x2 = false;
   // rounding_scheme STOCHASTIC for the requantization of this layer (REQUANT mode only)
@@ -283,6 +285,7 @@ int launch_direct(const GemmProblem& p);
 bool tensor_path_supported(const GemmProblem& p);
 size_t tensor_path_workspace(const GemmProblem& p);
 int launch_tensor(const GemmProblem& p);
+bool tensor_path_taps(const GemmProblem& p);             // whether launch_tensor takes `p`, which has taps set
 bool tensor_path_can_pool_boxes(const GemmProblem& p);   // whether launch_tensor takes `p`, which has box_pool set
 bool tensor_path_can_pool(const GemmProblem& p);   // whether launch_tensor takes `p` with pool_w set
 int tensor_path_tiles(const GemmProblem& p, bool* split);   // its output tiles (0: cannot run), and whether it splits K

@@ -58,7 +58,8 @@ constexpr int kEpiGeneric = 0, kEpiFast = 1, kEpiStochastic = 2, kEpiFastStochas
 // because the issuing warp's code decides the main loop's speed: with the bookkeeping of the third in the second
 // 64 x 224 x 224 x 64 -> 64 took 595 us against 515.)
 // kLoopPixels: neighbouring output pixels share a row of the GEMM, see PixelPlan.
-constexpr int kLoopPlain = 0, kLoopGrouped = 1, kLoopPartial = 2, kLoopPixels = 3;
+// kLoopHalo, kLoopTaps: the activations of a tile are copied once for all filter taps, see HaloPlan.
+constexpr int kLoopPlain = 0, kLoopGrouped = 1, kLoopPartial = 2, kLoopPixels = 3, kLoopHalo = 4, kLoopTaps = 5;
 
 // Division by a number fixed for the launch: q = (n * mul >> 32) >> shift for 0 <= n < 2^31 (mul =
 // ceil(2^(32 + shift) / d) with 2^(shift + 1) >= d > 2^shift; mul = 0 stands for d = 1).  An integer division costs a
@@ -118,6 +119,25 @@ struct BoxPlan {
   FastDiv div_w, div_h;
 };
 
+// One copy of a tile's activations for all filter taps (kLoopHalo, kLoopTaps), for convolutions of stride 1 on boxes of 8
+// columns x 16 rows: the copied box has the filter's margin around it, `w` pixels per row of it, and the operand of a tap is
+// the same rows of shared memory begun (r w + s) pixels further on: the eight rows of a swizzle group are eight pixels of
+// an image row, and the groups lie `w` pixels apart whatever the tap.  (The swizzle is a function of the address, so rows
+// may begin anywhere in its pattern.)  Copies deliver one row per two cycles whatever its length, and they write shared
+// memory while the MMAs read it: 3x3 filters take 180 rows per tile this way, 1152 before.  us, before -> now: 16 bits, 64 x
+// 224 x 224 x 64 -> 64 488 -> 322 (pooled 441 -> 329), 64 x 112 x 112 x 64 -> 128 185 -> 161; 8 bits, 128 images 385 -> 338
+// (439 -> 342), 128 x 112 x 112 x 128 -> 128 192 -> 169 (173 -> 146).
+// kLoopTaps is the same for the pixels of 16 bytes of a first layer, unswizzled: a step of 32 bytes is two taps, whose
+// distance is the operand's leading offset.  No packed copy of the image is written and read back.
+constexpr int kHaloW = 8, kHaloH = 16, kMaxTapSteps = 5;
+struct HaloPlan {
+  int w, R, S;
+  int steps;                       // kLoopTaps: steps of 32 bytes (0: kLoopHalo)
+  uint32_t px_u;                   // a pixel in 16-byte units
+  uint32_t b_row_u;                // kLoopTaps: weights of a step in 16-byte units
+  uint32_t a_lo[kMaxTapSteps];     // kLoopTaps: low descriptor word of a step relative to the tile's first pixel
+};
+
 struct TcParams {
   int M, N;
   int tile_m;                 // rows per tile: 128, or 256 for a CTA pair
@@ -131,10 +151,10 @@ struct TcParams {
   // a stage holds `kps` consecutive k-blocks of `kb_bytes` each (short k-blocks are grouped so
   // that the per-stage hand-shake is amortised over enough MMAs)
   int kps;
-  uint32_t kb_bytes;
+  uint32_t kb_bytes, tx_bytes;     // tx_bytes: what the copies of a k-block deliver
   // weights resident in shared memory (one column tile, short reduction): the ring then holds
   // only activation planes and all weight k-blocks are loaded once per CTA at this offset
-  int b_resident;
+  int b_resident, b_blocks;        // b_blocks: weight k-blocks (kLoopTaps: slabs of a tap) that are resident
   uint32_t b_res_off;
   int acc_bufs, acc_shift;    // 1, 2 or 4 accumulator sets, and the power of two
   FastDiv div_tiles_n, div_splits, div_ow, div_oh, div_s, div_cblks;
@@ -180,6 +200,7 @@ struct TcParams {
   uint32_t const_off;         // offset of the per-column epilogue constants (8 bytes per column and group)
   PixelPlan px;
   BoxPlan box;
+  HaloPlan halo;
 };
 
 // Optional per-role time stamps of CTA 0 (development builds only: -DADAPTION_TIMELINE).
@@ -771,6 +792,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                const __grid_constant__ TcParams p) {
   constexpr int NACC = NAX + NBW - 1;
   constexpr bool GROUPED = LOOP == kLoopGrouped, PARTIAL = LOOP == kLoopPartial, PIX = LOOP == kLoopPixels;
+  constexpr bool HALO = LOOP == kLoopHalo, TAPS = LOOP == kLoopTaps;
   constexpr bool FAST = EPI == kEpiFast;
   constexpr bool STOCH = EPI == kEpiStochastic, FASTST = EPI == kEpiFastStochastic;
   extern __shared__ uint8_t smem_raw[];
@@ -827,7 +849,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     // Planes that are streamed through the ring: all of them, or only the activation planes when
     // the weights are resident.  With fewer streamed planes than producer warps, several warps
     // share a plane and take turns stage by stage.
-    const bool b_res = PIX || (GROUPED && p.b_resident);
+    const bool b_res = PIX || HALO || TAPS || (GROUPED && p.b_resident);
     const int nact = b_res ? NAX : NPLANES;
     const int kps = GROUPED ? p.kps : 1;
     const int nsub = nact >= kProducerWarps ? 1 : kProducerWarps / nact;   // warps per streamed plane
@@ -850,7 +872,17 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         // all reporting to one barrier
         // (in a pair each CTA fetches its own half of the weight rows; the bytes of both are counted
         // on the leader's barrier, which the leader arms for both)
-        if (PIX) {
+        if (TAPS) {
+          // a slab of 16-byte rows per tap (the one behind the last tap of an odd number arrives as zeros)
+          if (elect_one()) {
+            const uint32_t bar = smem_u32(&ctrl.b_ready);
+            mbar_expect_tx(bar, NBW * p.b_bytes);
+            for (int tap = 0; tap < p.b_blocks; ++tap)
+              for (int bplane = 0; bplane < NBW; ++bplane)
+                tma_load_3d<false>(ring + p.b_res_off + (uint32_t)bplane * p.b_bytes + (uint32_t)(tap * p.BN * 16),
+                                   bplane == 0 ? &map_b0 : &map_b1, bar, 0, tap, 0);
+          }
+        } else if (PIX) {
           if (elect_one()) {
             const uint32_t bar = smem_u32(&ctrl.b_ready);
             mbar_expect_tx(bar, NBW * p.px.b_plane);
@@ -865,16 +897,16 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           }
         } else if (elect_one()) {
           uint32_t bar = smem_u32(&ctrl.b_ready);
-          if (rank == 0) mbar_expect_tx(bar, (PAIR ? 2u : 1u) * (uint32_t)p.num_kb * NBW * p.b_bytes);
+          const int tiles_n = HALO ? p.tiles_n : 1;
+          if (rank == 0) mbar_expect_tx(bar, (PAIR ? 2u : 1u) * (uint32_t)(tiles_n * p.b_blocks) * NBW * p.b_bytes);
           if (PAIR) bar = mapa_rank(bar, 0);
-          for (int kb = 0; kb < p.num_kb; ++kb) {
-            const int kcol = p.is_conv ? (kb / p.cblks) * p.w_pitch + (kb % p.cblks) * p.BK : kb * p.BK;
-            for (int bplane = 0; bplane < NBW; ++bplane) {
-              const uint32_t dst =
-                  ring + p.b_res_off + (uint32_t)kb * (NBW * p.b_bytes) + (uint32_t)bplane * p.b_bytes;
-              tma_load_2d<PAIR>(dst, bplane == 0 ? &map_b0 : &map_b1, bar, kcol, (int)rank * b_rows);
+          uint32_t dst = ring + p.b_res_off;
+          for (int tn = 0; tn < tiles_n; ++tn)
+            for (int kb = 0; kb < p.b_blocks; ++kb) {
+              const int kcol = p.is_conv ? (kb / p.cblks) * p.w_pitch + (kb % p.cblks) * p.BK : kb * p.BK;
+              for (int bplane = 0; bplane < NBW; ++bplane, dst += p.b_bytes)
+                tma_load_2d<PAIR>(dst, bplane == 0 ? &map_b0 : &map_b1, bar, kcol, tn * p.BN + (int)rank * b_rows);
             }
-          }
         }
         __syncwarp();
       }
@@ -900,7 +932,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           base_w = ow * p.stride_w - p.pad_w;
           base_h = oh * p.stride_h - p.pad_h;
         }
-        if (p.is_conv) {
+        if (p.is_conv && !HALO && !TAPS) {
           tap = p.div_cblks.quot(tc.kb_begin);
           cb = tc.kb_begin - tap * p.cblks;
           r = p.div_s.quot(tap);
@@ -911,7 +943,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           const int nkb = GROUPED ? min(kps, tc.kb_end - kb) : 1;      // k-blocks in this stage
           const bool my_turn = turn == sub;           // ring slots have fixed owners
           if (++turn == nsub) turn = 0;
-          if ((GROUPED || PIX) && !my_turn) {
+          if ((GROUPED || PIX || HALO || TAPS) && !my_turn) {
             if (++s == p.stages) { s = 0; ph ^= 1u; turn = 0; }
             continue;
           }
@@ -930,11 +962,15 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             if (PAIR) full = mapa_rank(full, 0);
             dst = ring + (uint32_t)s * p.stage_bytes;
             if (act_plane == 0 && rank == 0 && elect_one())
-              mbar_expect_tx(smem_u32(&ctrl.full[s]), (PAIR ? 2u : 1u) * (uint32_t)nkb * p.kb_bytes);
+              mbar_expect_tx(smem_u32(&ctrl.full[s]), (PAIR ? 2u : 1u) * (uint32_t)nkb * p.tx_bytes);
           }
           for (int j = 0; j < nkb; ++j) {
             if (my_turn && elect_one()) {
-              if (p.is_conv) {
+              if (TAPS) {
+                tma_load_3d<PAIR>(dst + my_off, my_map, full, 2 * base_w, base_h, img);
+              } else if (HALO) {
+                tma_load_4d<PAIR>(dst + my_off, my_map, full, kb * p.BK, base_w, base_h, img);
+              } else if (p.is_conv) {
                 if (PIX) {
                   int d = sx + p.px.first;                     // (the block order begins with a full one)
                   if (d >= p.px.blocks) d -= p.px.blocks;
@@ -954,7 +990,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
               }
             }
             dst += p.kb_bytes;
-            if (p.is_conv) {
+            if (p.is_conv && !HALO && !TAPS) {
               if (++cb == p.cblks) {
                 cb = 0;
                 ++tap;
@@ -1009,7 +1045,9 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       const uint32_t id_uu = make_idesc(false, false, id_n, tile_rows);
       const uint32_t dhi_b = smem_desc_hi(256, 6);                  // PIX: weight rows of 32 bytes
       const uint32_t dhi = smem_desc_hi(p.sbo, p.layout_type);
-      const uint32_t ring_lo = smem_desc_lo(ring);
+      // (weights of a tile that is copied with its margin: rows of their own; kLoopTaps gives leading offsets step by step)
+      const uint32_t dhi_rows = TAPS ? smem_desc_hi(128, 0) : smem_desc_hi((uint32_t)(8 * p.BK), p.layout_type);
+      const uint32_t ring_lo = TAPS ? smem_desc_lo(ring) - (1u << 16) : smem_desc_lo(ring);
       const uint32_t stage_u = p.stage_bytes >> 4, a_u = p.a_bytes >> 4, b_u = p.b_bytes >> 4;
       const uint32_t kb_u = p.kb_bytes >> 4;
       const uint32_t off_a1 = a_u, off_b0 = NAX * a_u;
@@ -1019,9 +1057,12 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       uint32_t a0 = ring_lo, full_bar = full_bar0, empty_bar = empty_bar0;
       int s = 0;
       bool ok = true;
-      const bool b_res = PIX || (GROUPED && p.b_resident);
+      const bool b_res = PIX || HALO || TAPS || (GROUPED && p.b_resident);
       const int kps = GROUPED ? p.kps : 1;
-      const uint32_t bres_lo = smem_desc_lo(ring + p.b_res_off), bres_u = NBW * b_u;
+      const uint32_t bres_lo = smem_desc_lo(ring + p.b_res_off) + (TAPS ? (uint32_t)(p.BN - 1) << 16 : 0u), bres_u = NBW * b_u;
+      const uint32_t issue = HALO || TAPS ? (elect_one() ? 1u : 0u) : 0u;
+      const int halo_r = p.halo.R, halo_s = p.halo.S;
+      const uint32_t px_u = p.halo.px_u, row_u = (uint32_t)p.halo.w * px_u, tap_u = (uint32_t)p.cblks * bres_u;
       if (b_res) {
         ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&ctrl.b_ready), 0u, &ctrl, p, false));
         tc_fence_after();
@@ -1047,7 +1088,8 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         const uint32_t d0 = dset + hh_sel * (uint32_t)(3 * p.BN);
         const uint32_t d1 = dset + (uint32_t)p.BN, d2 = dset + 2u * (uint32_t)p.BN;
         uint32_t bres = bres_lo + (uint32_t)tc.kb_begin * bres_u;   // resident weights of this k-block
-        const bool stagger = !GROUPED && !PIX && NAX == 2 && NBW == 2 && p.tail_stagger != 0;
+        if (HALO && tc.n0 != 0) bres += (uint32_t)p.b_blocks * bres_u;
+        const bool stagger = !GROUPED && !PIX && !HALO && !TAPS && NAX == 2 && NBW == 2 && p.tail_stagger != 0;
         const int kb_main_end = stagger ? tc.kb_end - 2 : tc.kb_end;
         int cb = PARTIAL ? tc.kb_begin % p.cblks : 0;               // channel block of its tap
         int pb = 0;                                                 // block of input pixels
@@ -1071,7 +1113,36 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           if (!ok) break;
           tc_fence_after();
           const uint32_t acc = kb == tc.kb_begin ? 0u : 1u;
-          if (elect_one()) {
+          if (HALO) {
+            // the taps of this channel block: the same copied rows from different pixels on
+            uint32_t a = a0, b = bres + (uint32_t)kb * bres_u, first = acc;
+            const int steps = kb == p.cblks - 1 ? p.ksteps_last : ksteps_full;
+#pragma unroll 1
+            for (int r = 0; r < halo_r; ++r) {
+              uint32_t at = a;
+#pragma unroll 1
+              for (int sx = 0; sx < halo_s; ++sx) {
+                mma_kblock_if<NAX, NBW, PAIR>(issue, d0, d1, d2, at, off_a1, b, b_u, dhi, dhi_rows, id_ss, id_su, id_us, id_uu,
+                                              steps, first);
+                first = 1u;
+                at += px_u;
+                b += tap_u;
+              }
+              a += row_u;
+            }
+            tc_commit_if<PAIR>(issue, empty_bar);              // stage reusable once these MMAs retire
+          } else if (TAPS) {
+            uint32_t b = bres_lo, first = 0u;
+#pragma unroll 1
+            for (int i = 0; i < p.halo.steps; ++i) {
+              const uint32_t a = a0 + p.halo.a_lo[i];
+              mma_kstep_if<NAX, NBW, false>(issue, d0, d1, d2, a, a + off_a1, b, b + b_u, dhi, dhi_rows, id_ss, id_su, id_us,
+                                            id_uu, first);
+              first = 1u;
+              b += p.halo.b_row_u;
+            }
+            tc_commit_if<PAIR>(issue, empty_bar);
+          } else if (elect_one()) {
             // a0 / ak: low descriptor word of the first A plane of a k-block; the other planes and
             // the k-steps are fixed offsets (16-byte units) from it (weights: in the stage or
             // resident).  The first k-block is straight-line code; grouped stages loop over the rest.
@@ -1590,6 +1661,9 @@ struct TcConfig {
   size_t workspace_bytes = 0;
   PixelPlan px{};              // px.G > 1: pixels grouped (make_pixel_config)
   BoxPlan box{};               // box.on: tiles are boxes of pixels
+  HaloPlan halo{};             // halo.w > 0: one copy of activations for all taps (make_halo_config)
+  int b_blocks = 0;            // weight k-blocks that are resident
+  uint32_t a_tx = 0;           // bytes of one copy of activations, where they are not a_bytes
 };
 
 // Boxes of 2^w x 2^h x 2^n pixels over OW x OH pixels of `images` images.
@@ -1814,6 +1888,7 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   if (c.tiles_n == 1 && c.splits == 1 && c.tiles_m >= 4 * sms && (!c.pair || knob(kBres) != 2) &&
       res_bytes + 3 * (size_t)c.kps * c.nax * c.a_bytes + 1024 <= budget && knob(kBres) != 0) {
     c.b_resident = true;
+    c.b_blocks = c.num_kb;
     c.b_res_bytes = (uint32_t)res_bytes;
     c.kb_bytes = c.nax * c.a_bytes;
   }
@@ -1952,6 +2027,102 @@ TcConfig make_pixel_config(const GemmProblem& g) {
   return TcConfig();
 }
 
+// One copy of the activations for all taps (see HaloPlan), where the weights stay resident beside at least two tiles'
+// copies of them: operands of one width, 8 x 16 boxes without much margin.
+TcConfig make_halo_config(const GemmProblem& g) {
+  TcConfig c;
+  if (knob(kHalo) == 0 || !g.is_conv || g.pool_w || g.cs.stride_h != 1 || g.cs.stride_w != 1 || g.cs.R > 15 || g.cs.S > 15 ||
+      g.M > (int64_t)1 << 30 || g.x.c_stride != g.w.c_stride)
+    return c;
+  for (Knob k : {kSplits, kPair, kStages, kBK, kBN, kKps, kBres, kWide, kStageBufs})
+    if (knob(k) != kKnobDefaults[k]) return TcConfig();        // an override of the other tiles asks for them
+  const int sms = num_sms(), taps = g.cs.R * g.cs.S;
+  const int64_t cs = g.x.c_stride;
+  c.nax = g.x.fmt.n_bits > 8 ? 2 : 1;
+  c.nbw = g.w.fmt.n_bits > 8 ? 2 : 1;
+  c.nacc = c.nax + c.nbw - 1;
+  if (c.nax != c.nbw || g.N > 128) return c;
+  c.BN = g.N <= 32 ? 32 : (g.N <= 64 ? 64 : 128);
+  c.tiles_n = 1;
+  c.box = box_plan(3, 4, 0, g.OW, g.OH, g.cs.N, g.box_pool);
+  const int64_t boxes = box_count(c.box);
+  if (boxes > (1 << 23) || boxes * kBM * 16 > g.M * 17) return c;
+  HaloPlan& h = c.halo;
+  h.w = kHaloW + g.cs.S - 1;
+  h.R = g.cs.R;
+  h.S = g.cs.S;
+  if (g.taps) {
+    // pixels of 16 bytes: two taps are a step of 32
+    h.steps = (taps + 1) / 2;
+    if (cs != 16 || h.steps > kMaxTapSteps) return c;
+    c.BK = 16;
+    h.px_u = 1;
+    h.b_row_u = (uint32_t)(2 * c.BN);
+    for (int i = 0; i < h.steps; ++i) {
+      const int t0 = 2 * i, t1 = 2 * i + 1 < taps ? 2 * i + 1 : 2 * i;     // (behind the last tap the weights are zero)
+      const int at0 = t0 / g.cs.S * h.w + t0 % g.cs.S, at1 = t1 / g.cs.S * h.w + t1 % g.cs.S;
+      h.a_lo[i] = (uint32_t)at0 | (uint32_t)(at1 - at0) << 16;
+    }
+    c.num_kb = 1;
+    c.ksteps_last = 1;
+    c.b_blocks = 2 * h.steps;
+    c.b_bytes = (uint32_t)(c.b_blocks * c.BN * 16);
+    c.b_res_bytes = (uint32_t)c.nbw * c.b_bytes;
+    c.tiles_m = (int)boxes;
+  } else {
+    if (taps < 4 || cs % 32 != 0 || cs < 64 || c.BN < 64 || (sms & 1) != 0 || taps * cs > kMaxKPerAccumulation) return c;
+    c.BK = cs > 64 ? 128 : 64;
+    c.cblks = (int)((cs + c.BK - 1) / c.BK);
+    c.ksteps_last = (int)(cs - (int64_t)(c.cblks - 1) * c.BK) / 32;
+    c.swizzle = c.BK == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    c.layout_type = c.BK == 128 ? 2u : 4u;
+    h.px_u = (uint32_t)(c.BK / 16);
+    c.pair = true;
+    c.tile_m = 2 * kBM;
+    c.num_kb = c.cblks;
+    c.b_blocks = taps * c.cblks;
+    c.b_bytes = (uint32_t)(c.BN / 2 * c.BK);
+    // 16-bit operands: two tiles of 64 columns rather than one of 128, whose three accumulators could not be doubled
+    // (64 x 112 x 112 x 64 -> 128: 205 us with one, 158 with two)
+    if (c.nacc == 3 && c.BN == 128) {
+      c.BN = 64;
+      c.b_bytes /= 2;
+      c.tiles_n = 2;
+    }
+    // (8 bits, 128 columns over 64 channels: the epilogue bounds either form, 145 us against 138 with 128 images)
+    if (c.nacc == 1 && c.BN == 128 && cs == 64) return c;
+    c.b_res_bytes = (uint32_t)(c.tiles_n * c.b_blocks * c.nbw) * c.b_bytes;
+    c.tiles_m = (int)((boxes + 1) / 2);
+    if (c.tiles_m < sms / 2) return c;
+  }
+  c.kb_per_split = c.num_kb;
+  c.a_tx = (uint32_t)(h.w * (kHaloH + g.cs.R - 1) * c.BK);
+  c.a_bytes = (c.a_tx + 1023u) & ~1023u;
+  c.kb_bytes = c.stage_bytes = (uint32_t)c.nax * c.a_bytes;
+  c.acc_bufs = 512 / (c.nacc * c.BN);
+  if (c.acc_bufs > kMaxAccBufs) c.acc_bufs = kMaxAccBufs;
+  if (c.acc_bufs == 3) c.acc_bufs = 2;
+  while (c.tmem_cols < (uint32_t)(c.acc_bufs * c.nacc * c.BN)) c.tmem_cols <<= 1;
+  const int out_planes = g.y.fmt.n_bits > 8 ? 2 : 1;
+  c.staged = g.mode == ADAPTION_MODE_REQUANT && g.y.q16 == nullptr && g.y.lo != nullptr && g.y.c_stride >= c.BN &&
+             g.y.c_stride % 16 == 0 && knob(kStaged) != 0;
+  if (g.box_pool && !c.staged) return c;
+  c.epi_groups = c.acc_bufs;
+  const int most_groups = c.BN <= 64 ? 4 : 2;
+  while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
+  c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) / (g.box_pool ? 4u : 1u) : 0u;
+  c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
+  const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
+  c.b_resident = true;
+  if (c.b_res_bytes + 2 * c.stage_bytes + 1024 > budget) return c;
+  c.stages = (int)((budget - 1024 - c.b_res_bytes) / c.stage_bytes);
+  if (c.stages > kMaxStages) c.stages = kMaxStages;
+  c.stage_off = (uint32_t)(((size_t)c.stages * c.stage_bytes + c.b_res_bytes + 1023) & ~(size_t)1023);
+  c.smem_bytes = (size_t)c.stage_off + 1024 + c.stage_out_bytes + c.const_bytes;
+  c.ok = true;
+  return c;
+}
+
 template <int NAX, int NBW, bool PAIR, int LOOP, int EPI>
 int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
   // The dynamic shared-memory limit is a per-device attribute of the kernel: remember, per device
@@ -2024,6 +2195,10 @@ template <int NAX, int NBW>
 int launch_either(bool pair, const CUtensorMap* maps, const TcParams& p, int grid, size_t smem,
                   cudaStream_t stream) {
   if (p.px.G > 1) return launch_epi<NAX, NBW, false, kLoopPixels>(maps, p, grid, smem, stream);
+  if constexpr (NAX == NBW) {
+    if (p.halo.steps > 0) return launch_epi<NAX, NBW, false, kLoopTaps>(maps, p, grid, smem, stream);
+    if (p.halo.w > 0) return launch_epi<NAX, NBW, true, kLoopHalo>(maps, p, grid, smem, stream);
+  }
   return pair ? launch_loop<NAX, NBW, true>(maps, p, grid, smem, stream)
               : launch_loop<NAX, NBW, false>(maps, p, grid, smem, stream);
 }
@@ -2142,14 +2317,18 @@ extern "C" __attribute__((visibility("default"))) int adaption_debug_timeline(lo
 
 bool tensor_path_supported(const GemmProblem& g) { return make_config(g).ok; }
 
+// A first layer whose pixels of 16 bytes are read by the layer kernel itself (`g.taps`).
+bool tensor_path_taps(const GemmProblem& g) { return make_halo_config(g).ok; }
+
 // The whole 2x2 max-pool in the layer's epilogue (`g.box_pool`): box tiles.  (The columns of a pitch behind the last tile's
 // would stay unwritten.  Layers over 32 channels are grouped by pixels, which gains more than the pooling pass costs.)
 bool tensor_path_can_pool_boxes(const GemmProblem& g) {
   if (knob(kBox) == 0) return false;
   GemmProblem half = g;
   half.box_pool = false;
-  if (make_pixel_config(half).ok) return false;
-  const TcConfig c = make_config(g);
+  TcConfig c = make_halo_config(g);
+  if (!c.ok && (g.taps || make_pixel_config(half).ok)) return false;
+  if (!c.ok) c = make_config(g);
   return c.ok && c.box.on && c.staged && c.splits == 1 && g.y.c_stride <= (int64_t)c.tiles_n * c.BN;
 }
 
@@ -2202,8 +2381,9 @@ int launch_tensor(const GemmProblem& g) {
   const RequantParams rq = g.mode == ADAPTION_MODE_REQUANT ? make_requant(g.acc_frac_bits, g.y.fmt, g.relu)
                                                            : RequantParams{0, g.relu ? 1 : 0, 0, 0, 1};
   // (with grouped pixels only the rounding 32-bit epilogue pools)
-  TcConfig c;
-  if (!g.box_pool) c = make_pixel_config(g);
+  TcConfig c = make_halo_config(g);
+  if (!c.ok && g.taps) return ADAPTION_ERR_UNSUPPORTED;
+  if (!c.ok && !g.box_pool) c = make_pixel_config(g);
   if (!c.ok || (g.pool_w && !(c.staged && fast_epilogue(g, c, rq) == 1))) c = make_config(g);
   if (!c.ok) return ADAPTION_ERR_UNSUPPORTED;
   const int G = c.px.G > 1 ? c.px.G : 1;       // output pixels per row
@@ -2226,10 +2406,19 @@ int launch_tensor(const GemmProblem& g) {
   for (int i = 0; i < 2; ++i) {
     bool ok;
     if (c.box.on) {
+      // (with the filter's margin around it where all taps share one copy)
       const uint64_t px = (uint64_t)g.x.c_stride, W = (uint64_t)g.cs.W, H = (uint64_t)g.cs.H;
-      const uint64_t dims[4] = {px, W, H, (uint64_t)g.cs.N}, strides[3] = {px, px * W, px * W * H};
-      const uint32_t box[4] = {(uint32_t)c.BK, 1u << c.box.w, 1u << c.box.h, 1u << c.box.n};
-      ok = encode_tiled(&maps[i], xa[i], 4, dims, strides, box, nullptr, c.swizzle);
+      const uint32_t bw = c.halo.w > 0 ? (uint32_t)c.halo.w : 1u << c.box.w;
+      const uint32_t bh = c.halo.w > 0 ? (uint32_t)(kHaloH + g.cs.R - 1) : 1u << c.box.h;
+      if (c.halo.steps > 0) {
+        const uint64_t dims[3] = {2 * W, H, (uint64_t)g.cs.N}, strides[2] = {px * W, px * W * H};
+        const uint32_t box[3] = {2 * bw, bh, 1u};
+        ok = encode_tiled_words(&maps[i], xa[i], 3, dims, strides, box);
+      } else {
+        const uint64_t dims[4] = {px, W, H, (uint64_t)g.cs.N}, strides[3] = {px, px * W, px * W * H};
+        const uint32_t box[4] = {(uint32_t)c.BK, bw, bh, 1u << c.box.n};
+        ok = encode_tiled(&maps[i], xa[i], 4, dims, strides, box, nullptr, c.swizzle);
+      }
     } else if (g.is_conv)
       ok = encode_im2col_nhwc(&maps[i], xa[i], cs, g.x.c_stride * G, (uint32_t)c.BK, (uint32_t)kBM, c.swizzle);
     else
@@ -2238,6 +2427,13 @@ int launch_tensor(const GemmProblem& g) {
     if (!ok) return ADAPTION_ERR_CUDA;
     const uint64_t wk = g.is_conv ? (uint64_t)g.cs.R * g.cs.S * g.w.c_stride : (uint64_t)g.K;
     const uint64_t wpitch = g.is_conv ? wk : (uint64_t)g.w.c_stride;
+    if (c.halo.steps > 0) {
+      const uint64_t taps = (uint64_t)g.cs.R * g.cs.S;
+      const uint64_t dims[3] = {2, taps, (uint64_t)g.N}, strides[2] = {16, 16 * taps};
+      const uint32_t box[3] = {2u, 1u, (uint32_t)c.BN};
+      if (!encode_tiled_words(&maps[2 + i], wb[i], 3, dims, strides, box)) return ADAPTION_ERR_CUDA;
+      continue;
+    }
     const bool rows32 = G > 1;                 // grouped pixels: weight rows of one 32-byte step
     if (!encode_tiled_2d(&maps[2 + i], wb[i], wk, (uint64_t)g.N, wpitch, rows32 ? 32u : (uint32_t)c.BK,
                          (uint32_t)(rows32 ? c.px.ys : (c.pair ? c.BN / 2 : c.BN)),
@@ -2279,11 +2475,14 @@ int launch_tensor(const GemmProblem& g) {
   p.BN = c.BN; p.BK = c.BK; p.ksteps = c.BK / 32;
   p.px = c.px;
   p.box = c.box;
+  p.halo = c.halo;
   p.ksteps_last = g.is_conv ? c.ksteps_last : p.ksteps;
-  p.sbo = (uint32_t)(8 * c.BK); p.layout_type = c.layout_type;
+  p.sbo = (uint32_t)((c.halo.w > 0 ? c.halo.w : 8) * c.BK); p.layout_type = c.layout_type;
   p.stages = c.stages; p.a_bytes = c.a_bytes; p.b_bytes = c.b_bytes; p.stage_bytes = c.stage_bytes;
   p.kps = c.kps; p.kb_bytes = c.kb_bytes;
+  p.tx_bytes = c.a_tx != 0 ? (uint32_t)c.nax * c.a_tx : c.kb_bytes;
   p.b_resident = c.b_resident ? 1 : 0;
+  p.b_blocks = c.b_blocks;
   p.b_res_off = (uint32_t)c.stages * c.stage_bytes;
   p.acc_bufs = c.acc_bufs;
   p.acc_shift = c.acc_bufs == 4 ? 2 : (c.acc_bufs == 2 ? 1 : 0);
@@ -2326,7 +2525,7 @@ int launch_tensor(const GemmProblem& g) {
   p.fast_stochastic = fast == 2 ? 1 : 0;
   p.byte_out = p.fast_relu && c.nacc == 1 && c.staged && rq.shift >= 1 && rq.out_planes == 1 && rq.qmax == 127 ? 1 : 0;
   p.fast_range = g.mode == ADAPTION_MODE_RANGE && c.splits == 1 && knob(kFast) != 0 && fits_32_bits(g, c, 0) ? 1 : 0;
-  const bool grouped_kernel = c.kps > 1 || c.b_resident;
+  const bool grouped_kernel = c.kps > 1 || c.b_resident;     // (resident: also the tiles copied with their margin)
   p.tail_stagger = (p.split_hh && p.fast_relu && !grouped_kernel && c.kb_per_split >= 3 && c.stages >= 3 &&
                     c.nax == 2 && c.nbw == 2 && knob(kStagger) != 0) ? 1 : 0;
   p.ws = (long long*)g.workspace; p.ws_ld = g.N;

@@ -9,10 +9,10 @@ namespace adaption {
 static const char* const kKnobNames[kNumKnobs] = {
     "splits", "pair", "fast", "staged", "stages", "bk", "bn", "kps", "bres", "wide", "epigroups", "timeout_us", "stall_at",
     "split_hh", "pdl", "stagger", "stage_bufs", "cluster", "cluster_size", "cluster_bn",
-    "pixels", "box"};
-const int kKnobDefaults[kNumKnobs] = {0, -1, 1, 1, 0, 0, 0, 0, 1, 1, 4, 0, -1, 1, 1, 1, 2, 1, 0, 0, 1, 1};
+    "pixels", "box", "halo"};
+const int kKnobDefaults[kNumKnobs] = {0, -1, 1, 1, 0, 0, 0, 0, 1, 1, 4, 0, -1, 1, 1, 1, 2, 1, 0, 0, 1, 1, 1};
 std::atomic<int> g_knobs[kNumKnobs] = {{0}, {-1}, {1}, {1}, {0}, {0}, {0}, {0}, {1}, {1}, {4}, {0}, {-1}, {1}, {1},
-                                       {1}, {2}, {1}, {0}, {0}, {1}, {1}};
+                                       {1}, {2}, {1}, {0}, {0}, {1}, {1}, {1}};
 
 int debug_set(const char* name, int value) {
   if (name == nullptr) return ADAPTION_ERR_INVALID_ARG;

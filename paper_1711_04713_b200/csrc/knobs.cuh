@@ -6,7 +6,7 @@
 namespace adaption {
 
 enum Knob { kSplits, kPair, kFast, kStaged, kStages, kBK, kBN, kKps, kBres, kWide, kEpiGroups, kTimeoutUs, kStallAt,
-            kSplitHh, kPdl, kStagger, kStageBufs, kCluster, kClusterSize, kClusterBN, kPixels, kBox, kNumKnobs };
+            kSplitHh, kPdl, kStagger, kStageBufs, kCluster, kClusterSize, kClusterBN, kPixels, kBox, kHalo, kNumKnobs };
 
 // Each holds its default until set; the setter is the only writer.
 extern std::atomic<int> g_knobs[kNumKnobs];

@@ -444,6 +444,82 @@ __device__ __forceinline__ void mma_kblock(uint32_t d0, uint32_t d1, uint32_t d2
   }
 }
 
+// The same in warp-uniform control flow: every lane of the issuing warp comes along and the one with `issue` != 0 (elect_one
+// once, before the loop) issues.  Operands stay in uniform registers that way, and a rolled loop stays in the instruction
+// cache of a scheduler that also runs the epilogue: as straight-line code in a branch of one lane, filter taps copied once
+// (two 8-bit instructions each) took 270 to 320 cycles apiece, twice what the tensor core needs.
+template <bool PAIR>
+__device__ __forceinline__ void mma_i8_if(uint32_t issue, uint32_t d, uint32_t a, uint32_t b, uint32_t dha, uint32_t dhb,
+                                          uint32_t id, uint32_t acc) {
+#define ADAPTION_MMA_IF(CG)                                              \
+  asm volatile(                                                          \
+      "{\n"                                                              \
+      ".reg .pred p, e;\n"                                               \
+      ".reg .b64 da, db;\n"                                              \
+      "setp.ne.b32 e, %0, 0;\n"                                          \
+      "setp.ne.b32 p, %7, 0;\n"                                          \
+      "mov.b64 da, {%2, %4};\n"                                          \
+      "mov.b64 db, {%3, %5};\n"                                          \
+      "@e tcgen05.mma.cta_group::" CG ".kind::i8 [%1], da, db, %6, p;\n" \
+      "}\n" ::"r"(issue),                                                \
+      "r"(d), "r"(a), "r"(b), "r"(dha), "r"(dhb), "r"(id), "r"(acc)      \
+      : "memory")
+  if (PAIR)
+    ADAPTION_MMA_IF("2");
+  else
+    ADAPTION_MMA_IF("1");
+#undef ADAPTION_MMA_IF
+}
+// One 32-byte k-step of all products.
+template <int NAX, int NBW, bool PAIR>
+__device__ __forceinline__ void mma_kstep_if(uint32_t issue, uint32_t d0, uint32_t d1, uint32_t d2, uint32_t a0, uint32_t a1,
+                                             uint32_t b0, uint32_t b1, uint32_t dha, uint32_t dhb, uint32_t id_ss,
+                                             uint32_t id_su, uint32_t id_us, uint32_t id_uu, uint32_t acc) {
+  mma_i8_if<PAIR>(issue, d0, a0, b0, dha, dhb, id_ss, acc);
+  if (NAX == 2 && NBW == 2) {
+    mma_i8_if<PAIR>(issue, d1, a0, b1, dha, dhb, id_su, acc);
+    mma_i8_if<PAIR>(issue, d2, a1, b1, dha, dhb, id_uu, acc);
+    mma_i8_if<PAIR>(issue, d1, a1, b0, dha, dhb, id_us, 1u);
+  } else if (NAX == 2) {
+    mma_i8_if<PAIR>(issue, d1, a1, b0, dha, dhb, id_us, acc);
+  } else if (NBW == 2) {
+    mma_i8_if<PAIR>(issue, d1, a0, b1, dha, dhb, id_su, acc);
+  }
+}
+template <int NAX, int NBW, bool PAIR>
+__device__ __forceinline__ void mma_kblock_if(uint32_t issue, uint32_t d0, uint32_t d1, uint32_t d2, uint32_t a0, uint32_t off_a1,
+                                              uint32_t b0, uint32_t b_u, uint32_t dha, uint32_t dhb, uint32_t id_ss,
+                                              uint32_t id_su, uint32_t id_us, uint32_t id_uu, int ksteps, uint32_t acc) {
+#pragma unroll 1
+  for (int k = 0; k < ksteps; ++k) {
+    mma_kstep_if<NAX, NBW, PAIR>(issue, d0, d1, d2, a0, a0 + off_a1, b0, b0 + b_u, dha, dhb, id_ss, id_su, id_us, id_uu, acc);
+    acc = 1u;
+    a0 += 2u;
+    b0 += 2u;
+  }
+}
+template <bool PAIR>
+__device__ __forceinline__ void tc_commit_if(uint32_t issue, uint32_t bar) {
+  if (PAIR)
+    asm volatile(
+        "{\n"
+        ".reg .pred e;\n"
+        "setp.ne.b32 e, %2, 0;\n"
+        "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n"
+        "}\n" ::"r"(bar),
+        "h"((uint16_t)3), "r"(issue)
+        : "memory");
+  else
+    asm volatile(
+        "{\n"
+        ".reg .pred e;\n"
+        "setp.ne.b32 e, %1, 0;\n"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+        "}\n" ::"r"(bar),
+        "r"(issue)
+        : "memory");
+}
+
 // Instruction descriptor: int32 accumulate, 8-bit operands with independent signedness,
 // both K-major, M = 128, N = bn.
 __device__ __forceinline__ uint32_t make_idesc(bool a_signed, bool b_signed, int bn, int m) {

@@ -38,8 +38,8 @@ bool load_tensor_map_encoders() {
   return g_encode_tiled != nullptr && g_encode_im2col != nullptr;
 }
 
-bool encode_tiled(CUtensorMap* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
-                  const uint32_t* box, const uint32_t* estr, CUtensorMapSwizzle swz, bool long_rows) {
+static bool encode(CUtensorMap* map, CUtensorMapDataType type, const void* base, int rank, const uint64_t* dims,
+                   const uint64_t* strides, const uint32_t* box, const uint32_t* estr, CUtensorMapSwizzle swz, bool long_rows) {
   cuuint64_t d[5], s[4];
   cuuint32_t b[5], e[5];
   for (int i = 0; i < rank; ++i) {
@@ -48,10 +48,20 @@ bool encode_tiled(CUtensorMap* map, const void* base, int rank, const uint64_t* 
     e[i] = estr != nullptr ? estr[i] : 1u;
     if (i > 0) s[i - 1] = strides[i - 1];
   }
-  return g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, (cuuint32_t)rank, const_cast<void*>(base), d, s, b, e,
+  return g_encode_tiled(map, type, (cuuint32_t)rank, const_cast<void*>(base), d, s, b, e,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
                         long_rows ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool encode_tiled(CUtensorMap* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
+                  const uint32_t* box, const uint32_t* estr, CUtensorMapSwizzle swz, bool long_rows) {
+  return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, base, rank, dims, strides, box, estr, swz, long_rows);
+}
+
+bool encode_tiled_words(CUtensorMap* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
+                        const uint32_t* box) {
+  return encode(map, CU_TENSOR_MAP_DATA_TYPE_INT64, base, rank, dims, strides, box, nullptr, CU_TENSOR_MAP_SWIZZLE_NONE, false);
 }
 
 bool encode_im2col_nhwc(CUtensorMap* map, const void* base, const adaption_conv_shape& s, int64_t c_stride,

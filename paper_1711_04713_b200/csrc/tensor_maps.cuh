@@ -17,6 +17,10 @@ bool load_tensor_map_encoders();
 bool encode_tiled(CUtensorMap* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
                   const uint32_t* box, const uint32_t* estr, CUtensorMapSwizzle swz, bool long_rows = false);
 
+// The same over elements of 8 bytes without swizzle: boxes of up to 256 of them, copied as contiguous rows.
+bool encode_tiled_words(CUtensorMap* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
+                        const uint32_t* box);
+
 inline bool encode_tiled_2d(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint64_t pitch_bytes,
                             uint32_t box_inner, uint32_t box_rows, CUtensorMapSwizzle swz, bool long_rows = false) {
   const uint64_t dims[2] = {inner, rows}, strides[1] = {pitch_bytes};

@@ -1,9 +1,13 @@
-"""GPU parity of the persistent layer kernel on tiles that are boxes of pixels, where its epilogue makes the whole 2x2 max-pool:
-every box shape, margins behind the last column, row and image, every epilogue."""
+"""GPU parity of the persistent layer kernel on tiles that are boxes of pixels: the whole 2x2 max-pool in its epilogue,
+activations copied once for all filter taps, first layers read without packing.  Every box shape, margins behind the last
+column, row and image, every epilogue."""
+import numpy as np
 import pytest
 
+from oracle import reference as orc
 from paper_1711_04713_b200 import binding as B
-from tests.test_gpu_layers import run_pool_case
+from tests.test_gpu_layers import _pick_f_out, _rand_q, run_conv_case, run_pool_case
+from tests.util import Guards, dev, from_qtensor, stats_tuple, to_qtensor
 
 pytestmark = pytest.mark.gpu
 
@@ -29,6 +33,8 @@ CASES = [
     (2, 32, 32, 96, 20, 3, 1, 1, 16, 8, 16, True),         # 32-column tiles, mixed widths
     (2, 34, 34, 64, 64, 3, 0, 1, 16, 16, 8, True),         # no padding, bytes from 16-bit operands
     (64, 48, 48, 64, 64, 3, 1, 1, 8, 8, 8, True),          # many tiles per block
+    (5, 64, 64, 64, 64, 3, 1, 1, 16, 16, 16, True),        # with one copy for all taps
+    (5, 64, 64, 128, 128, 3, 1, 1, 8, 8, 8, True),
 ]
 
 
@@ -48,3 +54,78 @@ def test_an_int16_copy_is_pooled_by_its_own_pass():
     before = B.adaption_launches()
     run_pool_case(CASES[0], True)
     assert B.adaption_launches() - before == 4
+
+
+# 74 pairs of boxes of 8 x 16 pixels and more: activations copied once for all taps
+HALO = [
+    # N, H, W, Cin, K, R, pad, nx, nw, n_out, relu
+    (5, 64, 64, 64, 64, 3, 1, 16, 16, 16, True),
+    (7, 48, 56, 64, 64, 3, 1, 8, 8, 8, True),              # an odd number of boxes
+    (5, 64, 62, 64, 128, 3, 1, 16, 16, 16, True),          # two column tiles; columns behind the last
+    (5, 63, 64, 64, 100, 3, 1, 16, 16, 16, True),          # the second one ragged; rows behind the last
+    (5, 64, 64, 96, 128, 3, 1, 8, 8, 8, True),             # partial k-block
+    (5, 64, 64, 160, 72, 3, 1, 8, 8, 8, True),             # two channel blocks, the second partial
+    (5, 64, 64, 128, 128, 3, 1, 8, 8, 16, False),          # signed outputs of 8-bit operands
+    (5, 66, 66, 64, 61, 3, 0, 16, 16, 16, True),           # no padding, 64-bit epilogue
+    (5, 64, 64, 64, 64, 5, 2, 16, 16, 12, True),
+    (5, 65, 65, 64, 64, 2, 0, 16, 16, 16, True),           # even filter
+    (3, 112, 112, 64, 64, 3, 1, 16, 16, 16, True),         # several tiles per pair
+]
+
+
+@pytest.mark.parametrize("case", HALO)
+@pytest.mark.parametrize("fast,staged,stochastic", [(1, 1, False), (0, 1, False), (1, 0, False), (1, 1, True)])
+def test_one_copy_for_all_taps(case, fast, staged, stochastic):
+    N, H, W, Cin, K, R, pad, nx, nw, n_out, relu = case
+    B.adaption_debug_set("fast", fast)
+    B.adaption_debug_set("staged", staged)
+    run_conv_case(np.random.default_rng(sum(case)), N, H, W, Cin, K, R, pad, 1, nx, nw, n_out, relu, B.ALGO_AUTO,
+                  with_q16=False, stochastic_seed=77 if stochastic else None)
+
+
+# first layers over pixels of 16 bytes
+TAPS = [
+    # N, H, W, Cin, K, R, pad, nx, nw, n_out, relu
+    (2, 32, 32, 3, 64, 3, 1, 16, 16, 16, True),
+    (2, 32, 32, 3, 64, 3, 1, 8, 8, 8, True),
+    (3, 48, 40, 3, 16, 1, 0, 16, 16, 16, True),            # one tap, no margin
+    (2, 34, 34, 4, 100, 3, 0, 16, 16, 12, True),           # no padding, 128 columns, ragged
+    (1, 65, 63, 1, 32, 2, 0, 16, 16, 16, False),           # even filter, columns and rows behind the last, signed
+    (1, 64, 64, 2, 61, 3, 1, 8, 8, 8, True),               # 64-bit epilogue
+    (9, 112, 112, 3, 64, 3, 1, 16, 16, 16, True),          # many tiles per block
+]
+
+
+@pytest.mark.parametrize("case", TAPS)
+@pytest.mark.parametrize("fast,staged,stochastic", [(1, 1, False), (0, 1, False), (1, 0, False), (1, 1, True)])
+def test_first_layers_without_packing(case, fast, staged, stochastic):
+    N, H, W, Cin, K, R, pad, nx, nw, n_out, relu = case
+    B.adaption_debug_set("fast", fast)
+    B.adaption_debug_set("staged", staged)
+    before = B.adaption_launches()
+    run_conv_case(np.random.default_rng(sum(case)), N, H, W, Cin, K, R, pad, 1, nx, nw, n_out, relu, B.ALGO_AUTO,
+                  with_q16=False, stochastic_seed=77 if stochastic else None, cs=16)
+    assert B.adaption_launches() - before == 2             # (one to measure, one to store)
+
+
+@pytest.mark.parametrize("n_bits", [16, 8])
+def test_first_layer_with_its_pool(n_bits):
+    N, H, W, C, K = 3, 48, 40, 3, 64
+    rng = np.random.default_rng(n_bits)
+    xq, wq, bq = _rand_q(rng, (N, H, W, C), n_bits, 0.3), _rand_q(rng, (K, 3, 3, C), n_bits), _rand_q(rng, (K,), n_bits)
+    fx, fw = n_bits - 3, n_bits - 1
+    acc = orc.conv_acc(xq, wq, (1, 1), (1, 1))
+    _, f = _pick_f_out(acc, bq, fw, fx + fw, True, n_bits)
+    conv_y, cnt = orc.epilogue(acc, bq, fw, fx + fw, True, n_bits, f)
+    want = orc.maxpool2x2(conv_y)
+    x, w = to_qtensor(xq.reshape(-1, C), n_bits, fx, 16), to_qtensor(wq.reshape(-1, C), n_bits, fw, 16)
+    guards = Guards()
+    y = guards.qtensor(N * H * W // 4, K, n_bits, f, 64)
+    shp = B.conv_shape(N, H, W, C, K, 3, 3, 1, 1)
+    need = B.adaption_lp_conv_pool_workspace_bytes(shp, x.fmt(), w.fmt(), y.fmt(), 16, 64, B.ALGO_AUTO)
+    ws, st, before = guards.alloc(need), B.new_stats(), B.adaption_launches()
+    B.adaption_lp_conv_pool_fwd(shp, x, w, dev(bq), fw, True, B.ALGO_AUTO, y, st, ws)
+    assert B.adaption_launches() - before == 1
+    assert np.array_equal(from_qtensor(y).reshape(want.shape), want)
+    assert stats_tuple(st) == (cnt.zeros, cnt.sat_pos, cnt.sat_neg)
+    guards.check()
