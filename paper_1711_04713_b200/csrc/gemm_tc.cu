@@ -194,6 +194,10 @@ struct TcParams {
   int fast_range;             // range mode: 32-bit keys decide what is worth the exact 64-bit value
   int pool_w;                 // store max(row 2j, row 2j+1) of the tile: half of a 2x2 max-pool (staged only)
   int epi_groups;             // 1, 2 or 4 groups of epilogue warps that take turns tile by tile
+  // four groups: every warp makes, stages and stores 32 whole rows of a tile by itself, with no barrier among the warps (8
+  // bits, 128 x 224 x 224, 3 -> 64 230 -> 214 us; 128 x 112 x 112, one copy for all taps, us with two groups and four: 64 ->
+  // 128 146 and 114, 128 -> 128 174 and 140)
+  int own_rows;
   int staged;                 // outputs leave through shared memory and bulk-tensor stores
   int stage_bufs;             // staging buffers per epilogue group: 1, or 2 used in turn (narrow tiles)
   uint32_t stage_off;         // offset of the staging planes from the ring base
@@ -220,7 +224,7 @@ struct Ctrl {
   unsigned long long tmem_full[kMaxAccBufs];
   unsigned long long tmem_empty[kMaxAccBufs];
   unsigned long long part_full[2];   // staggered tail: low accumulator complete, middle accumulator complete
-  unsigned long long drain;     // the issuing warp's last commit before an early exit
+  unsigned long long drain[2];  // an issuing warp's last commit before an early exit
   unsigned long long b_ready;   // resident weights have landed
   uint32_t tmem_base;
   volatile uint32_t abort;
@@ -479,6 +483,12 @@ __device__ __forceinline__ void load_acc16(uint32_t taddr, uint32_t first_off, i
   if (NACC == 3) tmem_ld16(taddr + 2u * (uint32_t)bn, x.a[2], y.a[2]);
 }
 template <int NACC>
+__device__ __forceinline__ void load_acc8(uint32_t taddr, uint32_t first_off, int bn, Acc8<NACC>& x) {
+  tmem_ld8(taddr + first_off, x.a[0]);
+  if (NACC >= 2) tmem_ld8(taddr + (uint32_t)bn, x.a[1]);
+  if (NACC == 3) tmem_ld8(taddr + 2u * (uint32_t)bn, x.a[2]);
+}
+template <int NACC>
 __device__ __forceinline__ void pin_acc8(Acc8<NACC>& x) {
   pin_after_wait(x.a[0]);
   if (NACC >= 2) pin_after_wait(x.a[1]);
@@ -675,6 +685,17 @@ __device__ __forceinline__ void store16_global(const uint32_t* w, const TcParams
   }
 }
 
+// ... of eight outputs (8 bytes per plane)
+__device__ __forceinline__ void store8_global(const uint32_t* w, const TcParams& p, bool row_ok, int m, int col) {
+  if (row_ok && col < p.y_stride) {
+    const size_t off = (size_t)m * (size_t)p.y_stride + (size_t)col;
+    *reinterpret_cast<uint2*>(p.y_lo + off) = make_uint2(__byte_perm(w[0], w[1], 0x6420), __byte_perm(w[2], w[3], 0x6420));
+    if (p.rq.out_planes == 2)
+      *reinterpret_cast<uint2*>(p.y_hi + off) = make_uint2(__byte_perm(w[0], w[1], 0x7531), __byte_perm(w[2], w[3], 0x7531));
+    if (p.y_q16 != nullptr) *reinterpret_cast<uint4*>(p.y_q16 + off) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
 // Staged stores: the tile's byte planes are assembled in shared memory (rows of BN bytes, 16-byte
 // chunks swizzled the way the bulk-tensor store expects for that row length, which also keeps the
 // 16-byte writes of a quarter warp on distinct banks) and leave as one bulk-tensor store per plane.
@@ -689,6 +710,9 @@ __device__ __forceinline__ uint32_t staged_offset(int row, int chunk, int bn, in
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint4 v) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
                : "memory");
+}
+__device__ __forceinline__ void st_shared_v2(uint32_t addr, uint32_t a, uint32_t b) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
 __device__ __forceinline__ void st_shared_b32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
@@ -794,6 +818,11 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
   constexpr bool GROUPED = LOOP == kLoopGrouped, PARTIAL = LOOP == kLoopPartial, PIX = LOOP == kLoopPixels;
   constexpr bool HALO = LOOP == kLoopHalo, TAPS = LOOP == kLoopTaps;
   constexpr bool FAST = EPI == kEpiFast;
+  // Where one copy serves all taps and a step is one product, the last copying warp issues MMAs too, every other tile: they
+  // take the tensor core less time than one warp needs for its loop (64 channels: 105 cycles an instruction, 40 where
+  // nothing else bounds them; 8 bits, 128 x 224 x 224 x 64 -> 64 340 -> 290 us).  With four products a step one warp
+  // keeps up, and two tiles' instructions in turn cost the tensor core more (16 bits, 64 images 329 -> 453 us).
+  constexpr int kIssuers = (HALO || TAPS) && NAX * NBW == 1 ? 2 : 1, kCopyWarps = kProducerWarps + 1 - kIssuers;
   constexpr bool STOCH = EPI == kEpiStochastic, FASTST = EPI == kEpiFastStochastic;
   extern __shared__ uint8_t smem_raw[];
   __shared__ Ctrl ctrl;
@@ -820,7 +849,8 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     }
     mbar_init(smem_u32(&ctrl.part_full[0]), 1);
     mbar_init(smem_u32(&ctrl.part_full[1]), 1);
-    mbar_init(smem_u32(&ctrl.drain), 1);
+    mbar_init(smem_u32(&ctrl.drain[0]), 1);
+    mbar_init(smem_u32(&ctrl.drain[1]), 1);
     mbar_init(smem_u32(&ctrl.b_ready), 1);
     ctrl.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -839,7 +869,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
   pdl_wait();
   pdl_launch_dependents();
 
-  if (warp < kProducerWarps) {
+  if (warp < kCopyWarps) {
     // ------------------------------------------------------------------ TMA producers
     // Operand planes are numbered A planes first, then B planes.  Every producer warp walks the same
     // sequence of stages and issues only the copies of its own planes (warp w takes planes w and
@@ -852,10 +882,10 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     const bool b_res = PIX || HALO || TAPS || (GROUPED && p.b_resident);
     const int nact = b_res ? NAX : NPLANES;
     const int kps = GROUPED ? p.kps : 1;
-    const int nsub = nact >= kProducerWarps ? 1 : kProducerWarps / nact;   // warps per streamed plane
-    const int act_plane = nact >= kProducerWarps ? warp : warp % nact;
-    const int sub = nact >= kProducerWarps ? 0 : warp / nact;
-    const bool two_planes = act_plane + kProducerWarps < nact;             // this warp also owns a second plane
+    const int nsub = nact >= kCopyWarps ? 1 : kCopyWarps / nact;           // warps per streamed plane
+    const int act_plane = nact >= kCopyWarps ? warp : warp % nact;
+    const int sub = nact >= kCopyWarps ? 0 : warp / nact;
+    const bool two_planes = act_plane + kCopyWarps < nact;                 // this warp also owns a second plane
     {
       const bool is_a = act_plane < NAX;
       const int plane = is_a ? act_plane : act_plane - NAX;
@@ -867,7 +897,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       uint32_t it = 0, ph = 0;
       int s = 0, turn = 0;                     // turn: s modulo nsub
       bool ok = true;
-      if (b_res && warp == kProducerWarps - 1) {
+      if (b_res && warp == kCopyWarps - 1) {
         // the whole weight matrix of this (single) column tile, one copy per k-block and plane,
         // all reporting to one barrier
         // (in a pair each CTA fetches its own half of the weight rows; the bytes of both are counted
@@ -1001,7 +1031,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           if (++s == p.stages) { s = 0; ph ^= 1u; turn = 0; }
         }
       }
-      const bool is_b_loader = b_res && warp == kProducerWarps - 1;
+      const bool is_b_loader = b_res && warp == kCopyWarps - 1;
       if (ctrl.abort && lane == 0 && is_b_loader) {
         // another role gave up: let the resident-weight copies land before the CTA exits (the
         // follower of a pair cannot see the leader's barrier: it waits a fixed time)
@@ -1060,6 +1090,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       const bool b_res = PIX || HALO || TAPS || (GROUPED && p.b_resident);
       const int kps = GROUPED ? p.kps : 1;
       const uint32_t bres_lo = smem_desc_lo(ring + p.b_res_off) + (TAPS ? (uint32_t)(p.BN - 1) << 16 : 0u), bres_u = NBW * b_u;
+      const uint32_t issuer = kIssuers == 2 && warp != kMmaWarp ? 1u : 0u;
       const uint32_t issue = HALO || TAPS ? (elect_one() ? 1u : 0u) : 0u;
       const int halo_r = p.halo.R, halo_s = p.halo.S;
       const uint32_t px_u = p.halo.px_u, row_u = (uint32_t)p.halo.w * px_u, tap_u = (uint32_t)p.cblks * bres_u;
@@ -1068,6 +1099,13 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         tc_fence_after();
       }
       for (int t = worker; t < p.total_tiles && ok; t += workers, ++tile_iter) {
+        if (kIssuers == 2 && (tile_iter & 1u) != issuer) {            // the other warp's tile: pass over its stages
+          for (s += p.num_kb; s >= p.stages; s -= p.stages) ph ^= 1u;
+          a0 = ring_lo + (uint32_t)s * stage_u;
+          full_bar = full_bar0 + 8u * (uint32_t)s;
+          empty_bar = empty_bar0 + 8u * (uint32_t)s;
+          continue;
+        }
         const TileCoord tc = decode_tile(t, p);
         const uint32_t buf = tile_iter & (uint32_t)(p.acc_bufs - 1);
         const uint32_t bph = (tile_iter >> p.acc_shift) & 1u;
@@ -1245,9 +1283,9 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       }
       if ((!ok || ctrl.abort) && lane == 0) {
         // make sure no MMA still reads shared memory or writes TMEM when the CTAs tear down
-        tc_commit<PAIR>(smem_u32(&ctrl.drain));
+        tc_commit<PAIR>(smem_u32(&ctrl.drain[issuer]));
         const unsigned long long t0 = global_ns();
-        while (!mbar_try_wait(smem_u32(&ctrl.drain), 0) && global_ns() - t0 < 50000000ull) {
+        while (!mbar_try_wait(smem_u32(&ctrl.drain[issuer]), 0) && global_ns() - t0 < 50000000ull) {
         }
       }
     }
@@ -1278,9 +1316,11 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     uint32_t stage_hi = stage_lo + (uint32_t)plane_bytes;
     uint32_t stage_turn = 0;
     // per-column epilogue constants of the current tile, one array per group, behind the staging planes
+    // (one per warp where warps work by themselves: then no barrier separates readers and writers)
+    const bool own = p.own_rows != 0;
     long long* colconst = reinterpret_cast<long long*>(smem_raw + (ring - smem_u32(smem_raw)) + p.const_off) +
-                          group * p.BN;
-    const bool store_leader = ew == 0 && lane == 0;
+                          (own ? warp - kFirstEpiWarp : group) * p.BN;
+    const bool store_leader = (own || ew == 0) && lane == 0;
     uint32_t tile_iter = (uint32_t)group;
     Counts cnt;
     long long vmax = 0;
@@ -1295,7 +1335,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       // writes from its readers): bias aligned to the accumulator, plus the rounding half on the
       // fast path.  Kept when the tile covers the same columns as the previous one.
       if (tc.n0 != const_n0) {
-        for (int c = 32 * ew + lane; c < p.BN; c += gthreads) {
+        for (int c = own ? lane : 32 * ew + lane; c < p.BN; c += own ? 32 : gthreads) {
           const int n = tc.n0 + c;
           long long b = 0;
           const int ch = PIX ? n & (p.px.ys - 1) : n;
@@ -1330,7 +1370,12 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       bool w = wait_bar(smem_u32(stagger ? &ctrl.part_full[0] : &ctrl.tmem_full[buf]), bph, &ctrl, p);
       // one decision for all epilogue warps (they meet at barriers below), which also publishes the
       // constants and the free staging planes
-      w = epi_bar_all(group, gthreads, w);
+      if (own) {
+        w = __all_sync(0xffffffffu, w);
+        __syncwarp();
+      } else {
+        w = epi_bar_all(group, gthreads, w);
+      }
       if (lane == 0 && (ew & 3) == 0) TL_STAMP(2 + (ew >> 2), tile_iter, 1);
       if (!w) { ok = false; break; }
       tc_fence_after();
@@ -1523,7 +1568,48 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           }
         }
       }
-      for (int c0 = col_begin; !FAST && (c0 < col_end || !released); c0 += 16) {
+      if (STOCH || FASTST) {
+        // Stochastic rounding: a rolled loop over eight columns.  The generator's rounds are long straight-line code: with
+        // sixteen columns a step (eight blocks of it) the warps waited for instructions (16 images, 3 -> 16 channels at
+        // 224 x 224, 1x1: 61 us with sixteen, 48 with eight, 7x7 over 16 channels at 112 x 112 81 and 69, 64 -> 64 47 and 39; the
+        // generator's rounds as a loop: 53, 69, 43).
+#pragma unroll 1
+        for (int c0 = col_begin; c0 < col_end; c0 += 8) {
+          const int col = tc.n0 + c0;
+          Acc8<NACC> v;
+          load_acc8<NACC>(taddr + (uint32_t)c0, hh_off, p.BN, v);
+          tmem_ld_wait();
+          pin_acc8<NACC>(v);
+          if (c0 + 8 >= col_end) {
+            release_accumulators<PAIR>(bar_rest, lane);
+            if (split) release_accumulators<PAIR>(bar_hh, lane);
+            released = true;
+          }
+          uint32_t wq[4];
+          if (FASTST) {
+            const int* cl = reinterpret_cast<const int*>(colconst) + c0;
+            stochastic8<NACC, PIX>(v, cl, cl + p.BN, p, row_ok, m, col, cnt, wq);
+          } else if (p.rq.relu) {
+            requant8<NACC, true, true, PIX>(v, colconst + c0, p, row_ok, m, col, cnt, wq);
+          } else {
+            requant8<NACC, false, true, PIX>(v, colconst + c0, p, row_ok, m, col, cnt, wq);
+          }
+          if (p.staged) {
+            const uint32_t off = staged_offset(row, c0 >> 4, p.BN) + (uint32_t)(c0 & 8);
+            st_shared_v2(stage_lo + off, __byte_perm(wq[0], wq[1], 0x6420), __byte_perm(wq[2], wq[3], 0x6420));
+            if (p.rq.out_planes == 2)
+              st_shared_v2(stage_hi + off, __byte_perm(wq[0], wq[1], 0x7531), __byte_perm(wq[2], wq[3], 0x7531));
+          } else {
+            store8_global(wq, p, row_ok, m, col);
+          }
+        }
+        if (!released) {                     // a warp without columns only hands the accumulators back
+          release_accumulators<PAIR>(bar_rest, lane);
+          if (split) release_accumulators<PAIR>(bar_hh, lane);
+          released = true;
+        }
+      }
+      for (int c0 = col_begin; !FAST && !STOCH && !FASTST && (c0 < col_end || !released); c0 += 16) {
         const bool have = c0 < col_end;
         Acc8<NACC> xa, xb;
         if (have) {
@@ -1549,16 +1635,12 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           partial_or_range8<NACC, PIX>(xb, bcol + 8, p, row_ok, m, col + 8, vmax);
         } else {
           uint32_t wq[8];
-          if (FASTST) {
-            const int* cl = reinterpret_cast<const int*>(colconst) + c0;
-            stochastic8<NACC, PIX>(xa, cl, cl + p.BN, p, row_ok, m, col, cnt, wq);
-            stochastic8<NACC, PIX>(xb, cl + 8, cl + p.BN + 8, p, row_ok, m, col + 8, cnt, wq + 4);
-          } else if (p.rq.relu) {
-            requant8<NACC, true, STOCH, PIX>(xa, bcol, p, row_ok, m, col, cnt, wq);
-            requant8<NACC, true, STOCH, PIX>(xb, bcol + 8, p, row_ok, m, col + 8, cnt, wq + 4);
+          if (p.rq.relu) {
+            requant8<NACC, true, false, PIX>(xa, bcol, p, row_ok, m, col, cnt, wq);
+            requant8<NACC, true, false, PIX>(xb, bcol + 8, p, row_ok, m, col + 8, cnt, wq + 4);
           } else {
-            requant8<NACC, false, STOCH, PIX>(xa, bcol, p, row_ok, m, col, cnt, wq);
-            requant8<NACC, false, STOCH, PIX>(xb, bcol + 8, p, row_ok, m, col + 8, cnt, wq + 4);
+            requant8<NACC, false, false, PIX>(xa, bcol, p, row_ok, m, col, cnt, wq);
+            requant8<NACC, false, false, PIX>(xb, bcol + 8, p, row_ok, m, col + 8, cnt, wq + 4);
           }
           if (!PIX && p.box.pool) {
             store_window_max(wq, lane, down, window, c0 >> 4, p, stage_lo, stage_hi);
@@ -1590,10 +1672,27 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         // the same barrier also carries the verdict on this tile's later waits, so that all warps
         // of the group leave together if one of them gave up
         if (!epi_bar_all(group, gthreads, tile_ok)) { ok = false; break; }
+      } else if (own) {
+        __syncwarp();
       } else {
         epi_bar_sync(group, gthreads);
       }
-      if (!PIX && p.box.on && p.staged && store_leader) {
+      if (own && p.staged && store_leader) {
+        // this warp's rows (a quarter of the tile, whose stored rows are consecutive whatever the pool)
+        const int first = 32 * quarter;
+        const uint32_t so = (uint32_t)(quarter * (plane_bytes >> (p.pool_w && !PIX ? 3 : 2)));
+        if (!PIX && p.box.on) {
+          const int oh = (bc.oh + ((first >> p.box.w) & ((1 << p.box.h) - 1))) >> p.box.pool, ow = bc.ow >> p.box.pool;
+          const int img = bc.img + (first >> (p.box.w + p.box.h));
+          tma_store_4d(&map_y_lo, stage_lo + so, tc.n0, ow, oh, img);
+          if (p.rq.out_planes == 2) tma_store_4d(&map_y_hi, stage_hi + so, tc.n0, ow, oh, img);
+        } else {
+          const int m_first = (tc.m0 + (int)rank * kBM + first) >> (p.pool_w && !PIX ? 1 : 0);
+          tma_store_2d(&map_y_lo, stage_lo + so, tc.n0, m_first);
+          if (p.rq.out_planes == 2) tma_store_2d(&map_y_hi, stage_hi + so, tc.n0, m_first);
+        }
+        bulk_commit();
+      } else if (!PIX && p.box.on && p.staged && store_leader) {
         const int ow = bc.ow >> p.box.pool, oh = bc.oh >> p.box.pool;
         for (int sub = 0; sub * 128 < p.BN; ++sub) {
           const uint32_t so = (uint32_t)sub * (uint32_t)(plane_rows * 128);
@@ -1654,6 +1753,7 @@ struct TcConfig {
   bool pair = false;           // two CTAs per 256-row tile (cta_group::2)
   int tile_m = kBM;
   int epi_groups = 1;
+  bool own_rows = false;
   bool staged = false;         // outputs staged in shared memory and written by bulk-tensor stores
   uint32_t stage_out_bytes = 0, stage_off = 0, const_bytes = 0;
   int stage_bufs = 1;
@@ -1852,7 +1952,8 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
   c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) / (c.box.pool ? 4u : 1u) : 0u;
   // dynamic shared memory: everything up to the per-block limit except the control block
-  c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
+  c.own_rows = c.epi_groups * 4 == kEpiWarps && c.BN <= 128;
+  c.const_bytes = (uint32_t)(c.BN * (c.own_rows ? kEpiWarps : c.epi_groups) * sizeof(long long));
   const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
   // group short k-blocks so that a stage carries roughly 768 tensor-pipe cycles of work or more.  512 with one product
   // per step (128 -> 128 channels at 112 x 112, 8 bits, batch 128 231 us with two k-blocks, 264 with three), but not for
@@ -1999,7 +2100,8 @@ TcConfig make_pixel_config(const GemmProblem& g, int G) {
   const int most_groups = c.BN <= 64 ? 4 : 2;
   while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
   c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) / (g.pool_w ? 2u : 1u) : 0u;
-  c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
+  c.own_rows = c.epi_groups * 4 == kEpiWarps && c.BN <= 128;
+  c.const_bytes = (uint32_t)(c.BN * (c.own_rows ? kEpiWarps : c.epi_groups) * sizeof(long long));
   const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
   c.b_resident = true;
   c.b_res_bytes = c.nbw * px.b_plane;
@@ -2089,8 +2191,6 @@ TcConfig make_halo_config(const GemmProblem& g) {
       c.b_bytes /= 2;
       c.tiles_n = 2;
     }
-    // (8 bits, 128 columns over 64 channels: the epilogue bounds either form, 145 us against 138 with 128 images)
-    if (c.nacc == 1 && c.BN == 128 && cs == 64) return c;
     c.b_res_bytes = (uint32_t)(c.tiles_n * c.b_blocks * c.nbw) * c.b_bytes;
     c.tiles_m = (int)((boxes + 1) / 2);
     if (c.tiles_m < sms / 2) return c;
@@ -2108,10 +2208,11 @@ TcConfig make_halo_config(const GemmProblem& g) {
              g.y.c_stride % 16 == 0 && knob(kStaged) != 0;
   if (g.box_pool && !c.staged) return c;
   c.epi_groups = c.acc_bufs;
-  const int most_groups = c.BN <= 64 ? 4 : 2;
+  const int most_groups = c.BN <= 64 || c.nacc == 1 ? 4 : 2;
   while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
   c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) / (g.box_pool ? 4u : 1u) : 0u;
-  c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
+  c.own_rows = c.epi_groups * 4 == kEpiWarps && c.BN <= 128;
+  c.const_bytes = (uint32_t)(c.BN * (c.own_rows ? kEpiWarps : c.epi_groups) * sizeof(long long));
   const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
   c.b_resident = true;
   if (c.b_res_bytes + 2 * c.stage_bytes + 1024 > budget) return c;
@@ -2456,12 +2557,17 @@ int launch_tensor(const GemmProblem& g) {
         const int half = c.box.pool;
         const uint64_t W = (uint64_t)(g.OW >> half), H = (uint64_t)(g.OH >> half);
         const uint64_t dims[4] = {ypitch, W, H, (uint64_t)g.cs.N}, strides[3] = {ypitch, ypitch * W, ypitch * W * H};
-        const uint32_t box[4] = {(uint32_t)ybox, 1u << (c.box.w - half), 1u << (c.box.h - half), 1u << c.box.n};
+        uint32_t box[4] = {(uint32_t)ybox, 1u << (c.box.w - half), 1u << (c.box.h - half), 1u << c.box.n};
+        if (c.own_rows) {        // 32 of the tile's rows
+          const int h = c.box.w + c.box.h < 5 ? c.box.h : 5 - c.box.w;
+          box[2] = 1u << (h - half);
+          box[3] = 1u << (5 - c.box.w - h);
+        }
         if (!encode_tiled(&maps[4 + i], planes[i], 4, dims, strides, box, nullptr, yswz)) return ADAPTION_ERR_CUDA;
         continue;
       }
       if (!encode_tiled_2d(&maps[4 + i], planes[i], ypitch, (uint64_t)(halve_rows ? M / 2 : M), ypitch, (uint32_t)ybox,
-                           (uint32_t)(halve_rows ? kBM / 2 : kBM), yswz))
+                           (uint32_t)((halve_rows ? kBM / 2 : kBM) / (c.own_rows ? 4 : 1)), yswz))
         return ADAPTION_ERR_CUDA;
     }
   }
@@ -2512,6 +2618,7 @@ int launch_tensor(const GemmProblem& g) {
   if (g.box_pool && !(c.staged && c.box.pool)) return ADAPTION_ERR_UNSUPPORTED;
   p.pool_w = g.pool_w ? 1 : 0;
   p.epi_groups = c.epi_groups;
+  p.own_rows = c.own_rows ? 1 : 0;
   p.staged = c.staged ? 1 : 0;
   p.stage_bufs = c.stage_bufs;
   p.stage_off = c.stage_off;

@@ -245,6 +245,13 @@ __device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint32_t a_lo, uint32_t 
                                        uint32_t accumulate) {
   mma_i8<PAIR>(d_tmem, a_lo, b_lo, desc_hi, idesc, accumulate, desc_hi);
 }
+// eight consecutive columns
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, int32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
 // sixteen consecutive columns: the first eight into `lo`, the next eight into `hi`
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, int32_t (&lo)[8], int32_t (&hi)[8]) {
   asm volatile(
