@@ -202,7 +202,12 @@ __device__ __forceinline__ void finish_group(const long long (&v)[G], int nreal,
 #pragma unroll
     for (int j = 0; j < G; ++j) keep_range(v[j], p, vmax);
   } else if constexpr (KIND == kFinishStochastic) {
-    if (G == 8 && step == 1 && nreal == G && (index & 3) == 0) {     // two whole generator blocks
+    if (G == 8) {      // (a convolution of N % 8 = 0 channels, finish_tile: two whole generator blocks, or padding)
+      if (nreal == 0) {
+#pragma unroll
+        for (int j = 0; j < G; ++j) q[j] = 0;
+        return;
+      }
 #pragma unroll
       for (int b = 0; b < G / 4; ++b) {
         const uint64_t blk = (index >> 2) + (uint64_t)b;
