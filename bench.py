@@ -395,8 +395,8 @@ def run_gpu(args):
                 e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
                 e0.record()
             if fused:
-                # convolution with the horizontal half of the pooling in its epilogue, then (outside the
-                # layer-GEMM events) the vertical half
+                # convolution with the pooling (or its horizontal half) in its epilogue, then, outside the
+                # layer-GEMM events, what is left of it
                 P = net.layers[i + 1]
                 net._run_conv_pool(L, P, a, B.PHASE_CONV)
             else:
