@@ -339,6 +339,15 @@ ADAPTION_API int adaption_probe_i8_peak(int32_t bn, int32_t pair, int32_t iters,
  * do not change overrides while another host thread is inside a layer call. */
 ADAPTION_API int adaption_debug_set(const char* h_name, int32_t value);
 
+/* Test aid: which kernel the calling host thread's last layer call launched.  h_name is a host string:
+ *   "loop"    main loop of the persistent layer kernel: 0 one k-block per stage, 1 several k-blocks per stage or resident
+ *             weights, 2 partial k-blocks, 3 grouped pixels, 4 one copy for all taps, 5 first layer without packing; -1 if
+ *             another kernel ran (one cluster per tile, direct)
+ *   "stages"  depth of its shared-memory ring      "tiles"  output tiles (of a pair, where CTAs are paired)
+ *   "staged"  1 if outputs are staged in shared memory
+ * Returns ADAPTION_ERR_INVALID_ARG for an unknown name. */
+ADAPTION_API int adaption_debug_get(const char* h_name, int32_t* h_value);
+
 /* Kernels that calls of the calling host thread have launched so far (memsets and copies are not counted). */
 ADAPTION_API uint64_t adaption_launches(void);
 

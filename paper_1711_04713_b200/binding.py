@@ -60,7 +60,7 @@ EXPORTS = [
     "adaption_choose_frac_bits_from_hist", "adaption_choose_frac_bits_from_widths",
     "adaption_lp_act_stochastic", "adaption_lp_conv_pool_workspace_bytes", "adaption_lp_conv_pool_fwd",
     "adaption_quantize_batch", "adaption_quantize_batch_stochastic", "adaption_debug_set", "adaption_lp_conv_fwd_stochastic",
-    "adaption_lp_ip_fwd_stochastic", "adaption_launches",
+    "adaption_lp_ip_fwd_stochastic", "adaption_launches", "adaption_debug_get",
 ]
 HIST_BINS = 17
 
@@ -125,6 +125,7 @@ def load(path: str | None = None):
     lib.adaption_choose_frac_bits_from_widths.argtypes = [C.POINTER(C.c_uint64), I32, I32, C.c_double,
                                                           C.POINTER(adaption_qfmt)]
     lib.adaption_debug_set.argtypes = [C.c_char_p, C.c_int32]
+    lib.adaption_debug_get.argtypes = [C.c_char_p, C.POINTER(C.c_int32)]
     lib.adaption_status_string.argtypes = [C.c_int]
     lib.adaption_status_string.restype = C.c_char_p
     for name in EXPORTS:
@@ -164,6 +165,13 @@ def _calls():
 def adaption_debug_set(name: str, value: int = 0):
     """Test / experiment override of the tensor-core path's heuristics (see the header)."""
     _check(load().adaption_debug_set(name.encode(), int(value)), f"adaption_debug_set({name})")
+
+
+def adaption_debug_get(name: str) -> int:
+    """What this host thread's last layer call launched: "loop", "stages", "tiles" or "staged" (see the header)."""
+    out = C.c_int32()
+    _check(load().adaption_debug_get(name.encode(), C.byref(out)), "adaption_debug_get")
+    return out.value
 
 
 def adaption_launches() -> int:

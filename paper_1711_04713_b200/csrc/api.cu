@@ -1,6 +1,7 @@
 // extern "C" entry points: argument validation and dispatch.  See include/adaption.h.
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 
 #include "common.cuh"
 
@@ -37,6 +38,15 @@ int debug_set(const char* name, int value);
 
 static thread_local uint64_t t_launches = 0;
 void count_launch() { ++t_launches; }
+
+static const char* const kLayerFields[] = {"loop", "stages", "tiles", "staged"};
+static thread_local int32_t t_layer[4] = {-1, 0, 0, 0};
+void note_layer(int loop, int stages, int tiles, int staged) {
+  t_layer[0] = loop;
+  t_layer[1] = stages;
+  t_layer[2] = tiles;
+  t_layer[3] = staged;
+}
 
 // Longest reduction the direct kernels and the int64 workspace can take without overflow:
 // |q_x * q_w| <= 2^30, so 2^31 terms still leave a sign bit and headroom for the bias.
@@ -459,6 +469,16 @@ int adaption_probe_i8_peak(int32_t bn, int32_t pair, int32_t iters, int32_t comm
 uint64_t adaption_launches(void) { return t_launches; }
 
 int adaption_debug_set(const char* h_name, int32_t value) { return debug_set(h_name, value); }
+
+int adaption_debug_get(const char* h_name, int32_t* h_value) {
+  if (h_name == nullptr || h_value == nullptr) return ADAPTION_ERR_INVALID_ARG;
+  for (int i = 0; i < 4; ++i)
+    if (std::strcmp(h_name, kLayerFields[i]) == 0) {
+      *h_value = t_layer[i];
+      return ADAPTION_OK;
+    }
+  return ADAPTION_ERR_INVALID_ARG;
+}
 
 const char* adaption_status_string(int status) {
   switch (status) {

@@ -869,6 +869,7 @@ int launch_cluster(const GemmProblem& g) {
   if (g.pool_w) return ADAPTION_ERR_UNSUPPORTED;
   const CgPlan c = make_plan(g, g.pool2x2);
   if (!c.ok) return ADAPTION_ERR_UNSUPPORTED;
+  note_layer(-1, 0, 0, 0);
   if (!load_tensor_map_encoders()) return ADAPTION_ERR_CUDA;
   const CUtensorMapSwizzle swz = c.BK == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
                                              : (c.BK == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);

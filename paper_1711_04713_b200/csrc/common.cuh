@@ -230,6 +230,8 @@ __device__ __forceinline__ void pdl_prologue() {
 }
 
 void count_launch();     // one more kernel launched by this host thread (adaption_launches)
+// what the host thread's last layer call launched (adaption_debug_get); loop -1: not the persistent layer kernel
+void note_layer(int loop, int stages, int tiles, int staged);
 bool pdl_enabled();      // process-wide switch (adaption_debug_set "pdl")
 
 // Launch of a kernel whose first statement is pdl_prologue().

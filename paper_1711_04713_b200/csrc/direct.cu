@@ -162,6 +162,7 @@ static int grid_for(size_t items) {
 }
 
 int launch_direct(const GemmProblem& g) {
+  note_layer(-1, 0, 0, 0);
   DirectParams p{};
   p.M = g.M; p.N = g.N; p.K = g.K;
   p.is_conv = g.is_conv ? 1 : 0;

@@ -219,7 +219,12 @@ __device__ long long g_timeline[8192];
 #endif
 
 struct Ctrl {
-  unsigned long long full[kMaxStages];
+  // A slot's copies report to the barrier of the warp that issues the MMAs on them (the first kMaxStages, or the second
+  // where there are two issuing warps).  A wait on an mbarrier tells phases apart only modulo two: a warp that waits may
+  // be at most one fill behind.  With one barrier per slot, counted in laps of the ring, a warp waiting for a fill whose
+  // predecessor was the other warp's, and had not landed yet, was let through by the one before that.  A barrier of its
+  // own, whose fills it counts itself, cannot run ahead: its next fill needs the slot that this warp hands back.
+  unsigned long long full[2 * kMaxStages];
   unsigned long long empty[kMaxStages];
   unsigned long long tmem_full[kMaxAccBufs];
   unsigned long long tmem_empty[kMaxAccBufs];
@@ -271,6 +276,18 @@ __device__ __forceinline__ bool wait_bar_inline(uint32_t bar, uint32_t parity, C
     }
   }
   return true;
+}
+
+// Two issuing warps: which barrier of its slot fill number `j` of the ring reports to, and with which parity (the tile's
+// warp, and how many of that warp's fills the slot had before).
+struct Fill {
+  uint32_t bar, parity;
+};
+__device__ __noinline__ Fill fill_of(uint32_t j, uint32_t stages, uint32_t num_kb) {
+  Fill f{(j / num_kb) & 1u, 0u};
+  for (uint32_t i = j % stages; i < j; i += stages) f.parity ^= ((i / num_kb) & 1u) == f.bar ? 1u : 0u;
+  f.bar = j % stages + f.bar * (uint32_t)kMaxStages;
+  return f;
 }
 
 struct TileCoord {
@@ -841,6 +858,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(smem_u32(&ctrl.full[s]), 1);
+      mbar_init(smem_u32(&ctrl.full[kMaxStages + s]), 1);
       mbar_init(smem_u32(&ctrl.empty[s]), 1);
     }
     for (int b = 0; b < kMaxAccBufs; ++b) {
@@ -942,7 +960,9 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       }
       const bool in_tile_loop = sub < nsub;
       bool stalled = false;
-      for (int t = worker; t < p.total_tiles && ok && in_tile_loop && !stalled; t += workers) {
+      int to = 0;                              // two issuing warps: the tile's row of barriers
+      for (int t = worker; t < p.total_tiles && ok && in_tile_loop && !stalled;
+           t += workers, to = kIssuers == 2 ? kMaxStages - to : 0) {
         const TileCoord tc = decode_tile(t, p);
         const int m_begin = tc.m0 + (int)rank * kBM;        // first of the 128 rows this CTA stages
         const int n_begin = tc.n0 + (int)rank * b_rows;     // first weight row this CTA stages
@@ -988,11 +1008,11 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             ok = __all_sync(0xffffffffu, wait_bar(smem_u32(&ctrl.empty[s]), ph ^ 1u, &ctrl, p));
             if (!ok) break;
             // bytes are reported to the leader's barrier; the leader arms it for both CTAs' copies
-            full = smem_u32(&ctrl.full[s]);
+            full = smem_u32(&ctrl.full[s + to]);
             if (PAIR) full = mapa_rank(full, 0);
             dst = ring + (uint32_t)s * p.stage_bytes;
             if (act_plane == 0 && rank == 0 && elect_one())
-              mbar_expect_tx(smem_u32(&ctrl.full[s]), (PAIR ? 2u : 1u) * (uint32_t)nkb * p.tx_bytes);
+              mbar_expect_tx(smem_u32(&ctrl.full[s + to]), (PAIR ? 2u : 1u) * (uint32_t)nkb * p.tx_bytes);
           }
           for (int j = 0; j < nkb; ++j) {
             if (my_turn && elect_one()) {
@@ -1049,15 +1069,15 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         // (In a pair the bytes are counted on the leader's barriers, so the follower just waits.)
         const uint32_t n = it < (uint32_t)p.stages ? it : (uint32_t)p.stages;
         for (uint32_t j = it - n; j < it; ++j) {
-          const int sj = (int)(j % (uint32_t)p.stages);
-          const uint32_t pj = (j / (uint32_t)p.stages) & 1u;
+          Fill f{j % (uint32_t)p.stages, (j / (uint32_t)p.stages) & 1u};
+          if (kIssuers == 2) f = fill_of(j, (uint32_t)p.stages, (uint32_t)p.num_kb);
           const unsigned long long t0 = global_ns();
           if (PAIR && rank != 0) {
             while (global_ns() - t0 < 2000000ull) {
             }
             break;
           }
-          while (!mbar_try_wait(smem_u32(&ctrl.full[sj]), pj) && global_ns() - t0 < 50000000ull) {
+          while (!mbar_try_wait(smem_u32(&ctrl.full[f.bar]), f.parity) && global_ns() - t0 < 50000000ull) {
           }
         }
       }
@@ -1082,15 +1102,15 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       const uint32_t kb_u = p.kb_bytes >> 4;
       const uint32_t off_a1 = a_u, off_b0 = NAX * a_u;
       const int ksteps_full = p.ksteps;
-      const uint32_t full_bar0 = smem_u32(&ctrl.full[0]), empty_bar0 = smem_u32(&ctrl.empty[0]);
-      uint32_t tile_iter = 0, ph = 0;
+      const uint32_t issuer = kIssuers == 2 && warp != kMmaWarp ? 1u : 0u;
+      const uint32_t full_bar0 = smem_u32(&ctrl.full[issuer * kMaxStages]), empty_bar0 = smem_u32(&ctrl.empty[0]);
+      uint32_t tile_iter = 0, ph = 0;      // (two issuing warps: bit s of ph is the parity of this warp's next fill of slot s)
       uint32_t a0 = ring_lo, full_bar = full_bar0, empty_bar = empty_bar0;
       int s = 0;
       bool ok = true;
       const bool b_res = PIX || HALO || TAPS || (GROUPED && p.b_resident);
       const int kps = GROUPED ? p.kps : 1;
       const uint32_t bres_lo = smem_desc_lo(ring + p.b_res_off) + (TAPS ? (uint32_t)(p.BN - 1) << 16 : 0u), bres_u = NBW * b_u;
-      const uint32_t issuer = kIssuers == 2 && warp != kMmaWarp ? 1u : 0u;
       const uint32_t issue = HALO || TAPS ? (elect_one() ? 1u : 0u) : 0u;
       const int halo_r = p.halo.R, halo_s = p.halo.S;
       const uint32_t px_u = p.halo.px_u, row_u = (uint32_t)p.halo.w * px_u, tap_u = (uint32_t)p.cblks * bres_u;
@@ -1100,7 +1120,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       }
       for (int t = worker; t < p.total_tiles && ok; t += workers, ++tile_iter) {
         if (kIssuers == 2 && (tile_iter & 1u) != issuer) {            // the other warp's tile: pass over its stages
-          for (s += p.num_kb; s >= p.stages; s -= p.stages) ph ^= 1u;
+          for (s += p.num_kb; s >= p.stages;) s -= p.stages;
           a0 = ring_lo + (uint32_t)s * stage_u;
           full_bar = full_bar0 + 8u * (uint32_t)s;
           empty_bar = empty_bar0 + 8u * (uint32_t)s;
@@ -1143,7 +1163,8 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
 #ifdef ADAPTION_TIMELINE
           const long long tw0 = clock64();
 #endif
-          ok = __all_sync(0xffffffffu, wait_bar(full_bar, ph, &ctrl, p, false));
+          ok = __all_sync(0xffffffffu, wait_bar(full_bar, kIssuers == 2 ? (ph >> s) & 1u : ph, &ctrl, p, false));
+          if (kIssuers == 2) ph ^= 1u << s;
 #ifdef ADAPTION_TIMELINE
           if (lane == 0 && blockIdx.x == 0 && tile_iter < 32u)
             g_timeline[(1 * 32 + tile_iter) * 8 + 3] += clock64() - tw0;   // time waiting for data
@@ -1221,7 +1242,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           empty_bar += 8u;
           if (++s == p.stages) {
             s = 0;
-            ph ^= 1u;
+            if (kIssuers == 1) ph ^= 1u;
             a0 = ring_lo;
             full_bar = full_bar0;
             empty_bar = empty_bar0;
@@ -2226,6 +2247,7 @@ TcConfig make_halo_config(const GemmProblem& g) {
 
 template <int NAX, int NBW, bool PAIR, int LOOP, int EPI>
 int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
+  note_layer(LOOP, p.stages, p.total_tiles, p.staged);
   // The dynamic shared-memory limit is a per-device attribute of the kernel: remember, per device
   // ordinal, the largest size it has been raised to (a racing thread at worst sets it once more).
   constexpr int kMaxDevices = 64;

@@ -10,6 +10,7 @@ from tests.test_gpu_layers import _pick_f_out, _rand_q, run_conv_case, run_pool_
 from tests.util import Guards, dev, from_qtensor, stats_tuple, to_qtensor
 
 pytestmark = pytest.mark.gpu
+ONE_COPY, UNPACKED = 4, 5          # adaption_debug_get("loop")
 
 
 @pytest.fixture(autouse=True)
@@ -81,6 +82,46 @@ def test_one_copy_for_all_taps(case, fast, staged, stochastic):
     B.adaption_debug_set("staged", staged)
     run_conv_case(np.random.default_rng(sum(case)), N, H, W, Cin, K, R, pad, 1, nx, nw, n_out, relu, B.ALGO_AUTO,
                   with_q16=False, stochastic_seed=77 if stochastic else None)
+
+
+# 8 bits: two warps issue every other tile's MMAs from one ring, whose slots change hands between them where its depth is no
+# multiple of twice a tile's channel blocks.  At least twice as many tiles per pair of SMs as stages.
+RINGS = [
+    # N, H, W, Cin, K, n_out, pooled, stages when stored
+    (16, 112, 112, 128, 128, 8, False, 3),
+    (16, 112, 112, 128, 128, 8, True, 5),
+    (28, 112, 112, 64, 128, 8, False, 9),
+    (22, 112, 112, 128, 64, 8, True, 7),
+    (10, 112, 112, 256, 64, 16, False, 3),                  # two channel blocks
+    (8, 112, 112, 256, 128, 8, True, 2),
+    (8, 112, 112, 512, 64, 8, True, 2),                     # four
+]
+
+
+@pytest.mark.parametrize("N,H,W,Cin,K,n_out,pooled,stages", RINGS)
+def test_rings_shared_by_two_issuing_warps(N, H, W, Cin, K, n_out, pooled, stages):
+    case = (N, H, W, Cin, K, 3, 1, 1, 8, 8, n_out, True)
+    if pooled:
+        run_pool_case(case, False)
+    else:
+        run_conv_case(np.random.default_rng(sum(case)), *case, B.ALGO_AUTO, with_q16=False)
+    assert [B.adaption_debug_get(k) for k in ("loop", "staged", "stages")] == [ONE_COPY, 1, stages]
+    assert B.adaption_debug_get("tiles") >= 2 * stages * 74
+
+
+def test_range_mode_on_a_ring_of_two_stages():
+    """Calibration's measuring pass over two channel blocks: nothing is staged, and two stages are left."""
+    N, H, W, Cin, K = 8, 112, 112, 256, 128
+    rng = np.random.default_rng(5)
+    xq, wq, bq = _rand_q(rng, (N, H, W, Cin), 8, 0.4), _rand_q(rng, (K, 3, 3, Cin), 8), _rand_q(rng, (K,), 8)
+    x, w = to_qtensor(xq.reshape(-1, Cin), 8, 5, Cin), to_qtensor(wq.reshape(-1, Cin), 8, 7, Cin)
+    want = orc.epilogue_range(orc.conv_acc(xq, wq, (1, 1), (1, 1)), bq, 7, 12, True)
+    st = B.new_stats()
+    B.adaption_lp_conv_fwd(B.conv_shape(N, H, W, Cin, K, 3, 3, 1, 1), x, w, dev(bq), 7, True, B.MODE_RANGE, B.ALGO_AUTO, None,
+                           st, None)
+    s = B.read_stats(st)
+    assert s.status == 0 and int(s.max_abs_acc) == want
+    assert [B.adaption_debug_get(k) for k in ("loop", "staged", "stages")] == [ONE_COPY, 0, 2]
 
 
 # first layers over pixels of 16 bytes
