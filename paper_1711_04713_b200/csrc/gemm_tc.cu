@@ -60,6 +60,11 @@ constexpr int kEpiGeneric = 0, kEpiFast = 1, kEpiStochastic = 2, kEpiFastStochas
 // kLoopPixels: neighbouring output pixels share a row of the GEMM, see PixelPlan.
 // kLoopHalo, kLoopTaps: the activations of a tile are copied once for all filter taps, see HaloPlan.
 constexpr int kLoopPlain = 0, kLoopGrouped = 1, kLoopPartial = 2, kLoopPixels = 3, kLoopHalo = 4, kLoopTaps = 5;
+// Added to the first three: tiles are boxes of pixels whose epilogue stores whole pooled windows, see BoxPlan.  (The last two
+// are always boxes, pooled or not.  Kernels of their own, because the box's coordinates stay live beside the 64-bit
+// epilogue's accumulators: with them in the kernels of all other layers too, 16 x 112 x 112, 64 -> 64, took 21.6 us instead of
+// 18.0 (1x1, 16 bits) and 28.6 instead of 23.5 (3x3, 8 by 16 bits); 126 random layers 3 % on average, at most 18.)
+constexpr int kLoopBoxes = 8;
 
 // Division by a number fixed for the launch: q = (n * mul >> 32) >> shift for 0 <= n < 2^31 (mul =
 // ceil(2^(32 + shift) / d) with 2^(shift + 1) >= d > 2^shift; mul = 0 stands for d = 1).  An integer division costs a
@@ -832,8 +837,10 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                const __grid_constant__ CUtensorMap map_y_hi, const __grid_constant__ CUtensorMap map_y_lo,
                const __grid_constant__ TcParams p) {
   constexpr int NACC = NAX + NBW - 1;
-  constexpr bool GROUPED = LOOP == kLoopGrouped, PARTIAL = LOOP == kLoopPartial, PIX = LOOP == kLoopPixels;
-  constexpr bool HALO = LOOP == kLoopHalo, TAPS = LOOP == kLoopTaps;
+  constexpr int MAIN = LOOP & (kLoopBoxes - 1);
+  constexpr bool GROUPED = MAIN == kLoopGrouped, PARTIAL = MAIN == kLoopPartial, PIX = MAIN == kLoopPixels;
+  constexpr bool HALO = MAIN == kLoopHalo, TAPS = MAIN == kLoopTaps, BOX = HALO || TAPS || LOOP != MAIN;
+  const bool box_pool = BOX && (LOOP != MAIN || p.box.pool != 0);
   constexpr bool FAST = EPI == kEpiFast;
   // Where one copy serves all taps and a step is one product, the last copying warp issues MMAs too, every other tile: they
   // take the tensor core less time than one warp needs for its loop (64 channels: 105 cycles an instruction, 40 where
@@ -969,7 +976,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         int img = 0, base_h = 0, base_w = 0;
         int tap = 0, cb = 0, r = 0, sx = 0;       // position of kb in the (tap, channel block) order
         if (lane == 0 && warp == 0) TL_STAMP(0, (uint32_t)((t - worker) / workers), 0);
-        if (p.box.on) {
+        if (BOX) {
           const BoxCoord bc = decode_box(m_begin >> 7, p.box);
           img = bc.img;
           base_w = bc.ow - p.pad_w;
@@ -1025,7 +1032,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                   int d = sx + p.px.first;                     // (the block order begins with a full one)
                   if (d >= p.px.blocks) d -= p.px.blocks;
                   tma_load_im2col<false>(dst + my_off, my_map, full, 0, base_w, base_h, img, (uint16_t)d, (uint16_t)r);
-                } else if (is_a && p.box.on)
+                } else if (is_a && BOX)
                   tma_load_4d<PAIR>(dst + my_off, my_map, full, cb * p.BK, base_w + sx, base_h + r, img);
                 else if (is_a)
                   tma_load_im2col<PAIR>(dst + my_off, my_map, full, cb * p.BK, base_w, base_h, img, (uint16_t)sx,
@@ -1326,12 +1333,13 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     const int col_begin = min(p.BN, (ew >> 2) * cols_per_warp);
     const int col_end = min(p.BN, col_begin + cols_per_warp);
     const int row = quarter * 32 + lane;   // row of the tile (and of this CTA's staging planes)
-    const int plane_rows = p.box.pool ? kBM / 4 : kBM;
+    const int plane_rows = box_pool ? kBM / 4 : kBM;
     const int plane_bytes = plane_rows * (PIX && p.pool_w ? p.BN >> 1 : p.BN);
     const int planes_bytes = plane_bytes * p.rq.out_planes;
     // box tiles: the lane of the pixel below, and the row of the stored tile that a 2x2 window becomes
     const int down = 1 << p.box.w;
-    const int window = ((row >> (p.box.w + 1)) << (p.box.w - p.box.pool)) | ((row & (down - 1)) >> 1);
+    const int pool = box_pool ? 1 : 0;
+    const int window = ((row >> (p.box.w + 1)) << (p.box.w - pool)) | ((row & (down - 1)) >> 1);
     const uint32_t stage_group = ring + p.stage_off + (uint32_t)(group * planes_bytes * p.stage_bufs);
     uint32_t stage_lo = stage_group;
     uint32_t stage_hi = stage_lo + (uint32_t)plane_bytes;
@@ -1403,7 +1411,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       int m = tc.m0 + (int)rank * kBM + row;
       bool row_ok = m < p.M;
       BoxCoord bc{0, 0, 0};
-      if (!PIX && p.box.on) {
+      if (BOX) {
         bc = decode_box(m >> 7, p.box);
         const int ow = bc.ow + (row & (down - 1)), oh = bc.oh + ((row >> p.box.w) & ((1 << p.box.h) - 1));
         const int img = bc.img + (row >> (p.box.w + p.box.h));
@@ -1533,7 +1541,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             if (NACC == 1 && p.byte_out) {
               uint32_t b[4];
               fast_bytes16<PIX>(t, half, p.rq.shift, row_ok, col, p, cnt, b);
-              if (!PIX && p.box.pool) {
+              if (box_pool) {
                 int first;
                 window_max<true>(b, lane, down, first);
                 st_shared_b32(stage_lo + staged_offset(window, (c0 >> 4) + half, p.BN, kBM / 4) + (uint32_t)first, b[0]);
@@ -1560,7 +1568,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             else
               fast_outputs16<NACC, false, PIX>(t, h, half, p.rq.shift, p.rq.qmax, row_ok, col, p, cnt, wq);
             const int chunk = (c0 >> 4) + half;
-            if (!PIX && p.box.pool) {
+            if (box_pool) {
               store_window_max(wq, lane, down, window, chunk, p, stage_lo, stage_hi);
             } else if (pool_px) {
               // the right pixel of a pair: its maximum with the left one, one chunk of the pooled row
@@ -1663,7 +1671,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             requant8<NACC, false, false, PIX>(xa, bcol, p, row_ok, m, col, cnt, wq);
             requant8<NACC, false, false, PIX>(xb, bcol + 8, p, row_ok, m, col + 8, cnt, wq + 4);
           }
-          if (!PIX && p.box.pool) {
+          if (box_pool) {
             store_window_max(wq, lane, down, window, c0 >> 4, p, stage_lo, stage_hi);
           } else if (p.staged && p.pool_w) {
             // Horizontal half of a 2x2 max-pool: rows 2j and 2j+1 of the tile are neighbouring
@@ -1702,8 +1710,8 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         // this warp's rows (a quarter of the tile, whose stored rows are consecutive whatever the pool)
         const int first = 32 * quarter;
         const uint32_t so = (uint32_t)(quarter * (plane_bytes >> (p.pool_w && !PIX ? 3 : 2)));
-        if (!PIX && p.box.on) {
-          const int oh = (bc.oh + ((first >> p.box.w) & ((1 << p.box.h) - 1))) >> p.box.pool, ow = bc.ow >> p.box.pool;
+        if (BOX) {
+          const int oh = (bc.oh + ((first >> p.box.w) & ((1 << p.box.h) - 1))) >> pool, ow = bc.ow >> pool;
           const int img = bc.img + (first >> (p.box.w + p.box.h));
           tma_store_4d(&map_y_lo, stage_lo + so, tc.n0, ow, oh, img);
           if (p.rq.out_planes == 2) tma_store_4d(&map_y_hi, stage_hi + so, tc.n0, ow, oh, img);
@@ -1713,8 +1721,8 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           if (p.rq.out_planes == 2) tma_store_2d(&map_y_hi, stage_hi + so, tc.n0, m_first);
         }
         bulk_commit();
-      } else if (!PIX && p.box.on && p.staged && store_leader) {
-        const int ow = bc.ow >> p.box.pool, oh = bc.oh >> p.box.pool;
+      } else if (BOX && p.staged && store_leader) {
+        const int ow = bc.ow >> pool, oh = bc.oh >> pool;
         for (int sub = 0; sub * 128 < p.BN; ++sub) {
           const uint32_t so = (uint32_t)sub * (uint32_t)(plane_rows * 128);
           tma_store_4d(&map_y_lo, stage_lo + so, tc.n0 + sub * 128, ow, oh, bc.img);
@@ -2247,7 +2255,7 @@ TcConfig make_halo_config(const GemmProblem& g) {
 
 template <int NAX, int NBW, bool PAIR, int LOOP, int EPI>
 int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
-  note_layer(LOOP, p.stages, p.total_tiles, p.staged);
+  note_layer(LOOP & (kLoopBoxes - 1), p.stages, p.total_tiles, p.staged);
   // The dynamic shared-memory limit is a per-device attribute of the kernel: remember, per device
   // ordinal, the largest size it has been raised to (a racing thread at worst sets it once more).
   constexpr int kMaxDevices = 64;
@@ -2302,16 +2310,20 @@ int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t s
 template <int NAX, int NBW, bool PAIR, int LOOP>
 int launch_epi(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
   if (p.fast_relu != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiFast>(maps, p, grid, smem, stream);
-  if (p.fast_stochastic != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiFastStochastic>(maps, p, grid, smem, stream);
-  if (p.st.enabled != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiStochastic>(maps, p, grid, smem, stream);
+  if constexpr ((LOOP & kLoopBoxes) == 0) {                // (the pooling call rounds to nearest)
+    if (p.fast_stochastic != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiFastStochastic>(maps, p, grid, smem, stream);
+    if (p.st.enabled != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiStochastic>(maps, p, grid, smem, stream);
+  } else if (p.st.enabled != 0) {
+    return ADAPTION_ERR_UNSUPPORTED;
+  }
   return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiGeneric>(maps, p, grid, smem, stream);
 }
 
-template <int NAX, int NBW, bool PAIR>
+template <int NAX, int NBW, bool PAIR, int BOXES>
 int launch_loop(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
-  if (p.kps > 1 || p.b_resident != 0) return launch_epi<NAX, NBW, PAIR, kLoopGrouped>(maps, p, grid, smem, stream);
-  if (p.ksteps_last != p.ksteps) return launch_epi<NAX, NBW, PAIR, kLoopPartial>(maps, p, grid, smem, stream);
-  return launch_epi<NAX, NBW, PAIR, kLoopPlain>(maps, p, grid, smem, stream);
+  if (p.kps > 1 || p.b_resident != 0) return launch_epi<NAX, NBW, PAIR, kLoopGrouped + BOXES>(maps, p, grid, smem, stream);
+  if (p.ksteps_last != p.ksteps) return launch_epi<NAX, NBW, PAIR, kLoopPartial + BOXES>(maps, p, grid, smem, stream);
+  return launch_epi<NAX, NBW, PAIR, kLoopPlain + BOXES>(maps, p, grid, smem, stream);
 }
 
 template <int NAX, int NBW>
@@ -2322,8 +2334,11 @@ int launch_either(bool pair, const CUtensorMap* maps, const TcParams& p, int gri
     if (p.halo.steps > 0) return launch_epi<NAX, NBW, false, kLoopTaps>(maps, p, grid, smem, stream);
     if (p.halo.w > 0) return launch_epi<NAX, NBW, true, kLoopHalo>(maps, p, grid, smem, stream);
   }
-  return pair ? launch_loop<NAX, NBW, true>(maps, p, grid, smem, stream)
-              : launch_loop<NAX, NBW, false>(maps, p, grid, smem, stream);
+  if (p.box.on != 0)
+    return pair ? launch_loop<NAX, NBW, true, kLoopBoxes>(maps, p, grid, smem, stream)
+                : launch_loop<NAX, NBW, false, kLoopBoxes>(maps, p, grid, smem, stream);
+  return pair ? launch_loop<NAX, NBW, true, 0>(maps, p, grid, smem, stream)
+              : launch_loop<NAX, NBW, false, 0>(maps, p, grid, smem, stream);
 }
 
 
