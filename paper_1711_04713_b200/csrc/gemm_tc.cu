@@ -199,9 +199,11 @@ struct TcParams {
   int fast_range;             // range mode: 32-bit keys decide what is worth the exact 64-bit value
   int pool_w;                 // store max(row 2j, row 2j+1) of the tile: half of a 2x2 max-pool (staged only)
   int epi_groups;             // 1, 2 or 4 groups of epilogue warps that take turns tile by tile
-  // four groups: every warp makes, stages and stores 32 whole rows of a tile by itself, with no barrier among the warps (8
-  // bits, 128 x 224 x 224, 3 -> 64 230 -> 214 us; 128 x 112 x 112, one copy for all taps, us with two groups and four: 64 ->
-  // 128 146 and 114, 128 -> 128 174 and 140)
+  // One copy for all taps, four groups: every warp makes, stages and stores 32 whole rows of a tile by itself, with no
+  // barrier among the warps (8 bits, 128 x 224 x 224, 3 -> 64 230 -> 214 us; 128 x 112 x 112, us with two groups and four: 64
+  // -> 128 146 and 114, 128 -> 128 174 and 140).  Not in the other loops, whose kernels spilled for it: 48 x 62 x 137, 38 -> 92,
+  // 3x3 at 12 bits 164 us with it and 148 without, 61 x 36 x 197, 8 -> 72, 1x1 63 and 61, 51 x 200 x 158, 41 -> 22 at 8 bits 43.5
+  // and 40.3.
   int own_rows;
   int staged;                 // outputs leave through shared memory and bulk-tensor stores
   int stage_bufs;             // staging buffers per epilogue group: 1, or 2 used in turn (narrow tiles)
@@ -1346,7 +1348,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     uint32_t stage_turn = 0;
     // per-column epilogue constants of the current tile, one array per group, behind the staging planes
     // (one per warp where warps work by themselves: then no barrier separates readers and writers)
-    const bool own = p.own_rows != 0;
+    const bool own = (HALO || TAPS) && p.own_rows != 0;
     long long* colconst = reinterpret_cast<long long*>(smem_raw + (ring - smem_u32(smem_raw)) + p.const_off) +
                           (own ? warp - kFirstEpiWarp : group) * p.BN;
     const bool store_leader = (own || ew == 0) && lane == 0;
@@ -1981,8 +1983,7 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
   c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) / (c.box.pool ? 4u : 1u) : 0u;
   // dynamic shared memory: everything up to the per-block limit except the control block
-  c.own_rows = c.epi_groups * 4 == kEpiWarps && c.BN <= 128;
-  c.const_bytes = (uint32_t)(c.BN * (c.own_rows ? kEpiWarps : c.epi_groups) * sizeof(long long));
+  c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
   const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
   // group short k-blocks so that a stage carries roughly 768 tensor-pipe cycles of work or more.  512 with one product
   // per step (128 -> 128 channels at 112 x 112, 8 bits, batch 128 231 us with two k-blocks, 264 with three), but not for
@@ -2129,8 +2130,7 @@ TcConfig make_pixel_config(const GemmProblem& g, int G) {
   const int most_groups = c.BN <= 64 ? 4 : 2;
   while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
   c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) / (g.pool_w ? 2u : 1u) : 0u;
-  c.own_rows = c.epi_groups * 4 == kEpiWarps && c.BN <= 128;
-  c.const_bytes = (uint32_t)(c.BN * (c.own_rows ? kEpiWarps : c.epi_groups) * sizeof(long long));
+  c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
   const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
   c.b_resident = true;
   c.b_res_bytes = c.nbw * px.b_plane;
