@@ -188,9 +188,11 @@ __device__ __forceinline__ void store_group(const CgParams& p, size_t off, const
   }
 }
 
-// What happens to a finished sum.  Each kind has an epilogue of its own, so that a launch only fetches the
+// What happens to a finished sum.  Each kind has a kernel of its own, so that a launch only fetches the
 // instructions it runs: with the generator inlined beside the deterministic path the final stage of a
-// 128 x 128 tile took 29 k cycles, nearly all of it instruction fetches.
+// 128 x 128 tile took 29 k cycles, nearly all of it instruction fetches.  (Three epilogues in one kernel: 150 registers
+// where rounding alone takes 94, and every change of one moved the others; weights not in L2, us, one kernel and three: 5
+// rows, 4096 -> 1000, 16 bits 7.33 and 7.18, 8 by 16 bits 6.57 and 6.42; 2 rows, 284 -> 813 4.91 and 4.75.)
 constexpr int kFinishRound = 0, kFinishStochastic = 1, kFinishRange = 2;
 
 // `G` finished sums (the first `nreal` are real outputs, the rest padding with sum 0) of the elements `index`,
@@ -344,7 +346,7 @@ __device__ __forceinline__ void finish_tile(const CgParams& p, const Slots& slot
   }
 }
 
-template <int NAX, int NBW>
+template <int NAX, int NBW, int KIND>
 __global__ void __launch_bounds__(kClusterThreads, 1)
 lp_cluster_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
                   const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
@@ -613,14 +615,7 @@ lp_cluster_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_const
   // ---- the columns this CTA owns: sum over the CTAs, bias, ReLU, requantize, store
   const bool aborted = ctrl.abort != 0;
   const int col_first = c0 + (int)rank * cpo;
-  if (aborted)
-    ;                           // nothing sensible to store; the status says so
-  else if (p.mode == ADAPTION_MODE_RANGE)
-    finish_tile<kFinishRange>(p, slots, ctrl, cpo, r0, col_first);
-  else if (p.st.enabled)
-    finish_tile<kFinishStochastic>(p, slots, ctrl, cpo, r0, col_first);
-  else
-    finish_tile<kFinishRound>(p, slots, ctrl, cpo, r0, col_first);
+  if (!aborted) finish_tile<KIND>(p, slots, ctrl, cpo, r0, col_first);      // (else the status says that nothing was stored)
   if (warp == kFirstTableWarp) CG_STAMP(8);
   // zeros in the padding behind the last column tile (channels), if the pitch reaches that far
   const int pad_first = p.is_conv ? p.tiles_c * p.BN : (p.N + kRows - 1) / kRows * kRows;
@@ -790,7 +785,7 @@ CgPlan make_plan(const GemmProblem& g, bool pool) {
   return c;
 }
 
-template <int NAX, int NBW>
+template <int NAX, int NBW, int KIND>
 int launch_cg(const CUtensorMap* maps, const CgParams& p, int grid, size_t smem, cudaStream_t stream) {
   // (per device ordinal: the largest dynamic shared-memory size the kernel has been allowed)
   constexpr int kMaxDevices = 64;
@@ -799,7 +794,7 @@ int launch_cg(const CUtensorMap* maps, const CgParams& p, int grid, size_t smem,
   if (cudaGetDevice(&dev) != cudaSuccess) return ADAPTION_ERR_CUDA;
   const bool cached = dev >= 0 && dev < kMaxDevices;
   if (!cached || smem > attr_size[dev].load(std::memory_order_acquire)) {
-    const cudaError_t ae = cudaFuncSetAttribute(lp_cluster_kernel<NAX, NBW>,
+    const cudaError_t ae = cudaFuncSetAttribute(lp_cluster_kernel<NAX, NBW, KIND>,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (ae != cudaSuccess) return cuda_failure(ae, "lp_cluster_kernel shared-memory attribute");
     if (cached) {
@@ -831,12 +826,19 @@ int launch_cg(const CUtensorMap* maps, const CgParams& p, int grid, size_t smem,
   cfg.attrs = n_attr ? attr : nullptr;
   cfg.numAttrs = n_attr;
   count_launch();
-  const cudaError_t le = cudaLaunchKernelEx(&cfg, lp_cluster_kernel<NAX, NBW>, maps[0], maps[1], maps[2], maps[3], p);
+  const cudaError_t le = cudaLaunchKernelEx(&cfg, lp_cluster_kernel<NAX, NBW, KIND>, maps[0], maps[1], maps[2], maps[3], p);
   if (le != cudaSuccess) {
     (void)cudaGetLastError();
     return cuda_failure(le, "lp_cluster_kernel launch");
   }
   return ADAPTION_OK;
+}
+
+template <int NAX, int NBW>
+int launch_kind(const CUtensorMap* maps, const CgParams& p, int grid, size_t smem, cudaStream_t stream) {
+  if (p.mode == ADAPTION_MODE_RANGE) return launch_cg<NAX, NBW, kFinishRange>(maps, p, grid, smem, stream);
+  if (p.st.enabled) return launch_cg<NAX, NBW, kFinishStochastic>(maps, p, grid, smem, stream);
+  return launch_cg<NAX, NBW, kFinishRound>(maps, p, grid, smem, stream);
 }
 
 }  // namespace
@@ -941,10 +943,10 @@ int launch_cluster(const GemmProblem& g) {
   p.timeout_ns = wait_limit_ns();
   p.stall_at = knob(kStallAt);
   const int grid = c.tiles_r * c.tiles_c * c.S;
-  if (c.nax == 2 && c.nbw == 2) return launch_cg<2, 2>(maps, p, grid, c.smem, g.stream);
-  if (c.nax == 2) return launch_cg<2, 1>(maps, p, grid, c.smem, g.stream);
-  if (c.nbw == 2) return launch_cg<1, 2>(maps, p, grid, c.smem, g.stream);
-  return launch_cg<1, 1>(maps, p, grid, c.smem, g.stream);
+  if (c.nax == 2 && c.nbw == 2) return launch_kind<2, 2>(maps, p, grid, c.smem, g.stream);
+  if (c.nax == 2) return launch_kind<2, 1>(maps, p, grid, c.smem, g.stream);
+  if (c.nbw == 2) return launch_kind<1, 2>(maps, p, grid, c.smem, g.stream);
+  return launch_kind<1, 1>(maps, p, grid, c.smem, g.stream);
 }
 
 }  // namespace adaption
