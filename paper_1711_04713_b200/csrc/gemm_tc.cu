@@ -2158,6 +2158,41 @@ TcConfig make_pixel_config(const GemmProblem& g) {
   return TcConfig();
 }
 
+// Whether one copy for all taps beats a copy per tap.  It waits for all of the weights before its first MMA and gains by
+// the rows that it does not copy: `bytes` per pixel and plane otherwise.  Ratio of times, streaming / this, over images of 16 to
+// 224 columns (T: tiles of a pair of SMs):
+//   one tile per pair or fewer: 0.81 to 1.02 whatever the filter;
+//   256 to 448 bytes (2x2 over 64 channels): 0.77 to 1.0 up to T = 4800; 512: 0.83 to 1.0 at 100 to 600, 1.02 to 1.1 at 1200;
+//   measuring only, with two column tiles 0.83 to 1.05 up to T = 222, 0.97 to 1.1 from 296 on; 512 bytes 1.08 to 1.12 from 600 on;
+//   three accumulators: two column tiles, which read the copy twice, 64 -> 128 0.85 to 0.96 up to 600, 0.98 at 1200, 0.99 to 1.06
+//     from 2400 on, but 1.12 to 1.6 from 600 on where the streamed tile of 128 columns is wider than the output's pitch and
+//     cannot be staged (64 -> 72); the 64-bit epilogue, 64 -> 61 and 100 0.94 to 1.0 (5x5 1.05 to 1.38), 96 -> 50 0.92 to 1.0 up to
+//     148, 1.0 to 1.2 beyond; 640 and 768 bytes of wide blocks 0.9 to 1.07 at 100 and 148, 1.06 to 1.3 from 300 on;
+//   one accumulator, where a streamed tile is a single CTA's: 64 -> 64 0.95 to 1.06 up to T = 148, 1.05 to 1.3 at 150 to 290, 0.91
+//     to 1.06 from 296 on, where the streamed weights stay resident too, 1.03 to 1.25 from 700 on; 64 -> 128 0.81 to 1.06 up to 784,
+//     1.0 to 1.08 from 1200 on; 128 -> 128 with 640 bytes 0.92 to 0.97 at 100 to 300, 768 to 1024 0.93 to 0.98 at 100 and 148, 1.02
+//     to 1.16 at 300, 1152 and more 1.03 and more; 128 columns through the 64-bit epilogue, whose four groups take a tile each:
+//     128 -> 99 and 96 -> 70 0.91 to 1.08 up to 300, 1.02 to 1.13 from 600 on, 64 -> 100 0.97, 1.0 and 1.03 at 600, 1200 and 2400.
+// Everything else measured 0.94 to 1.27 at 100 and 148, 0.97 to 2.3 beyond.
+bool one_copy_pays(const TcConfig& c, const GemmProblem& g, int taps) {
+  const int pairs = num_sms() / 2, T = c.tiles_m, bytes = taps * c.cblks * c.BK;
+  const bool wide_sums = g.N % 8 != 0;         // the 64-bit epilogue
+  if (T <= pairs) return false;
+  if (g.mode != ADAPTION_MODE_REQUANT)
+    return bytes < 576 ? bytes >= 512 && T >= 8 * pairs : c.tiles_n == 1 || T >= 4 * pairs;
+  if (bytes < 576) return bytes >= 512 && c.tiles_n == 1 && T >= 16 * pairs;
+  if (c.nacc == 3) {
+    if (wide_sums && c.BK == 64 && bytes < 1024) return false;
+    if (c.tiles_n > 1) return T >= (g.y.c_stride < 128 ? 4 : 32) * pairs;
+    return c.BK == 64 || (bytes >= 1152 && !wide_sums) || T > 2 * pairs;
+  }
+  if (c.BN == 128 && wide_sums) return T >= (c.BK == 64 ? 16 : 9) * pairs;
+  if (c.BK == 64 && bytes < 1024)
+    return c.BN == 128 ? T >= 16 * pairs : T >= 9 * pairs || (T > 2 * pairs && T < 4 * pairs);
+  if (c.BK == 128 && bytes < 1152) return T >= (bytes < 768 ? 9 : 4) * pairs;
+  return true;
+}
+
 // One copy of the activations for all taps (see HaloPlan), where the weights stay resident beside at least two tiles'
 // copies of them: operands of one width, 8 x 16 boxes without much margin.
 TcConfig make_halo_config(const GemmProblem& g) {
@@ -2222,7 +2257,7 @@ TcConfig make_halo_config(const GemmProblem& g) {
     }
     c.b_res_bytes = (uint32_t)(c.tiles_n * c.b_blocks * c.nbw) * c.b_bytes;
     c.tiles_m = (int)((boxes + 1) / 2);
-    if (c.tiles_m < sms / 2) return c;
+    if (!one_copy_pays(c, g, taps) && knob(kHalo) < 2) return c;
   }
   c.kb_per_split = c.num_kb;
   c.a_tx = (uint32_t)(h.w * (kHaloH + g.cs.R - 1) * c.BK);

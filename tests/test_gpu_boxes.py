@@ -124,6 +124,26 @@ def test_range_mode_on_a_ring_of_two_stages():
     assert [B.adaption_debug_get(k) for k in ("loop", "staged", "stages")] == [ONE_COPY, 0, 2]
 
 
+# 3x3 over images of 16 columns, 16 rows a tile of a pair: either side of the sizes where one copy for all taps is taken
+LINES = [
+    # tiles, Cin, K, n_bits, taken
+    (74, 64, 64, 16, False), (75, 64, 64, 16, True),
+    (74, 128, 128, 8, False), (75, 128, 128, 8, True),
+    (148, 64, 64, 8, False), (149, 64, 64, 8, True), (295, 64, 64, 8, True), (296, 64, 64, 8, False),
+    (665, 64, 64, 8, False), (666, 64, 64, 8, True),
+    (665, 128, 99, 8, False), (666, 128, 99, 8, True),       # 64-bit epilogue, 128 columns
+    (295, 64, 72, 12, False), (296, 64, 72, 12, True),       # two column tiles, the output's pitch is narrower than one of 128
+    (400, 64, 61, 16, False),
+]
+
+
+@pytest.mark.parametrize("tiles,Cin,K,n_bits,taken", LINES)
+def test_one_copy_is_taken_where_it_pays(tiles, Cin, K, n_bits, taken):
+    case = (1, 16 * tiles, 16, Cin, K, 3, 1, 1, n_bits, n_bits, n_bits, True)
+    run_conv_case(np.random.default_rng(tiles), *case, B.ALGO_AUTO, with_q16=False)
+    assert (B.adaption_debug_get("loop") == ONE_COPY) == taken
+
+
 # first layers over pixels of 16 bytes
 TAPS = [
     # N, H, W, Cin, K, R, pad, nx, nw, n_out, relu
