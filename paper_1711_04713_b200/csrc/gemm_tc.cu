@@ -2272,7 +2272,11 @@ TcConfig make_halo_config(const GemmProblem& g) {
              g.y.c_stride % 16 == 0 && knob(kStaged) != 0;
   if (g.box_pool && !c.staged) return c;
   c.epi_groups = c.acc_bufs;
-  const int most_groups = c.BN <= 64 || c.nacc == 1 ? 4 : 2;
+  // (first layers through the 64-bit epilogue with up to two tiles per SM: a tile's chain counts, so twice the warps share it;
+  // 8 bits, 3 -> 100, us with four groups and two, 76 tiles 11.6 and 10.1, 222 14.8 and 13.6, 300 16.9 and 18.2; 3 -> 61 7.7 and 6.9,
+  // 9.6 and 9.1, 10.1 and 11.5)
+  const bool two_groups = g.taps && g.N % 8 != 0 && c.tiles_m <= 2 * sms;
+  const int most_groups = !two_groups && (c.BN <= 64 || c.nacc == 1) ? 4 : 2;
   while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
   c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) / (g.box_pool ? 4u : 1u) : 0u;
   c.own_rows = c.epi_groups * 4 == kEpiWarps && c.BN <= 128;

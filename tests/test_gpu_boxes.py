@@ -154,6 +154,8 @@ TAPS = [
     (1, 65, 63, 1, 32, 2, 0, 16, 16, 16, False),           # even filter, columns and rows behind the last, signed
     (1, 64, 64, 2, 61, 3, 1, 8, 8, 8, True),               # 64-bit epilogue
     (9, 112, 112, 3, 64, 3, 1, 16, 16, 16, True),          # many tiles per block
+    (3, 112, 112, 3, 100, 3, 1, 8, 8, 8, True),            # 294 tiles through the 64-bit epilogue: two groups of warps
+    (1, 2400, 16, 3, 100, 3, 1, 8, 8, 8, True),            # 300: four
 ]
 
 
