@@ -63,7 +63,9 @@ constexpr int kLoopPlain = 0, kLoopGrouped = 1, kLoopPartial = 2, kLoopPixels = 
 // Added to the first three: tiles are boxes of pixels whose epilogue stores whole pooled windows, see BoxPlan.  (The last two
 // are always boxes, pooled or not.  Kernels of their own, because the box's coordinates stay live beside the 64-bit
 // epilogue's accumulators: with them in the kernels of all other layers too, 16 x 112 x 112, 64 -> 64, took 21.6 us instead of
-// 18.0 (1x1, 16 bits) and 28.6 instead of 23.5 (3x3, 8 by 16 bits); 126 random layers 3 % on average, at most 18.)
+// 18.0 (1x1, 16 bits) and 28.6 instead of 23.5 (3x3, 8 by 16 bits); 126 random layers 3 % on average, at most 18.  Partial
+// blocks with the 32-bit epilogue are one kernel for both: split, 12 x 45 x 37, 96 -> 168 took 25.2 us instead of 24.8, seven
+// others 0.3 % less.)
 constexpr int kLoopBoxes = 8;
 
 // Division by a number fixed for the launch: q = (n * mul >> 32) >> shift for 0 <= n < 2^31 (mul =
@@ -842,7 +844,8 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
   constexpr int MAIN = LOOP & (kLoopBoxes - 1);
   constexpr bool GROUPED = MAIN == kLoopGrouped, PARTIAL = MAIN == kLoopPartial, PIX = MAIN == kLoopPixels;
   constexpr bool HALO = MAIN == kLoopHalo, TAPS = MAIN == kLoopTaps, BOX = HALO || TAPS || LOOP != MAIN;
-  const bool box_pool = BOX && (LOOP != MAIN || p.box.pool != 0);
+  const bool boxes = BOX || (LOOP == kLoopPartial && EPI == kEpiFast && p.box.on != 0);
+  const bool box_pool = boxes && (LOOP != MAIN || p.box.pool != 0);
   constexpr bool FAST = EPI == kEpiFast;
   // Where one copy serves all taps and a step is one product, the last copying warp issues MMAs too, every other tile: they
   // take the tensor core less time than one warp needs for its loop (64 channels: 105 cycles an instruction, 40 where
@@ -978,7 +981,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         int img = 0, base_h = 0, base_w = 0;
         int tap = 0, cb = 0, r = 0, sx = 0;       // position of kb in the (tap, channel block) order
         if (lane == 0 && warp == 0) TL_STAMP(0, (uint32_t)((t - worker) / workers), 0);
-        if (BOX) {
+        if (boxes) {
           const BoxCoord bc = decode_box(m_begin >> 7, p.box);
           img = bc.img;
           base_w = bc.ow - p.pad_w;
@@ -1034,7 +1037,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                   int d = sx + p.px.first;                     // (the block order begins with a full one)
                   if (d >= p.px.blocks) d -= p.px.blocks;
                   tma_load_im2col<false>(dst + my_off, my_map, full, 0, base_w, base_h, img, (uint16_t)d, (uint16_t)r);
-                } else if (is_a && BOX)
+                } else if (is_a && boxes)
                   tma_load_4d<PAIR>(dst + my_off, my_map, full, cb * p.BK, base_w + sx, base_h + r, img);
                 else if (is_a)
                   tma_load_im2col<PAIR>(dst + my_off, my_map, full, cb * p.BK, base_w, base_h, img, (uint16_t)sx,
@@ -1413,7 +1416,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       int m = tc.m0 + (int)rank * kBM + row;
       bool row_ok = m < p.M;
       BoxCoord bc{0, 0, 0};
-      if (BOX) {
+      if (boxes) {
         bc = decode_box(m >> 7, p.box);
         const int ow = bc.ow + (row & (down - 1)), oh = bc.oh + ((row >> p.box.w) & ((1 << p.box.h) - 1));
         const int img = bc.img + (row >> (p.box.w + p.box.h));
@@ -1712,7 +1715,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         // this warp's rows (a quarter of the tile, whose stored rows are consecutive whatever the pool)
         const int first = 32 * quarter;
         const uint32_t so = (uint32_t)(quarter * (plane_bytes >> (p.pool_w && !PIX ? 3 : 2)));
-        if (BOX) {
+        if (boxes) {
           const int oh = (bc.oh + ((first >> p.box.w) & ((1 << p.box.h) - 1))) >> pool, ow = bc.ow >> pool;
           const int img = bc.img + (first >> (p.box.w + p.box.h));
           tma_store_4d(&map_y_lo, stage_lo + so, tc.n0, ow, oh, img);
@@ -1723,7 +1726,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
           if (p.rq.out_planes == 2) tma_store_2d(&map_y_hi, stage_hi + so, tc.n0, m_first);
         }
         bulk_commit();
-      } else if (BOX && p.staged && store_leader) {
+      } else if (boxes && p.staged && store_leader) {
         const int ow = bc.ow >> pool, oh = bc.oh >> pool;
         for (int sub = 0; sub * 128 < p.BN; ++sub) {
           const uint32_t so = (uint32_t)sub * (uint32_t)(plane_rows * 128);
@@ -2348,7 +2351,8 @@ int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t s
 
 template <int NAX, int NBW, bool PAIR, int LOOP>
 int launch_epi(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
-  if (p.fast_relu != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiFast>(maps, p, grid, smem, stream);
+  constexpr int FAST_LOOP = LOOP == kLoopPartial + kLoopBoxes ? kLoopPartial : LOOP;
+  if (p.fast_relu != 0) return launch_kernel<NAX, NBW, PAIR, FAST_LOOP, kEpiFast>(maps, p, grid, smem, stream);
   if constexpr ((LOOP & kLoopBoxes) == 0) {                // (the pooling call rounds to nearest)
     if (p.fast_stochastic != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiFastStochastic>(maps, p, grid, smem, stream);
     if (p.st.enabled != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiStochastic>(maps, p, grid, smem, stream);
