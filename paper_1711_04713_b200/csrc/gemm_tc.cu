@@ -63,9 +63,10 @@ constexpr int kLoopPlain = 0, kLoopGrouped = 1, kLoopPartial = 2, kLoopPixels = 
 // Added to the first three: tiles are boxes of pixels whose epilogue stores whole pooled windows, see BoxPlan.  (The last two
 // are always boxes, pooled or not.  Kernels of their own, because the box's coordinates stay live beside the 64-bit
 // epilogue's accumulators: with them in the kernels of all other layers too, 16 x 112 x 112, 64 -> 64, took 21.6 us instead of
-// 18.0 (1x1, 16 bits) and 28.6 instead of 23.5 (3x3, 8 by 16 bits); 126 random layers 3 % on average, at most 18.  Partial
-// blocks with the 32-bit epilogue are one kernel for both: split, 12 x 45 x 37, 96 -> 168 took 25.2 us instead of 24.8, seven
-// others 0.3 % less.)
+// 18.0 (1x1, 16 bits) and 28.6 instead of 23.5 (3x3, 8 by 16 bits); 126 random layers 3 % on average, at most 18.)
+// Partial blocks with the 32-bit epilogue are an exception: their kernel for boxes takes other tiles of 128 columns too, which
+// the compiler schedules better in it (12 x 45 x 37, 96 -> 168, 12 bits 24.3 us, 25.2 in the kernel without boxes; seven others
+// within 1 %), but not narrower ones (16 x 56 x 56, 96 -> 32, 16 bits 18.1 us, 17.2 without).
 constexpr int kLoopBoxes = 8;
 
 // Division by a number fixed for the launch: q = (n * mul >> 32) >> shift for 0 <= n < 2^31 (mul =
@@ -203,7 +204,8 @@ struct TcParams {
   int epi_groups;             // 1, 2 or 4 groups of epilogue warps that take turns tile by tile
   // One copy for all taps, four groups: every warp makes, stages and stores 32 whole rows of a tile by itself, with no
   // barrier among the warps (8 bits, 128 x 224 x 224, 3 -> 64 230 -> 214 us; 128 x 112 x 112, us with two groups and four: 64
-  // -> 128 146 and 114, 128 -> 128 174 and 140).  Not in the other loops, whose kernels spilled for it: 48 x 62 x 137, 38 -> 92,
+  // -> 128 146 and 114, 128 -> 128 174 and 140), and in the one kernel that takes box tiles and others.  Not in the other
+  // loops, whose kernels spilled for it: 48 x 62 x 137, 38 -> 92,
   // 3x3 at 12 bits 164 us with it and 148 without, 61 x 36 x 197, 8 -> 72, 1x1 63 and 61, 51 x 200 x 158, 41 -> 22 at 8 bits 43.5
   // and 40.3.
   int own_rows;
@@ -844,8 +846,10 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
   constexpr int MAIN = LOOP & (kLoopBoxes - 1);
   constexpr bool GROUPED = MAIN == kLoopGrouped, PARTIAL = MAIN == kLoopPartial, PIX = MAIN == kLoopPixels;
   constexpr bool HALO = MAIN == kLoopHalo, TAPS = MAIN == kLoopTaps, BOX = HALO || TAPS || LOOP != MAIN;
-  const bool boxes = BOX || (LOOP == kLoopPartial && EPI == kEpiFast && p.box.on != 0);
-  const bool box_pool = boxes && (LOOP != MAIN || p.box.pool != 0);
+  // (the exception that kLoopBoxes tells of)
+  constexpr bool EITHER = LOOP == kLoopPartial + kLoopBoxes && EPI == kEpiFast;
+  const bool boxes = BOX && (!EITHER || p.box.on != 0);
+  const bool box_pool = boxes && ((LOOP != MAIN && !EITHER) || p.box.pool != 0);
   constexpr bool FAST = EPI == kEpiFast;
   // Where one copy serves all taps and a step is one product, the last copying warp issues MMAs too, every other tile: they
   // take the tensor core less time than one warp needs for its loop (64 channels: 105 cycles an instruction, 40 where
@@ -1351,7 +1355,7 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     uint32_t stage_turn = 0;
     // per-column epilogue constants of the current tile, one array per group, behind the staging planes
     // (one per warp where warps work by themselves: then no barrier separates readers and writers)
-    const bool own = (HALO || TAPS) && p.own_rows != 0;
+    const bool own = (HALO || TAPS || EITHER) && p.own_rows != 0;
     long long* colconst = reinterpret_cast<long long*>(smem_raw + (ring - smem_u32(smem_raw)) + p.const_off) +
                           (own ? warp - kFirstEpiWarp : group) * p.BN;
     const bool store_leader = (own || ew == 0) && lane == 0;
@@ -1986,7 +1990,9 @@ TcConfig make_config_impl(const GemmProblem& g, bool allow_wide) {
   while (c.epi_groups > 1 && (c.epi_groups > most_groups || c.epi_groups > knob(kEpiGroups))) c.epi_groups /= 2;
   c.stage_out_bytes = c.staged ? (uint32_t)(kBM * c.BN * out_planes * c.epi_groups) / (c.box.pool ? 4u : 1u) : 0u;
   // dynamic shared memory: everything up to the per-block limit except the control block
-  c.const_bytes = (uint32_t)(c.BN * c.epi_groups * sizeof(long long));
+  // (box tiles over partial blocks with the 32-bit epilogue: launch_tensor)
+  c.own_rows = partial && c.box.on && c.epi_groups * 4 == kEpiWarps;
+  c.const_bytes = (uint32_t)(c.BN * (c.own_rows ? kEpiWarps : c.epi_groups) * sizeof(long long));
   const size_t budget = 232448 - sizeof(Ctrl) - 256 - c.stage_out_bytes - c.const_bytes;
   // group short k-blocks so that a stage carries roughly 768 tensor-pipe cycles of work or more.  512 with one product
   // per step (128 -> 128 channels at 112 x 112, 8 bits, batch 128 231 us with two k-blocks, 264 with three), but not for
@@ -2351,8 +2357,7 @@ int launch_kernel(const CUtensorMap* maps, const TcParams& p, int grid, size_t s
 
 template <int NAX, int NBW, bool PAIR, int LOOP>
 int launch_epi(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
-  constexpr int FAST_LOOP = LOOP == kLoopPartial + kLoopBoxes ? kLoopPartial : LOOP;
-  if (p.fast_relu != 0) return launch_kernel<NAX, NBW, PAIR, FAST_LOOP, kEpiFast>(maps, p, grid, smem, stream);
+  if (p.fast_relu != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiFast>(maps, p, grid, smem, stream);
   if constexpr ((LOOP & kLoopBoxes) == 0) {                // (the pooling call rounds to nearest)
     if (p.fast_stochastic != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiFastStochastic>(maps, p, grid, smem, stream);
     if (p.st.enabled != 0) return launch_kernel<NAX, NBW, PAIR, LOOP, kEpiStochastic>(maps, p, grid, smem, stream);
@@ -2365,6 +2370,8 @@ int launch_epi(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem
 template <int NAX, int NBW, bool PAIR, int BOXES>
 int launch_loop(const CUtensorMap* maps, const TcParams& p, int grid, size_t smem, cudaStream_t stream) {
   if (p.kps > 1 || p.b_resident != 0) return launch_epi<NAX, NBW, PAIR, kLoopGrouped + BOXES>(maps, p, grid, smem, stream);
+  if (p.ksteps_last != p.ksteps && p.fast_relu != 0 && p.BN == 128)
+    return launch_kernel<NAX, NBW, PAIR, kLoopPartial + kLoopBoxes, kEpiFast>(maps, p, grid, smem, stream);
   if (p.ksteps_last != p.ksteps) return launch_epi<NAX, NBW, PAIR, kLoopPartial + BOXES>(maps, p, grid, smem, stream);
   return launch_epi<NAX, NBW, PAIR, kLoopPlain + BOXES>(maps, p, grid, smem, stream);
 }
@@ -2578,6 +2585,9 @@ int launch_tensor(const GemmProblem& g) {
     cs.S = cs.W - OW + 2 * cs.pad_w + 1;        // (the filter width that gives OW)
   }
   if (!load_tensor_map_encoders()) return ADAPTION_ERR_CUDA;
+  const int fast = fast_epilogue(g, c, rq);
+  // (the kernels that know it)
+  c.own_rows = c.own_rows && (c.halo.w > 0 || (fast == 1 && c.kps == 1 && !c.b_resident && c.ksteps_last != c.BK / 32));
 
   // plane 0 is the high byte plane when there are two, else the single plane
   const void* xa[2] = {c.nax == 2 ? g.x.hi : g.x.lo, g.x.lo};
@@ -2707,7 +2717,6 @@ int launch_tensor(const GemmProblem& g) {
   // finalize kernel when the reduction is split
   p.st = g.stochastic;
   if (g.mode != ADAPTION_MODE_REQUANT || c.splits > 1) p.st.enabled = 0;
-  const int fast = fast_epilogue(g, c, rq);
   p.fast_relu = fast == 1 ? 1 : 0;
   p.fast_stochastic = fast == 2 ? 1 : 0;
   p.byte_out = p.fast_relu && c.nacc == 1 && c.staged && rq.shift >= 1 && rq.out_planes == 1 && rq.qmax == 127 ? 1 : 0;

@@ -34,6 +34,8 @@ CASES = [
     (2, 46, 32, 64, 61, 3, 1, 1, 16, 16, 16, True),        # channel count no multiple of 8: 64-bit epilogue
     (2, 32, 32, 96, 20, 3, 1, 1, 16, 8, 16, True),         # 32-column tiles, mixed widths
     (2, 34, 34, 64, 64, 3, 0, 1, 16, 16, 8, True),         # no padding, bytes from 16-bit operands
+    (2, 48, 32, 96, 32, 3, 1, 1, 16, 16, 16, True),        # partial blocks, warps that store their own rows
+    (17, 40, 40, 160, 64, 3, 1, 1, 16, 8, 16, True),       # ... of boxes with two images
     (64, 48, 48, 64, 64, 3, 1, 1, 8, 8, 8, True),          # many tiles per block
     (5, 64, 64, 64, 64, 3, 1, 1, 16, 16, 16, True),        # with one copy for all taps
     (5, 64, 64, 128, 128, 3, 1, 1, 8, 8, 8, True),
