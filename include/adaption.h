@@ -196,8 +196,10 @@ ADAPTION_API int adaption_lp_act(const float* d_x_f32, const adaption_qtensor* h
  * NULL) has bias_frac_bits <= x.fmt.frac_bits + w.fmt.frac_bits.  In RANGE mode y is ignored.
  * The workspace query returns the bytes the call needs (possibly 0); the workspace contents
  * need no initialisation.  (Layers with at most 4 input channels whose R*S*C taps fit 32 bytes,
- * e.g. the first 3x3 layer of an RGB network, gather their taps into packed planes there: 64 bytes
- * per output pixel.)  d_stats must not be NULL. */
+ * e.g. the first 3x3 layer of an RGB network, may gather their taps into packed planes there: 64 bytes
+ * per output pixel.  Those of stride 1, at most ten taps, operands of one width and at most 128 outputs over a
+ * pitch of 16 whose images fill boxes of 8 x 16 pixels are read where they are and leave the workspace untouched.)
+ * d_stats must not be NULL. */
 ADAPTION_API size_t adaption_lp_conv_workspace_bytes(const adaption_conv_shape* h_shape, adaption_qfmt fx,
                                         adaption_qfmt fw, int64_t c_stride, int32_t algo);
 ADAPTION_API int adaption_lp_conv_fwd(const adaption_conv_shape* h_shape, adaption_qtensor x,
@@ -236,7 +238,7 @@ ADAPTION_API int adaption_lp_ip_fwd_stochastic(int64_t B, int64_t K, int64_t O, 
  * lives in the workspace: where the tensor-core path can, only the maxima of horizontal pixel
  * pairs are stored there (half the bytes written and read back), otherwise all of it.  (Layers with
  * few output tiles, and those whose image sizes are covered by 128-pixel boxes, pool inside their kernel: y is
- * then written in the convolution's phase.)
+ * then written in the convolution's phase, unless it has an int16 copy, q16.)
  * phases: ADAPTION_PHASE_CONV | ADAPTION_PHASE_POOL runs the whole layer pair; the two phases may
  * also be issued by two calls with otherwise identical arguments (convolution first, same stream
  * order, workspace untouched in between), e.g. to time them apart.
@@ -329,6 +331,9 @@ ADAPTION_API int adaption_probe_i8_peak(int32_t bn, int32_t pair, int32_t iters,
  *   "cluster_size" 1|2|4|8, "cluster_bn" n   its cluster size and column width          (default 0: heuristic)
  *   "pixels" 0|2|4 convolutions over a pitch of 32 channels without grouped pixels / in groups of two / of at most
  *                  four whatever the number of tiles                                 (default 1: heuristic)
+ *   "box" 0        2x2 max-pools are not taken into the persistent kernel's epilogue as box tiles (default 1)
+ *   "halo" 0|2     activations are copied once per filter tap and first layers are packed / one copy serves all taps
+ *                  wherever it can, whatever the number of tiles                     (default 1: heuristic)
  *   "pdl" 0        layer kernels are launched without programmatic stream serialization (default 1)
  *   "timeout_us" t limit of every device-side wait in microseconds (default 0: two seconds)
  *   "stall_at" i   the copy-issuing warps of every block stop before their i-th stage with nothing

@@ -13,7 +13,8 @@
 // One persistent CTA per SM walks over output tiles (128 rows x BN columns):
 //   warps 0-2  : TMA producers, spread over the operand planes (im2col / tiled loads into a ring
 //                of shared-memory stages; a single warp issues bulk-tensor copies too slowly)
-//   warp  3    : MMA issue; also owns the TMEM allocation
+//   warp  3    : MMA issue; also owns the TMEM allocation (with one product a step and one copy for all taps
+//                warp 2 issues every other tile's MMAs, and two warps copy: kIssuers)
 //   warps 4-19 : epilogue (tcgen05.ld -> 64-bit recombination -> bias, ReLU, requantize with
 //                saturation, zero / saturation counters; byte planes staged in shared memory and
 //                written by bulk-tensor stores; or range / split-K)
@@ -41,7 +42,8 @@ constexpr int kMaxStages = 12;
 constexpr int kMaxAccBufs = 4;
 constexpr int kEpiWarps = 16;                // four per TMEM lane quarter, each takes a quarter of the columns
 constexpr int kProducerWarps = 3;            // spread over the operand planes: TMA issue is slow per warp
-// One MMA-issuing warp (a second one, alternating stages, measured no faster).
+// One MMA-issuing warp of its own (a second one, alternating stages of a tile, measured no faster; see kIssuers for the loops
+// in which a copying warp issues every other tile).
 constexpr int kMmaWarps = 1;
 constexpr int kMmaWarp = kProducerWarps;
 constexpr int kFirstEpiWarp = kProducerWarps + kMmaWarps;
@@ -932,8 +934,8 @@ lp_gemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
       int s = 0, turn = 0;                     // turn: s modulo nsub
       bool ok = true;
       if (b_res && warp == kCopyWarps - 1) {
-        // the whole weight matrix of this (single) column tile, one copy per k-block and plane,
-        // all reporting to one barrier
+        // the whole weight matrix (of the single column tile, or of both that kLoopHalo may have), one copy per
+        // k-block and plane, all reporting to one barrier
         // (in a pair each CTA fetches its own half of the weight rows; the bytes of both are counted
         // on the leader's barrier, which the leader arms for both)
         if (TAPS) {

@@ -471,7 +471,8 @@ __device__ __forceinline__ void quantize_padded_chunk(const QuantItem& it, const
 }
 
 // With a generator three blocks per SM for a single tensor, registers for more independent chains: 268 M elements 345 us with
-// four, 331 with three; a batch 83.6 and 91.
+// four, 331 with three; 2 to 4 % from 2 M elements on, dense or rows of 13 to 1000 in their pitch, equal below (rows of 3: 0.5 %
+// slower); a batch 83.6 and 91.
 template <bool STOCH, bool PADDED, int CAP>
 __global__ void __launch_bounds__(kQThreads, STOCH ? (CAP == 1 ? 3 : 4) : (PADDED ? 6 : 5)) quantize_kernel(const __grid_constant__ QuantArgs<CAP> a) {
   constexpr int kFlat = 2 * (kFlatBytes + 16);
