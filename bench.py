@@ -697,7 +697,7 @@ def run_kernel(args):
         return B.adaption_choose_frac_bits_from_acc(int(s.max_abs_acc), fx + fw, a.n_bits)
 
     if a.kernel == "conv":
-        cs = B.pad_to(a.C, 32)
+        cs = B.pad_to(a.C, 16 if a.C <= 4 else 32)         # (the network input keeps the smallest pitch)
         x = torch.randn(a.N * a.H * a.H, a.C, device="cuda", generator=g).clamp_(min=0)
         w = torch.randn(a.K * a.R * a.R, a.C, device="cuda", generator=g) * math.sqrt(2.0 / (a.R * a.R * a.C))
         xq, wq = quantized(x, a.N * a.H * a.H, a.C, cs), quantized(w, a.K * a.R * a.R, a.C, cs)
